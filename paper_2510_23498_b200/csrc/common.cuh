@@ -114,9 +114,13 @@ struct GemmArgs {
     //   2 (with EPI_DGRAD): the accumulators are hbar (primal) and gbar (tangent); with s = act'(H) from hprev and U from uprev
     //     (both [m_split, N], leading dimension ldh): out = Q16(s hbar + s (1 - s) U gbar), out2 = Q16(s gbar), non-finite flagged.
     int cnf_pair; void* pair_out; const void* uprev;
+    // EPI_WGRAD on the plain CUDA-core kernel: the row sums of A (bias gradient), row_sum[m] = beta row_sum[m] + sum; scaled by tau
+    // into row_sum_time[m * ldo] (the appended time column); and the bare sums into row_sum_raw[m].  Each may be null.
+    float *row_sum, *row_sum_time, *row_sum_raw;
 };
 
-void launch_gemm_simt(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* launches);
+// returns whether the plain-operand kernel ran (the one that takes GemmArgs::row_sum)
+bool launch_gemm_simt(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* launches);
 
 // ---------------------------------------------------------------- elementwise / reduction kernels
 struct Terms {                      // up to 4 low-format arrays with fp32 coefficients

@@ -10,12 +10,13 @@ namespace mpode {
 thread_local Profiler* tl_profiler = nullptr;
 thread_local PathCounters* tl_counters = nullptr;
 
-// returns which kernel ran: 0 the CUDA-core kernel, 1 the general tensor-core kernel, 2 the 64-channel convolution kernel
+// returns which kernel ran: 0 the general CUDA-core kernel, 1 the general tensor-core kernel, 2 the 64-channel convolution kernel,
+// 3 the CUDA-core kernel of plain operands (which also took GemmArgs::row_sum)
 int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* L) {
     Profiler* pr = tl_profiler;
     int klass = g.epi == EPI_FWD ? 0 : (g.epi == EPI_WGRAD ? 2 : 1);
     if (pr && pr->enabled) pr->begin(klass, 2.0 * g.M * g.N * (double)g.K, st);
-    bool done = false, halo = false;
+    bool done = false, halo = false, dense = false;
     if (g.epi == EPI_WGRAD) done = wgrad_tc_eligible(dt, g) && launch_wgrad_tc(dt, g, st, L);
     else {
         done = halo = conv_halo_eligible(dt, g) && launch_conv_halo(dt, g, st, L);
@@ -25,10 +26,10 @@ int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long 
     if (!done) {
         GemmArgs s = g;
         if (s.epi == EPI_WGRAD && s.split_k <= 1) s.partial = nullptr;
-        launch_gemm_simt(dt, s, st, L);
+        dense = launch_gemm_simt(dt, s, st, L);
     }
     if (pr && pr->enabled) pr->end(st);
-    return halo ? 2 : (done ? 1 : 0);
+    return halo ? 2 : (done ? 1 : (dense ? 3 : 0));
 }
 
 }  // namespace mpode

@@ -204,6 +204,7 @@ public:
         for (int l = L_ - 1; l >= 0; --l) {
             const void* X = (l == 0) ? yin : at(ws, H_[j][l]);
             int in_full = w_[l] + ((time_ && l == 0) ? 1 : 0);
+            bool sums_done;
             {   // weight gradient: dW_l[n, k] (+)= sum_m dZ[m, n] X[m, k]
                 GemmArgs g = base_args(ws, lay_);
                 g.A = dZ; g.a_rs = 1; g.a_ks = w_[l + 1];
@@ -211,10 +212,15 @@ public:
                 g.M = w_[l + 1]; g.N = w_[l]; g.K = B_;
                 g.epi = EPI_WGRAD; g.out = dg + woff_[l]; g.ldo = in_full; g.beta = beta;
                 g.partial = wgrad_tc_scratch_bytes(g.M, g.N, g.K) <= wgpart_bytes_ ? (float*)at(ws, wgpart_) : nullptr;
-                launch_contraction(dt_, g, st, L);
+                // the CUDA-core kernel takes the bias and time-column gradients (row sums of the same operand) along
+                g.row_sum = bias_ ? dg + boff_[l] : nullptr;
+                g.row_sum_time = (time_ && l == 0) ? dg + woff_[l] + w_[l] : nullptr;
+                g.tau = tau16;
+                g.row_sum_raw = (float*)at(ws, colsum_);
+                sums_done = launch_contraction(dt_, g, st, L) == 3;
             }
             if (bias_ || (time_ && l == 0)) {
-                const int R = launch_colsum(dt_, dZ, B_, w_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
+                const int R = sums_done ? 1 : launch_colsum(dt_, dZ, B_, w_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
                                             (time_ && l == 0) ? dg + woff_[l] + w_[l] : nullptr, in_full, tau16, beta, st, L, colsum_counters(ws, lay_));
                 if (lay_->time_gradient && time_ && l == 0) {      // d tau_j = w_t . colsum(dZ_1)
                     StageTimeArgs ta{};

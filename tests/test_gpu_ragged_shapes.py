@@ -1,0 +1,17 @@
+"""GPU parity at sizes where tiles, slices and padded rows end: just inside, on and just past their edges."""
+import pytest
+
+from paper_2510_23498_b200 import inputs
+from _harness import TOL, assert_parity, run_gpu, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+# CUDA-core contractions: 64 x 64 tiles, reduction chunks of 32, clusters of 1, 2, 4 and 8 reduction slices, vector and scalar loads.
+# Tolerance: the float32 mode's 1e-5 against the exact fp64 solution (sums of at most 1025 terms, 1025 * 2^-24 = 6e-5 at worst, 1e-6 typical).
+@pytest.mark.parametrize("batch,d,hidden", [(1, 8, 16), (63, 8, 65), (64, 12, 64), (65, 5, 33), (300, 33, 130), (1025, 24, 64)])
+def test_float32_mlp_at_tile_edges(batch, d, hidden):
+    wl = inputs.mlp_block(batch=batch, n_steps=2, d=d, hidden=hidden, low="f32")
+    gpu = run_gpu(wl, low="f32")
+    assert_parity(gpu, run_oracle(wl, exact=True), TOL["f32"])
+    assert gpu["stats"]["tc_contractions"] == 0 and gpu["stats"]["simt_contractions"] > 0
