@@ -95,6 +95,7 @@ struct GemmArgs {
     const float* conv_tbias;
     int epi;
     void* out; long long ldo;
+    int crop_m, crop_n;             // EPI_WGRAD: only the first crop_m x crop_n entries are written (0 = all; the rest belongs to padding)
     void* out2; int m_split;        // rows >= m_split are written to out2 (row m - m_split) without bias/activation
     const void* bias;               // low format [N] or null
     const void* wt; float tau;      // time column of the first layer, low format [N] or null
@@ -129,8 +130,9 @@ struct Terms {                      // up to 4 low-format arrays with fp32 coeff
     int n;
 };
 
+// dst [rows_p][cols_p] and dst_t [cols_p][rows_p] may be larger than the source (0 = as large): zero beyond it
 void launch_quantize_matrix(mpode_dtype dt, const float* src, long long src_ld, int rows, int cols, void* dst,
-                            void* dst_t, cudaStream_t st, long long* launches);
+                            void* dst_t, cudaStream_t st, long long* launches, int rows_p = 0, int cols_p = 0);
 void launch_quantize_conv_weights(mpode_dtype dt, const float* src, int cout, int cin_total, int cin_keep, void* dst,
                                   void* dst_flip_t, cudaStream_t st, long long* launches, float sign = 1.f);
 // Instance normalisation of an NHWC tensor [B][HW][C] per (image, channel) plane (Sec. 6.3): Z = Q16((S - mean) rstd), and its
@@ -180,9 +182,11 @@ void launch_conv_class_bias(mpode_dtype dt, const void* b, const void* w, int ci
                             cudaStream_t st, long long* launches);
 void launch_init_state(mpode_dtype dt, const float* y0, float* y, void* traj0, int B, int d, int D, cudaStream_t st,
                        long long* launches);
-void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* out, long long n, cudaStream_t st,
+// `ds` in the launches below: row length of the internal state buffers (k, Y, v, kappa, psi), >= d, zero columns behind d; base and
+// traj have rows of d, y and a rows of D
+void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* out, int B, int d, int ds, cudaStream_t st,
                         long long* launches);
-void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_next, int B, int d, int D,
+void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_next, int B, int d, int ds, int D,
                           int round_increment, float h, cudaStream_t st, long long* launches);
 void launch_column_combine(mpode_dtype dt, float* y, int D, int col, const Terms& t, int B, int round_increment,
                            float h, cudaStream_t st, long long* launches);
@@ -190,13 +194,13 @@ void launch_copy_amax(const float* src, float* dst, long long n, float* amax, un
                       long long* launches);
 // v = Q16(2^e a); optionally also kappa_last = Q16(b_last * v), the cotangent of the last stage.  With `e_dev` the exponent is
 // read from the device (dynamic scaling); the commits below then take coef = h and apply 2^-e themselves.
-void launch_seed(mpode_dtype dt, const float* a, int e, void* v, void* v_l, int B, int d, int D, unsigned* flag,
+void launch_seed(mpode_dtype dt, const float* a, int e, void* v, void* v_l, int B, int d, int ds, int D, unsigned* flag,
                  cudaStream_t st, long long* launches, void* kappa_last = nullptr, float b_last = 0.f, const int* e_dev = nullptr);
 void launch_kappa(mpode_dtype dt, const void* v, float bj, const Terms& t, void* out, long long n, unsigned* flag,
                   cudaStream_t st, long long* launches);
 // the commits do nothing when *skip_if_set != 0 (dynamic scaling: the attempt overflowed and will be repeated)
 // `add` (nullable, fp32 [B, D]): a running-cost cotangent w_i dR/dy_i added after the update (Alg. 2, adjoint update)
-void launch_commit_a(mpode_dtype dt, float* a, const Terms& psis, float coef, int B, int d, int D, float* amax,
+void launch_commit_a(mpode_dtype dt, float* a, const Terms& psis, float coef, int B, int d, int ds, int D, float* amax,
                      cudaStream_t st, long long* launches, const unsigned* skip_if_set = nullptr, const float* add = nullptr,
                      const int* e_dev = nullptr);
 
@@ -233,16 +237,16 @@ void launch_check_as_low(mpode_dtype dt, const float* x, long long n, unsigned* 
 void launch_fill(float* x, float v, long long n, cudaStream_t st, long long* launches);
 void launch_scale(float* x, float v, long long n, cudaStream_t st, long long* launches);      // x <- v * x
 void launch_fill_low(mpode_dtype dt, void* x, float v, long long n, cudaStream_t st, long long* launches);   // low-format array
-// column sums of a low-format [M, N] matrix, deterministic two-pass; dst1[n*s1] (+)= sum, dst2[n*s2] (+)= scale2*sum
+// column sums of a low-format [M, N] matrix (row length ld), deterministic two-pass; dst1[n*s1] (+)= sum, dst2[n*s2] (+)= scale2*sum
 // returns the number of partial rows it left in `partial` ([rows][N])
 constexpr int kColsumCounters = 32;   // column blocks a one-launch column sum can count (words of the caller's `counters`)
-int launch_colsum(mpode_dtype dt, const void* x, int M, int N, float* partial, float* dst1, long long s1, float* dst2,
+int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* partial, float* dst1, long long s1, float* dst2,
                   long long s2, float scale2, float beta, cudaStream_t st, long long* launches, unsigned* counters = nullptr);
 // column sums of a low-format [M, N] matrix per group of 128 rows (the layout the fused backward kernel also writes)
 void launch_colsum_groups(mpode_dtype dt, const void* x, int M, int N, float* out, cudaStream_t st, long long* launches);
 // out[m * ldo + n] = (beta ? out : 0) + sum_z partial[z][m][n], z in ascending order
 void launch_splitk_reduce(const float* partial, int S, int M, int N, float* out, long long ldo, float beta, cudaStream_t st,
-                          long long* launches);
+                          long long* launches, int crop_m = 0, int crop_n = 0);
 // One launch that turns the fused backward kernel's scratch into the step's parameter gradient, layer by layer:
 //   dW_l[m][n]  = sum over slices z (ascending) of partial[z][m][n]
 //   db_l[m]     = sum over stages j and batch slices r of colpart[col_off[j] + (r * M + m) * 8]    (bias_off >= 0)
@@ -250,7 +254,7 @@ void launch_splitk_reduce(const float* partial, int S, int M, int N, float* out,
 // and writes out[i] = (beta != 0 ? beta * out[i] : 0) + coef * value: either the step gradient itself (beta 0, coef 1)
 // or straight into the running gradient g <- g + (h / S) dg of Alg. 2 (beta 1, coef h / S).
 struct GradFinishLayer {
-    const float* partial; int splits, M, N;
+    const float* partial; int splits, M, N, Mp, Np;     // M x N entries kept of the Mp x Np slices
     long long w_off; int ldo;
     const float* colpart; long long col_off[4]; float tau[4]; int terms, rows;
     long long bias_off, time_off;
@@ -265,11 +269,11 @@ void launch_grad_finish(const GradFinishArgs& a, cudaStream_t st, long long* lau
 // CNF helpers (Sec. 6.1 joint state)
 void launch_cnf_tangent_act(mpode_dtype dt, int act, const void* H, const void* U, void* G, long long n,
                             cudaStream_t st, long long* launches);
-void launch_cnf_trace(mpode_dtype dt, const signed char* eps, const void* U, void* k_l, int B, int d, cudaStream_t st,
+void launch_cnf_trace(mpode_dtype dt, const signed char* eps, const void* U, void* k_l, int B, int d, int ds, cudaStream_t st,
                       long long* launches);
-void launch_cnf_probe_to_low(mpode_dtype dt, const signed char* eps, void* out, long long n, cudaStream_t st,
+void launch_cnf_probe_to_low(mpode_dtype dt, const signed char* eps, void* out, int B, int d, int ds, cudaStream_t st,
                              long long* launches);
-void launch_cnf_ubar_last(mpode_dtype dt, const void* kappa_l, const signed char* eps, void* ubar, int B, int d,
+void launch_cnf_ubar_last(mpode_dtype dt, const void* kappa_l, const signed char* eps, void* ubar, int B, int d, int ds,
                           unsigned* flag, cudaStream_t st, long long* launches);
 void launch_cnf_backprop_act(mpode_dtype dt, int act, const void* H, const void* U, const float* hbar,
                              const float* gbar, void* zeta, void* ubar, long long n, unsigned* flag, cudaStream_t st,

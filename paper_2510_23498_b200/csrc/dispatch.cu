@@ -26,6 +26,7 @@ int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long 
     if (!done) {
         GemmArgs s = g;
         if (s.epi == EPI_WGRAD && s.split_k <= 1) s.partial = nullptr;
+        if (s.crop_m > 0) { s.M = s.crop_m; s.N = s.crop_n; }
         dense = launch_gemm_simt(dt, s, st, L);
     }
     if (pr && pr->enabled) pr->end(st);

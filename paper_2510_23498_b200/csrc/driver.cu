@@ -162,7 +162,7 @@ void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes&
                     ++t.n;
                 }
             }
-            launch_stage_input(dt, traj_i, t, at(ws, c->lay.ybuf[j]), nBd, st, L);
+            launch_stage_input(dt, traj_i, t, at(ws, c->lay.ybuf[j]), c->B, c->d, c->lay.ds, st, L);
             yin = at(ws, c->lay.ybuf[j]);
         }
         c->v->forward(st, ws, j, yin, tm.tau16[j], L);
@@ -380,7 +380,7 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
             t.c[j] = c->pol.round_increment ? (float)c->tb[j] : (float)((double)tm.h * c->tb[j]);
         }
         char* traj_next = (char*)traj_dev + (size_t)(i + 1) * nBd * es;
-        launch_final_combine(dt, yT_dev, t, traj_next, c->B, c->d, c->D, c->pol.round_increment, tm.h, st, L);
+        launch_final_combine(dt, yT_dev, t, traj_next, c->B, c->d, c->lay.ds, c->D, c->pol.round_increment, tm.h, st, L);
         if (c->D > c->d) {
             for (int j = 0; j < c->stages; ++j) t.p[j] = at(ws, c->lay.klbuf[j]);
             launch_column_combine(dt, yT_dev, c->D, c->d, t, c->B, c->pol.round_increment, tm.h, st, L);
@@ -561,7 +561,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             DotPairs pr{};
             pr.n = s;
             for (int j = 0; j < s; ++j) {
-                pr.x[j] = at(ws, c->lay.kbuf[j]); pr.ldx[j] = c->d; pr.y[j] = a; pr.y_f32[j] = 1; pr.ldy[j] = c->D; pr.coef[j] = (float)c->tb[j];
+                pr.x[j] = at(ws, c->lay.kbuf[j]); pr.ldx[j] = c->lay.ds; pr.y[j] = a; pr.y_f32[j] = 1; pr.ldy[j] = c->D; pr.coef[j] = (float)c->tb[j];
             }
             launch_dot_partial(dt, pr, c->B, c->d, part_phi, st, L);
         }
@@ -577,7 +577,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             // velocities that write kappa_{j-1} from their own epilogues (state without extra columns) get kappa_s from the seed
             const bool kappa_in_vjp = !fused && c->D == c->d && c->v->can_write_next_kappa();
             const bool seeded_kappa = kappa_in_vjp;
-            launch_seed(dt, a, e, at(ws, c->lay.v), c->D > c->d ? at(ws, c->lay.vl) : nullptr, c->B, c->d, c->D,
+            launch_seed(dt, a, e, at(ws, c->lay.v), c->D > c->d ? at(ws, c->lay.vl) : nullptr, c->B, c->d, c->lay.ds, c->D,
                         vjp_flag, sr, L, fused ? c->v->fused_kappa_last(ws) : (seeded_kappa ? at(ws, c->v->kappa_offset(c->lay)) : nullptr),
                         (float)c->tb[s - 1], e_dev);                                             // seed Q16(S a)
             // without a finiteness decision the step gradient goes straight into g <- g + (h / S) dg
@@ -603,7 +603,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
                     }
                 }
                 void* kappa = at(ws, c->v->kappa_offset(c->lay));
-                if (!kappa_ready) launch_kappa(dt, at(ws, c->lay.v), (float)c->tb[j], t, kappa, nBd, vjp_flag, st, L);
+                if (!kappa_ready) launch_kappa(dt, at(ws, c->lay.v), (float)c->tb[j], t, kappa, (long long)c->B * c->lay.ds, vjp_flag, st, L);
                 // can this stage's vector-Jacobian product also write kappa_{j-1}?  Yes when the tableau couples stage j - 1 to
                 // stage j alone (a_lj = 0 for l > j: Euler, midpoint, RK4, ...)
                 kappa_ready = false;
@@ -630,7 +630,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
                     for (int l = 0; l < j; ++l)
                         if (c->ta[j * s + l] != 0.0 && pr.n < 8) {
                             const int q = pr.n++;
-                            pr.x[q] = at(ws, c->lay.psi[j]); pr.ldx[q] = c->d; pr.y[q] = at(ws, c->lay.kbuf[l]); pr.y_f32[q] = 0; pr.ldy[q] = c->d;
+                            pr.x[q] = at(ws, c->lay.psi[j]); pr.ldx[q] = c->lay.ds; pr.y[q] = at(ws, c->lay.kbuf[l]); pr.y_f32[q] = 0; pr.ldy[q] = c->lay.ds;
                             pr.coef[q] = (float)c->ta[j * s + l];
                         }
                 launch_dot_partial(dt, pr, c->B, c->d, part_dh, st, L);
@@ -648,7 +648,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             // behind them records the attempt (growth test on the new ||a||_inf) or the failure
             cudaMemsetAsync(amax, 0, 4, st);
             if (tg) launch_tgrad_update(tprime, i, tvals, tm.h, flag, st, L, e_dev);        // before a changes: it holds Phi^T a_{i+1} already
-            launch_commit_a(dt, a, ps, tm.h, c->B, c->d, c->D, amax, st, L, flag, cot_i, e_dev);
+            launch_commit_a(dt, a, ps, tm.h, c->B, c->d, c->lay.ds, c->D, amax, st, L, flag, cot_i, e_dev);
             launch_commit_g(g, dg, tm.h, p, st, L, flag, e_dev);
             launch_scale_decide(flag, amax, sstate, mirror, i, i == fail_step ? fail_count + 1 : 1, c->pol.growth_rule, precision_bits(dt),
                                 kExpMin, kExpMax, slog_exp, slog_att, slog_dbl, st, L);
@@ -676,7 +676,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         } else {
             float coef = (float)((double)tm.h * ldexp(1.0, -e));
             if (tg) launch_tgrad_update(tprime, i, tvals, coef, nullptr, st, L);
-            launch_commit_a(dt, a, ps, coef, c->B, c->d, c->D, nullptr, sr, L, nullptr, cot_i);
+            launch_commit_a(dt, a, ps, coef, c->B, c->d, c->lay.ds, c->D, nullptr, sr, L, nullptr, cot_i);
             if (!(fused && !checked)) launch_commit_g(g, dg, coef, p, st, L);
             if (log) { log->attempts[i] = 1; log->exp_used[i] = e; log->doubled[i] = 0; }
         }

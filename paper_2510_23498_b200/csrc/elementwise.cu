@@ -28,9 +28,9 @@ inline bool aligned_to(const void* p, size_t a) { return ((uintptr_t)p % a) == 0
     } while (0)
 
 // ---------------------------------------------------------------- theta -> Q16(theta) (Alg. 1, Alg. 2: weights in low precision)
-// src: fp32 [rows, src_ld] (only the first `cols` columns are taken); dst: low [rows, cols]; dst_t: low [cols, rows].
+// src: fp32 [rows, src_ld] (only the first `cols` columns are taken); dst: low [rp, cp]; dst_t: low [cp, rp], zero beyond [rows, cols].
 template <typename T>
-__global__ void quantize_matrix_kernel(const float* __restrict__ src, long long src_ld, int rows, int cols,
+__global__ void quantize_matrix_kernel(const float* __restrict__ src, long long src_ld, int rows, int cols, int rp, int cp,
                                        T* __restrict__ dst, T* __restrict__ dst_t) {
     __shared__ float tile[32][33];
     int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
@@ -38,13 +38,13 @@ __global__ void quantize_matrix_kernel(const float* __restrict__ src, long long 
         int r = r0 + i, c = c0 + threadIdx.x;
         float v = (r < rows && c < cols) ? src[(long long)r * src_ld + c] : 0.f;
         tile[i][threadIdx.x] = v;
-        if (dst != nullptr && r < rows && c < cols) dst[(long long)r * cols + c] = Low<T>::from_f(v);
+        if (dst != nullptr && r < rp && c < cp) dst[(long long)r * cp + c] = Low<T>::from_f(v);
     }
     __syncthreads();
     if (dst_t != nullptr) {
         for (int i = threadIdx.y; i < 32; i += blockDim.y) {
             int c = c0 + i, r = r0 + threadIdx.x;
-            if (r < rows && c < cols) dst_t[(long long)c * rows + r] = Low<T>::from_f(tile[threadIdx.x][i]);
+            if (r < rp && c < cp) dst_t[(long long)c * rp + r] = Low<T>::from_f(tile[threadIdx.x][i]);
         }
     }
 }
@@ -247,9 +247,24 @@ __global__ void stage_input_kernel(const T* __restrict__ base, Terms t, T* __res
     }
 }
 
+// the same with rows of `d` in and rows of `ds` out (k too), zero behind d
+template <typename T>
+__global__ void stage_input_rows_kernel(const T* __restrict__ base, Terms t, T* __restrict__ out, int B, int d, int ds) {
+    const long long n = (long long)B * ds;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const unsigned row = (unsigned)(i / ds), col = (unsigned)(i - (long long)row * ds);
+        float acc = 0.f;
+        if ((int)col < d) {
+            acc = Low<T>::to_f(base[(long long)row * d + col]);
+            for (int l = 0; l < t.n; ++l) acc = fmaf(t.c[l], Low<T>::to_f(((const T*)t.p[l])[i]), acc);
+        }
+        out[i] = Low<T>::from_f(acc);
+    }
+}
+
 // ---------------------------------------------------------------- Alg. 1 accumulate and store: y += h Phi (fp32), traj[i+1] = Q16(y)
 template <typename T, int V>
-__global__ void final_combine_kernel(float* __restrict__ y, Terms t, T* __restrict__ traj_next, int B, int d, int D,
+__global__ void final_combine_kernel(float* __restrict__ y, Terms t, T* __restrict__ traj_next, int B, int d, int ds, int D,
                                      int round_increment, float h) {
     int dv = d / V;
     long long nv = (long long)B * dv;
@@ -260,7 +275,7 @@ __global__ void final_combine_kernel(float* __restrict__ y, Terms t, T* __restri
 #pragma unroll
         for (int k = 0; k < V; ++k) acc[k] = 0.f;
         for (int l = 0; l < t.n; ++l) {
-            Pack<T, V> kk = *reinterpret_cast<const Pack<T, V>*>((const T*)t.p[l] + row * d + col);
+            Pack<T, V> kk = *reinterpret_cast<const Pack<T, V>*>((const T*)t.p[l] + row * ds + col);
 #pragma unroll
             for (int k = 0; k < V; ++k) acc[k] = fmaf(t.c[l], Low<T>::to_f(kk.v[k]), acc[k]);
         }
@@ -338,7 +353,7 @@ __global__ void copy_amax_kernel(const float* __restrict__ src, float* __restric
 
 // ---------------------------------------------------------------- Eq. (vjp) seed: v = Q16(S a), S = 2^e
 template <typename T, int V>
-__global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ v, T* __restrict__ v_l, int B, int d,
+__global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ v, T* __restrict__ v_l, int B, int d, int ds,
                             int D, unsigned* __restrict__ flag, T* __restrict__ kap, float bk, const int* __restrict__ e_dev) {
     if (e_dev != nullptr) e = *e_dev;               // the exponent lives on the device (dynamic scaling)
     int dv = d / V;
@@ -354,7 +369,7 @@ __global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ 
             q.v[k] = Low<T>::from_f(ldexpf(aa.v[k], e));
             bad |= Low<T>::nonfinite(q.v[k]);
         }
-        *reinterpret_cast<Pack<T, V>*>(v + row * d + col) = q;
+        *reinterpret_cast<Pack<T, V>*>(v + row * ds + col) = q;
         if (kap != nullptr) {   // cotangent of the last stage, kappa_s = Q16(b_s v), for the fused backward kernel
             Pack<T, V> kq;
 #pragma unroll
@@ -362,7 +377,16 @@ __global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ 
                 kq.v[k] = Low<T>::from_f(bk * Low<T>::to_f(q.v[k]));
                 bad |= Low<T>::nonfinite(kq.v[k]);
             }
-            *reinterpret_cast<Pack<T, V>*>(kap + row * d + col) = kq;
+            *reinterpret_cast<Pack<T, V>*>(kap + row * ds + col) = kq;
+        }
+    }
+    if (ds > d) {                                   // padded rows end in zeros
+        const int pad = ds - d;
+        const long long np = (long long)B * pad;
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x) {
+            const long long o = (i / pad) * ds + d + i % pad;
+            v[o] = Low<T>::from_f(0.f);
+            if (kap != nullptr) kap[o] = Low<T>::from_f(0.f);
         }
     }
     if (D > d) {
@@ -403,7 +427,7 @@ __global__ void kappa_kernel(const T* __restrict__ v, float bj, Terms t, T* __re
 
 // ---------------------------------------------------------------- Alg. 2 adjoint update: a <- a + (h / S) sum_j psi_j, and ||a||_inf
 template <typename T, int V>
-__global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, int B, int d, int D,
+__global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, int B, int d, int ds, int D,
                                 float* __restrict__ amax, const unsigned* __restrict__ skip_if_set, const float* __restrict__ add,
                                 const int* __restrict__ e_dev) {
     if (skip_if_set != nullptr && *skip_if_set != 0u) return;   // a non-finite attempt is not committed (it is repeated)
@@ -418,7 +442,7 @@ __global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, i
 #pragma unroll
         for (int k = 0; k < V; ++k) da[k] = 0.f;
         for (int l = 0; l < psis.n; ++l) {
-            Pack<T, V> pp = *reinterpret_cast<const Pack<T, V>*>((const T*)psis.p[l] + row * d + col);
+            Pack<T, V> pp = *reinterpret_cast<const Pack<T, V>*>((const T*)psis.p[l] + row * ds + col);
 #pragma unroll
             for (int k = 0; k < V; ++k) da[k] += Low<T>::to_f(pp.v[k]);
         }
@@ -534,7 +558,7 @@ constexpr int kRowLanes = 8;
 // With `counters` (one zero word per column block, left zero again) the block that finishes a column block last also adds the
 // partial rows in ascending order and writes the result as colsum_final_kernel would.
 template <typename T>
-__global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int rows_per_block,
+__global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int ld, int rows_per_block,
                                       float* __restrict__ partial, unsigned* __restrict__ counters, float* __restrict__ dst1,
                                       long long s1, float* __restrict__ dst2, long long s2, float scale2, float beta) {
     __shared__ float sm[kRowLanes][kColsPerBlock];
@@ -544,9 +568,18 @@ __global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int
     int r0 = blockIdx.y * rows_per_block;
     int r1 = min(M, r0 + rows_per_block);
     float a0 = 0.f, a1 = 0.f;
-    for (int r = r0 + rl; r < r1; r += kRowLanes) {
-        if (c < N) a0 += Low<T>::to_f(x[(long long)r * N + c]);
-        if (c + 1 < N) a1 += Low<T>::to_f(x[(long long)r * N + c + 1]);
+    if (sizeof(T) == 2 && (ld & 1) == 0 && ((uintptr_t)x & 3) == 0 && c + 1 < ld) {      // both columns in one load, four rows in flight
+#pragma unroll 4
+        for (int r = r0 + rl; r < r1; r += kRowLanes) {
+            const Pack<T, 2> v = *reinterpret_cast<const Pack<T, 2>*>(x + (long long)r * ld + c);
+            a0 += Low<T>::to_f(v.v[0]);
+            a1 += Low<T>::to_f(v.v[1]);
+        }
+    } else {
+        for (int r = r0 + rl; r < r1; r += kRowLanes) {
+            if (c < N) a0 += Low<T>::to_f(x[(long long)r * ld + c]);
+            if (c + 1 < N) a1 += Low<T>::to_f(x[(long long)r * ld + c + 1]);
+        }
     }
     sm[rl][lane * 2] = a0;
     sm[rl][lane * 2 + 1] = a1;
@@ -565,10 +598,19 @@ __global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const int cc = blockIdx.x * kColsPerBlock + threadIdx.x;
+    // four threads per column take every fourth partial row each, their sums are added in order
+    const int cc = blockIdx.x * kColsPerBlock + (threadIdx.x & (kColsPerBlock - 1)), pr = threadIdx.x / kColsPerBlock;
+    float t = 0.f;
+    if (cc < N) {
+#pragma unroll 8
+        for (int r = pr; r < (int)gridDim.y; r += kThreads / kColsPerBlock) t += __ldcg(partial + (long long)r * N + cc);
+    }
+    sm[pr][threadIdx.x & (kColsPerBlock - 1)] = t;
+    __syncthreads();
     if (threadIdx.x < kColsPerBlock && cc < N) {
         float s = 0.f;
-        for (int r = 0; r < (int)gridDim.y; ++r) s += __ldcg(partial + (long long)r * N + cc);
+#pragma unroll
+        for (int i = 0; i < kThreads / kColsPerBlock; ++i) s += sm[i][threadIdx.x];
         if (dst1 != nullptr) dst1[cc * s1] = (beta != 0.f ? dst1[cc * s1] : 0.f) + s;
         if (dst2 != nullptr) dst2[cc * s2] = (beta != 0.f ? dst2[cc * s2] : 0.f) + scale2 * s;
     }
@@ -605,11 +647,12 @@ __global__ void grad_finish_kernel(GradFinishArgs a) {
     const GradFinishLayer& L = a.layer[blockIdx.y];
     const int wblocks = (int)gridDim.x - kFinishBiasBlocks;
     if ((int)blockIdx.x < wblocks) {
-        const long long n_el = (long long)L.M * L.N;
+        const long long n_el = (long long)L.Mp * L.Np;
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_el; i += (long long)wblocks * blockDim.x) {
+            if (i / L.Np >= L.M || i % L.Np >= L.N) continue;
             float s = 0.f;
             for (int z = 0; z < L.splits; ++z) s += L.partial[(long long)z * n_el + i];
-            float* o = a.out + L.w_off + (i / L.N) * L.ldo + (i % L.N);
+            float* o = a.out + L.w_off + (i / L.Np) * L.ldo + (i % L.Np);
             *o = (a.beta != 0.f ? a.beta * *o : 0.f) + a.coef * s;
         }
     } else if (L.bias_off >= 0 || L.time_off >= 0) {
@@ -620,7 +663,7 @@ __global__ void grad_finish_kernel(GradFinishArgs a) {
             float sb = 0.f, stime = 0.f;
             for (int t = lane; t < terms; t += 32) {
                 const int j = t / L.rows, r = t - j * L.rows;      // stage j, batch slice r: column 0 of the stored ones-product
-                const float v = L.colpart[L.col_off[j] + ((long long)r * L.M + m) * 8];
+                const float v = L.colpart[L.col_off[j] + ((long long)r * L.Mp + m) * 8];
                 sb += v;
                 stime = fmaf(L.tau[j], v, stime);
             }
@@ -911,13 +954,13 @@ __global__ void cnf_tangent_act_kernel(int act, const T* __restrict__ H, const T
 // k_l[b] = Q16(-sum_n eps[b, n] U[b, n]); one warp per sample
 template <typename T>
 __global__ void cnf_trace_kernel(const signed char* __restrict__ eps, const T* __restrict__ U, T* __restrict__ k_l,
-                                 int B, int d) {
+                                 int B, int d, int ds) {
     int warps_per_block = blockDim.x >> 5;
     int lane = threadIdx.x & 31;
     for (long long b = blockIdx.x * (long long)warps_per_block + (threadIdx.x >> 5); b < B;
          b += (long long)gridDim.x * warps_per_block) {
         float s = 0.f;
-        for (int n = lane; n < d; n += 32) s += (float)eps[b * d + n] * Low<T>::to_f(U[b * d + n]);
+        for (int n = lane; n < d; n += 32) s += (float)eps[b * d + n] * Low<T>::to_f(U[b * ds + n]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) k_l[b] = Low<T>::from_f(-s);
@@ -925,21 +968,28 @@ __global__ void cnf_trace_kernel(const signed char* __restrict__ eps, const T* _
 }
 
 template <typename T>
-__global__ void cnf_probe_to_low_kernel(const signed char* __restrict__ eps, T* __restrict__ out, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = Low<T>::from_f((float)eps[i]);
+__global__ void cnf_probe_to_low_kernel(const signed char* __restrict__ eps, T* __restrict__ out, int B, int d, int ds) {
+    const long long n = (long long)B * ds;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const long long row = i / ds, col = i - row * ds;
+        out[i] = Low<T>::from_f(col < d ? (float)eps[row * d + col] : 0.f);
+    }
 }
 
-// cotangent of the last tangent output: ubar[b, n] = Q16(-kappa_l[b] * eps[b, n])
+// cotangent of the last tangent output: ubar[b, n] = Q16(-kappa_l[b] * eps[b, n]), rows of ds with zeros behind d
 template <typename T>
 __global__ void cnf_ubar_last_kernel(const T* __restrict__ kappa_l, const signed char* __restrict__ eps,
-                                     T* __restrict__ ubar, int B, int d, unsigned* __restrict__ flag) {
-    long long n = (long long)B * d;
+                                     T* __restrict__ ubar, int B, int d, int ds, unsigned* __restrict__ flag) {
     bool bad = false;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        T q = Low<T>::from_f(-Low<T>::to_f(kappa_l[i / d]) * (float)eps[i]);
-        bad |= Low<T>::nonfinite(q);
-        ubar[i] = q;
+    for (int row = blockIdx.x; row < B; row += gridDim.x) {
+        const float k = Low<T>::to_f(kappa_l[row]);
+        const signed char* er = eps + (long long)row * d;
+        T* ur = ubar + (long long)row * ds;
+        for (int col = threadIdx.x; col < ds; col += blockDim.x) {
+            const T q = Low<T>::from_f(col < d ? -k * (float)er[col] : 0.f);
+            bad |= Low<T>::nonfinite(q);
+            ur[col] = q;
+        }
     }
     warp_flag_or(flag, bad);
 }
@@ -970,9 +1020,10 @@ __global__ void cnf_backprop_act_kernel(int act, const T* __restrict__ H, const 
 #define COUNT(l) do { if (l) ++*(l); } while (0)
 
 void launch_quantize_matrix(mpode_dtype dt, const float* src, long long src_ld, int rows, int cols, void* dst,
-                            void* dst_t, cudaStream_t st, long long* launches) {
-    dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
-    MPODE_DISPATCH_T(dt, T, (quantize_matrix_kernel<T><<<grid, block, 0, st>>>(src, src_ld, rows, cols, (T*)dst, (T*)dst_t)));
+                            void* dst_t, cudaStream_t st, long long* launches, int rows_p, int cols_p) {
+    const int rp = rows_p > rows ? rows_p : rows, cp = cols_p > cols ? cols_p : cols;
+    dim3 grid((cp + 31) / 32, (rp + 31) / 32), block(32, 8);
+    MPODE_DISPATCH_T(dt, T, (quantize_matrix_kernel<T><<<grid, block, 0, st>>>(src, src_ld, rows, cols, rp, cp, (T*)dst, (T*)dst_t)));
     COUNT(launches);
 }
 
@@ -1054,8 +1105,14 @@ void launch_init_state(mpode_dtype dt, const float* y0, float* y, void* traj0, i
     COUNT(launches);
 }
 
-void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* out, long long n, cudaStream_t st,
+void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* out, int B, int d, int ds, cudaStream_t st,
                         long long* launches) {
+    const long long n = (long long)B * ds;
+    if (ds != d) {
+        MPODE_DISPATCH_T(dt, T, (stage_input_rows_kernel<T><<<grid_for(n), kThreads, 0, st>>>((const T*)base, t, (T*)out, B, d, ds)));
+        COUNT(launches);
+        return;
+    }
     bool v8 = (n % 8 == 0) && aligned_to(base, 32) && aligned_to(out, 32);
     for (int l = 0; l < t.n; ++l) v8 = v8 && aligned_to(t.p[l], 32);
     if (v8 && n % 16 == 0 && dt != MPODE_F32) {   // 32 bytes per operand and thread in flight: needed to fill the memory pipe
@@ -1068,7 +1125,7 @@ void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* 
     COUNT(launches);
 }
 
-void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_next, int B, int d, int D,
+void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_next, int B, int d, int ds, int D,
                           int round_increment, float h, cudaStream_t st, long long* launches) {
     bool v8 = vec8_ok(d, D, {y, traj_next});
     for (int l = 0; l < t.n; ++l) v8 = v8 && aligned_to(t.p[l], 32);
@@ -1076,13 +1133,13 @@ void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_n
     for (int l = 0; l < t.n; ++l) v16 = v16 && aligned_to(t.p[l], 64);
     if (v16) {
         MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, D, round_increment, h)));
+                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     } else if (v8) {
         MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, D, round_increment, h)));
+                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     } else {
         MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, D, round_increment, h)));
+                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     }
     COUNT(launches);
 }
@@ -1099,16 +1156,16 @@ void launch_copy_amax(const float* src, float* dst, long long n, float* amax, un
     COUNT(launches);
 }
 
-void launch_seed(mpode_dtype dt, const float* a, int e, void* v, void* v_l, int B, int d, int D, unsigned* flag,
+void launch_seed(mpode_dtype dt, const float* a, int e, void* v, void* v_l, int B, int d, int ds, int D, unsigned* flag,
                  cudaStream_t st, long long* launches, void* kappa_last, float b_last, const int* e_dev) {
     if (vec16_ok(dt, d, D, {a, v, kappa_last})) {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, D, flag,
+        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                         (T*)kappa_last, b_last, e_dev)));
     } else if (vec8_ok(d, D, {a, v, kappa_last})) {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, D, flag,
+        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                       (T*)kappa_last, b_last, e_dev)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, D, flag,
+        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                   (T*)kappa_last, b_last, e_dev)));
     }
     COUNT(launches);
@@ -1128,18 +1185,18 @@ void launch_kappa(mpode_dtype dt, const void* v, float bj, const Terms& t, void*
     COUNT(launches);
 }
 
-void launch_commit_a(mpode_dtype dt, float* a, const Terms& psis, float coef, int B, int d, int D, float* amax,
+void launch_commit_a(mpode_dtype dt, float* a, const Terms& psis, float coef, int B, int d, int ds, int D, float* amax,
                      cudaStream_t st, long long* launches, const unsigned* skip_if_set, const float* add, const int* e_dev) {
     bool v8 = vec8_ok(d, D, {a, add});
     for (int l = 0; l < psis.n; ++l) v8 = v8 && aligned_to(psis.p[l], 32);
     bool v16 = v8 && vec16_ok(dt, d, D, {a, add});
     for (int l = 0; l < psis.n; ++l) v16 = v16 && aligned_to(psis.p[l], 64);
     if (v16) {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, psis, coef, B, d, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     } else if (v8) {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, psis, coef, B, d, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, psis, coef, B, d, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     }
     COUNT(launches);
 }
@@ -1235,7 +1292,7 @@ void launch_tgrad_update(float* tprime, int i, const float* vals, float coef, co
     COUNT(launches);
 }
 
-int launch_colsum(mpode_dtype dt, const void* x, int M, int N, float* partial, float* dst1, long long s1, float* dst2,
+int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* partial, float* dst1, long long s1, float* dst2,
                   long long s2, float scale2, float beta, cudaStream_t st, long long* launches, unsigned* counters) {
     // row chunks: enough blocks to fill the GPU, at most 64 partial rows (the scratch holds 64 * N floats)
     int col_blocks = (N + kColsPerBlock - 1) / kColsPerBlock;
@@ -1248,7 +1305,7 @@ int launch_colsum(mpode_dtype dt, const void* x, int M, int N, float* partial, f
     R = (M + rows_per_block - 1) / rows_per_block;
     dim3 grid(col_blocks, R);
     if (counters != nullptr && col_blocks > kColsumCounters) counters = nullptr;
-    MPODE_DISPATCH_T(dt, T, (colsum_partial_kernel<T><<<grid, kThreads, 0, st>>>((const T*)x, M, N, rows_per_block, partial, counters, dst1, s1, dst2,
+    MPODE_DISPATCH_T(dt, T, (colsum_partial_kernel<T><<<grid, kThreads, 0, st>>>((const T*)x, M, N, ld, rows_per_block, partial, counters, dst1, s1, dst2,
                                                                                    s2, scale2, beta)));
     COUNT(launches);
     if (counters == nullptr) {
@@ -1276,24 +1333,24 @@ void launch_cnf_tangent_act(mpode_dtype dt, int act, const void* H, const void* 
     COUNT(launches);
 }
 
-void launch_cnf_trace(mpode_dtype dt, const signed char* eps, const void* U, void* k_l, int B, int d, cudaStream_t st,
+void launch_cnf_trace(mpode_dtype dt, const signed char* eps, const void* U, void* k_l, int B, int d, int ds, cudaStream_t st,
                       long long* launches) {
     int blocks = (B + 7) / 8;
     if (blocks > kSMs * 8) blocks = kSMs * 8;
-    MPODE_DISPATCH_T(dt, T, (cnf_trace_kernel<T><<<blocks, kThreads, 0, st>>>(eps, (const T*)U, (T*)k_l, B, d)));
+    MPODE_DISPATCH_T(dt, T, (cnf_trace_kernel<T><<<blocks, kThreads, 0, st>>>(eps, (const T*)U, (T*)k_l, B, d, ds)));
     COUNT(launches);
 }
 
-void launch_cnf_probe_to_low(mpode_dtype dt, const signed char* eps, void* out, long long n, cudaStream_t st,
+void launch_cnf_probe_to_low(mpode_dtype dt, const signed char* eps, void* out, int B, int d, int ds, cudaStream_t st,
                              long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_probe_to_low_kernel<T><<<grid_for(n), kThreads, 0, st>>>(eps, (T*)out, n)));
+    MPODE_DISPATCH_T(dt, T, (cnf_probe_to_low_kernel<T><<<grid_for((long long)B * ds), kThreads, 0, st>>>(eps, (T*)out, B, d, ds)));
     COUNT(launches);
 }
 
-void launch_cnf_ubar_last(mpode_dtype dt, const void* kappa_l, const signed char* eps, void* ubar, int B, int d,
+void launch_cnf_ubar_last(mpode_dtype dt, const void* kappa_l, const signed char* eps, void* ubar, int B, int d, int ds,
                           unsigned* flag, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_ubar_last_kernel<T><<<grid_for((long long)B * d), kThreads, 0, st>>>(
-                                (const T*)kappa_l, eps, (T*)ubar, B, d, flag)));
+    MPODE_DISPATCH_T(dt, T, (cnf_ubar_last_kernel<T><<<B < kSMs * 8 ? B : kSMs * 8, kThreads, 0, st>>>(
+                                (const T*)kappa_l, eps, (T*)ubar, B, d, ds, flag)));
     COUNT(launches);
 }
 

@@ -314,9 +314,10 @@ bool launch_dense(const GemmArgs& g, cudaStream_t st) {
 }
 
 __global__ void splitk_reduce_kernel(const float* __restrict__ partial, int S, int M, int N, float* __restrict__ out,
-                                     long long ldo, float beta) {
+                                     long long ldo, float beta, int keep_m, int keep_n) {
     long long n_el = (long long)M * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_el; i += (long long)gridDim.x * blockDim.x) {
+        if (i / N >= keep_m || i % N >= keep_n) continue;
         float s = 0.f;
         for (int z = 0; z < S; ++z) s += partial[(long long)z * n_el + i];
         float* o = out + (i / N) * ldo + (i % N);
@@ -324,45 +325,57 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ partial, int S, i
     }
 }
 
-// The same four columns at a time (N, ldo multiples of 4, 16-byte aligned pointers, fewer than 2^31 elements): the slices are
-// still added in ascending order per element
-__global__ void splitk_reduce4_kernel(const float4* __restrict__ partial, int S, unsigned n4, unsigned N4, float* __restrict__ out,
-                                      long long ldo, float beta) {
+// The same four columns at a time (N a multiple of 4, fewer than 2^31 elements): the slices are still added in ascending order per
+// element.  VEC: the destination rows are 16-byte aligned too; otherwise (a row with an appended column, cropped padding) its four
+// elements are written one by one.
+template <bool VEC>
+__global__ void splitk_reduce4_kernel(const float4* __restrict__ partial, int S, unsigned slice4, unsigned n4, unsigned N4, float* __restrict__ out,
+                                      long long ldo, float beta, unsigned keep_n) {
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {
         float4 s = partial[i];
         for (int z = 1; z < S; ++z) {
-            const float4 v = partial[(size_t)z * n4 + i];
+            const float4 v = partial[(size_t)z * slice4 + i];
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
-        const unsigned row = i / N4, col = i - row * N4;
-        float4* o = reinterpret_cast<float4*>(out + (long long)row * ldo) + col;
-        if (beta != 0.f) {
-            const float4 old = *o;
-            s.x += old.x; s.y += old.y; s.z += old.z; s.w += old.w;
+        const unsigned row = i / N4, col = 4 * (i - row * N4);
+        float* o = out + (long long)row * ldo + col;
+        if (VEC) {
+            if (beta != 0.f) {
+                const float4 old = *reinterpret_cast<const float4*>(o);
+                s.x += old.x; s.y += old.y; s.z += old.z; s.w += old.w;
+            }
+            *reinterpret_cast<float4*>(o) = s;
+        } else {
+            const float v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (col + e < keep_n) o[e] = (beta != 0.f ? o[e] : 0.f) + v[e];
         }
-        *o = s;
     }
 }
 
-void reduce_slices(const float* partial, int S, int M, int N, float* out, long long ldo, float beta, cudaStream_t st) {
+void reduce_slices(const float* partial, int S, int M, int N, float* out, long long ldo, float beta, cudaStream_t st, int crop_m = 0, int crop_n = 0) {
+    const int keep_m = crop_m > 0 ? crop_m : M, keep_n = crop_n > 0 ? crop_n : N;
     const long long n_el = (long long)M * N;
-    if (N % 4 == 0 && ldo % 4 == 0 && n_el < 0x7fffffffLL && ((((uintptr_t)partial) | ((uintptr_t)out)) & 15) == 0 && S >= 1) {
-        const unsigned n4 = (unsigned)(n_el / 4);
+    if (N % 4 == 0 && n_el < 0x7fffffffLL && ((uintptr_t)partial & 15) == 0 && S >= 1) {
+        const unsigned N4 = (unsigned)(N / 4), n4 = (unsigned)keep_m * N4, slice4 = (unsigned)(n_el / 4);
         int blocks = (int)((n4 + 255) / 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
-        splitk_reduce4_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(partial), S, n4, (unsigned)(N / 4), out, ldo, beta);
+        const float4* p4 = reinterpret_cast<const float4*>(partial);
+        if (keep_n == N && ldo % 4 == 0 && ((uintptr_t)out & 15) == 0) splitk_reduce4_kernel<true><<<blocks, 256, 0, st>>>(p4, S, slice4, n4, N4, out, ldo, beta, N);
+        else splitk_reduce4_kernel<false><<<blocks, 256, 0, st>>>(p4, S, slice4, n4, N4, out, ldo, beta, keep_n);
         return;
     }
     int blocks = (int)((n_el + 255) / 256);
     if (blocks > 148 * 8) blocks = 148 * 8;
-    splitk_reduce_kernel<<<blocks, 256, 0, st>>>(partial, S, M, N, out, ldo, beta);
+    splitk_reduce_kernel<<<blocks, 256, 0, st>>>(partial, S, M, N, out, ldo, beta, keep_m, keep_n);
 }
 
 }  // namespace
 
 void launch_splitk_reduce(const float* partial, int S, int M, int N, float* out, long long ldo, float beta, cudaStream_t st,
-                          long long* launches) {
-    reduce_slices(partial, S, M, N, out, ldo, beta, st);
+                          long long* launches, int crop_m, int crop_n) {
+    reduce_slices(partial, S, M, N, out, ldo, beta, st, crop_m, crop_n);
     if (launches) ++*launches;
 }
 

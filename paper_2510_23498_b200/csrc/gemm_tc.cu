@@ -473,7 +473,7 @@ bool tc_eligible(mpode_dtype dt, const GemmArgs& g) {
     if (g.K % 8 != 0 || g.N % 8 != 0 || g.a_rs % 8 != 0 || g.b_rs % 8 != 0 || g.ldo % 8 != 0) return false;
     if (g.hprev != nullptr && g.ldh % 8 != 0) return false;
     if (((uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.out | (uintptr_t)g.out2 | (uintptr_t)g.hprev) & 15) return false;
-    if (g.M < 128 || g.N < 64 || g.K < 64) return false;  // tiny problems stay on the CUDA cores
+    if (g.M < 64 || g.N < 8 || g.K < 8) return false;    // a handful of rows stays on the CUDA cores
     if (g.err == nullptr) return false;
     return true;
 }
@@ -559,7 +559,7 @@ bool wgrad_tc_eligible(mpode_dtype dt, const GemmArgs& g) {
     if (g.a_rs != 1 || g.b_rs != 1) return false;                       // operands are [reduction rows, M] and [rows, N]
     if (g.M % 8 != 0 || g.N % 8 != 0 || g.a_ks % 8 != 0 || g.b_ks % 8 != 0) return false;
     if (((uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.partial) & 15) return false;
-    if (g.M < 64 || g.N < 64 || g.K < 128) return false;
+    if (g.M < 8 || g.N < 8 || g.K < 128) return false;
     if (g.err == nullptr || g.partial == nullptr) return false;
     return true;
 }
@@ -574,7 +574,7 @@ bool launch_wgrad_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lo
     TcParams p{};
     p.M = g.M; p.N = g.N; p.K = g.K; p.epi = EPI_WGRAD; p.err = g.err;
     p.splits = splits; p.kb_per_split = per; p.partial = g.partial;
-    p.direct = splits == 1 && g.ldo % 4 == 0 && (((uintptr_t)g.out) & 15) == 0;
+    p.direct = splits == 1 && (g.crop_m == 0 || (g.crop_m == g.M && g.crop_n == g.N)) && g.ldo % 4 == 0 && (((uintptr_t)g.out) & 15) == 0;
     p.out = g.out; p.ldo = g.ldo; p.beta = g.beta;
     bool ok;
     if (dt == MPODE_BF16) {
@@ -586,7 +586,7 @@ bool launch_wgrad_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lo
     }
     if (!ok) return false;
     if (launches) ++*launches;
-    if (!p.direct) launch_splitk_reduce(g.partial, splits, g.M, g.N, (float*)g.out, g.ldo, g.beta, st, launches);
+    if (!p.direct) launch_splitk_reduce(g.partial, splits, g.M, g.N, (float*)g.out, g.ldo, g.beta, st, launches, g.crop_m, g.crop_n);
     return true;
 }
 

@@ -17,9 +17,11 @@ namespace {
 
 inline char* at(void* ws, size_t off) { return (char*)ws + off; }
 
-void plan_common(Layout& lay, int B, int d, int D, size_t p, mpode_dtype dt, int ybuf_rows_factor, bool own_kappa = true) {
+// d: row length of the internal state buffers (the state width, padded where the velocity asks for it); wide: the state has a log-density column
+void plan_common(Layout& lay, int B, int d, bool wide, size_t p, mpode_dtype dt, int ybuf_rows_factor, bool own_kappa = true) {
     const size_t es = low_size(dt);
     lay.scal = lay.take(256);
+    lay.ds = d;
     // one slab per family, stage slots back to back (the fused kernels address a slot through a 3-D tensor map)
     const size_t slot = (size_t)B * d * es;
     const size_t k0 = lay.take(4 * slot), y0 = lay.take(4 * ybuf_rows_factor * slot), p0 = lay.take(4 * slot);
@@ -30,7 +32,7 @@ void plan_common(Layout& lay, int B, int d, int D, size_t p, mpode_dtype dt, int
     }
     lay.v = lay.take((size_t)B * d * es);
     if (own_kappa) lay.kappa = lay.take((size_t)B * d * es);
-    if (D > d) {
+    if (wide) {
         for (int j = 0; j < 4; ++j) lay.klbuf[j] = lay.take((size_t)B * es);
         lay.vl = lay.take((size_t)B * es);
         lay.kappal = lay.take((size_t)B * es);
@@ -63,33 +65,37 @@ public:
             if (bias_) off += w_[l + 1];
         }
         p_ = off;
+        // 16-bit formats: every internal row length is rounded up to 8 elements (16 bytes, what a bulk tensor copy needs); the pad
+        // columns of weights, biases, states and cotangents are zero, so that they add nothing to any sum
+        for (int w : w_) wp_.push_back(dt_ == MPODE_F32 ? w : (w + 7) / 8 * 8);
     }
     size_t param_count() const override { return p_; }
 
     bool supports_time_gradient() const override { return true; }
+    bool needs_input_copy() const override { return wp_[0] != w_[0]; }     // the trajectory's rows are not padded
 
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
         keep_k_ = lay.time_gradient;          // the time-grid gradient reads every k_j after the vector-Jacobian products
         fused_ok_ = fused_shape_ok();
-        plan_common(lay, B_, w_[0], w_[0], p_, dt_, 1, !fused_ok_);
+        plan_common(lay, B_, wp_[0], false, p_, dt_, 1, !fused_ok_);
         if (fused_ok_) {     // kappa_j of three consecutive stages (slot j % 3); the layer-by-layer path uses the first slot
-            kappaslab_ = lay.take((size_t)3 * B_ * w_[0] * es);
+            kappaslab_ = lay.take((size_t)3 * B_ * wp_[0] * es);
             lay.kappa = kappaslab_;
         }
         int maxw = 0;
         for (int l = 0; l < L_; ++l) {
-            W16_.push_back(lay.take((size_t)w_[l + 1] * w_[l] * es));
-            W16T_.push_back(lay.take((size_t)w_[l + 1] * w_[l] * es));
-            b16_.push_back(bias_ ? lay.take((size_t)w_[l + 1] * es) : 0);
-            maxw = w_[l + 1] > maxw ? w_[l + 1] : maxw;
+            W16_.push_back(lay.take((size_t)wp_[l + 1] * wp_[l] * es));
+            W16T_.push_back(lay.take((size_t)wp_[l + 1] * wp_[l] * es));
+            b16_.push_back(bias_ ? lay.take((size_t)wp_[l + 1] * es) : 0);
+            maxw = wp_[l + 1] > maxw ? wp_[l + 1] : maxw;
         }
-        wt16_ = time_ ? lay.take((size_t)w_[1] * es) : 0;
+        wt16_ = time_ ? lay.take((size_t)wp_[1] * es) : 0;
         hslab_.assign(L_, 0);
-        for (int l = 1; l < L_; ++l) hslab_[l] = lay.take((size_t)4 * B_ * w_[l] * es);   // H_l of the four stages
+        for (int l = 1; l < L_; ++l) hslab_[l] = lay.take((size_t)4 * B_ * wp_[l] * es);   // H_l of the four stages
         for (int j = 0; j < 4; ++j) {
             std::vector<size_t> hs(L_, 0);
-            for (int l = 1; l < L_; ++l) hs[l] = hslab_[l] + (size_t)j * B_ * w_[l] * es;
+            for (int l = 1; l < L_; ++l) hs[l] = hslab_[l] + (size_t)j * B_ * wp_[l] * es;
             H_.push_back(hs);
         }
         // dZ_l: one buffer, or for the fused backward two stage slots (its weight gradients lag one stage behind the
@@ -98,9 +104,9 @@ public:
         dzslab_.assign(L_ + 1, 0);
         dz_stride_.assign(L_ + 1, 0);
         dZ_.assign(L_, 0);
-        size_t k_free = 4 * (size_t)B_ * w_[0] * es, k_at = lay.kbuf[0];
+        size_t k_free = 4 * (size_t)B_ * wp_[0] * es, k_at = lay.kbuf[0];
         for (int l = 1; l < L_; ++l) {
-            const size_t slot = (size_t)B_ * w_[l] * es;
+            const size_t slot = (size_t)B_ * wp_[l] * es;
             if (fused_ok_ && slot <= k_free && !keep_k_) {
                 dzslab_[l] = k_at;                              // slot 0 in the k slab (lower address), slot 1 its own buffer
                 dZ_[l] = lay.take(slot);
@@ -109,7 +115,7 @@ public:
             } else {
                 dzslab_[l] = lay.take((fused_ok_ ? 2 : 1) * slot);
                 dZ_[l] = dzslab_[l];
-                dz_stride_[l] = (long long)B_ * w_[l];
+                dz_stride_[l] = (long long)B_ * wp_[l];
             }
         }
         colsum_ = lay.take((size_t)64 * maxw * sizeof(float));
@@ -126,7 +132,7 @@ public:
             // dZ^T * 1 against a block of ones, into [stage][slice][width][8] partial sums (only column 0 is read back)
             size_t cp = 0;
             for (int j = 0; j < 4; ++j)
-                for (int l = 1; l <= L_; ++l) { col_off_[j][l] = (long long)cp; cp += (size_t)wg_splits_ * w_[l] * kOnesKeep; }
+                for (int l = 1; l <= L_; ++l) { col_off_[j][l] = (long long)cp; cp += (size_t)wg_splits_ * wp_[l] * kOnesKeep; }
             colpart_elems_ = cp;
             wg = (wg_part_elems_ + cp) * sizeof(float);      // the column-sum partials sit right behind the weight partials
             ones_ = lay.take((size_t)B_ * 64 * es);
@@ -136,7 +142,7 @@ public:
             f_cnt_ = lay.take(((size_t)RK_MAX_PHASES * cnt_stride_ + 2) * sizeof(unsigned));
         } else if (dt_ != MPODE_F32) {      // slice partial sums of the tensor-core weight gradient
             for (int l = 0; l < L_; ++l) {
-                size_t b = wgrad_tc_scratch_bytes(w_[l + 1], w_[l], B_);
+                size_t b = wgrad_tc_scratch_bytes(wp_[l + 1], wp_[l], B_);
                 wg = b > wg ? b : wg;
             }
         }
@@ -149,8 +155,8 @@ public:
     void plan_wgrad() {
         long long tiles = 0;
         for (int l = 0; l < L_; ++l) {
-            wg_bn_[l] = w_[l] >= 256 ? 256 : (w_[l] >= 128 ? 128 : 64);
-            tiles += (long long)((w_[l + 1] + 127) / 128) * ((w_[l] + wg_bn_[l] - 1) / wg_bn_[l]);
+            wg_bn_[l] = wp_[l] >= 256 ? 256 : (wp_[l] >= 128 ? 128 : 64);
+            tiles += (long long)((wp_[l + 1] + 127) / 128) * ((wp_[l] + wg_bn_[l] - 1) / wg_bn_[l]);
         }
         const int kb_rows = (B_ + 63) / 64;
         int splits = (int)((sm_count() + tiles / 2) / tiles);
@@ -163,8 +169,8 @@ public:
         wg_items_max_ = 0;
         for (int l = 0; l < L_; ++l) {
             wg_part_off_[l] = (long long)wg_part_elems_;
-            wg_part_elems_ += (size_t)wg_splits_ * w_[l + 1] * w_[l];
-            int items = ((w_[l + 1] + 127) / 128) * ((w_[l] + wg_bn_[l] - 1) / wg_bn_[l]) * wg_splits_;
+            wg_part_elems_ += (size_t)wg_splits_ * wp_[l + 1] * wp_[l];
+            int items = ((wp_[l + 1] + 127) / 128) * ((wp_[l] + wg_bn_[l] - 1) / wg_bn_[l]) * wg_splits_;
             wg_items_max_ = items > wg_items_max_ ? items : wg_items_max_;
         }
     }
@@ -172,10 +178,10 @@ public:
     void prepare(cudaStream_t st, void* ws, const float* theta, const signed char*, long long* L) override {
         for (int l = 0; l < L_; ++l) {
             int in_full = w_[l] + ((time_ && l == 0) ? 1 : 0);
-            launch_quantize_matrix(dt_, theta + woff_[l], in_full, w_[l + 1], w_[l], at(ws, W16_[l]), at(ws, W16T_[l]), st, L);
+            launch_quantize_matrix(dt_, theta + woff_[l], in_full, w_[l + 1], w_[l], at(ws, W16_[l]), at(ws, W16T_[l]), st, L, wp_[l + 1], wp_[l]);
             if (time_ && l == 0)
-                launch_quantize_matrix(dt_, theta + woff_[l] + w_[l], in_full, w_[l + 1], 1, at(ws, wt16_), nullptr, st, L);
-            if (bias_) launch_quantize_matrix(dt_, theta + boff_[l], w_[l + 1], 1, w_[l + 1], at(ws, b16_[l]), nullptr, st, L);
+                launch_quantize_matrix(dt_, theta + woff_[l] + w_[l], in_full, w_[l + 1], 1, at(ws, wt16_), nullptr, st, L, wp_[l + 1], 1);
+            if (bias_) launch_quantize_matrix(dt_, theta + boff_[l], w_[l + 1], 1, w_[l + 1], at(ws, b16_[l]), nullptr, st, L, 1, wp_[l + 1]);
         }
     }
 
@@ -183,12 +189,12 @@ public:
         const void* X = yin;
         for (int l = 0; l < L_; ++l) {
             GemmArgs g = base_args(ws, lay_);
-            g.A = X; g.a_rs = w_[l]; g.a_ks = 1;
-            g.B = at(ws, W16_[l]); g.b_rs = w_[l]; g.b_ks = 1;
-            g.M = B_; g.N = w_[l + 1]; g.K = w_[l];
+            g.A = X; g.a_rs = wp_[l]; g.a_ks = 1;
+            g.B = at(ws, W16_[l]); g.b_rs = wp_[l]; g.b_ks = 1;
+            g.M = B_; g.N = wp_[l + 1]; g.K = wp_[l];
             g.epi = EPI_FWD;
             g.out = (l == L_ - 1) ? at(ws, lay_->kbuf[j]) : at(ws, H_[j][l + 1]);
-            g.ldo = w_[l + 1];
+            g.ldo = wp_[l + 1];
             g.bias = bias_ ? at(ws, b16_[l]) : nullptr;
             g.wt = (time_ && l == 0) ? at(ws, wt16_) : nullptr;
             g.tau = tau16;
@@ -207,9 +213,10 @@ public:
             bool sums_done;
             {   // weight gradient: dW_l[n, k] (+)= sum_m dZ[m, n] X[m, k]
                 GemmArgs g = base_args(ws, lay_);
-                g.A = dZ; g.a_rs = 1; g.a_ks = w_[l + 1];
-                g.B = X; g.b_rs = 1; g.b_ks = w_[l];
-                g.M = w_[l + 1]; g.N = w_[l]; g.K = B_;
+                g.A = dZ; g.a_rs = 1; g.a_ks = wp_[l + 1];
+                g.B = X; g.b_rs = 1; g.b_ks = wp_[l];
+                g.M = wp_[l + 1]; g.N = wp_[l]; g.K = B_;
+                g.crop_m = w_[l + 1]; g.crop_n = w_[l];
                 g.epi = EPI_WGRAD; g.out = dg + woff_[l]; g.ldo = in_full; g.beta = beta;
                 g.partial = wgrad_tc_scratch_bytes(g.M, g.N, g.K) <= wgpart_bytes_ ? (float*)at(ws, wgpart_) : nullptr;
                 // the CUDA-core kernel takes the bias and time-column gradients (row sums of the same operand) along
@@ -220,7 +227,7 @@ public:
                 sums_done = launch_contraction(dt_, g, st, L) == 3;
             }
             if (bias_ || (time_ && l == 0)) {
-                const int R = sums_done ? 1 : launch_colsum(dt_, dZ, B_, w_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
+                const int R = sums_done ? 1 : launch_colsum(dt_, dZ, B_, w_[l + 1], wp_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
                                             (time_ && l == 0) ? dg + woff_[l] + w_[l] : nullptr, in_full, tau16, beta, st, L, colsum_counters(ws, lay_));
                 if (lay_->time_gradient && time_ && l == 0) {      // d tau_j = w_t . colsum(dZ_1)
                     StageTimeArgs ta{};
@@ -231,14 +238,14 @@ public:
             }
             {   // input gradient: dX[m, k] = sum_n dZ[m, n] W_l[n, k], then the activation derivative of the layer below
                 GemmArgs g = base_args(ws, lay_);
-                g.A = dZ; g.a_rs = w_[l + 1]; g.a_ks = 1;
-                g.B = at(ws, W16T_[l]); g.b_rs = w_[l + 1]; g.b_ks = 1;
-                g.M = B_; g.N = w_[l]; g.K = w_[l + 1];
+                g.A = dZ; g.a_rs = wp_[l + 1]; g.a_ks = 1;
+                g.B = at(ws, W16T_[l]); g.b_rs = wp_[l + 1]; g.b_ks = 1;
+                g.M = B_; g.N = wp_[l]; g.K = wp_[l + 1];
                 g.epi = EPI_DGRAD; g.flag = flag;
                 g.out = (l == 0) ? psi_out : at(ws, dZ_[l]);
-                g.ldo = w_[l];
+                g.ldo = wp_[l];
                 g.hprev = (l == 0) ? nullptr : at(ws, H_[j][l]);
-                g.ldh = w_[l];
+                g.ldh = wp_[l];
                 g.act = act_;
                 launch_contraction(dt_, g, st, L);
                 dZ = g.out;
@@ -296,12 +303,10 @@ public:
         return true;
     }
 
-    // ---- fused Runge-Kutta path (16-bit formats, every width a multiple of 8)
+    // ---- fused Runge-Kutta path (16-bit formats, state width a multiple of 8; hidden widths are padded to one)
     virtual bool fused_shape_ok() const {
         if (dt_ != MPODE_BF16 && dt_ != MPODE_F16) return false;
-        if (L_ > 4) return false;
-        for (int w : w_) if (w % 8 != 0) return false;
-        return true;
+        return L_ <= 4 && w_[0] % 8 == 0;
     }
     // output-tile width of a contraction with N columns: wide tiles for the tensor pipe, narrower ones when that
     // wastes fewer padded columns or when wide tiles would leave SMs without work
@@ -321,7 +326,7 @@ public:
     bool fused_forward(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
         if (!fused_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
         if (((uintptr_t)fs.traj & 31) != 0) return false;       // the epilogues move 32-byte pieces of trajectory rows
-        const int s = fs.stages, d = w_[0];
+        const int s = fs.stages, d = wp_[0];
         if (s * L_ > RK_MAX_PHASES) return false;
         RkMaps maps;
         int nm = 0;
@@ -331,12 +336,12 @@ public:
         int m_h[8] = {0}, m_w[8] = {0}, bn[8] = {0};
         for (int l = 1; l < L_; ++l) {
             m_h[l] = nm++;
-            if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, w_[l], (long long)B_ * w_[l], w_[l], 128, dt_, &maps.m[m_h[l]])) return false;
+            if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, wp_[l], (long long)B_ * wp_[l], wp_[l], 128, dt_, &maps.m[m_h[l]])) return false;
         }
         for (int l = 0; l < L_; ++l) {
-            bn[l] = choose_bn(w_[l + 1]);
+            bn[l] = choose_bn(wp_[l + 1]);
             m_w[l] = nm++;
-            if (!get_tensor_map(at(ws, W16_[l]), w_[l + 1], w_[l], w_[l], bn[l], dt_, &maps.m[m_w[l]])) return false;
+            if (!get_tensor_map(at(ws, W16_[l]), wp_[l + 1], wp_[l], wp_[l], bn[l], dt_, &maps.m[m_w[l]])) return false;
         }
         std::vector<RkPhase> ph;
         for (int j = 0; j < s; ++j)
@@ -346,7 +351,7 @@ public:
                 q.a_slot = (l == 0 && j > 0) ? j : 0;          // hidden outputs are consumed at once: one slot serves all stages
                 q.a_slot_step = (l == 0 && j == 0) ? 1 : 0;
                 q.b_map = m_w[l];
-                q.N = w_[l + 1]; q.K = w_[l]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
+                q.N = wp_[l + 1]; q.K = wp_[l]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
                 q.epi = l == L_ - 1 ? RK_EPI_STAGE_OUT : RK_EPI_HIDDEN;
                 q.act = act_; q.stage = j; q.layer = l; q.out_slot = 0;
                 q.dep_phase = ph.empty() ? s * L_ - 1 : (int)ph.size() - 1;      // the chain is linear: previous phase,
@@ -385,7 +390,7 @@ public:
         (void)L;
         if (!fused_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
         if (((uintptr_t)fs.traj & 31) != 0) return false;
-        const int s = fs.stages, d = w_[0];
+        const int s = fs.stages, d = wp_[0];
         b_stages_ = s;
         // ---------------- recompute program: stage inputs live in the Y slab (slot 0 = copy of the stored state)
         {
@@ -395,12 +400,12 @@ public:
             int m_h[8] = {0}, m_w[8] = {0}, bn[8] = {0};
             for (int l = 1; l < L_; ++l) {
                 m_h[l] = nm++;
-                if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, w_[l], (long long)B_ * w_[l], w_[l], 128, dt_, &maps_r_.m[m_h[l]])) return false;
+                if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, wp_[l], (long long)B_ * wp_[l], wp_[l], 128, dt_, &maps_r_.m[m_h[l]])) return false;
             }
             for (int l = 0; l < L_; ++l) {
-                bn[l] = choose_bn(w_[l + 1]);
+                bn[l] = choose_bn(wp_[l + 1]);
                 m_w[l] = nm++;
-                if (!get_tensor_map(at(ws, W16_[l]), w_[l + 1], w_[l], w_[l], bn[l], dt_, &maps_r_.m[m_w[l]])) return false;
+                if (!get_tensor_map(at(ws, W16_[l]), wp_[l + 1], wp_[l], wp_[l], bn[l], dt_, &maps_r_.m[m_w[l]])) return false;
             }
             std::vector<RkPhase> ph;
             for (int j = 0; j < s; ++j)
@@ -410,7 +415,7 @@ public:
                     q.a_map = l == 0 ? m_y : m_h[l];
                     q.a_slot = j; q.a_slot_step = 0;
                     q.b_map = m_w[l];
-                    q.N = w_[l + 1]; q.K = w_[l]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
+                    q.N = wp_[l + 1]; q.K = wp_[l]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
                     q.epi = l == L_ - 1 ? RK_EPI_STAGE_OUT : RK_EPI_HIDDEN;
                     q.act = act_; q.stage = j; q.layer = l; q.out_slot = j;
                     q.dep_phase = (int)ph.size() - 1;
@@ -430,14 +435,14 @@ public:
             int m_dz[8] = {0}, m_wt[8] = {0}, m_hs[8] = {0}, bn[8] = {0};
             for (int l = 1; l < L_; ++l) {
                 m_dz[l] = nm++;
-                if (!get_tensor_map_3d(at(ws, dzslab_[l]), 2, B_, w_[l], dz_stride_[l], w_[l], 128, dt_, &maps_v_.m[m_dz[l]])) return false;
+                if (!get_tensor_map_3d(at(ws, dzslab_[l]), 2, B_, wp_[l], dz_stride_[l], wp_[l], 128, dt_, &maps_v_.m[m_dz[l]])) return false;
                 m_hs[l] = nm++;     // stored layer outputs H_l (4 stage slots), staged into shared memory for the derivative product
-                if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, w_[l], (long long)B_ * w_[l], w_[l], 128, dt_, &maps_v_.m[m_hs[l]])) return false;
+                if (!get_tensor_map_3d(at(ws, hslab_[l]), 4, B_, wp_[l], (long long)B_ * wp_[l], wp_[l], 128, dt_, &maps_v_.m[m_hs[l]])) return false;
             }
             for (int l = 0; l < L_; ++l) {       // input gradient of layer l: N = w_l, K = w_{l+1}, operand W_l^T [w_l][w_{l+1}]
-                bn[l] = choose_bn(w_[l]);
+                bn[l] = choose_bn(wp_[l]);
                 m_wt[l] = nm++;
-                if (!get_tensor_map(at(ws, W16T_[l]), w_[l], w_[l + 1], w_[l + 1], bn[l], dt_, &maps_v_.m[m_wt[l]])) return false;
+                if (!get_tensor_map(at(ws, W16T_[l]), wp_[l], wp_[l + 1], wp_[l + 1], bn[l], dt_, &maps_v_.m[m_wt[l]])) return false;
             }
             // weight-gradient operands, read with the batch as the reduction index: boxes of [64 rows][64 columns]
             int m_ga[8] = {0}, m_gb[8] = {0};
@@ -445,11 +450,11 @@ public:
                 m_ga[l] = nm++;     // dZ_{l+1} (2 slots), kappa for the last layer (3 slots)
                 const bool last = l == L_ - 1;
                 const void* a_ptr = last ? at(ws, kappaslab_) : at(ws, dzslab_[l + 1]);
-                if (!get_tensor_map_3d(a_ptr, last ? 3 : 2, B_, w_[l + 1], last ? (long long)B_ * d : dz_stride_[l + 1], w_[l + 1], 64, dt_,
+                if (!get_tensor_map_3d(a_ptr, last ? 3 : 2, B_, wp_[l + 1], last ? (long long)B_ * d : dz_stride_[l + 1], wp_[l + 1], 64, dt_,
                                        &maps_v_.m[m_ga[l]])) return false;
                 m_gb[l] = nm++;     // layer input: Y slab for the first layer, H_l otherwise, 4 slots
                 const void* b_ptr = l == 0 ? at(ws, lay_->ybuf[0]) : at(ws, hslab_[l]);
-                if (!get_tensor_map_3d(b_ptr, 4, B_, w_[l], (long long)B_ * w_[l], w_[l], 64, dt_, &maps_v_.m[m_gb[l]])) return false;
+                if (!get_tensor_map_3d(b_ptr, 4, B_, wp_[l], (long long)B_ * wp_[l], wp_[l], 64, dt_, &maps_v_.m[m_gb[l]])) return false;
             }
             const int m_ones = nm++;
             if (!get_tensor_map_3d(at(ws, ones_), 1, B_, 64, (long long)B_ * 64, 64, 64, dt_, &maps_v_.m[m_ones])) return false;
@@ -466,7 +471,7 @@ public:
                     q.epi = RK_EPI_WGRAD;
                     q.a_map = m_ga[l]; q.a_slot = l == L_ - 1 ? j % 3 : (j & 1);
                     q.b_map = m_gb[l]; q.b_slot = j;
-                    q.M = w_[l + 1]; q.N = w_[l]; q.K = B_; q.bn = wg_bn_[l];
+                    q.M = wp_[l + 1]; q.N = wp_[l]; q.K = B_; q.bn = wg_bn_[l];
                     q.tiles_m = (q.M + 127) / 128; q.tiles_n = (q.N + q.bn - 1) / q.bn;
                     q.splits = wg_splits_; q.kb_per_split = wg_kb_per_split_;
                     q.part_off = wg_part_off_[l];
@@ -501,7 +506,7 @@ public:
                     // their last readers are that stage's weight-gradient items
                     if (j + 2 <= s - 1) q.wait_wg_total = wg_items_through_stage[j + 2];
                     q.b_map = m_wt[l];
-                    q.N = w_[l]; q.K = w_[l + 1]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
+                    q.N = wp_[l]; q.K = wp_[l + 1]; q.bn = bn[l]; q.tiles_n = (q.N + q.bn - 1) / q.bn;
                     q.epi = l == 0 ? RK_EPI_PSI : RK_EPI_DGRAD;
                     q.act = act_; q.stage = j; q.layer = l; q.out_slot = j & 1; q.h_slot = j; q.h_map = l >= 1 ? m_hs[l] : 0;
                     q.queue = j == s - 1 ? 2 : 0;      // no weight-gradient work exists yet during the first stage's chain
@@ -527,7 +532,7 @@ public:
 
     void fused_recompute(cudaStream_t st, void* ws, const FusedSolve& fs, int step, long long* L) override {
         const size_t es = low_size(dt_);
-        const size_t slot = (size_t)B_ * w_[0] * es;
+        const size_t slot = (size_t)B_ * wp_[0] * es;
         cudaMemcpyAsync(at(ws, lay_->ybuf[0]), (const char*)fs.traj + (size_t)step * slot, slot, cudaMemcpyDeviceToDevice, st);
         if (n_phases_r_ == 0) return;
         RkParams p{};
@@ -545,12 +550,12 @@ public:
     }
 
     void* fused_kappa_last(void* ws) const override {
-        return at(ws, kappaslab_) + (size_t)((b_stages_ - 1) % 3) * B_ * w_[0] * low_size(dt_);
+        return at(ws, kappaslab_) + (size_t)((b_stages_ - 1) % 3) * B_ * wp_[0] * low_size(dt_);
     }
 
     void fused_vjp(cudaStream_t st, void* ws, const FusedSolve& fs, int step, float* out, float beta, float coef, unsigned* flag,
                    long long* L, cudaEvent_t after_kernel, cudaStream_t st_finish) override {
-        const int s = b_stages_, d = w_[0];
+        const int s = b_stages_, d = wp_[0];
         const RkStepScalars& sc = scal_host_[step];
         RkParams p{};
         fill_common_params(p, ws, fs, n_phases_v_);
@@ -575,7 +580,7 @@ public:
             StageTimeArgs ta{};
             ta.colsum = (const float*)at(ws, wgpart_) + wg_part_elems_;
             for (int j = 0; j < s; ++j) ta.off[j] = col_off_[j][1];
-            ta.terms = s; ta.rows = wg_splits_; ta.M = w_[1]; ta.stride = kOnesKeep;
+            ta.terms = s; ta.rows = wg_splits_; ta.M = wp_[1]; ta.stride = kOnesKeep;
             ta.wt = at(ws, wt16_); ta.dtau = (float*)at(ws, lay_->tdots) + 2 * kDotBlocks;
             launch_stage_time_cot(dt_, ta, st, L);
         }
@@ -586,7 +591,7 @@ public:
             GradFinishLayer& g = ga.layer[l];
             const int in_full = w_[l] + ((time_ && l == 0) ? 1 : 0);
             g.partial = (const float*)at(ws, wgpart_) + wg_part_off_[l];
-            g.splits = wg_splits_; g.M = w_[l + 1]; g.N = w_[l];
+            g.splits = wg_splits_; g.M = w_[l + 1]; g.N = w_[l]; g.Mp = wp_[l + 1]; g.Np = wp_[l];
             g.w_off = (long long)woff_[l]; g.ldo = in_full;
             g.colpart = (const float*)at(ws, wgpart_) + wg_part_elems_;
             g.terms = s; g.rows = wg_splits_;
@@ -598,7 +603,7 @@ public:
     }
 
     void fill_common_params(RkParams& p, void* ws, const FusedSolve& fs, int n_phases) const {
-        p.B = B_; p.rb = rb_; p.d = w_[0]; p.D = w_[0]; p.stages = fs.stages;
+        p.B = B_; p.rb = rb_; p.d = wp_[0]; p.D = wp_[0]; p.stages = fs.stages;
         p.n_phases = n_phases;
         p.round_increment = fs.round_increment;
         p.scalars = (const RkStepScalars*)at(ws, f_scalars_);
@@ -608,8 +613,8 @@ public:
         p.wait_ns = fs.wait_ns;
         for (int l = 0; l < L_; ++l) p.bias[l] = bias_ ? at(ws, b16_[l]) : nullptr;
         p.wt = time_ ? at(ws, wt16_) : nullptr;
-        for (int l = 0; l <= L_; ++l) p.w[l] = w_[l];
-        for (int l = 1; l < L_; ++l) { p.hslab[l] = at(ws, hslab_[l]); p.h_slot_stride[l] = (long long)B_ * w_[l]; }
+        for (int l = 0; l <= L_; ++l) p.w[l] = wp_[l];
+        for (int l = 1; l < L_; ++l) { p.hslab[l] = at(ws, hslab_[l]); p.h_slot_stride[l] = (long long)B_ * wp_[l]; }
         p.kslab = at(ws, lay_->kbuf[0]); p.yslab = at(ws, lay_->ybuf[0]); p.psislab = at(ws, lay_->psi[0]);
         p.traj = const_cast<void*>(fs.traj);
     }
@@ -623,7 +628,7 @@ protected:
     bool time_, bias_;
     int L_;
     int max_steps_;
-    std::vector<int> w_;
+    std::vector<int> w_, wp_;      // layer widths; padded row lengths of the internal buffers
     std::vector<size_t> woff_, boff_, W16_, W16T_, b16_, dZ_;
     std::vector<std::vector<size_t>> H_;
     std::vector<size_t> hslab_, dzslab_;
@@ -660,37 +665,37 @@ public:
 
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
-        const int d = w_[0];
-        plan_common(lay, B_, d, d + 1, p_, dt_, 2);
+        const int d = wp_[0];
+        plan_common(lay, B_, d, true, p_, dt_, 2);
         int maxw = 0;
         for (int l = 0; l < L_; ++l) {
-            W16_.push_back(lay.take((size_t)w_[l + 1] * w_[l] * es));
-            W16T_.push_back(lay.take((size_t)w_[l + 1] * w_[l] * es));
-            b16_.push_back(bias_ ? lay.take((size_t)w_[l + 1] * es) : 0);
-            maxw = w_[l + 1] > maxw ? w_[l + 1] : maxw;
+            W16_.push_back(lay.take((size_t)wp_[l + 1] * wp_[l] * es));
+            W16T_.push_back(lay.take((size_t)wp_[l + 1] * wp_[l] * es));
+            b16_.push_back(bias_ ? lay.take((size_t)wp_[l + 1] * es) : 0);
+            maxw = wp_[l + 1] > maxw ? wp_[l + 1] : maxw;
         }
-        wt16_ = time_ ? lay.take((size_t)w_[1] * es) : 0;
+        wt16_ = time_ ? lay.take((size_t)wp_[1] * es) : 0;
         for (int j = 0; j < 4; ++j) {
             std::vector<size_t> hg(L_, 0), u(L_, 0);
             for (int l = 1; l < L_; ++l) {
-                hg[l] = lay.take((size_t)2 * B_ * w_[l] * es);   // [H_l; G_l]
-                u[l] = lay.take((size_t)B_ * w_[l] * es);        // U_l
+                hg[l] = lay.take((size_t)2 * B_ * wp_[l] * es);   // [H_l; G_l]
+                u[l] = lay.take((size_t)B_ * wp_[l] * es);        // U_l
             }
             H_.push_back(hg);
             U_.push_back(u);
         }
         uL_ = lay.take((size_t)B_ * d * es);
         cot_.assign(L_ + 1, 0);
-        for (int l = 1; l <= L_; ++l) cot_[l] = lay.take((size_t)2 * B_ * w_[l] * es);   // [zeta_l; ubar_l]
+        for (int l = 1; l <= L_; ++l) cot_[l] = lay.take((size_t)2 * B_ * wp_[l] * es);   // [zeta_l; ubar_l]
         // fp32 [hbar; gbar] of the backward step through an activation: not needed where the tensor-core epilogue takes that
         // step (tiles of sample pairs; every such contraction is eligible when the widths are multiples of 8 and at least 64)
         pair_bwd_ = pair_tiles();
-        for (int l = 1; l <= L_; ++l) pair_bwd_ = pair_bwd_ && w_[l] >= 64 && w_[l] % 8 == 0;
+        for (int l = 1; l <= L_; ++l) pair_bwd_ = pair_bwd_ && wp_[l] % 8 == 0;
         wide_ = pair_bwd_ ? 0 : lay.take((size_t)2 * B_ * maxw * sizeof(float));
         colsum_ = lay.take((size_t)64 * maxw * sizeof(float));
         size_t wg = 0;
         for (int l = 0; l < L_; ++l) {
-            size_t b = wgrad_tc_scratch_bytes(w_[l + 1], w_[l], 2 * B_);
+            size_t b = wgrad_tc_scratch_bytes(wp_[l + 1], wp_[l], 2 * B_);
             wg = b > wg ? b : wg;
         }
         wgpart_ = lay.take(wg);
@@ -703,8 +708,8 @@ public:
         MlpVelocity::prepare(st, ws, theta, probe, L);
         probe_ = probe;
         const size_t es = low_size(dt_);
-        const long long n = (long long)B_ * w_[0];
-        for (int j = 0; j < 4; ++j) launch_cnf_probe_to_low(dt_, probe, at(ws, lay_->ybuf[j]) + n * es, n, st, L);
+        const long long n = (long long)B_ * wp_[0];
+        for (int j = 0; j < 4; ++j) launch_cnf_probe_to_low(dt_, probe, at(ws, lay_->ybuf[j]) + n * es, B_, w_[0], wp_[0], st, L);
     }
 
     void forward(cudaStream_t st, void* ws, int j, const void* yin, float tau16, long long* L) override {
@@ -713,20 +718,20 @@ public:
         for (int l = 0; l < L_; ++l) {
             bool last = (l == L_ - 1);
             GemmArgs g = base_args(ws, lay_);
-            g.A = X; g.a_rs = w_[l]; g.a_ks = 1;
-            g.B = at(ws, W16_[l]); g.b_rs = w_[l]; g.b_ks = 1;
-            g.M = 2 * B_; g.N = w_[l + 1]; g.K = w_[l];
+            g.A = X; g.a_rs = wp_[l]; g.a_ks = 1;
+            g.B = at(ws, W16_[l]); g.b_rs = wp_[l]; g.b_ks = 1;
+            g.M = 2 * B_; g.N = wp_[l + 1]; g.K = wp_[l];
             g.epi = EPI_FWD;
             g.out = last ? at(ws, lay_->kbuf[j]) : at(ws, H_[j][l + 1]);
             g.out2 = last ? at(ws, uL_) : at(ws, U_[j][l + 1]);
             g.m_split = B_;
-            g.ldo = w_[l + 1];
+            g.ldo = wp_[l + 1];
             g.bias = bias_ ? at(ws, b16_[l]) : nullptr;
             g.wt = (time_ && l == 0) ? at(ws, wt16_) : nullptr;
             g.tau = tau16;
             g.act = last ? MPODE_ACT_NONE : act_;
             // tensor-core kernel: tiles of sample pairs, whose epilogue also writes G_l = Q16(sigma'(H_l) * U_l)
-            const long long n = (long long)B_ * w_[l + 1];
+            const long long n = (long long)B_ * wp_[l + 1];
             g.cnf_pair = pair_tiles() ? 1 : 0;
             g.pair_out = (g.cnf_pair && !last) ? at(ws, H_[j][l + 1]) + n * es : nullptr;
             const int path = launch_contraction(dt_, g, st, L);
@@ -736,50 +741,51 @@ public:
                 X = at(ws, H_[j][l + 1]);
             }
         }
-        launch_cnf_trace(dt_, probe_, at(ws, uL_), at(ws, lay_->klbuf[j]), B_, w_[0], st, L);
+        launch_cnf_trace(dt_, probe_, at(ws, uL_), at(ws, lay_->klbuf[j]), B_, w_[0], wp_[0], st, L);
     }
 
     void vjp(cudaStream_t st, void* ws, int j, const void* yin, float tau16, void* psi_out, float* dg, float beta,
              unsigned* flag, long long* L) override {
         const size_t es = low_size(dt_);
-        const int d = w_[0];
+        const int d = wp_[0];
         // cot_[L] = [kappa_z; ubar_L]: the driver wrote kappa_z into the first half
-        launch_cnf_ubar_last(dt_, at(ws, lay_->kappal), probe_, at(ws, cot_[L_]) + (size_t)B_ * d * es, B_, d, flag, st, L);
+        launch_cnf_ubar_last(dt_, at(ws, lay_->kappal), probe_, at(ws, cot_[L_]) + (size_t)B_ * d * es, B_, w_[0], d, flag, st, L);
         const void* C = at(ws, cot_[L_]);
         for (int l = L_ - 1; l >= 0; --l) {
             const void* Xpair = (l == 0) ? yin : at(ws, H_[j][l]);
             int in_full = w_[l] + ((time_ && l == 0) ? 1 : 0);
             {   // dW_l = zeta^T X + ubar^T G: one contraction over the 2B stacked rows
                 GemmArgs g = base_args(ws, lay_);
-                g.A = C; g.a_rs = 1; g.a_ks = w_[l + 1];
-                g.B = Xpair; g.b_rs = 1; g.b_ks = w_[l];
-                g.M = w_[l + 1]; g.N = w_[l]; g.K = 2 * B_;
+                g.A = C; g.a_rs = 1; g.a_ks = wp_[l + 1];
+                g.B = Xpair; g.b_rs = 1; g.b_ks = wp_[l];
+                g.M = wp_[l + 1]; g.N = wp_[l]; g.K = 2 * B_;
+                g.crop_m = w_[l + 1]; g.crop_n = w_[l];
                 g.epi = EPI_WGRAD; g.out = dg + woff_[l]; g.ldo = in_full; g.beta = beta;
                 g.partial = (float*)at(ws, wgpart_);
                 launch_contraction(dt_, g, st, L);
             }
             if (bias_ || (time_ && l == 0))   // bias and time column see the primal rows only
-                launch_colsum(dt_, C, B_, w_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
+                launch_colsum(dt_, C, B_, w_[l + 1], wp_[l + 1], (float*)at(ws, colsum_), bias_ ? dg + boff_[l] : nullptr, 1,
                               (time_ && l == 0) ? dg + woff_[l] + w_[l] : nullptr, in_full, tau16, beta, st, L, colsum_counters(ws, lay_));
             if (l > 0) {
-                const long long n = (long long)B_ * w_[l];
+                const long long n = (long long)B_ * wp_[l];
                 GemmArgs g = base_args(ws, lay_);
-                g.A = C; g.a_rs = w_[l + 1]; g.a_ks = 1;
-                g.B = at(ws, W16T_[l]); g.b_rs = w_[l + 1]; g.b_ks = 1;
-                g.M = 2 * B_; g.N = w_[l]; g.K = w_[l + 1];
+                g.A = C; g.a_rs = wp_[l + 1]; g.a_ks = 1;
+                g.B = at(ws, W16T_[l]); g.b_rs = wp_[l + 1]; g.b_ks = 1;
+                g.M = 2 * B_; g.N = wp_[l]; g.K = wp_[l + 1];
                 bool done = false;
                 if (pair_tiles()) {      // [hbar; gbar] through the activation in the epilogue of the tensor-core kernel
                     GemmArgs f = g;
                     f.epi = EPI_DGRAD; f.cnf_pair = 2; f.m_split = B_; f.act = act_; f.flag = flag;
-                    f.hprev = at(ws, H_[j][l]); f.ldh = w_[l]; f.uprev = at(ws, U_[j][l]);
-                    f.out = at(ws, cot_[l]); f.out2 = at(ws, cot_[l]) + n * es; f.ldo = w_[l];
+                    f.hprev = at(ws, H_[j][l]); f.ldh = wp_[l]; f.uprev = at(ws, U_[j][l]);
+                    f.out = at(ws, cot_[l]); f.out2 = at(ws, cot_[l]) + n * es; f.ldo = wp_[l];
                     done = tc_eligible(dt_, f) && launch_contraction(dt_, f, st, L) == 1;
                 }
                 if (!done && pair_bwd_) {
                     // no scratch was planned for the two-kernel form: report through the error word that the driver reads back
                     cudaMemsetAsync(g.err, 0xff, sizeof(unsigned), st);
                 } else if (!done) {
-                    g.epi = EPI_RAW32; g.out = at(ws, wide_); g.ldo = w_[l];
+                    g.epi = EPI_RAW32; g.out = at(ws, wide_); g.ldo = wp_[l];
                     launch_contraction(dt_, g, st, L);
                     float* wide = (float*)at(ws, wide_);
                     launch_cnf_backprop_act(dt_, act_, at(ws, H_[j][l]), at(ws, U_[j][l]), wide, wide + n, at(ws, cot_[l]),
@@ -788,10 +794,10 @@ public:
                 C = at(ws, cot_[l]);
             } else {
                 GemmArgs g = base_args(ws, lay_);
-                g.A = C; g.a_rs = w_[1]; g.a_ks = 1;
-                g.B = at(ws, W16T_[0]); g.b_rs = w_[1]; g.b_ks = 1;
-                g.M = B_; g.N = w_[0]; g.K = w_[1];
-                g.epi = EPI_DGRAD; g.flag = flag; g.out = psi_out; g.ldo = w_[0];
+                g.A = C; g.a_rs = wp_[1]; g.a_ks = 1;
+                g.B = at(ws, W16T_[0]); g.b_rs = wp_[1]; g.b_ks = 1;
+                g.M = B_; g.N = wp_[0]; g.K = wp_[1];
+                g.epi = EPI_DGRAD; g.flag = flag; g.out = psi_out; g.ldo = wp_[0];
                 launch_contraction(dt_, g, st, L);
             }
         }
@@ -822,7 +828,7 @@ public:
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
         const size_t pix = (size_t)B_ * H_ * W_;
-        plan_common(lay, B_, H_ * W_ * C_, H_ * W_ * C_, p_, dt_, 1);
+        plan_common(lay, B_, H_ * W_ * C_, false, p_, dt_, 1);
         w1_ = lay.take(n1_ * es);
         w1t_ = lay.take(n2_ * es);      // [C][9 flipped][C]: data channels only
         w2_ = lay.take(n2_ * es);
@@ -916,7 +922,7 @@ public:
                 launch_conv_class_grads(dt_, dz, B_, H_, W_, C_, ct, tau, class_scratch, ct > C_ ? out : nullptr, bias_out, beta, st, L);
             return;
         }
-        launch_colsum(dt_, dz, B_ * H_ * W_, C_, (float*)at(ws, colsum_), bias_out, 1, nullptr, 0, 0.f, beta, st, L, colsum_counters(ws, lay_));
+        launch_colsum(dt_, dz, B_ * H_ * W_, C_, C_, (float*)at(ws, colsum_), bias_out, 1, nullptr, 0, 0.f, beta, st, L, colsum_counters(ws, lay_));
         GemmArgs g = base_args(ws, lay_);
         g.A = dz; g.a_rs = 1; g.a_ks = C_;
         g.B = x; g.conv_on = 2; g.conv_h = H_; g.conv_w = W_; g.conv_cd = C_; g.conv_ct = ct; g.conv_tau = tau;
@@ -986,7 +992,7 @@ public:
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
         const size_t pix = (size_t)B_ * H_ * W_;
-        plan_common(lay, B_, H_ * W_ * C_, H_ * W_ * C_, p_, dt_, 1);
+        plan_common(lay, B_, H_ * W_ * C_, false, p_, dt_, 1);
         for (int i = 0; i < pieces_; ++i) {
             w_.push_back(lay.take(nw_ * es));        // W                (S = relu(conv(y, W) + b))
             wn_.push_back(lay.take(nw_ * es));       // -W               (dZ = -conv(kappa, W))
@@ -1085,7 +1091,7 @@ public:
         launch_instnorm_bwd(dt_, at(ws, dz_), at(ws, z_[j]), at(ws, s_[j]), (const float*)at(ws, r_[j]), at(ws, du_), B_, H_ * W_, C_,
                             MPODE_ACT_RELU, norm_ ? 1 : 0, flag, st, L);
         wgrad(st, ws, at(ws, du_), yin, dw, 1.f, 1.f, L);                  // S = relu(W y + b) as a function of W
-        launch_colsum(dt_, at(ws, du_), B_ * H_ * W_, C_, (float*)at(ws, colsum_), db, 1, nullptr, 0, 0.f, 1.f, st, L, colsum_counters(ws, lay_));
+        launch_colsum(dt_, at(ws, du_), B_ * H_ * W_, C_, C_, (float*)at(ws, colsum_), db, 1, nullptr, 0, 0.f, 1.f, st, L, colsum_counters(ws, lay_));
         g = conv_args(ws, at(ws, du_), at(ws, wt_[piece_]), EPI_DGRAD);
         g.flag = flag; g.out = psi_out;
         launch_contraction(dt_, g, st, L);
@@ -1115,7 +1121,7 @@ public:
     size_t param_count() const override { return 3; }
     bool supports_time_gradient() const override { return true; }
     void plan(Layout& lay) override {
-        plan_common(lay, B_, 1, 1, 3, dt_, 1);
+        plan_common(lay, B_, 1, false, 3, dt_, 1);
         scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
         log_ = lay.take(((size_t)4 * max_steps_ + 8) * sizeof(int));         // scale log, status words, t' [max_steps + 1]
     }
@@ -1185,7 +1191,7 @@ public:
     size_t param_count() const override { return hyper_param_count(h_, w_, d_); }
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
-        plan_common(lay, B_, d_, d_ + 1, param_count(), dt_, 1);
+        plan_common(lay, B_, d_, true, param_count(), dt_, 1);
         for (int j = 0; j < 4; ++j) {
             hyp_[j] = lay.take(hyper_stage_floats(h_, w_, d_) * sizeof(float));
             units_[j] = lay.take((size_t)w_ * B_ * es);

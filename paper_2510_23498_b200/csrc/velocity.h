@@ -40,11 +40,12 @@ struct Layout {
                               // bounded waits, [8..10] scale state (log2 S, failed step, bad input), [12..14] its copy when no mapped
                               // host words exist, [16] last-block counter of the convolution weight-gradient reduction,
                               // [17] that of the hypernetwork flow's cotangent sums, [20..23] those of its whole-step product, [24..55] those of the column sums
-    size_t kbuf[4] = {0};     // stage derivatives k_j, low [B, d]
+    int ds = 0;               // row length of k_j, Y_j, psi_j, v, kappa: d, or d rounded up with zero columns behind (velocities that ask for it)
+    size_t kbuf[4] = {0};     // stage derivatives k_j, low [B, ds]
     size_t klbuf[4] = {0};    // CNF: log-density component of k_j, low [B]
-    size_t ybuf[4] = {0};     // stage inputs Y_j, low [B, d] (CNF: [2B, d], second half = probe)
-    size_t psi[4] = {0};      // stage input cotangents psi_j, low [B, d]
-    size_t v = 0, vl = 0;     // seed Q16(S a): state part low [B, d], CNF log-density part low [B]
+    size_t ybuf[4] = {0};     // stage inputs Y_j, low [B, ds] (CNF: [2B, ds], second half = probe)
+    size_t psi[4] = {0};      // stage input cotangents psi_j, low [B, ds]
+    size_t v = 0, vl = 0;     // seed Q16(S a): state part low [B, ds], CNF log-density part low [B]
     size_t kappa = 0, kappal = 0;
     size_t dg = 0;            // per-step parameter gradient, fp32 [p]
     size_t slog = 0;          // dynamic scaling: the device-side scale log, int exponent [max_steps], int attempts [max_steps], byte doubled [max_steps]

@@ -15,3 +15,23 @@ def test_float32_mlp_at_tile_edges(batch, d, hidden):
     gpu = run_gpu(wl, low="f32")
     assert_parity(gpu, run_oracle(wl, exact=True), TOL["f32"])
     assert gpu["stats"]["tc_contractions"] == 0 and gpu["stats"]["simt_contractions"] > 0
+
+
+# 16-bit rows whose length is not a multiple of 8 elements are padded; hidden widths and state widths, each with its remainder, and
+# batches that are and are not whole tiles of 64 sample pairs.  Tolerances: those of the formats (rounding-emulating oracle).
+@pytest.mark.parametrize("batch,d,hidden,low", [(128, 63, 136, "bf16"), (64, 9, 71, "f16"), (130, 17, 65, "bf16"), (192, 64, 129, "f16")])
+def test_flow_with_odd_widths_runs_on_the_tensor_cores(batch, d, hidden, low):
+    wl = inputs.cnf_mlp(batch=batch, n_steps=2, d=d, hidden=hidden)
+    scaling = "dynamic" if low == "f16" else "none"
+    gpu = run_gpu(wl, low=low, scaling=scaling)
+    assert_parity(gpu, run_oracle(wl, low=low, scaling=scaling), TOL[low])
+    assert gpu["stats"]["simt_contractions"] == 0 and gpu["stats"]["tc_contractions"] > 0
+
+
+@pytest.mark.parametrize("batch,d,hidden,low", [(200, 64, 137, "bf16"), (130, 33, 100, "bf16"), (257, 71, 65, "f16"), (128, 9, 72, "f16")])
+def test_mlp_with_odd_widths_runs_on_the_tensor_cores(batch, d, hidden, low):
+    wl = inputs.mlp_block(batch=batch, n_steps=2, d=d, hidden=hidden)
+    scaling = "dynamic" if low == "f16" else "none"
+    gpu = run_gpu(wl, low=low, scaling=scaling)
+    assert_parity(gpu, run_oracle(wl, low=low, scaling=scaling), TOL[low])
+    assert gpu["stats"]["simt_contractions"] == 0
