@@ -148,7 +148,6 @@ void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes&
     const long long nBd = (long long)c->B * c->d;
     const char* traj_i = (const char*)c->traj + (size_t)i * nBd * es;
     long long* L = &c->stats.kernel_launches;
-    if (!c->v->needs_input_copy() && c->v->step_forward(st, ws, traj_i, step_scalars(c, i), c->stages, L)) return;
     for (int j = 0; j < c->stages; ++j) {
         const void* yin = traj_i;
         if (j > 0 || c->v->needs_input_copy()) {
@@ -367,7 +366,6 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
     launch_init_state(dt, y0_dev, yT_dev, traj_dev, c->B, c->d, c->D, st, L);                // y <- x, traj[0]
     // the whole loop in one persistent launch where the velocity has a fused kernel, else layer by layer
     FusedSolve fs = fused_solve(c, yT_dev);
-    c->v->prepare_solve(st, ws, fs, L);
     const bool fused = c->v->fused_forward(st, ws, fs, L);
     for (int i = 0; i < n_steps && !fused; ++i) {
         StepTimes tm = step_times(c, i);
@@ -447,6 +445,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             c->stats.retries = wb.retries;
             mpode_status cs = check_cuda(c, "mpode_backward");
             if (cs != MPODE_OK) return cs;
+            if (wb.status == MPODE_ERR_CUDA) return fail(c, MPODE_ERR_CUDA, "a device-side wait timed out");
             if (wb.status == MPODE_ERR_NONFINITE_INPUT) return fail(c, MPODE_ERR_NONFINITE_INPUT, "dL/dy_T is not finite");
             if (wb.status == MPODE_ERR_SCALE_FAILED) {
                 if (log) log->first_failed_step = wb.first_failed_step;
@@ -519,7 +518,6 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     c->v->prepare(st, ws, c->theta, c->probe, L);                                            // weights in low precision
     // fused kernels (one recompute launch per step, one VJP launch per attempt) where the velocity has them
     FusedSolve fs = fused_solve(c, nullptr);
-    c->v->prepare_solve(st, ws, fs, L);
     const bool fused = c->v->fused_backward_begin(st, ws, fs, L);
     // Without finiteness decisions nothing of step i - 1's recompute depends on step i's adjoint.  The two fused launches of
     // every step then follow each other on the caller's stream (recompute of step i - 1 right behind the VJP launch of
@@ -589,9 +587,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             } else if (fused && !checked) c->v->fused_vjp(st, ws, fs, i, g, 1.f, (float)((double)tm.h * ldexp(1.0, -e)), vjp_flag, L);
             else if (fused) c->v->fused_vjp(st, ws, fs, i, dg, 0.f, 1.f, vjp_flag, L);
             bool kappa_ready = seeded_kappa;          // stage s - 1: kappa = Q16(b_s v), written by the seed kernel
-            const bool by_step = !fused && !tg && !c->v->needs_input_copy() &&
-                                 c->v->step_vjp(st, ws, traj_i, step_scalars(c, i), s, dg, vjp_flag, L);
-            for (int j = s - 1; j >= 0 && !fused && !by_step; --j) {
+            for (int j = s - 1; j >= 0 && !fused; --j) {
                 Terms t{};
                 t.n = 0;
                 for (int l = j + 1; l < s; ++l) {

@@ -10,7 +10,6 @@ constexpr int HYPER_MAX_D = 8;
 size_t hyper_param_count(int h, int w, int d);       // A1, c1, A2, c2, A3, c3
 size_t hyper_stage_floats(int h, int w, int d);      // h1, h2, the w weight sets and the products U_j . W_j of one stage time
 size_t hyper_scratch_floats(int w, int d);           // the batch sums of the weight-set cotangents
-size_t hyper_step_scratch_floats(int h, int w, int d);   // whole-step product: those sums, the parts of the h2 cotangent, the stage gradients
 bool hyper_shape_ok(int h, int w, int d);            // the weight sets of one stage time fit the kernels' shared memory
 
 // k = [v; -tr] for one stage: `hyp` (hyper_stage_floats) receives the hypernetwork's rounded layers, A (low [w][B]) the units
@@ -23,26 +22,35 @@ void launch_hyper_vjp(mpode_dtype dt, const float* theta, float tau16, int h, in
                       void* Sb, const void* kappa, const void* kappa_l, void* psi, float* sums, float* dg, float beta, int B, unsigned* flag,
                       unsigned* counter, cudaStream_t st, long long* launches);
 
-// All stages of one Runge-Kutta step in one launch each way (the samples are independent of each other through a step).
-// The hypernetwork is evaluated for every stage time of the solve beforehand: launch_hyper_table fills table[count] (each
-// hyper_stage_floats) from the device array taus[count] of rounded stage times.
-// Per stage: hyp (hyper_stage_floats, an entry of that table), units A (low [w][B]), k (low [B, d]), kl (low [B]), the stage input y (low [B, d]; stage 0
-// reads the step's state instead), psi (low [B, d]), the unit cotangents sb (low [w][B]), the stage cotangent kap / kapl.
-struct HyperStagePtrs {
-    float* hyp[RK_MAX_STAGES];
-    void *A[RK_MAX_STAGES], *k[RK_MAX_STAGES], *kl[RK_MAX_STAGES], *y[RK_MAX_STAGES], *psi[RK_MAX_STAGES], *sb[RK_MAX_STAGES],
-        *kap[RK_MAX_STAGES], *kapl[RK_MAX_STAGES];
+// The whole solve (hyper_solve.cu).  launch_hyper_table evaluates the hypernetwork for every stage time of the solve into
+// table[step][4] (hyper_stage_floats each); the forward kernel runs Alg. 1, the backward kernel (a cooperative launch) Alg. 2 with its
+// scale decisions.
+struct HyperSolve {
+    int B, d, h, w, stages, n_steps, round_increment;
+    const float* theta;
+    const float* table; long long stage_floats;
+    const RkStepScalars* scal;          // device [n_steps]
+    void* traj;                         // low [(n_steps + 1)][B][d]
+    // forward
+    const float* y0; float* yT;         // fp32 [B][d], [B][d + 1]
+    // backward
+    const float* dLdyT; float* a; float* g; int accumulate;
+    const float* cot;                   // fp32 [n_steps][B][d + 1] running-cost cotangents, or null
+    int scaling, k_max, growth_rule, pbits, e0, e0_from_norm;
+    float* part;                        // hyper_solve_part_floats: every block's sums of the weight-set cotangents over its samples
+    float* tpart;                       // hyper_solve_tpart_floats: the weight sets' parts of the cotangent of h2
+    float* dg;                          // [p] the attempt's parameter gradient
+    float* a_new;                       // [B][d + 1] the adjoint the attempt would leave
+    unsigned* words;                    // 16 device words, zero at launch
+    unsigned long long wait_ns;         // limit of a grid barrier
+    int *log_exp, *log_attempts, *log_doubled, *status;     // device [n_steps] each; status [4], zero at launch
 };
-bool hyper_step_shape_ok(int h, int w, int d, int stages);      // the weight sets of all stage times fit shared memory
-// Y_j = Q16(ybar + sum_{l<j} (h a_jl) k_l) and k_j = f(tau_j, Y_j) for every stage (Alg. 1, increment)
-void launch_hyper_table(mpode_dtype dt, const float* theta, const float* taus, int count, int h, int w, int d, float* table, cudaStream_t st,
-                        long long* launches);
-void launch_hyper_step_forward(mpode_dtype dt, const RkStepScalars& sc, int stages, int h, int w, int d,
-                               const HyperStagePtrs& ptr, const void* ybar, int B, cudaStream_t st, long long* launches);
-// kappa_j = Q16(b_j v + sum_{l>j} (h a_lj) psi_l), psi_j and dg = sum_j dtheta_j (added last stage first) from the seed v (low
-// [B, d]) and v_l (low [B]).  scratch: hyper_step_scratch_floats; counters: `stages` device words that are zero between calls.
-void launch_hyper_step_vjp(mpode_dtype dt, const float* theta, const RkStepScalars& sc, int stages, int h, int w, int d,
-                           const HyperStagePtrs& ptr, const void* ybar, const void* v, const void* v_l, float* scratch, float* dg, int B,
-                           unsigned* flag, unsigned* counters, cudaStream_t st, long long* launches);
+bool hyper_solve_shape_ok(mpode_dtype dt, int h, int w, int d, int stages);
+size_t hyper_solve_part_floats(int w, int d);
+size_t hyper_solve_tpart_floats(int h, int w);
+void launch_hyper_table(mpode_dtype dt, const float* theta, const RkStepScalars* scal, int n_steps, int stages, int h, int w, int d, float* table,
+                        cudaStream_t st, long long* launches);
+bool launch_hyper_solve_forward(mpode_dtype dt, const HyperSolve& p, cudaStream_t st, long long* launches);
+bool launch_hyper_solve_backward(mpode_dtype dt, const HyperSolve& p, cudaStream_t st, long long* launches);
 
 }  // namespace mpode

@@ -1183,7 +1183,8 @@ private:
 
 // ---------------------------------------------------------------------------------------------------- hypernetwork flow, exact trace
 // Sec. 6.1 (two-dimensional flows): joint state [z; l], z' = (1/w) sum_j U_j(t) tanh(W_j(t) . z + b_j(t)), l' = -tr(dz'/dz) written
-// out; the weight sets come from t through three fully connected layers (hyper_cnf.cu).  Layer-by-layer path only.
+// out; the weight sets come from t through three fully connected layers.  Whole-solve kernels (hyper_solve.cu), or stage by stage
+// (hyper_cnf.cu) where the weight sets do not fit shared memory.
 class HyperCnfVelocity : public Velocity {
 public:
     HyperCnfVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps) : B_(B), dt_(dt), d_(v.d), h_(v.widths[0]),
@@ -1192,32 +1193,70 @@ public:
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
         plan_common(lay, B_, d_, true, param_count(), dt_, 1);
+        whole_ = hyper_solve_shape_ok(dt_, h_, w_, d_, RK_MAX_STAGES);
+        if (whole_) {
+            // the hypernetwork's layers and weight sets for every stage time of a solve; per-step scalars; scratch of the backward pass
+            table_ = lay.take((size_t)max_steps_ * RK_MAX_STAGES * hyper_stage_floats(h_, w_, d_) * sizeof(float));
+            scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
+            log_ = lay.take(((size_t)3 * max_steps_ + 4 + 16) * sizeof(int));       // scale log, status [4], words [16]
+            part_ = lay.take(hyper_solve_part_floats(w_, d_) * sizeof(float));
+            tpart_ = lay.take(hyper_solve_tpart_floats(h_, w_) * sizeof(float));
+            return;
+        }
         for (int j = 0; j < 4; ++j) {
             hyp_[j] = lay.take(hyper_stage_floats(h_, w_, d_) * sizeof(float));
             units_[j] = lay.take((size_t)w_ * B_ * es);
         }
-        // one set per stage of what a whole-step vector-Jacobian product keeps: unit cotangents, stage cotangents, batch sums
-        for (int j = 0; j < 4; ++j) {
-            sbar_[j] = lay.take((size_t)w_ * B_ * es);
-            kap_[j] = lay.take((size_t)B_ * d_ * es);
-            kapl_[j] = lay.take((size_t)B_ * es);
+        sbar_ = lay.take((size_t)w_ * B_ * es);
+        part_ = lay.take(hyper_scratch_floats(w_, d_) * sizeof(float));
+    }
+    void prepare(cudaStream_t, void*, const float* theta, const signed char*, long long*) override { theta_ = theta; }
+    HyperSolve solve_params(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, long long* L) const {
+        HyperSolve p{};
+        p.B = B_; p.d = d_; p.h = h_; p.w = w_; p.stages = fs.stages; p.n_steps = fs.n_steps; p.round_increment = fs.round_increment;
+        p.theta = theta; p.stage_floats = (long long)hyper_stage_floats(h_, w_, d_);
+        p.scal = (const RkStepScalars*)at(ws, scal_); p.traj = const_cast<void*>(fs.traj);
+        p.table = (const float*)at(ws, table_);
+        cudaMemcpyAsync(at(ws, scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
+        launch_hyper_table(dt_, theta, p.scal, fs.n_steps, fs.stages, h_, w_, d_, (float*)at(ws, table_), st, L);
+        return p;
+    }
+    bool whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
+                       long long* L) override {
+        if (!whole_ || fs.n_steps > max_steps_) return false;
+        HyperSolve p = solve_params(st, ws, fs, theta, L);
+        p.y0 = y0; p.yT = yT;
+        if (!launch_hyper_solve_forward(dt_, p, st, L)) return false;
+        if (tl_counters) ++tl_counters->whole;
+        return true;
+    }
+    bool whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
+        if (!whole_ || fs.n_steps > max_steps_) return false;
+        const int N = fs.n_steps;
+        HyperSolve p = solve_params(st, ws, fs, wb.theta, L);
+        p.dLdyT = wb.dLdyT; p.a = wb.a; p.g = wb.g; p.accumulate = wb.accumulate; p.cot = wb.cot;
+        p.scaling = wb.scaling; p.k_max = wb.k_max; p.growth_rule = wb.growth_rule; p.pbits = wb.pbits; p.e0 = wb.e0; p.e0_from_norm = wb.e0_from_norm;
+        p.part = (float*)at(ws, part_); p.tpart = (float*)at(ws, tpart_); p.dg = (float*)at(ws, lay_->dg);
+        p.a_new = (float*)at(ws, lay_->psi[0]);         // the psi slab: 4 B d low-format entries, at least 4 B (d + 1) bytes
+        int* logs = (int*)at(ws, log_);
+        p.log_exp = logs; p.log_attempts = logs + N; p.log_doubled = logs + 2 * N; p.status = logs + 3 * N; p.words = (unsigned*)(logs + 3 * N + 4);
+        p.wait_ns = fs.wait_ns;
+        const size_t ints = (size_t)3 * N + 4;
+        cudaMemsetAsync(logs, 0, (ints + 16) * sizeof(int), st);
+        if (!launch_hyper_solve_backward(dt_, p, st, L)) return false;
+        if (tl_counters) ++tl_counters->whole;
+        std::vector<int> hl(ints);
+        cudaMemcpyAsync(hl.data(), logs, ints * sizeof(int), cudaMemcpyDeviceToHost, st);
+        cudaStreamSynchronize(st);
+        const int* stp = hl.data() + 3 * N;
+        wb.status = stp[0]; wb.first_failed_step = wb.status == MPODE_ERR_SCALE_FAILED ? stp[1] : -1; wb.retries = stp[2];
+        for (int i = 0; i < N; ++i) {
+            if (wb.exp_used) wb.exp_used[i] = hl[i];
+            if (wb.attempts) wb.attempts[i] = hl[N + i];
+            if (wb.doubled) wb.doubled[i] = (unsigned char)hl[2 * N + i];
         }
-        part_ = lay.take(hyper_step_scratch_floats(h_, w_, d_) * sizeof(float));
-        // the hypernetwork's layers and weight sets for every stage time of a solve, and those times
-        table_ = lay.take((size_t)max_steps_ * 4 * hyper_stage_floats(h_, w_, d_) * sizeof(float));
-        taus_ = lay.take((size_t)max_steps_ * 4 * sizeof(float));
+        return true;
     }
-    void prepare(cudaStream_t, void*, const float* theta, const signed char*, long long*) override { theta_ = theta; by_step_ = false; }
-    void prepare_solve(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
-        by_step_ = hyper_step_shape_ok(h_, w_, d_, fs.stages) && fs.n_steps <= max_steps_;
-        if (!by_step_) return;
-        taus_host_.assign((size_t)fs.n_steps * 4, 0.f);
-        for (int i = 0; i < fs.n_steps; ++i)
-            for (int j = 0; j < fs.stages; ++j) taus_host_[(size_t)i * 4 + j] = fs.scalars[i].tau16[j];
-        cudaMemcpyAsync(at(ws, taus_), taus_host_.data(), taus_host_.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-        launch_hyper_table(dt_, theta_, (const float*)at(ws, taus_), fs.n_steps * 4, h_, w_, d_, (float*)at(ws, table_), st, L);
-    }
-    void set_step(int step, int) override { step_ = step; }
     void forward(cudaStream_t st, void* ws, int j, const void* yin, float tau16, long long* L) override {
         launch_hyper_forward(dt_, theta_, tau16, h_, w_, d_, (float*)at(ws, hyp_[j]), yin, at(ws, units_[j]), at(ws, lay_->kbuf[j]),
                              at(ws, lay_->klbuf[j]), B_, st, L);
@@ -1225,41 +1264,18 @@ public:
     void vjp(cudaStream_t st, void* ws, int j, const void* yin, float tau16, void* psi_out, float* dg, float beta, unsigned* flag,
              long long* L) override {
         unsigned* counter = (unsigned*)at(ws, lay_->scal) + 17;     // a word of the scalar slice: zero between kernels
-        launch_hyper_vjp(dt_, theta_, tau16, h_, w_, d_, (const float*)at(ws, hyp_[j]), yin, at(ws, units_[j]), at(ws, sbar_[0]),
+        launch_hyper_vjp(dt_, theta_, tau16, h_, w_, d_, (const float*)at(ws, hyp_[j]), yin, at(ws, units_[j]), at(ws, sbar_),
                          at(ws, lay_->kappa), at(ws, lay_->kappal), psi_out, (float*)at(ws, part_), dg, beta, B_, flag, counter, st, L);
-    }
-    bool step_forward(cudaStream_t st, void* ws, const void* ybar, const RkStepScalars& sc, int stages, long long* L) override {
-        if (!by_step_) return false;
-        launch_hyper_step_forward(dt_, sc, stages, h_, w_, d_, stage_ptrs(ws), ybar, B_, st, L);
-        return true;
-    }
-    bool step_vjp(cudaStream_t st, void* ws, const void* ybar, const RkStepScalars& sc, int stages, float* dg, unsigned* flag,
-                  long long* L) override {
-        if (!by_step_) return false;
-        unsigned* counter = (unsigned*)at(ws, lay_->scal) + 20;     // words 20 .. 23 of the scalar slice
-        launch_hyper_step_vjp(dt_, theta_, sc, stages, h_, w_, d_, stage_ptrs(ws), ybar, at(ws, lay_->v), at(ws, lay_->vl),
-                              (float*)at(ws, part_), dg, B_, flag, counter, st, L);
-        return true;
     }
     void bind(const Layout* lay) { lay_ = lay; }
 
 private:
-    HyperStagePtrs stage_ptrs(void* ws) const {
-        HyperStagePtrs p{};
-        for (int j = 0; j < 4; ++j) {
-            p.hyp[j] = (float*)at(ws, table_) + ((size_t)step_ * 4 + j) * hyper_stage_floats(h_, w_, d_); p.A[j] = at(ws, units_[j]); p.k[j] = at(ws, lay_->kbuf[j]); p.kl[j] = at(ws, lay_->klbuf[j]);
-            p.y[j] = at(ws, lay_->ybuf[j]); p.psi[j] = at(ws, lay_->psi[j]); p.sb[j] = at(ws, sbar_[j]); p.kap[j] = at(ws, kap_[j]);
-            p.kapl[j] = at(ws, kapl_[j]);
-        }
-        return p;
-    }
     int B_;
     mpode_dtype dt_;
     int d_, h_, w_;
-    int max_steps_, step_ = 0;
-    bool by_step_ = false;                 // this pass goes step by step on the table of weight sets
-    std::vector<float> taus_host_;
-    size_t hyp_[4] = {0}, units_[4] = {0}, sbar_[4] = {0}, kap_[4] = {0}, kapl_[4] = {0}, part_ = 0, table_ = 0, taus_ = 0;
+    int max_steps_;
+    bool whole_ = false;                   // whole-solve kernels
+    size_t hyp_[4] = {0}, units_[4] = {0}, sbar_ = 0, part_ = 0, tpart_ = 0, table_ = 0, scal_ = 0, log_ = 0;
     const float* theta_ = nullptr;
     const Layout* lay_ = nullptr;
 };

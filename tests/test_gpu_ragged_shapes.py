@@ -2,7 +2,7 @@
 import pytest
 
 from paper_2510_23498_b200 import inputs
-from _harness import TOL, assert_parity, run_gpu, run_oracle
+from _harness import TOL, assert_parity, assert_same_log, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +35,16 @@ def test_mlp_with_odd_widths_runs_on_the_tensor_cores(batch, d, hidden, low):
     gpu = run_gpu(wl, low=low, scaling=scaling)
     assert_parity(gpu, run_oracle(wl, low=low, scaling=scaling), TOL[low])
     assert gpu["stats"]["simt_contractions"] == 0
+
+
+# whole-solve kernels of the hypernetwork flow: one sample, a block's samples less and plus one, more sample groups than blocks, more
+# weight sets than blocks, a hypernetwork as wide as a block's threads, and sets too large for shared memory (stage by stage)
+@pytest.mark.parametrize("batch,d,hidden,w,n_steps", [(1, 2, 8, 16, 3), (7, 2, 32, 33, 2), (9, 3, 16, 200, 2), (2400, 2, 16, 32, 2), (40, 1, 128, 20, 2),
+                                                      (30, 6, 8, 600, 2)])
+def test_hypernetwork_flow_at_block_edges(batch, d, hidden, w, n_steps):
+    wl = inputs.hyper_cnf(batch=batch, n_steps=n_steps, d=d, hidden=hidden, w=w)
+    assert_parity(run_gpu(wl, "f32", "none"), run_oracle(wl, exact=True), TOL["f32"])
+    gpu, orc = run_gpu(wl, "f16", "dynamic"), run_oracle(wl, "f16", "dynamic")
+    assert_parity(gpu, orc, TOL["f16"])
+    assert_same_log(gpu["log"], orc["log"])
+    assert gpu["stats"]["whole_solve_launches"] == (0 if w == 600 else 2)
