@@ -1,7 +1,7 @@
 // Whole-solve kernels for very small dense velocities (state width <= 8, one hidden layer of <= 64 units, batch <= 1024):
-// at these sizes the time loop is pure launch latency, so the forward pass of Alg. 1 and the whole backward pass of
+// at these sizes the time loop is pure latency, so the forward pass of Alg. 1 and the whole backward pass of
 // Alg. 2 (recompute, vector-Jacobian products, finiteness test, halving / doubling of the adjoint scale, fp32 updates)
-// each run as ONE launch of a single CTA with one thread per sample and the rounded weights in shared memory.
+// each run as ONE launch, eight lanes per sample, the rounded weights in shared memory or registers; the backward pass is one cluster.
 #pragma once
 #include "common.cuh"
 #include "rk_fused.h"
@@ -34,7 +34,8 @@ struct TinyParams {
 };
 
 bool tiny_mlp_supported(int B, int d, int h, int n_layers, int p);
-void launch_tiny_forward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
-void launch_tiny_backward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
+// return false when the launch is refused (nothing has run then)
+bool launch_tiny_forward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
+bool launch_tiny_backward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
 
 }  // namespace mpode

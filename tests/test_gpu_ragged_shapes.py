@@ -48,3 +48,19 @@ def test_hypernetwork_flow_at_block_edges(batch, d, hidden, w, n_steps):
     assert_parity(gpu, orc, TOL["f16"])
     assert_same_log(gpu["log"], orc["log"])
     assert gpu["stats"]["whole_solve_launches"] == (0 if w == 600 else 2)
+
+
+# whole-solve kernels of very small networks: every variant (state width 2 / 4 / 8, hidden width 32 / 64), one sample, a full block,
+# one more than a block, a full cluster of 16 blocks
+@pytest.mark.parametrize("batch,d,hidden", [(1, 2, 32), (64, 1, 5), (65, 4, 33), (513, 3, 32), (1024, 2, 64), (1000, 8, 30), (130, 7, 39)])
+def test_tiny_network_variants(batch, d, hidden):
+    wl = inputs.toy_mlp(batch=batch, n_steps=4, hidden=hidden)
+    if d != 2:
+        widths = [d, hidden, d]
+        wl = inputs.mlp_block(batch=batch, n_steps=4, d=d, hidden=hidden, low="f16", scaling="dynamic")
+        wl.vel["widths"], wl.theta = widths, inputs.mlp_theta(3, widths, True)
+    gpu, orc = run_gpu(wl, "f16", "dynamic"), run_oracle(wl, "f16", "dynamic")
+    assert_parity(gpu, orc, TOL["f16"])
+    assert_same_log(gpu["log"], orc["log"])
+    assert gpu["stats"]["whole_solve_launches"] == 2
+    assert_parity(run_gpu(wl, "f32", "none"), run_oracle(wl, exact=True), TOL["f32"])
