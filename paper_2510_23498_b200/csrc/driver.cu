@@ -523,7 +523,10 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     // every step then follow each other on the caller's stream (recompute of step i - 1 right behind the VJP launch of
     // step i, whose layer outputs it overwrites), and the small kernels between them (gradient finish, adjoint commit,
     // next seed) run beside the recompute on a second stream.
-    bool overlap = fused && !checked && c->allow_side && !tg;
+    const bool all_done = fused && !dynamic && c->v->fused_backward_all(st, ws, fs, a, g, cot, e, vjp_flag, tprime, L);
+    if (all_done && log)
+        for (int i = 0; i < N; ++i) { log->attempts[i] = 1; log->exp_used[i] = e; log->doubled[i] = 0; }
+    bool overlap = fused && !checked && c->allow_side && !tg && !all_done;
     if (overlap && c->side == nullptr) {
         if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_ready, cudaEventDisableTiming) != cudaSuccess ||
@@ -555,7 +558,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         if (overlap) { /* queued on the second stream */ }
         else if (fused) c->v->fused_recompute(st, ws, fs, i, L);
         else run_stages(c, st, ws, i, tm);
-        if (tg) {      // Phi^T a_{i+1} with Phi = sum_j b_j k_j from the recomputed stages and the adjoint before its update
+        if (tg && !(fused && c->v->fused_has_time_terms())) {      // Phi^T a_{i+1} with Phi = sum_j b_j k_j from the recomputed stages and the adjoint before its update
             DotPairs pr{};
             pr.n = s;
             for (int j = 0; j < s; ++j) {
@@ -565,7 +568,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         }
     };
     for (;;) {
-    for (int i = start; i >= 0; --i) {
+    for (int i = start; i >= 0 && !all_done; --i) {
         if (recomputed != i) queue_recompute(i);     // a repeated attempt finds its step's stages still in place
         StepTimes tm = step_times(c, i);
         c->v->set_step(i, N);
@@ -575,7 +578,8 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             // velocities that write kappa_{j-1} from their own epilogues (state without extra columns) get kappa_s from the seed
             const bool kappa_in_vjp = !fused && c->D == c->d && c->v->can_write_next_kappa();
             const bool seeded_kappa = kappa_in_vjp;
-            launch_seed(dt, a, e, at(ws, c->lay.v), c->D > c->d ? at(ws, c->lay.vl) : nullptr, c->B, c->d, c->lay.ds, c->D,
+            if (!(fused && c->v->fused_seeds_itself(a, e, e_dev)))
+                launch_seed(dt, a, e, at(ws, c->lay.v), c->D > c->d ? at(ws, c->lay.vl) : nullptr, c->B, c->d, c->lay.ds, c->D,
                         vjp_flag, sr, L, fused ? c->v->fused_kappa_last(ws) : (seeded_kappa ? at(ws, c->v->kappa_offset(c->lay)) : nullptr),
                         (float)c->tb[s - 1], e_dev);                                             // seed Q16(S a)
             // without a finiteness decision the step gradient goes straight into g <- g + (h / S) dg
@@ -620,7 +624,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
                 const void* yin = (j > 0 || c->v->needs_input_copy()) ? (const void*)at(ws, c->lay.ybuf[j]) : (const void*)traj_i;
                 c->v->vjp(st, ws, j, yin, tm.tau16[j], at(ws, c->lay.psi[j]), dg, j == s - 1 ? 0.f : 1.f, vjp_flag, L);
             }
-            if (tg) {      // dt = sum_j dtau_j, dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>); Q16(dt), Q16(dh) join the test
+            if (tg && !(fused && c->v->fused_time_terms(st, tvals, vjp_flag, L))) {      // dt = sum_j dtau_j, dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>); Q16(dt), Q16(dh) join the test
                 DotPairs pr{};
                 for (int j = 1; j < s; ++j)
                     for (int l = 0; l < j; ++l)

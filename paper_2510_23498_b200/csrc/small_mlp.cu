@@ -1,0 +1,807 @@
+// Row-local kernels for small dense velocities in the 16-bit formats.  Samples are independent through the time loop, so a block
+// takes 16 (or 32) of them through the whole forward solve, or through the backward chain of several steps, without talking to any
+// other block: a layer is one contraction [16 x K] x [K x N] whose operands never leave the SM (activations in shared memory, weights
+// through L1), and the next layer starts after a block barrier.  What bounds this is the chain of layers, not bytes or tensor rate:
+// a tcgen05 tile needs 128 rows (64 at half rate) and a hand-over between its epilogue and the next tile's operands, about 8 us per
+// layer in rk_fused.cu, while mma.sync fragments of 16 rows spread the batch over the SMs and hand over in registers and shared memory.
+// Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
+// second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
+// Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.9 ms; MLP
+// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.5 ms.
+#include "small_mlp.h"
+
+#include "profiler.h"
+#include "tc_ptx.cuh"
+#include "tensormap.h"
+
+namespace mpode {
+using namespace tc;
+namespace {
+
+constexpr int kWarps = 8, kThreads = 32 * kWarps;
+
+template <typename T> __device__ __forceinline__ float lowf(T x) { return Low<T>::to_f(x); }
+template <typename T> __device__ __forceinline__ float q16(float x) { return Low<T>::to_f(Low<T>::from_f(x)); }
+
+template <typename T> __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
+template <> __device__ __forceinline__ void mma16816<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+template <> __device__ __forceinline__ void mma16816<__nv_bfloat16>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool on) {      // off: 16 zero bytes
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+
+__device__ __forceinline__ float act_f(int act, float z) {
+    switch (act) {
+        case MPODE_ACT_SOFTPLUS: return fast_act<MPODE_ACT_SOFTPLUS>(z);
+        case MPODE_ACT_RELU: return fast_act<MPODE_ACT_RELU>(z);
+        case MPODE_ACT_TANH: return fast_act<MPODE_ACT_TANH>(z);
+        default: return z;
+    }
+}
+__device__ __forceinline__ float act_df(int act, float h) {
+    switch (act) {
+        case MPODE_ACT_SOFTPLUS: return fast_act_deriv<MPODE_ACT_SOFTPLUS>(h);
+        case MPODE_ACT_RELU: return fast_act_deriv<MPODE_ACT_RELU>(h);
+        case MPODE_ACT_TANH: return fast_act_deriv<MPODE_ACT_TANH>(h);
+        default: return 1.f;
+    }
+}
+
+__host__ __device__ inline int k32(int w) { return (w + 31) / 32; }
+
+// ---------------------------------------------------------------- weights in fragment order, biases
+struct PackJob { long long first[2 * SMALL_MAX_L + 1]; };      // first 16-byte group of each (layer, direction)
+template <typename T>
+__global__ void __launch_bounds__(256) small_pack_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ PackJob job) {
+    const long long n = job.first[2 * p.L];
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        int q = 0;
+        while (i >= job.first[q + 1]) ++q;
+        const int l = q >> 1, back = q & 1;
+        const long long r = i - job.first[q];
+        const int kp = k32(back ? p.wp[l + 1] : p.wp[l]);
+        const int lane = (int)(r & 31), kk = (int)((r >> 5) % kp), tile = (int)((r >> 5) / kp);
+        const int in_full = p.wr[l] + ((p.time && l == 0) ? 1 : 0);
+        uint32_t w[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float v[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = kk * 32 + (g >> 1) * 16 + (g & 1) * 8 + 2 * (lane & 3) + h, c = tile * 8 + (lane >> 2);
+                const int out = back ? k : c, in = back ? c : k;
+                v[h] = out < p.wr[l + 1] && in < p.wr[l] ? p.theta[p.woff[l] + (long long)out * in_full + in] : 0.f;
+            }
+            w[g] = cvt_pack<T>(v[0], v[1]);
+        }
+        (back ? p.wb[l] : p.wf[l])[r] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    if (blockIdx.x == 0) {
+        for (int l = 0; l < p.L; ++l)
+            for (int c = threadIdx.x; c < p.wp[l + 1]; c += blockDim.x) {
+                const bool on = c < p.wr[l + 1];
+                if (p.bias) ((T*)p.b16[l])[c] = Low<T>::from_f(on ? p.theta[p.boff[l] + c] : 0.f);
+                if (p.time && l == 0) ((T*)p.wt16)[c] = Low<T>::from_f(on ? p.theta[p.woff[0] + (long long)c * (p.wr[0] + 1) + p.wr[0]] : 0.f);
+            }
+    }
+}
+
+// ---------------------------------------------------------------- one contraction of a block's rows
+// C[16 MT][8 tiles] = A[16 MT][32 kp] W, A in shared memory (row length lda), W packed.  Warp w takes the column tiles w, w + 8, ...,
+// four at a time; the next weights are requested before the present ones are used.  pre(g, col) runs before the reduction loop and
+// requests what the epilogue needs from memory for column tile g of the four; epi(g, m, row, col, c0, c1) gets two neighbouring columns.
+constexpr int kNG = 4;
+template <typename T, int MT, typename P, typename F>
+__device__ __forceinline__ void rows_gemm(const T* A, int lda, int kp, const uint4* __restrict__ W, int tiles, P&& pre, F&& epi) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t a0 = smem_u32(A) + (uint32_t)(((lane & 15) * lda + (lane >> 4) * 8) * 2);
+    for (int t0 = warp; t0 < tiles; t0 += kWarps * kNG) {
+        float acc[MT][kNG][4];
+        uint4 b[2][kNG];
+        auto fetch = [&](int k, uint4 (&d)[kNG]) {
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+                if (t0 + kWarps * g < tiles) d[g] = __ldg(W + ((t0 + kWarps * g) * kp + k) * 32 + lane);
+        };
+        auto step = [&](int k, const uint4 (&d)[kNG]) {
+            uint32_t a[MT][2][4];
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32) * 2), a[m][0]);
+                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32 + 16) * 2), a[m][1]);
+            }
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+                if (t0 + kWarps * g < tiles) {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][0], d[g].x, d[g].y);
+                }
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+                if (t0 + kWarps * g < tiles) {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][1], d[g].z, d[g].w);
+                }
+        };
+        fetch(0, b[0]);
+        if (kp > 1) fetch(1, b[1]);
+#pragma unroll
+        for (int g = 0; g < kNG; ++g)
+            if (t0 + kWarps * g < tiles) pre(g, (t0 + kWarps * g) * 8 + 2 * (lane & 3));
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[m][g][i] = 0.f;
+        for (int k = 0; k < kp; k += 2) {
+            {
+                uint4 cur[kNG];
+#pragma unroll
+                for (int g = 0; g < kNG; ++g) cur[g] = b[0][g];
+                if (k + 2 < kp) fetch(k + 2, b[0]);
+                step(k, cur);
+            }
+            if (k + 1 < kp) {
+                uint4 cur[kNG];
+#pragma unroll
+                for (int g = 0; g < kNG; ++g) cur[g] = b[1][g];
+                if (k + 3 < kp) fetch(k + 3, b[1]);
+                step(k + 1, cur);
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < kNG; ++g)
+            if (t0 + kWarps * g < tiles) {
+                const int col = (t0 + kWarps * g) * 8 + 2 * (lane & 3);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    epi(g, 2 * m, m * 16 + (lane >> 2), col, acc[m][g][0], acc[m][g][1]);
+                    epi(g, 2 * m + 1, m * 16 + (lane >> 2) + 8, col, acc[m][g][2], acc[m][g][3]);
+                }
+            }
+    }
+}
+
+// Shared memory of a block: two activation buffers (row length lda, zero behind the layer's width up to a multiple of 32), the stage
+// derivatives, stage cotangents, state and seed of its rows and the fp32 state or adjoint (row length wp_0), two steps' scalars, the
+// warps' sums of the time terms.
+constexpr int kScalarWords = sizeof(RkStepScalars) / sizeof(float);
+template <typename T> struct SmallSmem {
+    T *act0, *ks, *ps, *yb, *vv;
+    float *a, *scs, *red;
+    int lda, R, dp, d, half, pairs;
+    __device__ SmallSmem(const SmallMlp& p, unsigned char* base, int rows) : R(rows), dp(p.wp[0]), d(p.wr[0]) {
+        int kp = 0;
+        for (int l = 0; l <= p.L; ++l) kp = max(kp, k32(p.wp[l]));
+        lda = kp * 32 + 8;
+        half = dp / 2; pairs = R * half;
+        act0 = (T*)base;
+        ks = act0 + 2 * R * lda; ps = ks + p.stages * R * dp; yb = ps + p.stages * R * dp; vv = yb + R * dp;
+        a = (float*)(vv + R * dp);
+        scs = a + R * dp;
+        red = scs + 2 * kScalarWords;
+    }
+    __device__ __forceinline__ T* act(int i) const { return act0 + i * R * lda; }
+    __device__ __forceinline__ uint32_t* w(T* x) const { return reinterpret_cast<uint32_t*>(x); }
+    __device__ __forceinline__ const RkStepScalars& scalars(int n) const { return *(const RkStepScalars*)(scs + (n & 1) * kScalarWords); }
+};
+size_t small_smem(const SmallMlp& p, int rows) {
+    int kp = 0;
+    for (int l = 0; l <= p.L; ++l) kp = k32(p.wp[l]) > kp ? k32(p.wp[l]) : kp;
+    return (size_t)rows * 2 * (2 * (kp * 32 + 8) + (2 * p.stages + 2) * p.wp[0]) + (size_t)rows * p.wp[0] * 4 + (2 * kScalarWords + 3 * kWarps) * 4;
+}
+// a step's scalars travel to shared memory while the step before runs (asynchronous; wait with scalars_ready and a barrier)
+template <typename T>
+__device__ __forceinline__ void fetch_scalars(const SmallMlp& p, const SmallSmem<T>& sm, int n) {
+    if (threadIdx.x < kScalarWords) {
+        const float* src = (const float*)(p.scal + n) + threadIdx.x;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(sm.scs + (n & 1) * kScalarWords + threadIdx.x)), "l"(src) : "memory");
+    }
+}
+__device__ __forceinline__ void scalars_ready() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+template <typename T> __device__ __forceinline__ float lo_w(uint32_t w) { return lowf(from_bits<T>((unsigned short)(w & 0xFFFFu))); }
+template <typename T> __device__ __forceinline__ float hi_w(uint32_t w) { return lowf(from_bits<T>((unsigned short)(w >> 16))); }
+
+// zeros behind a layer's width, up to the next multiple of 32 columns
+template <typename T>
+__device__ __forceinline__ void zero_tail(T* act, int lda, int R, int w) {
+    const int pad = k32(w) * 32 - w;
+    if (pad == 0) return;
+    for (int i = threadIdx.x; i < R * pad; i += kThreads) act[(i / pad) * lda + w + i % pad] = Low<T>::from_f(0.f);
+}
+
+// All stages of one step for the rows r0 .. r0 + R - 1 from the state in sm.yb: k_j into sm.ks; with KEEP every layer input into the
+// slabs (slot `slot`).  `skip_last`: the last stage's derivative is not wanted.
+template <typename T, int MT, bool KEEP>
+__device__ __forceinline__ void small_stages(const SmallMlp& p, const SmallSmem<T>& sm, const RkStepScalars& sc, int r0, int slot, bool skip_last) {
+    const int R = 16 * MT, dp = sm.dp;
+    for (int j = 0; j < p.stages; ++j) {
+        float ha[RK_MAX_STAGES - 1];
+#pragma unroll
+        for (int l = 0; l < RK_MAX_STAGES - 1; ++l) ha[l] = l < j ? sc.ha[j][l] : 0.f;
+        T* x0 = KEEP ? (T*)p.xs[0] + ((long long)(slot * p.stages + j) * p.B + r0) * dp : nullptr;
+        for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
+            const int r = i / sm.half, c = 2 * (i - r * sm.half);
+            uint32_t q = sm.w(sm.yb)[i];
+            if (j > 0) {
+                float v0 = lo_w<T>(q), v1 = hi_w<T>(q);
+#pragma unroll
+                for (int l = 0; l < RK_MAX_STAGES - 1; ++l)
+                    if (l < j && ha[l] != 0.f) {
+                        const uint32_t k = sm.w(sm.ks)[l * sm.pairs + i];
+                        v0 = fmaf(ha[l], lo_w<T>(k), v0);
+                        v1 = fmaf(ha[l], hi_w<T>(k), v1);
+                    }
+                q = cvt_pack<T>(v0, v1);
+            }
+            *(uint32_t*)(sm.act(0) + r * sm.lda + c) = q;
+            if (KEEP && r0 + r < p.B) *(uint32_t*)(x0 + r * dp + c) = q;
+        }
+        zero_tail(sm.act(0), sm.lda, R, dp);
+        __syncthreads();
+        const float tau = sc.tau16[j];
+        for (int l = 0; l < p.L; ++l) {
+            const bool last = l == p.L - 1;
+            if (last && skip_last && j == p.stages - 1) break;
+            const int N = p.wp[l + 1];
+            const uint32_t* b16 = p.bias ? (const uint32_t*)p.b16[l] : nullptr;
+            const uint32_t* wt = p.time && l == 0 ? (const uint32_t*)p.wt16 : nullptr;
+            T* dst = last ? sm.ks + j * R * dp : sm.act((l + 1) & 1);
+            const int ld = last ? dp : sm.lda;
+            T* keep = KEEP && !last ? (T*)p.xs[l + 1] + ((long long)(slot * p.stages + j) * p.B + r0) * N : nullptr;
+            float2 bv[kNG];
+            rows_gemm<T, MT>(
+                sm.act(l & 1), sm.lda, k32(p.wp[l]), p.wf[l], N / 8,
+                [&](int g, int c) {
+                    bv[g] = make_float2(0.f, 0.f);
+                    if (b16 != nullptr) { const uint32_t w = __ldg(b16 + c / 2); bv[g] = make_float2(lo_w<T>(w), hi_w<T>(w)); }
+                    if (wt != nullptr) { const uint32_t w = __ldg(wt + c / 2); bv[g].x = fmaf(tau, lo_w<T>(w), bv[g].x); bv[g].y = fmaf(tau, hi_w<T>(w), bv[g].y); }
+                },
+                [&](int g, int, int r, int c, float v0, float v1) {
+                    v0 += bv[g].x; v1 += bv[g].y;
+                    if (!last) { v0 = act_f(p.act, v0); v1 = act_f(p.act, v1); }
+                    const uint32_t w = cvt_pack<T>(v0, v1);
+                    *(uint32_t*)(dst + r * ld + c) = w;
+                    if (KEEP && !last && r0 + r < p.B) *(uint32_t*)(keep + (long long)r * N + c) = w;
+                });
+            if (!last) zero_tail(dst, sm.lda, R, N);
+            __syncthreads();
+        }
+    }
+}
+
+template <typename T, int MT>
+__global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_constant__ SmallMlp p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int R = 16 * MT, r0 = blockIdx.x * R;
+    const SmallSmem<T> sm(p, smem, R);
+    const int d = sm.d, dp = sm.dp;
+    T* traj = (T*)p.traj;
+    fetch_scalars(p, sm, 0);
+    for (int i = threadIdx.x; i < R * dp; i += kThreads) {
+        const int r = i / dp, c = i - r * dp;
+        const bool on = r0 + r < p.B && c < d;
+        const float y = on ? p.y0[(long long)(r0 + r) * d + c] : 0.f;
+        const T q = Low<T>::from_f(y);
+        sm.yb[i] = q;
+        sm.a[i] = y;
+        if (on) traj[(long long)(r0 + r) * d + c] = q;
+    }
+    for (int n = 0; n < p.n_steps; ++n) {
+        scalars_ready();
+        __syncthreads();
+        if (n + 1 < p.n_steps) fetch_scalars(p, sm, n + 1);
+        const RkStepScalars& sc = sm.scalars(n);
+        small_stages<T, MT, false>(p, sm, sc, r0, 0, false);
+        float hb[RK_MAX_STAGES];
+#pragma unroll
+        for (int j = 0; j < RK_MAX_STAGES; ++j) hb[j] = j < p.stages ? sc.hb[j] : 0.f;
+        const float h = sc.h;
+        T* tn = traj + ((long long)(n + 1) * p.B + r0) * d;
+        for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
+            const int r = i / sm.half, c = 2 * (i - r * sm.half);
+            float v0 = 0.f, v1 = 0.f;
+#pragma unroll
+            for (int j = 0; j < RK_MAX_STAGES; ++j)
+                if (j < p.stages) {
+                    const uint32_t k = sm.w(sm.ks)[j * sm.pairs + i];
+                    v0 = fmaf(hb[j], lo_w<T>(k), v0);
+                    v1 = fmaf(hb[j], hi_w<T>(k), v1);
+                }
+            float2 y = reinterpret_cast<float2*>(sm.a)[i];
+            y.x += p.round_increment ? h * q16<T>(v0) : v0;
+            y.y += p.round_increment ? h * q16<T>(v1) : v1;
+            reinterpret_cast<float2*>(sm.a)[i] = y;
+            const uint32_t q = cvt_pack<T>(y.x, y.y);
+            sm.w(sm.yb)[i] = q;
+            if (r0 + r < p.B && c < d) {
+                if ((d & 1) == 0) *(uint32_t*)(tn + r * d + c) = q;
+                else {
+                    tn[r * d + c] = from_bits<T>((unsigned short)(q & 0xFFFFu));
+                    if (c + 1 < d) tn[r * d + c + 1] = from_bits<T>((unsigned short)(q >> 16));
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < R * d; i += kThreads) {
+        const int r = i / d, c = i - r * d;
+        if (r0 + r < p.B) p.yT[(long long)r0 * d + i] = sm.a[r * dp + c];
+    }
+}
+
+// The backward chain of `count` steps for a block's rows: recompute, seed, stage cotangents and layer cotangents; with commit also the
+// adjoint update, after which the next step follows at once.  Without commit (dynamic scaling: one step per launch, the update waits for
+// the finiteness decision) psi_j goes to memory.  With tpart also the block's share of the step's time terms: Phi^T a with
+// Phi = sum_j b_j k_j, dt = sum_j dtau_j and dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>), dtau_j = <dZ_1, w_t>.
+template <typename T, int MT>
+__global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_constant__ SmallMlp p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int R = 16 * MT, r0 = blockIdx.x * R;
+    const SmallSmem<T> sm(p, smem, R);
+    const int d = sm.d, dp = sm.dp;
+    const T* traj = (const T*)p.traj;
+    const float lim = OverflowLimit<T>::value();
+    const int e = p.e_dev != nullptr ? *p.e_dev : p.e;
+    const bool want_t = p.tpart != nullptr;
+    bool bad = false;
+    fetch_scalars(p, sm, p.step_hi);
+    if (p.vjp) {
+        for (int i = threadIdx.x; i < R * dp; i += kThreads) {
+            const int r = i / dp, c = i - r * dp;
+            sm.a[i] = r0 + r < p.B && c < d ? p.a[(long long)(r0 + r) * d + c] : 0.f;
+        }
+    }
+    for (int s = 0; s < p.count; ++s) {
+        const int n = p.step_hi - s;
+        scalars_ready();
+        __syncthreads();
+        if (s + 1 < p.count) fetch_scalars(p, sm, n - 1);
+        const RkStepScalars& sc = sm.scalars(n);
+        float t_phi = 0.f, t_dt = 0.f, t_dh = 0.f;
+        if (p.recompute) {
+            const T* tn = traj + ((long long)n * p.B + r0) * d;
+            for (int i = threadIdx.x; i < R * dp; i += kThreads) {
+                const int r = i / dp, c = i - r * dp;
+                sm.yb[i] = r0 + r < p.B && c < d ? tn[r * d + c] : Low<T>::from_f(0.f);
+            }
+            __syncthreads();
+            small_stages<T, MT, true>(p, sm, sc, r0, s, !want_t);
+        }
+        if (!p.vjp) continue;
+        for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {       // seed Q16(S a)
+            const float2 a = reinterpret_cast<const float2*>(sm.a)[i];
+            const float v0 = ldexpf(a.x, e), v1 = ldexpf(a.y, e);
+            bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
+            sm.w(sm.vv)[i] = cvt_pack<T>(v0, v1);
+            if (want_t) {
+                float p0 = 0.f, p1 = 0.f;
+                for (int j = 0; j < p.stages; ++j) {
+                    const uint32_t k = sm.w(sm.ks)[j * sm.pairs + i];
+                    p0 = fmaf(sc.b[j], lo_w<T>(k), p0);
+                    p1 = fmaf(sc.b[j], hi_w<T>(k), p1);
+                }
+                t_phi = fmaf(p0, a.x, fmaf(p1, a.y, t_phi));
+            }
+        }
+        for (int j = p.stages - 1; j >= 0; --j) {
+            // kappa_j = Q16(b_j v + sum_{l > j} (h a_lj) psi_l): each thread reads what it wrote itself, or what a barrier lies behind
+            float ha[RK_MAX_STAGES];
+#pragma unroll
+            for (int l = 1; l < RK_MAX_STAGES; ++l) ha[l] = l > j && l < p.stages ? sc.ha[l][j] : 0.f;
+            const float bj = sc.b[j], cj = sc.c[j];
+            float dtau = 0.f;
+            T* kap = (T*)p.zs[p.L] + ((long long)(s * p.stages + j) * p.B + r0) * dp;
+            const uint32_t* wt = want_t && p.time ? (const uint32_t*)p.wt16 : nullptr;
+            for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
+                const int r = i / sm.half, c = 2 * (i - r * sm.half);
+                const uint32_t v = sm.w(sm.vv)[i];
+                float v0 = bj * lo_w<T>(v), v1 = bj * hi_w<T>(v);
+#pragma unroll
+                for (int l = 1; l < RK_MAX_STAGES; ++l)
+                    if (ha[l] != 0.f) {
+                        const uint32_t q = sm.w(sm.ps)[l * sm.pairs + i];
+                        v0 = fmaf(ha[l], lo_w<T>(q), v0);
+                        v1 = fmaf(ha[l], hi_w<T>(q), v1);
+                    }
+                bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
+                const uint32_t q = cvt_pack<T>(v0, v1);
+                *(uint32_t*)(sm.act(0) + r * sm.lda + c) = q;
+                if (r0 + r < p.B) *(uint32_t*)(kap + r * dp + c) = q;
+                if (p.L == 1 && wt != nullptr) {
+                    const uint32_t w = __ldg(wt + c / 2);
+                    dtau = fmaf(lo_w<T>(q), lo_w<T>(w), fmaf(hi_w<T>(q), hi_w<T>(w), dtau));
+                }
+            }
+            zero_tail(sm.act(0), sm.lda, R, dp);
+            __syncthreads();
+            int cur = 0;
+            for (int l = p.L - 1; l >= 0; --l, cur ^= 1) {
+                const int N = p.wp[l];
+                const long long at = ((long long)(s * p.stages + j) * p.B + r0) * N;
+                const T* H = l > 0 ? (const T*)p.xs[l] + at : nullptr;
+                T* Z = l > 0 ? (T*)p.zs[l] + at : (p.commit ? nullptr : (T*)p.psi[j] + (long long)r0 * dp);
+                T* dst = l > 0 ? sm.act(cur ^ 1) : sm.ps + j * R * dp;
+                const int ld = l > 0 ? sm.lda : dp;
+                uint32_t hw[kNG][2 * MT];
+                rows_gemm<T, MT>(
+                    sm.act(cur), sm.lda, k32(p.wp[l + 1]), p.wb[l], N / 8,
+                    [&](int g, int c) {      // the stored layer outputs whose activation derivative multiplies the result
+#pragma unroll
+                        for (int q = 0; q < 2 * MT; ++q) {
+                            const int r = q * 8 + ((threadIdx.x & 31) >> 2);
+                            hw[g][q] = l > 0 && r0 + r < p.B ? *(const uint32_t*)(H + (long long)r * N + c) : 0u;
+                        }
+                    },
+                    [&](int g, int q, int r, int c, float v0, float v1) {
+                        if (l > 0) {
+                            v0 *= act_df(p.act, lo_w<T>(hw[g][q]));
+                            v1 *= act_df(p.act, hi_w<T>(hw[g][q]));
+                        }
+                        bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
+                        const uint32_t w = cvt_pack<T>(v0, v1);
+                        *(uint32_t*)(dst + r * ld + c) = w;
+                        if (Z != nullptr && r0 + r < p.B) *(uint32_t*)(Z + (long long)r * N + c) = w;
+                        if (l == 1 && wt != nullptr) {
+                            const uint32_t t = __ldg(wt + c / 2);
+                            dtau = fmaf(lo_w<T>(w), lo_w<T>(t), fmaf(hi_w<T>(w), hi_w<T>(t), dtau));
+                        }
+                    });
+                if (l > 0) zero_tail(dst, sm.lda, R, N);
+                __syncthreads();
+            }
+            if (want_t) {
+                t_dt += dtau;
+                t_dh = fmaf(cj, dtau, t_dh);
+                for (int l = 0; l < j; ++l) {
+                    const float ajl = sc.a[j][l];
+                    if (ajl == 0.f) continue;
+                    float dot = 0.f;
+                    for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
+                        const uint32_t q = sm.w(sm.ps)[j * sm.pairs + i], k = sm.w(sm.ks)[l * sm.pairs + i];
+                        dot = fmaf(lo_w<T>(q), lo_w<T>(k), fmaf(hi_w<T>(q), hi_w<T>(k), dot));
+                    }
+                    t_dh = fmaf(ajl, dot, t_dh);
+                }
+            }
+        }
+        if (p.commit) {      // a <- a + (h / S) sum_j psi_j (+ running cost)
+            const float coef = ldexpf(sc.h, -e);
+            for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
+                float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                for (int j = RK_MAX_STAGES - 1; j >= 0; --j)
+                    if (j < p.stages) {
+                        const uint32_t q = sm.w(sm.ps)[j * sm.pairs + i];
+                        d0 += lo_w<T>(q);
+                        d1 += hi_w<T>(q);
+                    }
+                float2 a = reinterpret_cast<float2*>(sm.a)[i];
+                a.x = fmaf(coef, d0, a.x); a.y = fmaf(coef, d1, a.y);
+                if (p.cot != nullptr) {
+                    const int r = i / sm.half, c = 2 * (i - r * sm.half);
+                    const float* ct = p.cot + ((long long)n * p.B + r0 + r) * d + c;
+                    if (r0 + r < p.B && c < d) a.x += ct[0];
+                    if (r0 + r < p.B && c + 1 < d) a.y += ct[1];
+                }
+                reinterpret_cast<float2*>(sm.a)[i] = a;
+            }
+        }
+        if (want_t) {      // lanes by shuffles, warps in ascending order
+            const int warp = threadIdx.x >> 5;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                t_phi += __shfl_xor_sync(0xffffffffu, t_phi, o);
+                t_dt += __shfl_xor_sync(0xffffffffu, t_dt, o);
+                t_dh += __shfl_xor_sync(0xffffffffu, t_dh, o);
+            }
+            if ((threadIdx.x & 31) == 0) { sm.red[warp] = t_phi; sm.red[kWarps + warp] = t_dt; sm.red[2 * kWarps + warp] = t_dh; }
+            __syncthreads();
+            if (threadIdx.x < 3) {
+                float x = 0.f;
+                for (int w = 0; w < kWarps; ++w) x += sm.red[threadIdx.x * kWarps + w];
+                p.tpart[((long long)s * gridDim.x + blockIdx.x) * 3 + threadIdx.x] = x;
+            }
+        }
+    }
+    if (p.commit) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < R * d; i += kThreads) {
+            const int r = i / d, c = i - r * d;
+            if (r0 + r < p.B) p.a[(long long)r0 * d + i] = sm.a[r * dp + c];
+        }
+    }
+    warp_flag_or(p.flag, bad);
+}
+
+// The time terms of the chunk's steps: the blocks' shares added in a fixed order; values {Phi^T a, dt, dh} of the last step to tvals, and
+// with tprime the two t' updates of Alg. 2 per step.  Q16(dt), Q16(dh) join the finiteness test.
+template <typename T>
+__global__ void __launch_bounds__(96) small_time_kernel(SmallMlp p, int blocks) {
+    __shared__ float v[3];
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int s = 0; s < p.count; ++s) {
+        float x = 0.f;
+        for (int b = lane; b < blocks; b += 32) x += p.tpart[((long long)s * blocks + b) * 3 + q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        __syncthreads();
+        if (lane == 0) v[q] = x;
+        __syncthreads();
+        if (threadIdx.x != 0) continue;
+        const float phi = v[0], dt = v[1], dh = v[2];
+        if (p.flag != nullptr && (Low<T>::nonfinite(Low<T>::from_f(dt)) || Low<T>::nonfinite(Low<T>::from_f(dh)))) atomicOr(p.flag, 1u);
+        if (p.tvals != nullptr) { p.tvals[0] = phi; p.tvals[1] = dt; p.tvals[2] = dh; }
+        if (p.tprime != nullptr) {
+            const int n = p.step_hi - s;
+            p.tprime[n] = p.tprime[n] + p.coef[s] * (dt - dh) - phi;
+            p.tprime[n + 1] = p.tprime[n + 1] + p.coef[s] * dh + phi;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- weight, bias and time-column gradients
+// One block per TM x TN piece of a layer's dW_l = sum over the rows of dZ_{l+1}^T X_l.  The rows of all stages of a step are one matrix
+// of stages * B rows; warp w takes the groups of 16 rows w, w + 8, ... through its own ring of asynchronous copies, so that no barrier
+// stands in the loop; the eight sums meet in shared memory in ascending order.  The bias gradient and the time column are two more
+// columns (ones, stage times) of the pieces in the first column of pieces.
+constexpr int kRing = 8;
+struct WgradItems { int first[SMALL_MAX_L + 1]; };
+template <typename T, int TM, int TN>
+__global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ WgradItems items) {
+    constexpr int LA = TM + 8, LB = TN + 8;                       // row lengths in shared memory: eight rows hit eight 16-byte slots
+    constexpr int kStage = 16 * (LA + LB);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    T* ring = (T*)smem + (size_t)warp * kRing * kStage;
+    int l = 0;
+    while ((int)blockIdx.x >= items.first[l + 1]) ++l;
+    const int M = p.wp[l + 1], N = p.wp[l], tn = (N + TN - 1) / TN;
+    const int tile = (int)blockIdx.x - items.first[l], m0 = (tile / tn) * TM, n0 = (tile % tn) * TN;
+    const bool time = p.time && l == 0, sums = n0 == 0 && (p.bias || time);
+    const int KR = p.stages * p.B;
+    const int groups = (KR + 15) / 16, per = (groups + kWarps - 1) / kWarps;      // groups of this step for each warp
+    const int total = per * p.count;
+    const T* Z = (const T*)p.zs[l + 1];
+    const T* X = (const T*)p.xs[l];
+    auto fetch = [&](int it) {
+        if (it < total) {
+            const int s = it / per, g = (it - s * per) * kWarps + warp;
+            T* dst = ring + (it % kRing) * kStage;
+            const T* zs = Z + (long long)s * KR * M;
+            const T* xs = X + (long long)s * KR * N;
+            constexpr int PA = TM / 8, PB = TN / 8;
+#pragma unroll
+            for (int q = lane; q < 16 * (PA + PB); q += 32) {
+                const bool isA = q < 16 * PA;
+                const int r = isA ? q / PA : (q - 16 * PA) / PB, c = 8 * (isA ? q % PA : (q - 16 * PA) % PB);
+                const int row = g * 16 + r;
+                const bool on = row < KR && (isA ? m0 + c < M : n0 + c < N);
+                const T* src = isA ? zs + (long long)row * M + m0 + c : xs + (long long)row * N + n0 + c;
+                cp_async16(smem_u32(dst + (isA ? r * LA : 16 * LA + r * LB) + c), on ? src : (isA ? Z : X), on);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float tot[TM / 16][TN / 8][4], acc[TM / 16][TN / 8][4], stot[TM / 16][4], sacc[TM / 16][4];
+#pragma unroll
+    for (int m = 0; m < TM / 16; ++m)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            stot[m][i] = sacc[m][i] = 0.f;
+#pragma unroll
+            for (int q = 0; q < TN / 8; ++q) tot[m][q][i] = acc[m][q][i] = 0.f;
+        }
+#pragma unroll
+    for (int k = 0; k < kRing - 1; ++k) fetch(k);
+    for (int it = 0; it < total; ++it) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
+        __syncwarp();
+        const T* buf = ring + (it % kRing) * kStage;
+        const int s = it / per, gi = it - s * per;
+        // fragments of dZ^T (rows = columns of dZ) and X from [16 rows][columns] blocks: transposing loads
+        uint32_t a[TM / 16][4], b[TN / 16][4];
+        const int r8 = lane & 7, id = lane >> 3;
+#pragma unroll
+        for (int m = 0; m < TM / 16; ++m) ldmatrix4_trans(smem_u32(buf + (r8 + (id >> 1) * 8) * LA + m * 16 + (id & 1) * 8), a[m]);
+#pragma unroll
+        for (int q = 0; q < TN / 16; ++q) ldmatrix4_trans(smem_u32(buf + 16 * LA + (r8 + (id & 1) * 8) * LB + q * 16 + (id >> 1) * 8), b[q]);
+#pragma unroll
+        for (int m = 0; m < TM / 16; ++m)
+#pragma unroll
+            for (int q = 0; q < TN / 8; ++q) mma16816<T>(acc[m][q], a[m], b[q >> 1][2 * (q & 1)], b[q >> 1][2 * (q & 1) + 1]);
+        if (sums) {      // column 0: ones, column 1: the rounded stage time of the row
+            uint32_t o0 = 0u, o1 = 0u;
+            const int c = lane >> 2;
+            if (c == 0) o0 = o1 = cvt_pack<T>(1.f, 1.f);
+            else if (c == 1 && time) {
+                const RkStepScalars& sc = p.scal[p.step_hi - s];
+                float t[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int row = (gi * kWarps + warp) * 16 + 2 * (lane & 3) + (i & 1) + (i >> 1) * 8;
+                    t[i] = row < KR ? sc.tau16[row / p.B] : 0.f;
+                }
+                o0 = cvt_pack<T>(t[0], t[1]);
+                o1 = cvt_pack<T>(t[2], t[3]);
+            }
+#pragma unroll
+            for (int m = 0; m < TM / 16; ++m) mma16816<T>(sacc[m], a[m], o0, o1);
+        }
+        __syncwarp();
+        fetch(it + kRing - 1);
+        if (gi == per - 1) {      // the step is complete
+            const float cf = p.coef[s];
+#pragma unroll
+            for (int m = 0; m < TM / 16; ++m)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    stot[m][i] = fmaf(cf, sacc[m][i], stot[m][i]); sacc[m][i] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < TN / 8; ++q) { tot[m][q][i] = fmaf(cf, acc[m][q][i], tot[m][q][i]); acc[m][q][i] = 0.f; }
+                }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    constexpr int LR = TN + 3;                                    // row of sums: TN columns, bias, time (odd stride)
+    float* red = (float*)smem;                                    // [warps][TM][LR]
+#pragma unroll
+    for (int m = 0; m < TM / 16; ++m)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = m * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
+            float* row = red + ((size_t)warp * TM + r) * LR;
+#pragma unroll
+            for (int q = 0; q < TN / 8; ++q) row[q * 8 + c] = tot[m][q][i];
+            if (c < 2) row[TN + c] = stot[m][i];
+        }
+    __syncthreads();
+    const int in_full = p.wr[l] + (time ? 1 : 0);
+    for (int i = threadIdx.x; i < TM * (TN + 2); i += kThreads) {
+        const int r = i / (TN + 2), c = i - r * (TN + 2), m = m0 + r, n = n0 + c;
+        if (m >= p.wr[l + 1]) continue;
+        long long at;
+        if (c < TN) {
+            if (n >= p.wr[l]) continue;
+            at = p.woff[l] + (long long)m * in_full + n;
+        } else if (c == TN) {
+            if (!sums || !p.bias) continue;
+            at = p.boff[l] + m;
+        } else {
+            if (!sums || !time) continue;
+            at = p.woff[l] + (long long)m * in_full + p.wr[l];
+        }
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) v += red[((size_t)w * TM + r) * LR + c];
+        p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + v;
+    }
+}
+
+template <typename K>
+bool allow_smem(K kernel, bool (&done)[kMaxDevices]) {
+    const int dev = current_device();
+    if (!done[dev]) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) { cudaGetLastError(); return false; }
+        done[dev] = true;
+    }
+    return true;
+}
+
+// rows per block: 16 while that is at most one block per SM, else 32 (half the weight traffic per row)
+int rows_tiles(int B) { return (B + 15) / 16 <= sm_count() ? 1 : 2; }
+
+template <typename T, int MT>
+bool forward_t(const SmallMlp& p, cudaStream_t st) {
+    static bool done[kMaxDevices] = {false};
+    if (!allow_smem(small_forward_kernel<T, MT>, done)) return false;
+    small_forward_kernel<T, MT><<<(p.B + 16 * MT - 1) / (16 * MT), kThreads, small_smem(p, 16 * MT), st>>>(p);
+    return true;
+}
+template <typename T, int MT>
+bool backward_t(const SmallMlp& p, cudaStream_t st) {
+    static bool done[kMaxDevices] = {false};
+    if (!allow_smem(small_backward_kernel<T, MT>, done)) return false;
+    small_backward_kernel<T, MT><<<(p.B + 16 * MT - 1) / (16 * MT), kThreads, small_smem(p, 16 * MT), st>>>(p);
+    return true;
+}
+template <typename T, int TM>
+bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st) {
+    static bool done[kMaxDevices] = {false};
+    if (!allow_smem(small_wgrad_kernel<T, TM, TM>, done)) return false;
+    const size_t ring = (size_t)kWarps * kRing * 16 * 2 * (TM + 8) * sizeof(T), red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
+    small_wgrad_kernel<T, TM, TM><<<items.first[p.L], kThreads, ring > red ? ring : red, st>>>(p, items);
+    return true;
+}
+WgradItems wgrad_items(const SmallMlp& p, int tm) {
+    WgradItems it{};
+    for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + tm - 1) / tm) * ((p.wp[l] + tm - 1) / tm);
+    return it;
+}
+
+}  // namespace
+
+size_t small_pack_bytes(int L, const int* wp) {
+    size_t n = 0;
+    for (int l = 0; l < L; ++l) n += (size_t)32 * ((wp[l + 1] / 8) * k32(wp[l]) + (wp[l] / 8) * k32(wp[l + 1]));
+    return n * sizeof(uint4);
+}
+
+bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp) {
+    if (dt != MPODE_BF16 && dt != MPODE_F16) return false;
+    if (L < 1 || L > SMALL_MAX_L) return false;
+    SmallMlp p{};
+    p.L = L; p.stages = RK_MAX_STAGES;
+    long long elems = 0;
+    for (int l = 0; l <= L; ++l) { p.wp[l] = p.wr[l] = wp[l]; if (l < L) elems += (long long)wp[l] * wp[l + 1]; }
+    return small_smem(p, 32) <= 200 * 1024 && elems <= 160 * 1024 && B <= 8192;
+}
+
+void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    PackJob job{};
+    for (int l = 0; l < p.L; ++l) {
+        job.first[2 * l + 1] = job.first[2 * l] + (long long)32 * (p.wp[l + 1] / 8) * k32(p.wp[l]);
+        job.first[2 * l + 2] = job.first[2 * l + 1] + (long long)32 * (p.wp[l] / 8) * k32(p.wp[l + 1]);
+    }
+    long long blocks = (job.first[2 * p.L] + 255) / 256;
+    if (blocks > 148 * 4) blocks = 148 * 4;
+    if (dt == MPODE_BF16) small_pack_kernel<__nv_bfloat16><<<(int)blocks, 256, 0, st>>>(p, job);
+    else small_pack_kernel<__half><<<(int)blocks, 256, 0, st>>>(p, job);
+    if (launches) ++*launches;
+}
+
+bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    const bool one = rows_tiles(p.B) == 1;
+    const bool ok = dt == MPODE_BF16 ? (one ? forward_t<__nv_bfloat16, 1>(p, st) : forward_t<__nv_bfloat16, 2>(p, st))
+                                     : (one ? forward_t<__half, 1>(p, st) : forward_t<__half, 2>(p, st));
+    if (ok && launches) ++*launches;
+    if (ok && tl_counters) ++tl_counters->fused;
+    return ok;
+}
+
+bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    const bool one = rows_tiles(p.B) == 1;
+    const bool ok = dt == MPODE_BF16 ? (one ? backward_t<__nv_bfloat16, 1>(p, st) : backward_t<__nv_bfloat16, 2>(p, st))
+                                     : (one ? backward_t<__half, 1>(p, st) : backward_t<__half, 2>(p, st));
+    if (ok && launches) ++*launches;
+    if (ok && tl_counters) ++tl_counters->fused;
+    return ok;
+}
+
+int small_blocks(int B) { return (B + 16 * rows_tiles(B) - 1) / (16 * rows_tiles(B)); }
+
+void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    if (dt == MPODE_BF16) small_time_kernel<__nv_bfloat16><<<1, 96, 0, st>>>(p, small_blocks(p.B));
+    else small_time_kernel<__half><<<1, 96, 0, st>>>(p, small_blocks(p.B));
+    if (launches) ++*launches;
+}
+
+bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    // 32 x 32 pieces where there are enough of them to occupy half the SMs, else 16 x 16 (each block reads its operands from L2: a
+    // smaller piece reads more in total but less per block)
+    WgradItems items = wgrad_items(p, 32);
+    const bool wide = items.first[p.L] >= sm_count() / 2;
+    if (!wide) items = wgrad_items(p, 16);
+    const bool ok = dt == MPODE_BF16 ? (wide ? wgrad_t<__nv_bfloat16, 32>(p, items, st) : wgrad_t<__nv_bfloat16, 16>(p, items, st))
+                                     : (wide ? wgrad_t<__half, 32>(p, items, st) : wgrad_t<__half, 16>(p, items, st));
+    if (ok && launches) ++*launches;
+    if (ok && tl_counters) ++tl_counters->fused;
+    return ok;
+}
+
+}  // namespace mpode

@@ -5,6 +5,7 @@
 #include "gemm_tc.h"
 #include "hyper_cnf.h"
 #include "profiler.h"
+#include "small_mlp.h"
 #include "tensormap.h"
 #include "tiny_mlp.h"
 #include "velocity.h"
@@ -148,6 +149,64 @@ public:
         }
         wgpart_ = lay.take(wg);
         wgpart_bytes_ = wg;
+        plan_small(lay);
+    }
+
+    // Row-local kernels (small_mlp.cu): packed weights, and the layer inputs and cotangents of a few steps at a time (8 MB at most, or
+    // one step's)
+    void plan_small(Layout& lay) {
+        small_ok_ = !tiny_ok_ && small_mlp_supported(dt_, B_, L_, wp_.data());
+        if (!small_ok_) return;
+        const size_t es = low_size(dt_);
+        size_t per_step = 0;
+        for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (wp_[l] + wp_[l + 1]) * es;
+        small_chunk_ = (int)(((size_t)8 << 20) / per_step);
+        if (small_chunk_ < 1) small_chunk_ = 1;
+        if (small_chunk_ > SMALL_MAX_CHUNK) small_chunk_ = SMALL_MAX_CHUNK;
+        if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
+        small_pack_ = lay.take(small_pack_bytes(L_, wp_.data()));
+        small_scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
+        for (int l = 0; l < L_; ++l) {
+            small_xs_[l] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * wp_[l] * es);
+            small_zs_[l + 1] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * wp_[l + 1] * es);
+        }
+        if (lay.time_gradient) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(B_) * 3 * sizeof(float));
+    }
+    SmallMlp small_params(void* ws) const {
+        SmallMlp p{};
+        p.B = B_; p.L = L_; p.act = act_; p.time = time_ ? 1 : 0; p.bias = bias_ ? 1 : 0;
+        p.theta = theta_;
+        size_t off = small_pack_;
+        for (int l = 0; l <= L_; ++l) { p.wr[l] = w_[l]; p.wp[l] = wp_[l]; }
+        for (int l = 0; l < L_; ++l) {
+            p.woff[l] = (long long)woff_[l]; p.boff[l] = (long long)boff_[l];
+            p.wf[l] = (uint4*)at(ws, off); off += (size_t)512 * (wp_[l + 1] / 8) * ((wp_[l] + 31) / 32);
+            p.wb[l] = (uint4*)at(ws, off); off += (size_t)512 * (wp_[l] / 8) * ((wp_[l + 1] + 31) / 32);
+            p.b16[l] = bias_ ? at(ws, b16_[l]) : nullptr;
+            p.xs[l] = at(ws, small_xs_[l]); p.zs[l + 1] = at(ws, small_zs_[l + 1]);
+        }
+        p.wt16 = time_ ? at(ws, wt16_) : nullptr;
+        p.scal = (const RkStepScalars*)at(ws, small_scal_);
+        for (int j = 0; j < 4; ++j) p.psi[j] = at(ws, lay_->psi[j]);
+        return p;
+    }
+    SmallMlp small_solve(cudaStream_t st, void* ws, const FusedSolve& fs) const {
+        cudaMemcpyAsync(at(ws, small_scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
+        SmallMlp p = small_params(ws);
+        p.stages = fs.stages; p.n_steps = fs.n_steps; p.round_increment = fs.round_increment; p.traj = const_cast<void*>(fs.traj);
+        return p;
+    }
+    // the test of the bounded waits (starve) is about the kernel that has them
+    bool small_usable(const FusedSolve& fs) const {
+        return small_ok_ && !fs.starve && fs.stages <= RK_MAX_STAGES && fs.n_steps <= max_steps_ && ((uintptr_t)fs.traj & 31) == 0;
+    }
+    template <typename F> bool small_timed(int klass, double flops, cudaStream_t st, F&& launch) {
+        Profiler* pr = tl_profiler;
+        const bool timed = pr != nullptr && pr->enabled;
+        if (timed) pr->begin(klass, flops, st);
+        const bool ok = launch();
+        if (timed) pr->end(st);
+        return ok;
     }
 
     // Weight-gradient tiling of the fused backward: every layer's dW tiles (128 x bn) times a common number of batch
@@ -176,6 +235,16 @@ public:
     }
 
     void prepare(cudaStream_t st, void* ws, const float* theta, const signed char*, long long* L) override {
+        theta_ = theta;
+        quantized_ = false;
+        if (small_ok_) launch_small_pack(dt_, small_params(ws), st, L);      // the other forms only if a pass turns out to need them
+        else quantize(st, ws, L);
+    }
+    // Q16(theta) in the layouts of the tensor-core and CUDA-core contractions, once per pass
+    void quantize(cudaStream_t st, void* ws, long long* L) {
+        if (quantized_) return;
+        quantized_ = true;
+        const float* theta = theta_;
         for (int l = 0; l < L_; ++l) {
             int in_full = w_[l] + ((time_ && l == 0) ? 1 : 0);
             launch_quantize_matrix(dt_, theta + woff_[l], in_full, w_[l + 1], w_[l], at(ws, W16_[l]), at(ws, W16T_[l]), st, L, wp_[l + 1], wp_[l]);
@@ -186,6 +255,7 @@ public:
     }
 
     void forward(cudaStream_t st, void* ws, int j, const void* yin, float tau16, long long* L) override {
+        quantize(st, ws, L);
         const void* X = yin;
         for (int l = 0; l < L_; ++l) {
             GemmArgs g = base_args(ws, lay_);
@@ -324,6 +394,12 @@ public:
     }
 
     bool fused_forward(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
+        if (small_usable(fs)) {
+            SmallMlp p = small_solve(st, ws, fs);
+            p.y0 = p.yT = fs.y;                       // the driver has put y_0 there
+            if (small_timed(0, (double)fs.n_steps * fs.stages * layer_flops(), st, [&] { return launch_small_forward(dt_, p, st, L); })) return true;
+        }
+        quantize(st, ws, L);
         if (!fused_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
         if (((uintptr_t)fs.traj & 31) != 0) return false;       // the epilogues move 32-byte pieces of trajectory rows
         const int s = fs.stages, d = wp_[0];
@@ -387,7 +463,14 @@ public:
     // ---- fused backward: per step one launch that recomputes the stages (keeping every layer output) and one launch
     // per attempt for the vector-Jacobian products and weight gradients.  begin() builds both phase tables.
     bool fused_backward_begin(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
-        (void)L;
+        b_small_ = small_usable(fs);
+        if (b_small_) {
+            small_bwd_ = small_solve(st, ws, fs);
+            b_stages_ = fs.stages;
+            scal_host_ = fs.scalars;
+            return true;
+        }
+        quantize(st, ws, L);
         if (!fused_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
         if (((uintptr_t)fs.traj & 31) != 0) return false;
         const int s = fs.stages, d = wp_[0];
@@ -530,7 +613,48 @@ public:
         return true;
     }
 
+    bool fused_seeds_itself(const float* a, int e, const int* e_dev) override {
+        if (!b_small_) return false;
+        small_bwd_.a = const_cast<float*>(a); small_bwd_.e = e; small_bwd_.e_dev = e_dev;
+        return true;
+    }
+
+    bool fused_has_time_terms() const override { return b_small_; }
+    bool fused_time_terms(cudaStream_t st, float* tvals, unsigned* flag, long long* L) override {
+        if (!b_small_) return false;
+        SmallMlp p = small_step_;
+        p.tvals = tvals; p.flag = flag;
+        launch_small_time(dt_, p, st, L);
+        return true;
+    }
+
+    // Chunks of steps: one launch for the chain of stages of all rows, one for the weight gradients of the chunk's steps
+    bool fused_backward_all(cudaStream_t st, void* ws, const FusedSolve& fs, float* a, float* g, const float* cot, int e, unsigned* flag,
+                            float* tprime, long long* L) override {
+        if (!b_small_) return false;
+        SmallMlp p = small_bwd_;
+        p.a = a; p.cot = cot; p.e = e; p.e_dev = nullptr; p.flag = flag; p.recompute = p.vjp = p.commit = 1;
+        p.out = g; p.beta = 1.f;
+        if (tprime != nullptr) { p.tpart = (float*)at(ws, small_tpart_); p.tprime = tprime; }
+        for (int hi = fs.n_steps - 1; hi >= 0; hi -= small_chunk_) {
+            p.step_hi = hi;
+            p.count = hi + 1 < small_chunk_ ? hi + 1 : small_chunk_;
+            for (int s = 0; s < p.count; ++s) p.coef[s] = ldexpf(fs.scalars[hi - s].h, -e);
+            const double f = (double)p.count * fs.stages * layer_flops();
+            if (!small_timed(3, 3.0 * f, st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, p, st, L); })) return false;
+            if (tprime != nullptr) launch_small_time(dt_, p, st, L);
+        }
+        return true;
+    }
+
     void fused_recompute(cudaStream_t st, void* ws, const FusedSolve& fs, int step, long long* L) override {
+        if (b_small_) {
+            if (lay_->time_gradient) return;          // the product wants the stage derivatives too: it recomputes them itself
+            SmallMlp p = small_bwd_;
+            p.step_hi = step; p.count = 1; p.recompute = 1;
+            small_timed(0, b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L); });
+            return;
+        }
         const size_t es = low_size(dt_);
         const size_t slot = (size_t)B_ * wp_[0] * es;
         cudaMemcpyAsync(at(ws, lay_->ybuf[0]), (const char*)fs.traj + (size_t)step * slot, slot, cudaMemcpyDeviceToDevice, st);
@@ -555,6 +679,17 @@ public:
 
     void fused_vjp(cudaStream_t st, void* ws, const FusedSolve& fs, int step, float* out, float beta, float coef, unsigned* flag,
                    long long* L, cudaEvent_t after_kernel, cudaStream_t st_finish) override {
+        if (b_small_) {
+            SmallMlp p = small_bwd_;
+            p.step_hi = step; p.count = 1; p.vjp = 1; p.flag = flag;
+            if (lay_->time_gradient) { p.recompute = 1; p.tpart = (float*)at(ws, small_tpart_); }
+            small_step_ = p;
+            p.out = out; p.beta = beta; p.coef[0] = coef;
+            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, p, st, L); });
+            if (after_kernel != nullptr) cudaEventRecord(after_kernel, st);
+            if (st_finish != nullptr && after_kernel != nullptr) cudaStreamWaitEvent(st_finish, after_kernel, 0);
+            return;
+        }
         const int s = b_stages_, d = wp_[0];
         const RkStepScalars& sc = scal_host_[step];
         RkParams p{};
@@ -637,6 +772,12 @@ protected:
     size_t f_scalars_ = 0, f_phases_[3] = {0, 0, 0}, f_cnt_ = 0, kappaslab_ = 0;
     size_t tiny_scal_ = 0, tiny_log_ = 0;
     bool tiny_ok_ = false;
+    bool small_ok_ = false, b_small_ = false, quantized_ = false;
+    int small_chunk_ = 1;
+    size_t small_pack_ = 0, small_scal_ = 0, small_xs_[SMALL_MAX_L] = {0}, small_zs_[SMALL_MAX_L + 1] = {0};
+    SmallMlp small_bwd_{}, small_step_{};
+    size_t small_tpart_ = 0;
+    const float* theta_ = nullptr;
     bool fused_ok_ = false;
     bool keep_k_ = false;
     int rb_ = 0, cnt_stride_ = 0;

@@ -107,6 +107,16 @@ public:
     // on `st` right behind the launch).
     virtual void fused_vjp(cudaStream_t st, void* ws, const FusedSolve& fs, int step, float* out, float beta, float coef,
                            unsigned* flag, long long* L, cudaEvent_t after_kernel = nullptr, cudaStream_t st_finish = nullptr) {}
+    // Fused kernels that form the seed Q16(S a) themselves are told where a and the exponent are (before fused_vjp) and return true: no seed
+    // kernel then
+    virtual bool fused_seeds_itself(const float* a, int e, const int* e_dev) { return false; }
+    // The whole backward loop of a pass without finiteness decisions (a in place, g += per step); false = not available, go step by step
+    virtual bool fused_backward_all(cudaStream_t st, void* ws, const FusedSolve& fs, float* a, float* g, const float* cot, int e, unsigned* flag,
+                                    float* tprime, long long* L) { return false; }
+    // Fused kernels that form the step's time terms {Phi^T a, dt, dh} with the vector-Jacobian product: written to tvals, non-finite ones
+    // raise the flag (called behind fused_vjp); false = the caller forms them
+    virtual bool fused_time_terms(cudaStream_t st, float* tvals, unsigned* flag, long long* L) { return false; }
+    virtual bool fused_has_time_terms() const { return false; }
     // where the seed kernel writes the last stage's cotangent kappa_s = Q16(b_s v) for fused_vjp
     virtual void* fused_kappa_last(void* ws) const { return nullptr; }
 };

@@ -64,3 +64,18 @@ def test_tiny_network_variants(batch, d, hidden):
     assert_same_log(gpu["log"], orc["log"])
     assert gpu["stats"]["whole_solve_launches"] == 2
     assert_parity(run_gpu(wl, "f32", "none"), run_oracle(wl, exact=True), TOL["f32"])
+
+
+# row-local kernels of small dense networks: one row, a block's 16 rows less and plus one, two row tiles per block (more than 16 rows per
+# SM), 1 to 4 layers, state widths that are not multiples of 8 or 16, both sizes of gradient pieces, several chunks of steps
+@pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (15, [40, 72, 40], 3), (17, [9, 33, 65, 9], 3), (300, [64, 64], 20),
+                                                  (200, [72, 200, 200, 72], 2), (2500, [24, 40, 24], 2), (130, [16, 32, 48, 32, 16], 3)])
+def test_small_networks_at_tile_edges(batch, widths, n_steps):
+    wl = inputs.mlp_block(batch=batch, n_steps=n_steps, d=widths[0], hidden=widths[1])
+    wl.vel["n_layers"], wl.vel["widths"], wl.theta = len(widths) - 1, widths, inputs.mlp_theta(3, widths, True)
+    for low, scaling in (("bf16", "none"), ("f16", "dynamic"), ("f16", "none_safe")):
+        gpu, orc = run_gpu(wl, low, scaling), run_oracle(wl, low, scaling)
+        assert_parity(gpu, orc, TOL[low])
+        assert gpu["stats"]["fused_launches"] > 0 and gpu["stats"]["simt_contractions"] == 0
+        if scaling == "dynamic":
+            assert_same_log(gpu["log"], orc["log"])
