@@ -117,7 +117,9 @@ struct GemmArgs {
     int cnf_pair; void* pair_out; const void* uprev;
     // EPI_WGRAD on the plain CUDA-core kernel: the row sums of A (bias gradient), row_sum[m] = beta row_sum[m] + sum; scaled by tau
     // into row_sum_time[m * ldo] (the appended time column); and the bare sums into row_sum_raw[m].  Each may be null.
+    // `alpha` (0 = 1) scales what is added to the outputs; with k_tau the time column weighs the reduction index k by k_tau[k / k_per]
     float *row_sum, *row_sum_time, *row_sum_raw;
+    float alpha; const float* k_tau; int k_per;
 };
 
 // returns whether the plain-operand kernel ran (the one that takes GemmArgs::row_sum)

@@ -50,7 +50,7 @@ __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, 
         return Low<T>::nonfinite(q);
     } else if (g.epi == EPI_WGRAD) {
         float* o = (float*)g.out + (long long)m * g.ldo + n;
-        *o = (g.beta != 0.f ? *o : 0.f) + v;
+        *o = fmaf(g.alpha != 0.f ? g.alpha : 1.f, v, g.beta != 0.f ? *o : 0.f);
     } else {
         ((float*)g.out)[(long long)m * g.ldo + n] = v;
     }
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     namespace cg = cooperative_groups;
     __shared__ __align__(16) float As[2][DK][kDenseLd];
     __shared__ __align__(16) float Bs[2][DK][kDenseLd];
-    __shared__ float rows[DM];
+    __shared__ float rows[2][DM], tau_s[2][DK];
     const T* A = (const T*)g.A;
     const T* B = (const T*)g.B;
     const int m0 = blockIdx.y * DM, n0 = blockIdx.x * DN, t = threadIdx.x;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     const int k_begin = blockIdx.z * per_slice, k_end = min(g.K, k_begin + per_slice);
     // the bias gradient is the row sum of A over the reduction range: taken along by the first column of tiles
     const bool sum_rows = !KFAST && (g.row_sum != nullptr || g.row_sum_time != nullptr) && blockIdx.x == 0;
-    float acc[4][4], rs[4] = {0.f, 0.f, 0.f, 0.f};
+    float acc[4][4], rs[4] = {0.f, 0.f, 0.f, 0.f}, rt[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             }
         }
     };
-    auto stash = [&](int buf) {
+    auto stash = [&](int buf, int k0) {
+        if (sum_rows && g.k_tau != nullptr && t < DK) tau_s[buf][t] = k0 + t < k_end ? g.k_tau[(k0 + t) / g.k_per] : 0.f;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             if (KFAST) {
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     };
     if (k_begin < k_end) {
         fetch(k_begin);
-        stash(0);
+        stash(0, k_begin);
     }
     __syncthreads();
     int buf = 0;
@@ -229,17 +230,23 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             if (sum_rows) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) rs[i] += a[i];
+                if (g.k_tau != nullptr) {
+                    const float tk = tau_s[buf][kk];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) rt[i] = fmaf(tk, a[i], rt[i]);
+                }
             }
         }
-        if (more) stash(buf ^ 1);
+        if (more) stash(buf ^ 1, k0 + DK);
         __syncthreads();
     }
 
-    auto put_row_sum = [&](int m, float s) {
-        if (g.row_sum != nullptr) g.row_sum[m] = (g.beta != 0.f ? g.row_sum[m] : 0.f) + s;
+    const float alpha = g.alpha != 0.f ? g.alpha : 1.f;
+    auto put_row_sum = [&](int m, float s, float st) {
+        if (g.row_sum != nullptr) g.row_sum[m] = fmaf(alpha, s, g.beta != 0.f ? g.row_sum[m] : 0.f);
         if (g.row_sum_time != nullptr) {
             float* o = g.row_sum_time + (long long)m * g.ldo;
-            *o = (g.beta != 0.f ? *o : 0.f) + g.tau * s;
+            *o = fmaf(alpha, g.k_tau != nullptr ? st : g.tau * s, g.beta != 0.f ? *o : 0.f);
         }
         if (g.row_sum_raw != nullptr) g.row_sum_raw[m] = s;
     };
@@ -254,7 +261,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
                 const int n = n0 + tx * 4 + j;
                 if (m < g.M && n < g.N) bad |= finish_element<T>(g, m, n, acc[i][j]);
             }
-            if (sum_rows && tx == 0 && m < g.M) put_row_sum(m, rs[i]);
+            if (sum_rows && tx == 0 && m < g.M) put_row_sum(m, rs[i], rt[i]);
         }
     } else {      // the slices of one tile are one cluster: rank r adds up the tile's rows [r, r + 1) * DM / S
         cg::cluster_group cl = cg::this_cluster();
@@ -262,7 +269,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             *reinterpret_cast<float4*>(&tile[ty * 4 + i][tx * 4]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            if (sum_rows && tx == 0) rows[ty * 4 + i] = rs[i];
+            if (sum_rows && tx == 0) { rows[0][ty * 4 + i] = rs[i]; rows[1][ty * 4 + i] = rt[i]; }
         }
         cl.sync();
         const int rank = (int)blockIdx.z, per = DM / S;
@@ -274,9 +281,12 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             bad |= finish_element<T>(g, m, n, v);
         }
         if (sum_rows && t < per && m0 + rank * per + t < g.M) {
-            float v = 0.f;
-            for (int z = 0; z < S; ++z) v += *cl.map_shared_rank(&rows[rank * per + t], z);
-            put_row_sum(m0 + rank * per + t, v);
+            float v = 0.f, vt = 0.f;
+            for (int z = 0; z < S; ++z) {
+                v += *cl.map_shared_rank(&rows[0][rank * per + t], z);
+                vt += *cl.map_shared_rank(&rows[1][rank * per + t], z);
+            }
+            put_row_sum(m0 + rank * per + t, v, vt);
         }
         cl.sync();      // no block leaves while another reads its shared memory
     }

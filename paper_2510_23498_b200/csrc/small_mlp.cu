@@ -1,13 +1,15 @@
-// Row-local kernels for small dense velocities in the 16-bit formats.  Samples are independent through the time loop, so a block
+// Row-local kernels for small dense velocities.  Samples are independent through the time loop, so a block
 // takes 16 (or 32) of them through the whole forward solve, or through the backward chain of several steps, without talking to any
 // other block: a layer is one contraction [16 x K] x [K x N] whose operands never leave the SM (activations in shared memory, weights
 // through L1), and the next layer starts after a block barrier.  What bounds this is the chain of layers, not bytes or tensor rate:
 // a tcgen05 tile needs 128 rows (64 at half rate) and a hand-over between its epilogue and the next tile's operands, about 8 us per
 // layer in rk_fused.cu, while mma.sync fragments of 16 rows spread the batch over the SMs and hand over in registers and shared memory.
+// float32 runs the same program on the CUDA cores, 8 rows to a block, bound by the weights' way from L2 (about 64 bytes a cycle).
 // Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
 // second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
 // Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.9 ms; MLP
-// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.5 ms.
+// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.2 ms; float32 MLP 64-256-256-64, 1024 samples, 16 RK4 steps
+// (before: a launch per layer) 10.8 -> 5.8 ms.
 #include "small_mlp.h"
 
 #include "profiler.h"
@@ -18,10 +20,32 @@ namespace mpode {
 using namespace tc;
 namespace {
 
-constexpr int kWarps = 8, kThreads = 32 * kWarps;
+constexpr int kWarps = 8, kThreads = 32 * kWarps;      // working warps; one more warp streams the weights
+constexpr int kPassCols = 256, kUnitBytes = 16384;
 
 template <typename T> __device__ __forceinline__ float lowf(T x) { return Low<T>::to_f(x); }
 template <typename T> __device__ __forceinline__ float q16(float x) { return Low<T>::to_f(Low<T>::from_f(x)); }
+
+// two neighbouring elements of a row, moved as one word
+template <typename T> struct Pair { using W = uint32_t; };
+template <> struct Pair<float> { using W = float2; };
+template <typename T> __device__ __forceinline__ typename Pair<T>::W pack_w(float a, float b) {
+    if constexpr (sizeof(T) == 4) return make_float2(a, b); else return cvt_pack<T>(a, b);
+}
+template <typename T> __device__ __forceinline__ T low_of(typename Pair<T>::W w) {
+    if constexpr (sizeof(T) == 4) return w.x; else return from_bits<T>((unsigned short)(w & 0xFFFFu));
+}
+template <typename T> __device__ __forceinline__ T high_of(typename Pair<T>::W w) {
+    if constexpr (sizeof(T) == 4) return w.y; else return from_bits<T>((unsigned short)(w >> 16));
+}
+template <typename T> __device__ __forceinline__ float lo_w(typename Pair<T>::W w) { return lowf(low_of<T>(w)); }
+template <typename T> __device__ __forceinline__ float hi_w(typename Pair<T>::W w) { return lowf(high_of<T>(w)); }
+// |v| at or above this is not finite in the format
+template <typename T> __device__ __forceinline__ float low_limit() {
+    if constexpr (sizeof(T) == 4) return INFINITY; else return OverflowLimit<T>::value();
+}
+// rows of a block: 16 per row tile of the matrix instructions; float32 runs on the CUDA cores with 8
+template <typename T, int MT> constexpr int kRows = (sizeof(T) == 4 ? 8 : 16) * MT;
 
 template <typename T> __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
 template <> __device__ __forceinline__ void mma16816<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -42,7 +66,8 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool o
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
 }
 
-__device__ __forceinline__ float act_f(int act, float z) {
+template <typename T> __device__ __forceinline__ float act_f(int act, float z) {
+    if constexpr (sizeof(T) == 4) return act_fwd(act, z);
     switch (act) {
         case MPODE_ACT_SOFTPLUS: return fast_act<MPODE_ACT_SOFTPLUS>(z);
         case MPODE_ACT_RELU: return fast_act<MPODE_ACT_RELU>(z);
@@ -50,7 +75,8 @@ __device__ __forceinline__ float act_f(int act, float z) {
         default: return z;
     }
 }
-__device__ __forceinline__ float act_df(int act, float h) {
+template <typename T> __device__ __forceinline__ float act_df(int act, float h) {
+    if constexpr (sizeof(T) == 4) return act_deriv_from_output(act, h);
     switch (act) {
         case MPODE_ACT_SOFTPLUS: return fast_act_deriv<MPODE_ACT_SOFTPLUS>(h);
         case MPODE_ACT_RELU: return fast_act_deriv<MPODE_ACT_RELU>(h);
@@ -70,9 +96,11 @@ __global__ void __launch_bounds__(256) small_pack_kernel(const __grid_constant__
         int q = 0;
         while (i >= job.first[q + 1]) ++q;
         const int l = q >> 1, back = q & 1;
-        const long long r = i - job.first[q];
-        const int kp = k32(back ? p.wp[l + 1] : p.wp[l]);
-        const int lane = (int)(r & 31), kk = (int)((r >> 5) % kp), tile = (int)((r >> 5) / kp);
+        // [pass of 32 column tiles][32 of the reduction][tile][lane]
+        const int r = (int)(i - job.first[q]), lane = r & 31;
+        const int kp = k32(back ? p.wp[l + 1] : p.wp[l]), tiles = (back ? p.wp[l] : p.wp[l + 1]) / 8;
+        const int pass = (r >> 5) / (32 * kp), in_pass = tiles - 32 * pass < 32 ? tiles - 32 * pass : 32, rr = (r >> 5) - pass * 32 * kp;
+        const int kk = rr / in_pass, tile = pass * 32 + rr % in_pass;
         const int in_full = p.wr[l] + ((p.time && l == 0) ? 1 : 0);
         uint32_t w[4];
 #pragma unroll
@@ -98,74 +126,134 @@ __global__ void __launch_bounds__(256) small_pack_kernel(const __grid_constant__
     }
 }
 
+// float32: forward [inputs][outputs], backward [outputs][inputs], zero in the padding
+__global__ void __launch_bounds__(256) small_pack_f32_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ PackJob job) {
+    const long long n = job.first[2 * p.L];
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        int q = 0;
+        while (i >= job.first[q + 1]) ++q;
+        // [pass of 256 columns][reduction][column]
+        const int l = q >> 1, back = q & 1, r = (int)(i - job.first[q]);
+        const int N = back ? p.wp[l] : p.wp[l + 1], K = back ? p.wp[l + 1] : p.wp[l];
+        const int pass = r / (kPassCols * K), in_pass = N - kPassCols * pass < kPassCols ? N - kPassCols * pass : kPassCols, rr = r - pass * kPassCols * K;
+        const int k = rr / in_pass, c = pass * kPassCols + rr % in_pass;
+        const int out = back ? k : c, in = back ? c : k;
+        const int in_full = p.wr[l] + ((p.time && l == 0) ? 1 : 0);
+        ((float*)(back ? p.wb[l] : p.wf[l]))[r] = out < p.wr[l + 1] && in < p.wr[l] ? p.theta[p.woff[l] + (long long)out * in_full + in] : 0.f;
+    }
+    if (blockIdx.x == 0) {
+        for (int l = 0; l < p.L; ++l)
+            for (int c = threadIdx.x; c < p.wp[l + 1]; c += blockDim.x) {
+                const bool on = c < p.wr[l + 1];
+                if (p.bias) ((float*)p.b16[l])[c] = on ? p.theta[p.boff[l] + c] : 0.f;
+                if (p.time && l == 0) ((float*)p.wt16)[c] = on ? p.theta[p.woff[0] + (long long)c * (p.wr[0] + 1) + p.wr[0]] : 0.f;
+            }
+    }
+}
+
+// ---------------------------------------------------------------- the weights on their way through shared memory
+// The order in which a block needs the weights is fixed, so one thread streams them ahead of the arithmetic: bulk copies of at most
+// 16 KB (32 of the reduction for up to 32 column tiles; in float32 16 rows of up to 256 columns) through a ring of buffers, across layer
+// and stage boundaries.  (Loaded by the warps themselves, even 16 loads ahead, each unit cost an L2 round trip of half a microsecond.)
+// Every wait is bounded; after one has given up the block runs on without waiting and the error word tells the host.
+struct Ring {
+    uint64_t *full, *empty;
+    unsigned char* buf;
+    int n, s;
+    uint32_t phase;
+    unsigned* err;
+    __device__ __forceinline__ void next() { if (++s == n) { s = 0; phase ^= 1u; } }
+    __device__ __forceinline__ unsigned char* stage() const { return buf + s * kUnitBytes; }
+};
+__device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }      // the working warps
+
+__device__ __forceinline__ void ring_wait(const Ring& r) {
+    if (!mbar_try_wait(&r.full[r.s], r.phase)) mbar_wait(&r.full[r.s], r.phase, r.err, 4u);
+}
+__device__ __forceinline__ void stream_units(Ring& r, const unsigned char* src, int bytes) {
+    if (r.n == 0) return;
+    if (!mbar_wait(&r.empty[r.s], r.phase ^ 1u, r.err, 1u)) {      // gave up: nothing more is issued, what is in flight lands first
+        const unsigned long long t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+        r.n = 0;
+        return;
+    }
+    mbar_arrive_expect_tx(&r.full[r.s], (uint32_t)bytes);
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(r.stage())), "l"(src), "r"(bytes),
+                 "r"(smem_u32(&r.full[r.s])) : "memory");
+    r.next();
+}
+// one contraction's weights: reduction K, N columns
+template <typename T> __device__ __forceinline__ void stream_layer(Ring& r, const uint4* W, int K, int N) {
+    const unsigned char* src = (const unsigned char*)W;
+    for (int c = 0; c < N; c += kPassCols) {
+        const int cols = min(kPassCols, N - c);
+        if constexpr (sizeof(T) == 4) {
+            for (int k = 0; k < K; k += 16) { const int b = min(16, K - k) * cols * 4; stream_units(r, src, b); src += b; }
+        } else {
+            const int b = cols * 64;
+            for (int k = 0; k < k32(K); ++k) { stream_units(r, src, b); src += b; }
+        }
+    }
+}
+
 // ---------------------------------------------------------------- one contraction of a block's rows
-// C[16 MT][8 tiles] = A[16 MT][32 kp] W, A in shared memory (row length lda), W packed.  Warp w takes the column tiles w, w + 8, ...,
-// four at a time; the next weights are requested before the present ones are used.  pre(g, col) runs before the reduction loop and
-// requests what the epilogue needs from memory for column tile g of the four; epi(g, m, row, col, c0, c1) gets two neighbouring columns.
+// C[16 MT][8 tiles] = A[16 MT][32 kp] W, A in shared memory (row length lda), W from the ring.  Warp w takes the column tiles w, w + 8, ...
+// of a pass.  pre(g, q, row, col) runs before the reduction loop and requests what the epilogue needs from memory for piece q of column
+// tile g; epi(g, q, row, col, c0, c1) gets two neighbouring columns.
 constexpr int kNG = 4;
 template <typename T, int MT, typename P, typename F>
-__device__ __forceinline__ void rows_gemm(const T* A, int lda, int kp, const uint4* __restrict__ W, int tiles, P&& pre, F&& epi) {
+__device__ __forceinline__ void rows_gemm(Ring& ring, const T* A, int lda, int kp, int tiles, P&& pre, F&& epi) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t a0 = smem_u32(A) + (uint32_t)(((lane & 15) * lda + (lane >> 4) * 8) * 2);
-    for (int t0 = warp; t0 < tiles; t0 += kWarps * kNG) {
+    for (int p0 = 0; p0 < tiles; p0 += 32) {
+        const int in_pass = min(32, tiles - p0);
         float acc[MT][kNG][4];
-        uint4 b[2][kNG];
-        auto fetch = [&](int k, uint4 (&d)[kNG]) {
-#pragma unroll
-            for (int g = 0; g < kNG; ++g)
-                if (t0 + kWarps * g < tiles) d[g] = __ldg(W + ((t0 + kWarps * g) * kp + k) * 32 + lane);
-        };
-        auto step = [&](int k, const uint4 (&d)[kNG]) {
-            uint32_t a[MT][2][4];
-#pragma unroll
-            for (int m = 0; m < MT; ++m) {
-                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32) * 2), a[m][0]);
-                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32 + 16) * 2), a[m][1]);
-            }
-#pragma unroll
-            for (int g = 0; g < kNG; ++g)
-                if (t0 + kWarps * g < tiles) {
-#pragma unroll
-                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][0], d[g].x, d[g].y);
-                }
-#pragma unroll
-            for (int g = 0; g < kNG; ++g)
-                if (t0 + kWarps * g < tiles) {
-#pragma unroll
-                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][1], d[g].z, d[g].w);
-                }
-        };
-        fetch(0, b[0]);
-        if (kp > 1) fetch(1, b[1]);
 #pragma unroll
         for (int g = 0; g < kNG; ++g)
-            if (t0 + kWarps * g < tiles) pre(g, (t0 + kWarps * g) * 8 + 2 * (lane & 3));
+            if (warp + kWarps * g < in_pass) {
+#pragma unroll
+                for (int q = 0; q < 2 * MT; ++q) pre(g, q, q * 8 + (lane >> 2), (p0 + warp + kWarps * g) * 8 + 2 * (lane & 3));
+            }
 #pragma unroll
         for (int m = 0; m < MT; ++m)
 #pragma unroll
             for (int g = 0; g < kNG; ++g)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[m][g][i] = 0.f;
-        for (int k = 0; k < kp; k += 2) {
-            {
-                uint4 cur[kNG];
+        for (int k = 0; k < kp; ++k) {
+            uint32_t a[MT][2][4];
 #pragma unroll
-                for (int g = 0; g < kNG; ++g) cur[g] = b[0][g];
-                if (k + 2 < kp) fetch(k + 2, b[0]);
-                step(k, cur);
+            for (int m = 0; m < MT; ++m) {
+                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32) * 2), a[m][0]);
+                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32 + 16) * 2), a[m][1]);
             }
-            if (k + 1 < kp) {
-                uint4 cur[kNG];
+            ring_wait(ring);
+            const uint4* W = (const uint4*)ring.stage() + warp * 32 + lane;
+            uint4 b[kNG];
 #pragma unroll
-                for (int g = 0; g < kNG; ++g) cur[g] = b[1][g];
-                if (k + 3 < kp) fetch(k + 3, b[1]);
-                step(k + 1, cur);
-            }
+            for (int g = 0; g < kNG; ++g)
+                if (warp + kWarps * g < in_pass) b[g] = W[g * kWarps * 32];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ring.empty[ring.s]);      // the fragments are in registers
+            ring.next();
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+                if (warp + kWarps * g < in_pass) {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][0], b[g].x, b[g].y);
+                }
+#pragma unroll
+            for (int g = 0; g < kNG; ++g)
+                if (warp + kWarps * g < in_pass) {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][1], b[g].z, b[g].w);
+                }
         }
 #pragma unroll
         for (int g = 0; g < kNG; ++g)
-            if (t0 + kWarps * g < tiles) {
-                const int col = (t0 + kWarps * g) * 8 + 2 * (lane & 3);
+            if (warp + kWarps * g < in_pass) {
+                const int col = (p0 + warp + kWarps * g) * 8 + 2 * (lane & 3);
 #pragma unroll
                 for (int m = 0; m < MT; ++m) {
                     epi(g, 2 * m, m * 16 + (lane >> 2), col, acc[m][g][0], acc[m][g][1]);
@@ -181,7 +269,7 @@ __device__ __forceinline__ void rows_gemm(const T* A, int lda, int kp, const uin
 constexpr int kScalarWords = sizeof(RkStepScalars) / sizeof(float);
 template <typename T> struct SmallSmem {
     T *act0, *ks, *ps, *yb, *vv;
-    float *a, *scs, *red;
+    float *a, *scs, *red, *scratch;
     int lda, R, dp, d, half, pairs;
     __device__ SmallSmem(const SmallMlp& p, unsigned char* base, int rows) : R(rows), dp(p.wp[0]), d(p.wr[0]) {
         int kp = 0;
@@ -193,15 +281,30 @@ template <typename T> struct SmallSmem {
         a = (float*)(vv + R * dp);
         scs = a + R * dp;
         red = scs + 2 * kScalarWords;
+        scratch = red + 3 * kWarps;
     }
     __device__ __forceinline__ T* act(int i) const { return act0 + i * R * lda; }
-    __device__ __forceinline__ uint32_t* w(T* x) const { return reinterpret_cast<uint32_t*>(x); }
+    __device__ __forceinline__ typename Pair<T>::W* w(T* x) const { return reinterpret_cast<typename Pair<T>::W*>(x); }
     __device__ __forceinline__ const RkStepScalars& scalars(int n) const { return *(const RkStepScalars*)(scs + (n & 1) * kScalarWords); }
 };
-size_t small_smem(const SmallMlp& p, int rows) {
+template <typename T> size_t small_smem(const SmallMlp& p, int rows) {
     int kp = 0;
     for (int l = 0; l <= p.L; ++l) kp = k32(p.wp[l]) > kp ? k32(p.wp[l]) : kp;
-    return (size_t)rows * 2 * (2 * (kp * 32 + 8) + (2 * p.stages + 2) * p.wp[0]) + (size_t)rows * p.wp[0] * 4 + (2 * kScalarWords + 3 * kWarps) * 4;
+    return (size_t)rows * sizeof(T) * (2 * (kp * 32 + 8) + (2 * p.stages + 2) * p.wp[0]) + (size_t)rows * p.wp[0] * 4 + (2 * kScalarWords + 3 * kWarps) * 4 +
+           (sizeof(T) == 4 ? (size_t)kThreads * rows * 4 : 0);
+}
+// the ring behind the block's own shared memory: `n` buffers, then the barriers
+__device__ __forceinline__ Ring make_ring(unsigned char* base, int n, unsigned* err) {
+    Ring r;
+    r.buf = base; r.n = n; r.s = 0; r.phase = 0; r.err = err;
+    r.full = (uint64_t*)(base + n * kUnitBytes);
+    r.empty = r.full + n;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < n; ++i) { mbar_init(&r.full[i], 1); mbar_init(&r.empty[i], kWarps); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    return r;
 }
 // a step's scalars travel to shared memory while the step before runs (asynchronous; wait with scalars_ready and a barrier)
 template <typename T>
@@ -213,8 +316,65 @@ __device__ __forceinline__ void fetch_scalars(const SmallMlp& p, const SmallSmem
 }
 __device__ __forceinline__ void scalars_ready() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <typename T> __device__ __forceinline__ float lo_w(uint32_t w) { return lowf(from_bits<T>((unsigned short)(w & 0xFFFFu))); }
-template <typename T> __device__ __forceinline__ float hi_w(uint32_t w) { return lowf(from_bits<T>((unsigned short)(w >> 16))); }
+// float32 on the CUDA cores: a thread has one column of the pass and all the block's rows, and where the pass has fewer than 256 columns
+// a share of each unit's 16 reduction steps; activations are broadcast from shared memory four reduction steps at a time.  The shares
+// meet in shared memory, added in order.
+template <int MT, typename P, typename F>
+__device__ __forceinline__ void rows_gemm_f32(Ring& ring, const SmallSmem<float>& sm, const float* A, int K, int N, P&& pre, F&& epi) {
+    constexpr int R = kRows<float, MT>;
+    const int lane = threadIdx.x & 31;
+    for (int c0 = 0; c0 < N; c0 += kPassCols) {
+        const int cols = min(kPassCols, N - c0);
+        int ct = 64;
+        while (ct < cols) ct *= 2;
+        const int kg = threadIdx.x / ct, tc = threadIdx.x % ct, KG = kThreads / ct, rows = 16 / KG;
+        const bool on = tc < cols;
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.f;
+        for (int k = 0; k < K; k += 16) {
+            ring_wait(ring);
+            const float* w = (const float*)ring.stage() + tc;
+            const int ke = min(16, K - k);                        // a multiple of 8
+            for (int i = kg * rows; i < kg * rows + rows && i < ke; i += 4) {
+                float wb[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) wb[q] = on ? w[(i + q) * cols] : 0.f;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float4 a = *reinterpret_cast<const float4*>(A + r * sm.lda + k + i);
+                    acc[r] = fmaf(a.w, wb[3], fmaf(a.z, wb[2], fmaf(a.y, wb[1], fmaf(a.x, wb[0], acc[r]))));
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ring.empty[ring.s]);
+            ring.next();
+        }
+        if (c0 > 0) work_sync();
+#pragma unroll
+        for (int r = 0; r < R; ++r) sm.scratch[(kg * R + r) * ct + tc] = acc[r];
+        work_sync();
+        const int hc = ct / 2;
+        for (int i = threadIdx.x; i < R * hc; i += kThreads) {
+            const int r = i / hc, c = 2 * (i - r * hc);
+            if (c >= cols) continue;
+            pre(0, 0, r, c0 + c);
+            float2 v = make_float2(0.f, 0.f);
+            for (int q = 0; q < KG; ++q) {
+                const float2 x = *reinterpret_cast<const float2*>(sm.scratch + (q * R + r) * ct + c);
+                v.x += x.x; v.y += x.y;
+            }
+            epi(0, 0, r, c0 + c, v.x, v.y);
+        }
+    }
+}
+
+// C[rows][N] = A[rows][K] W: A one of the activation buffers, W the next weights of the ring
+template <typename T, int MT, typename P, typename F>
+__device__ __forceinline__ void block_gemm(Ring& ring, const SmallSmem<T>& sm, const T* A, int K, int N, P&& pre, F&& epi) {
+    if constexpr (sizeof(T) == 4) rows_gemm_f32<MT>(ring, sm, A, K, N, pre, epi);
+    else rows_gemm<T, MT>(ring, A, sm.lda, k32(K), N / 8, pre, epi);
+}
 
 // zeros behind a layer's width, up to the next multiple of 32 columns
 template <typename T>
@@ -227,8 +387,9 @@ __device__ __forceinline__ void zero_tail(T* act, int lda, int R, int w) {
 // All stages of one step for the rows r0 .. r0 + R - 1 from the state in sm.yb: k_j into sm.ks; with KEEP every layer input into the
 // slabs (slot `slot`).  `skip_last`: the last stage's derivative is not wanted.
 template <typename T, int MT, bool KEEP>
-__device__ __forceinline__ void small_stages(const SmallMlp& p, const SmallSmem<T>& sm, const RkStepScalars& sc, int r0, int slot, bool skip_last) {
-    const int R = 16 * MT, dp = sm.dp;
+__device__ __forceinline__ void small_stages(const SmallMlp& p, Ring& ring, const SmallSmem<T>& sm, const RkStepScalars& sc, int r0, int slot, bool skip_last) {
+    using W = typename Pair<T>::W;
+    const int R = kRows<T, MT>, dp = sm.dp;
     for (int j = 0; j < p.stages; ++j) {
         float ha[RK_MAX_STAGES - 1];
 #pragma unroll
@@ -236,59 +397,68 @@ __device__ __forceinline__ void small_stages(const SmallMlp& p, const SmallSmem<
         T* x0 = KEEP ? (T*)p.xs[0] + ((long long)(slot * p.stages + j) * p.B + r0) * dp : nullptr;
         for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
             const int r = i / sm.half, c = 2 * (i - r * sm.half);
-            uint32_t q = sm.w(sm.yb)[i];
+            W q = sm.w(sm.yb)[i];
             if (j > 0) {
                 float v0 = lo_w<T>(q), v1 = hi_w<T>(q);
 #pragma unroll
                 for (int l = 0; l < RK_MAX_STAGES - 1; ++l)
                     if (l < j && ha[l] != 0.f) {
-                        const uint32_t k = sm.w(sm.ks)[l * sm.pairs + i];
+                        const W k = sm.w(sm.ks)[l * sm.pairs + i];
                         v0 = fmaf(ha[l], lo_w<T>(k), v0);
                         v1 = fmaf(ha[l], hi_w<T>(k), v1);
                     }
-                q = cvt_pack<T>(v0, v1);
+                q = pack_w<T>(v0, v1);
             }
-            *(uint32_t*)(sm.act(0) + r * sm.lda + c) = q;
-            if (KEEP && r0 + r < p.B) *(uint32_t*)(x0 + r * dp + c) = q;
+            *(W*)(sm.act(0) + r * sm.lda + c) = q;
+            if (KEEP && r0 + r < p.B) *(W*)(x0 + r * dp + c) = q;
         }
         zero_tail(sm.act(0), sm.lda, R, dp);
-        __syncthreads();
+        work_sync();
         const float tau = sc.tau16[j];
         for (int l = 0; l < p.L; ++l) {
             const bool last = l == p.L - 1;
             if (last && skip_last && j == p.stages - 1) break;
             const int N = p.wp[l + 1];
-            const uint32_t* b16 = p.bias ? (const uint32_t*)p.b16[l] : nullptr;
-            const uint32_t* wt = p.time && l == 0 ? (const uint32_t*)p.wt16 : nullptr;
+            const W* b16 = p.bias ? (const W*)p.b16[l] : nullptr;
+            const W* wt = p.time && l == 0 ? (const W*)p.wt16 : nullptr;
             T* dst = last ? sm.ks + j * R * dp : sm.act((l + 1) & 1);
             const int ld = last ? dp : sm.lda;
             T* keep = KEEP && !last ? (T*)p.xs[l + 1] + ((long long)(slot * p.stages + j) * p.B + r0) * N : nullptr;
             float2 bv[kNG];
-            rows_gemm<T, MT>(
-                sm.act(l & 1), sm.lda, k32(p.wp[l]), p.wf[l], N / 8,
-                [&](int g, int c) {
+            block_gemm<T, MT>(
+                ring, sm, sm.act(l & 1), p.wp[l], N,
+                [&](int g, int q, int, int c) {
+                    if (q != 0) return;               // the same for every row
                     bv[g] = make_float2(0.f, 0.f);
-                    if (b16 != nullptr) { const uint32_t w = __ldg(b16 + c / 2); bv[g] = make_float2(lo_w<T>(w), hi_w<T>(w)); }
-                    if (wt != nullptr) { const uint32_t w = __ldg(wt + c / 2); bv[g].x = fmaf(tau, lo_w<T>(w), bv[g].x); bv[g].y = fmaf(tau, hi_w<T>(w), bv[g].y); }
+                    if (b16 != nullptr) { const W w = __ldg(b16 + c / 2); bv[g] = make_float2(lo_w<T>(w), hi_w<T>(w)); }
+                    if (wt != nullptr) { const W w = __ldg(wt + c / 2); bv[g].x = fmaf(tau, lo_w<T>(w), bv[g].x); bv[g].y = fmaf(tau, hi_w<T>(w), bv[g].y); }
                 },
                 [&](int g, int, int r, int c, float v0, float v1) {
                     v0 += bv[g].x; v1 += bv[g].y;
-                    if (!last) { v0 = act_f(p.act, v0); v1 = act_f(p.act, v1); }
-                    const uint32_t w = cvt_pack<T>(v0, v1);
-                    *(uint32_t*)(dst + r * ld + c) = w;
-                    if (KEEP && !last && r0 + r < p.B) *(uint32_t*)(keep + (long long)r * N + c) = w;
+                    if (!last) { v0 = act_f<T>(p.act, v0); v1 = act_f<T>(p.act, v1); }
+                    const W w = pack_w<T>(v0, v1);
+                    *(W*)(dst + r * ld + c) = w;
+                    if (KEEP && !last && r0 + r < p.B) *(W*)(keep + (long long)r * N + c) = w;
                 });
             if (!last) zero_tail(dst, sm.lda, R, N);
-            __syncthreads();
+            work_sync();
         }
     }
 }
 
 template <typename T, int MT>
-__global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_constant__ SmallMlp p) {
+__global__ void __launch_bounds__(kThreads + 32, 1) small_forward_kernel(const __grid_constant__ SmallMlp p) {
+    using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int R = 16 * MT, r0 = blockIdx.x * R;
-    const SmallSmem<T> sm(p, smem, R);
+    const int R = kRows<T, MT>, r0 = blockIdx.x * R;
+    Ring ring = make_ring(smem, p.ring, p.err);
+    if (threadIdx.x >= kThreads) {
+        if (threadIdx.x == kThreads)
+            for (int n = 0; n < p.n_steps * p.stages; ++n)
+                for (int l = 0; l < p.L; ++l) stream_layer<T>(ring, p.wf[l], p.wp[l], p.wp[l + 1]);
+        return;
+    }
+    const SmallSmem<T> sm(p, smem + p.ring * (kUnitBytes + 16), R);
     const int d = sm.d, dp = sm.dp;
     T* traj = (T*)p.traj;
     fetch_scalars(p, sm, 0);
@@ -303,10 +473,10 @@ __global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_co
     }
     for (int n = 0; n < p.n_steps; ++n) {
         scalars_ready();
-        __syncthreads();
+        work_sync();
         if (n + 1 < p.n_steps) fetch_scalars(p, sm, n + 1);
         const RkStepScalars& sc = sm.scalars(n);
-        small_stages<T, MT, false>(p, sm, sc, r0, 0, false);
+        small_stages<T, MT, false>(p, ring, sm, sc, r0, 0, false);
         float hb[RK_MAX_STAGES];
 #pragma unroll
         for (int j = 0; j < RK_MAX_STAGES; ++j) hb[j] = j < p.stages ? sc.hb[j] : 0.f;
@@ -318,7 +488,7 @@ __global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_co
 #pragma unroll
             for (int j = 0; j < RK_MAX_STAGES; ++j)
                 if (j < p.stages) {
-                    const uint32_t k = sm.w(sm.ks)[j * sm.pairs + i];
+                    const W k = sm.w(sm.ks)[j * sm.pairs + i];
                     v0 = fmaf(hb[j], lo_w<T>(k), v0);
                     v1 = fmaf(hb[j], hi_w<T>(k), v1);
                 }
@@ -326,18 +496,18 @@ __global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_co
             y.x += p.round_increment ? h * q16<T>(v0) : v0;
             y.y += p.round_increment ? h * q16<T>(v1) : v1;
             reinterpret_cast<float2*>(sm.a)[i] = y;
-            const uint32_t q = cvt_pack<T>(y.x, y.y);
+            const W q = pack_w<T>(y.x, y.y);
             sm.w(sm.yb)[i] = q;
             if (r0 + r < p.B && c < d) {
-                if ((d & 1) == 0) *(uint32_t*)(tn + r * d + c) = q;
+                if ((d & 1) == 0) *(W*)(tn + r * d + c) = q;
                 else {
-                    tn[r * d + c] = from_bits<T>((unsigned short)(q & 0xFFFFu));
-                    if (c + 1 < d) tn[r * d + c + 1] = from_bits<T>((unsigned short)(q >> 16));
+                    tn[r * d + c] = low_of<T>(q);
+                    if (c + 1 < d) tn[r * d + c + 1] = high_of<T>(q);
                 }
             }
         }
     }
-    __syncthreads();
+    work_sync();
     for (int i = threadIdx.x; i < R * d; i += kThreads) {
         const int r = i / d, c = i - r * d;
         if (r0 + r < p.B) p.yT[(long long)r0 * d + i] = sm.a[r * dp + c];
@@ -349,13 +519,28 @@ __global__ void __launch_bounds__(kThreads) small_forward_kernel(const __grid_co
 // the finiteness decision) psi_j goes to memory.  With tpart also the block's share of the step's time terms: Phi^T a with
 // Phi = sum_j b_j k_j, dt = sum_j dtau_j and dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>), dtau_j = <dZ_1, w_t>.
 template <typename T, int MT>
-__global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_constant__ SmallMlp p) {
+__global__ void __launch_bounds__(kThreads + 32, 1) small_backward_kernel(const __grid_constant__ SmallMlp p) {
+    using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int R = 16 * MT, r0 = blockIdx.x * R;
-    const SmallSmem<T> sm(p, smem, R);
+    const int R = kRows<T, MT>, r0 = blockIdx.x * R;
+    Ring ring = make_ring(smem, p.ring, p.err);
+    if (threadIdx.x >= kThreads) {
+        if (threadIdx.x == kThreads)
+            for (int s = 0; s < p.count; ++s) {
+                if (p.recompute)
+                    for (int j = 0; j < p.stages; ++j)
+                        for (int l = 0; l < p.L; ++l)      // (the last stage's derivative only for the time terms)
+                            if (!(l == p.L - 1 && j == p.stages - 1 && p.tpart == nullptr)) stream_layer<T>(ring, p.wf[l], p.wp[l], p.wp[l + 1]);
+                if (p.vjp)
+                    for (int j = 0; j < p.stages; ++j)
+                        for (int l = p.L - 1; l >= 0; --l) stream_layer<T>(ring, p.wb[l], p.wp[l + 1], p.wp[l]);
+            }
+        return;
+    }
+    const SmallSmem<T> sm(p, smem + p.ring * (kUnitBytes + 16), R);
     const int d = sm.d, dp = sm.dp;
     const T* traj = (const T*)p.traj;
-    const float lim = OverflowLimit<T>::value();
+    const float lim = low_limit<T>();
     const int e = p.e_dev != nullptr ? *p.e_dev : p.e;
     const bool want_t = p.tpart != nullptr;
     bool bad = false;
@@ -369,7 +554,7 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
     for (int s = 0; s < p.count; ++s) {
         const int n = p.step_hi - s;
         scalars_ready();
-        __syncthreads();
+        work_sync();
         if (s + 1 < p.count) fetch_scalars(p, sm, n - 1);
         const RkStepScalars& sc = sm.scalars(n);
         float t_phi = 0.f, t_dt = 0.f, t_dh = 0.f;
@@ -379,19 +564,19 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
                 const int r = i / dp, c = i - r * dp;
                 sm.yb[i] = r0 + r < p.B && c < d ? tn[r * d + c] : Low<T>::from_f(0.f);
             }
-            __syncthreads();
-            small_stages<T, MT, true>(p, sm, sc, r0, s, !want_t);
+            work_sync();
+            small_stages<T, MT, true>(p, ring, sm, sc, r0, s, !want_t);
         }
         if (!p.vjp) continue;
         for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {       // seed Q16(S a)
             const float2 a = reinterpret_cast<const float2*>(sm.a)[i];
             const float v0 = ldexpf(a.x, e), v1 = ldexpf(a.y, e);
             bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
-            sm.w(sm.vv)[i] = cvt_pack<T>(v0, v1);
+            sm.w(sm.vv)[i] = pack_w<T>(v0, v1);
             if (want_t) {
                 float p0 = 0.f, p1 = 0.f;
                 for (int j = 0; j < p.stages; ++j) {
-                    const uint32_t k = sm.w(sm.ks)[j * sm.pairs + i];
+                    const W k = sm.w(sm.ks)[j * sm.pairs + i];
                     p0 = fmaf(sc.b[j], lo_w<T>(k), p0);
                     p1 = fmaf(sc.b[j], hi_w<T>(k), p1);
                 }
@@ -406,29 +591,29 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
             const float bj = sc.b[j], cj = sc.c[j];
             float dtau = 0.f;
             T* kap = (T*)p.zs[p.L] + ((long long)(s * p.stages + j) * p.B + r0) * dp;
-            const uint32_t* wt = want_t && p.time ? (const uint32_t*)p.wt16 : nullptr;
+            const W* wt = want_t && p.time ? (const W*)p.wt16 : nullptr;
             for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
                 const int r = i / sm.half, c = 2 * (i - r * sm.half);
-                const uint32_t v = sm.w(sm.vv)[i];
+                const W v = sm.w(sm.vv)[i];
                 float v0 = bj * lo_w<T>(v), v1 = bj * hi_w<T>(v);
 #pragma unroll
                 for (int l = 1; l < RK_MAX_STAGES; ++l)
                     if (ha[l] != 0.f) {
-                        const uint32_t q = sm.w(sm.ps)[l * sm.pairs + i];
+                        const W q = sm.w(sm.ps)[l * sm.pairs + i];
                         v0 = fmaf(ha[l], lo_w<T>(q), v0);
                         v1 = fmaf(ha[l], hi_w<T>(q), v1);
                     }
                 bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
-                const uint32_t q = cvt_pack<T>(v0, v1);
-                *(uint32_t*)(sm.act(0) + r * sm.lda + c) = q;
-                if (r0 + r < p.B) *(uint32_t*)(kap + r * dp + c) = q;
+                const W q = pack_w<T>(v0, v1);
+                *(W*)(sm.act(0) + r * sm.lda + c) = q;
+                if (r0 + r < p.B) *(W*)(kap + r * dp + c) = q;
                 if (p.L == 1 && wt != nullptr) {
-                    const uint32_t w = __ldg(wt + c / 2);
+                    const W w = __ldg(wt + c / 2);
                     dtau = fmaf(lo_w<T>(q), lo_w<T>(w), fmaf(hi_w<T>(q), hi_w<T>(w), dtau));
                 }
             }
             zero_tail(sm.act(0), sm.lda, R, dp);
-            __syncthreads();
+            work_sync();
             int cur = 0;
             for (int l = p.L - 1; l >= 0; --l, cur ^= 1) {
                 const int N = p.wp[l];
@@ -437,32 +622,28 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
                 T* Z = l > 0 ? (T*)p.zs[l] + at : (p.commit ? nullptr : (T*)p.psi[j] + (long long)r0 * dp);
                 T* dst = l > 0 ? sm.act(cur ^ 1) : sm.ps + j * R * dp;
                 const int ld = l > 0 ? sm.lda : dp;
-                uint32_t hw[kNG][2 * MT];
-                rows_gemm<T, MT>(
-                    sm.act(cur), sm.lda, k32(p.wp[l + 1]), p.wb[l], N / 8,
-                    [&](int g, int c) {      // the stored layer outputs whose activation derivative multiplies the result
-#pragma unroll
-                        for (int q = 0; q < 2 * MT; ++q) {
-                            const int r = q * 8 + ((threadIdx.x & 31) >> 2);
-                            hw[g][q] = l > 0 && r0 + r < p.B ? *(const uint32_t*)(H + (long long)r * N + c) : 0u;
-                        }
+                W hw[kNG][2 * MT];
+                block_gemm<T, MT>(
+                    ring, sm, sm.act(cur), p.wp[l + 1], N,
+                    [&](int g, int q, int r, int c) {      // the stored layer outputs whose activation derivative multiplies the result
+                        hw[g][q] = l > 0 && r0 + r < p.B ? *(const W*)(H + (long long)r * N + c) : W{};
                     },
                     [&](int g, int q, int r, int c, float v0, float v1) {
                         if (l > 0) {
-                            v0 *= act_df(p.act, lo_w<T>(hw[g][q]));
-                            v1 *= act_df(p.act, hi_w<T>(hw[g][q]));
+                            v0 *= act_df<T>(p.act, lo_w<T>(hw[g][q]));
+                            v1 *= act_df<T>(p.act, hi_w<T>(hw[g][q]));
                         }
                         bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
-                        const uint32_t w = cvt_pack<T>(v0, v1);
-                        *(uint32_t*)(dst + r * ld + c) = w;
-                        if (Z != nullptr && r0 + r < p.B) *(uint32_t*)(Z + (long long)r * N + c) = w;
+                        const W w = pack_w<T>(v0, v1);
+                        *(W*)(dst + r * ld + c) = w;
+                        if (Z != nullptr && r0 + r < p.B) *(W*)(Z + (long long)r * N + c) = w;
                         if (l == 1 && wt != nullptr) {
-                            const uint32_t t = __ldg(wt + c / 2);
+                            const W t = __ldg(wt + c / 2);
                             dtau = fmaf(lo_w<T>(w), lo_w<T>(t), fmaf(hi_w<T>(w), hi_w<T>(t), dtau));
                         }
                     });
                 if (l > 0) zero_tail(dst, sm.lda, R, N);
-                __syncthreads();
+                work_sync();
             }
             if (want_t) {
                 t_dt += dtau;
@@ -472,7 +653,7 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
                     if (ajl == 0.f) continue;
                     float dot = 0.f;
                     for (int i = threadIdx.x; i < sm.pairs; i += kThreads) {
-                        const uint32_t q = sm.w(sm.ps)[j * sm.pairs + i], k = sm.w(sm.ks)[l * sm.pairs + i];
+                        const W q = sm.w(sm.ps)[j * sm.pairs + i], k = sm.w(sm.ks)[l * sm.pairs + i];
                         dot = fmaf(lo_w<T>(q), lo_w<T>(k), fmaf(hi_w<T>(q), hi_w<T>(k), dot));
                     }
                     t_dh = fmaf(ajl, dot, t_dh);
@@ -486,7 +667,7 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
 #pragma unroll
                 for (int j = RK_MAX_STAGES - 1; j >= 0; --j)
                     if (j < p.stages) {
-                        const uint32_t q = sm.w(sm.ps)[j * sm.pairs + i];
+                        const W q = sm.w(sm.ps)[j * sm.pairs + i];
                         d0 += lo_w<T>(q);
                         d1 += hi_w<T>(q);
                     }
@@ -510,7 +691,7 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
                 t_dh += __shfl_xor_sync(0xffffffffu, t_dh, o);
             }
             if ((threadIdx.x & 31) == 0) { sm.red[warp] = t_phi; sm.red[kWarps + warp] = t_dt; sm.red[2 * kWarps + warp] = t_dh; }
-            __syncthreads();
+            work_sync();
             if (threadIdx.x < 3) {
                 float x = 0.f;
                 for (int w = 0; w < kWarps; ++w) x += sm.red[threadIdx.x * kWarps + w];
@@ -519,7 +700,7 @@ __global__ void __launch_bounds__(kThreads) small_backward_kernel(const __grid_c
         }
     }
     if (p.commit) {
-        __syncthreads();
+        work_sync();
         for (int i = threadIdx.x; i < R * d; i += kThreads) {
             const int r = i / d, c = i - r * d;
             if (r0 + r < p.B) p.a[(long long)r0 * d + i] = sm.a[r * dp + c];
@@ -693,31 +874,50 @@ __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_cons
     }
 }
 
+constexpr int kSmemCap = 220 * 1024;
+// ring buffers that fit beside the block's own shared memory: eight (128 KB ahead) at most, two at least
+template <typename T> int ring_buffers(const SmallMlp& p, int rows) {
+    const int left = kSmemCap - (int)small_smem<T>(p, rows), n = left / (kUnitBytes + 16);
+    return n > 8 ? 8 : n;
+}
 template <typename K>
 bool allow_smem(K kernel, bool (&done)[kMaxDevices]) {
     const int dev = current_device();
     if (!done[dev]) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap) != cudaSuccess) { cudaGetLastError(); return false; }
         done[dev] = true;
     }
     return true;
 }
 
-// rows per block: 16 while that is at most one block per SM, else 32 (half the weight traffic per row)
-int rows_tiles(int B) { return (B + 15) / 16 <= sm_count() ? 1 : 2; }
+// row tiles per block: one (16 rows, in float32 8) while that is at most one block per SM, else two (half the weight traffic per row)
+int rows_tiles(mpode_dtype dt, int B) {
+    const int r = dt == MPODE_F32 ? 8 : 16;
+    return (B + r - 1) / r <= sm_count() ? 1 : 2;
+}
 
 template <typename T, int MT>
 bool forward_t(const SmallMlp& p, cudaStream_t st) {
     static bool done[kMaxDevices] = {false};
     if (!allow_smem(small_forward_kernel<T, MT>, done)) return false;
-    small_forward_kernel<T, MT><<<(p.B + 16 * MT - 1) / (16 * MT), kThreads, small_smem(p, 16 * MT), st>>>(p);
+    SmallMlp q = p;
+    q.ring = ring_buffers<T>(p, kRows<T, MT>);
+    if (q.ring < 2) return false;
+    const int rows = kRows<T, MT>, blocks = (p.B + rows - 1) / rows;
+    const size_t smem = small_smem<T>(p, rows) + q.ring * (kUnitBytes + 16);
+    small_forward_kernel<T, MT><<<blocks, kThreads + 32, smem, st>>>(q);
     return true;
 }
 template <typename T, int MT>
 bool backward_t(const SmallMlp& p, cudaStream_t st) {
     static bool done[kMaxDevices] = {false};
     if (!allow_smem(small_backward_kernel<T, MT>, done)) return false;
-    small_backward_kernel<T, MT><<<(p.B + 16 * MT - 1) / (16 * MT), kThreads, small_smem(p, 16 * MT), st>>>(p);
+    SmallMlp q = p;
+    q.ring = ring_buffers<T>(p, kRows<T, MT>);
+    if (q.ring < 2) return false;
+    const int rows = kRows<T, MT>, blocks = (p.B + rows - 1) / rows;
+    const size_t smem = small_smem<T>(p, rows) + q.ring * (kUnitBytes + 16);
+    small_backward_kernel<T, MT><<<blocks, kThreads + 32, smem, st>>>(q);
     return true;
 }
 template <typename T, int TM>
@@ -736,62 +936,96 @@ WgradItems wgrad_items(const SmallMlp& p, int tm) {
 
 }  // namespace
 
-size_t small_pack_bytes(int L, const int* wp) {
+size_t small_pack_elems(mpode_dtype dt, int n, int k) {      // columns, reduction
+    return dt == MPODE_F32 ? (size_t)n * k : (size_t)(n / 8) * k32(k) * 256;
+}
+size_t small_pack_bytes(mpode_dtype dt, int L, const int* wp) {
     size_t n = 0;
-    for (int l = 0; l < L; ++l) n += (size_t)32 * ((wp[l + 1] / 8) * k32(wp[l]) + (wp[l] / 8) * k32(wp[l + 1]));
-    return n * sizeof(uint4);
+    for (int l = 0; l < L; ++l) n += small_pack_elems(dt, wp[l + 1], wp[l]) + small_pack_elems(dt, wp[l], wp[l + 1]);
+    return n * low_size(dt);
 }
 
 bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp) {
-    if (dt != MPODE_BF16 && dt != MPODE_F16) return false;
     if (L < 1 || L > SMALL_MAX_L) return false;
     SmallMlp p{};
     p.L = L; p.stages = RK_MAX_STAGES;
     long long elems = 0;
     for (int l = 0; l <= L; ++l) { p.wp[l] = p.wr[l] = wp[l]; if (l < L) elems += (long long)wp[l] * wp[l + 1]; }
-    return small_smem(p, 32) <= 200 * 1024 && elems <= 160 * 1024 && B <= 8192;
+    if (dt == MPODE_F32) return ring_buffers<float>(p, 16) >= 3 && elems <= 256 * 1024 && B <= 16 * sm_count();
+    return ring_buffers<__half>(p, 32) >= 3 && elems <= 160 * 1024 && B <= 8192;
+}
+
+int small_blocks(mpode_dtype dt, int B) {
+    const int r = (dt == MPODE_F32 ? 8 : 16) * rows_tiles(dt, B);
+    return (B + r - 1) / r;
 }
 
 void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
     PackJob job{};
+    const int unit = dt == MPODE_F32 ? 1 : 8;                // elements a thread writes
     for (int l = 0; l < p.L; ++l) {
-        job.first[2 * l + 1] = job.first[2 * l] + (long long)32 * (p.wp[l + 1] / 8) * k32(p.wp[l]);
-        job.first[2 * l + 2] = job.first[2 * l + 1] + (long long)32 * (p.wp[l] / 8) * k32(p.wp[l + 1]);
+        job.first[2 * l + 1] = job.first[2 * l] + (long long)small_pack_elems(dt, p.wp[l + 1], p.wp[l]) / unit;
+        job.first[2 * l + 2] = job.first[2 * l + 1] + (long long)small_pack_elems(dt, p.wp[l], p.wp[l + 1]) / unit;
     }
     long long blocks = (job.first[2 * p.L] + 255) / 256;
     if (blocks > 148 * 4) blocks = 148 * 4;
     if (dt == MPODE_BF16) small_pack_kernel<__nv_bfloat16><<<(int)blocks, 256, 0, st>>>(p, job);
-    else small_pack_kernel<__half><<<(int)blocks, 256, 0, st>>>(p, job);
+    else if (dt == MPODE_F16) small_pack_kernel<__half><<<(int)blocks, 256, 0, st>>>(p, job);
+    else small_pack_f32_kernel<<<(int)blocks, 256, 0, st>>>(p, job);
     if (launches) ++*launches;
 }
 
 bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    const bool one = rows_tiles(p.B) == 1;
+    const bool one = rows_tiles(dt, p.B) == 1;
     const bool ok = dt == MPODE_BF16 ? (one ? forward_t<__nv_bfloat16, 1>(p, st) : forward_t<__nv_bfloat16, 2>(p, st))
-                                     : (one ? forward_t<__half, 1>(p, st) : forward_t<__half, 2>(p, st));
+                  : dt == MPODE_F16  ? (one ? forward_t<__half, 1>(p, st) : forward_t<__half, 2>(p, st))
+                                     : (one ? forward_t<float, 1>(p, st) : forward_t<float, 2>(p, st));
     if (ok && launches) ++*launches;
     if (ok && tl_counters) ++tl_counters->fused;
     return ok;
 }
 
 bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    const bool one = rows_tiles(p.B) == 1;
+    const bool one = rows_tiles(dt, p.B) == 1;
     const bool ok = dt == MPODE_BF16 ? (one ? backward_t<__nv_bfloat16, 1>(p, st) : backward_t<__nv_bfloat16, 2>(p, st))
-                                     : (one ? backward_t<__half, 1>(p, st) : backward_t<__half, 2>(p, st));
+                  : dt == MPODE_F16  ? (one ? backward_t<__half, 1>(p, st) : backward_t<__half, 2>(p, st))
+                                     : (one ? backward_t<float, 1>(p, st) : backward_t<float, 2>(p, st));
     if (ok && launches) ++*launches;
     if (ok && tl_counters) ++tl_counters->fused;
     return ok;
 }
 
-int small_blocks(int B) { return (B + 16 * rows_tiles(B) - 1) / (16 * rows_tiles(B)); }
-
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    if (dt == MPODE_BF16) small_time_kernel<__nv_bfloat16><<<1, 96, 0, st>>>(p, small_blocks(p.B));
-    else small_time_kernel<__half><<<1, 96, 0, st>>>(p, small_blocks(p.B));
+    const int blocks = small_blocks(dt, p.B);
+    if (dt == MPODE_BF16) small_time_kernel<__nv_bfloat16><<<1, 96, 0, st>>>(p, blocks);
+    else if (dt == MPODE_F16) small_time_kernel<__half><<<1, 96, 0, st>>>(p, blocks);
+    else small_time_kernel<float><<<1, 96, 0, st>>>(p, blocks);
     if (launches) ++*launches;
 }
 
+// float32: the CUDA-core contraction per layer and step (the rows of all stages are its reduction range; it takes the bias and the time
+// column along)
+static bool small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launches) {
+    for (int s = 0; s < p.count; ++s)
+        for (int l = 0; l < p.L; ++l) {
+            const bool time = p.time && l == 0;
+            const size_t rows = (size_t)p.stages * p.B;
+            GemmArgs g{};
+            g.A = (const float*)p.zs[l + 1] + s * rows * p.wp[l + 1]; g.a_rs = 1; g.a_ks = p.wp[l + 1];
+            g.B = (const float*)p.xs[l] + s * rows * p.wp[l]; g.b_rs = 1; g.b_ks = p.wp[l];
+            g.M = p.wr[l + 1]; g.N = p.wr[l]; g.K = (int)rows;
+            g.epi = EPI_WGRAD; g.out = p.out + p.woff[l]; g.ldo = p.wr[l] + (time ? 1 : 0); g.beta = s == 0 ? p.beta : 1.f; g.alpha = p.coef[s];
+            g.split_k = 1;
+            g.row_sum = p.bias ? p.out + p.boff[l] : nullptr;
+            if (time) { g.row_sum_time = p.out + p.woff[l] + p.wr[l]; g.k_tau = p.scal[0].tau16 + (size_t)(p.step_hi - s) * (sizeof(RkStepScalars) / 4); g.k_per = p.B; }
+            if (!launch_gemm_simt(MPODE_F32, g, st, launches)) return false;
+            if (tl_counters) ++tl_counters->simt;
+        }
+    return true;
+}
+
 bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    if (dt == MPODE_F32) return small_wgrad_f32(p, st, launches);
     // 32 x 32 pieces where there are enough of them to occupy half the SMs, else 16 x 16 (each block reads its operands from L2: a
     // smaller piece reads more in total but less per block)
     WgradItems items = wgrad_items(p, 32);

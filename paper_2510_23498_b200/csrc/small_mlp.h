@@ -1,4 +1,4 @@
-// Row-local kernels for small dense velocities in the 16-bit formats: see small_mlp.cu.
+// Row-local kernels for small dense velocities: see small_mlp.cu.
 #pragma once
 #include "common.cuh"
 #include "rk_fused.h"
@@ -11,8 +11,7 @@ struct SmallMlp {
     int B, L, stages, act, time, bias, round_increment;
     int wr[SMALL_MAX_L + 1], wp[SMALL_MAX_L + 1];      // layer widths; rounded up to multiples of 8
     const float* theta; long long woff[SMALL_MAX_L], boff[SMALL_MAX_L];
-    // weights in the order the matrix instructions read them (launch_small_pack): [column tile of 8][32 of the reduction][lane] 16 bytes;
-    // forward: columns = outputs, reduction = inputs; backward: the other way round.  Biases and time column: low format, padded with zeros
+    // weights in the order they are used (launch_small_pack): matrix instruction fragments, or rows in float32; forward: columns = outputs, reduction = inputs; backward: the other way round.  Biases and time column: low format, padded with zeros
     uint4 *wf[SMALL_MAX_L], *wb[SMALL_MAX_L];
     void *b16[SMALL_MAX_L], *wt16;
     const RkStepScalars* scal;                         // device, indexed by absolute step
@@ -27,6 +26,8 @@ struct SmallMlp {
     void* zs[SMALL_MAX_L + 1];                         // cotangents dZ_l, l = 1 .. L (dZ_L = kappa_j): [slot][stages][B][wp_l]
     void* psi[4];                                      // without commit: psi_j, low [B][wp_0]
     unsigned* flag;
+    unsigned* err;                                     // a bounded wait that gave up
+    int ring;                                          // buffers of the weight stream (set by the launch)
     // time-grid gradient (null: not wanted): [slot][blocks][3] shares; results of the last step [3]; t' [n + 1], updated per step
     float *tpart, *tvals, *tprime;
     // weight gradient: out = beta out + sum over the slots of coef[slot] (parameter gradient of the step)
@@ -35,13 +36,14 @@ struct SmallMlp {
 constexpr int SMALL_MAX_CHUNK = 16;
 
 // bytes of packed weights (both directions); whether the kernels take these widths
-size_t small_pack_bytes(int L, const int* wp);
+size_t small_pack_elems(mpode_dtype dt, int n, int k);      // of one layer and direction: n columns, reduction of k
+size_t small_pack_bytes(mpode_dtype dt, int L, const int* wp);
 bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp);
 
 void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
-int small_blocks(int B);                               // blocks of the forward and backward kernels
+int small_blocks(mpode_dtype dt, int B);                               // blocks of the forward and backward kernels
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 

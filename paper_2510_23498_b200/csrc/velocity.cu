@@ -155,38 +155,44 @@ public:
     // Row-local kernels (small_mlp.cu): packed weights, and the layer inputs and cotangents of a few steps at a time (8 MB at most, or
     // one step's)
     void plan_small(Layout& lay) {
-        small_ok_ = !tiny_ok_ && small_mlp_supported(dt_, B_, L_, wp_.data());
+        small_w_.clear();
+        for (int w : w_) small_w_.push_back((w + 7) / 8 * 8);
+        // (the float32 buffers of the other paths are not padded: the state's rows have to agree)
+        small_ok_ = !tiny_ok_ && (dt_ != MPODE_F32 || w_[0] % 8 == 0) && small_mlp_supported(dt_, B_, L_, small_w_.data());
         if (!small_ok_) return;
         const size_t es = low_size(dt_);
         size_t per_step = 0;
-        for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (wp_[l] + wp_[l + 1]) * es;
+        for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
         small_chunk_ = (int)(((size_t)8 << 20) / per_step);
         if (small_chunk_ < 1) small_chunk_ = 1;
         if (small_chunk_ > SMALL_MAX_CHUNK) small_chunk_ = SMALL_MAX_CHUNK;
         if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
-        small_pack_ = lay.take(small_pack_bytes(L_, wp_.data()));
+        small_pack_ = lay.take(small_pack_bytes(dt_, L_, small_w_.data()));
+        for (int l = 0; l < L_; ++l) small_b_[l] = lay.take((size_t)small_w_[l + 1] * es);
+        small_wt_ = lay.take((size_t)small_w_[1] * es);
         small_scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
         for (int l = 0; l < L_; ++l) {
-            small_xs_[l] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * wp_[l] * es);
-            small_zs_[l + 1] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * wp_[l + 1] * es);
+            small_xs_[l] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
+            small_zs_[l + 1] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
         }
-        if (lay.time_gradient) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(B_) * 3 * sizeof(float));
+        if (lay.time_gradient) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
     }
     SmallMlp small_params(void* ws) const {
         SmallMlp p{};
         p.B = B_; p.L = L_; p.act = act_; p.time = time_ ? 1 : 0; p.bias = bias_ ? 1 : 0;
         p.theta = theta_;
         size_t off = small_pack_;
-        for (int l = 0; l <= L_; ++l) { p.wr[l] = w_[l]; p.wp[l] = wp_[l]; }
+        for (int l = 0; l <= L_; ++l) { p.wr[l] = w_[l]; p.wp[l] = small_w_[l]; }
         for (int l = 0; l < L_; ++l) {
             p.woff[l] = (long long)woff_[l]; p.boff[l] = (long long)boff_[l];
-            p.wf[l] = (uint4*)at(ws, off); off += (size_t)512 * (wp_[l + 1] / 8) * ((wp_[l] + 31) / 32);
-            p.wb[l] = (uint4*)at(ws, off); off += (size_t)512 * (wp_[l] / 8) * ((wp_[l + 1] + 31) / 32);
-            p.b16[l] = bias_ ? at(ws, b16_[l]) : nullptr;
+            p.wf[l] = (uint4*)at(ws, off); off += small_pack_elems(dt_, small_w_[l + 1], small_w_[l]) * low_size(dt_);
+            p.wb[l] = (uint4*)at(ws, off); off += small_pack_elems(dt_, small_w_[l], small_w_[l + 1]) * low_size(dt_);
+            p.b16[l] = bias_ ? at(ws, small_b_[l]) : nullptr;
             p.xs[l] = at(ws, small_xs_[l]); p.zs[l + 1] = at(ws, small_zs_[l + 1]);
         }
-        p.wt16 = time_ ? at(ws, wt16_) : nullptr;
+        p.wt16 = time_ ? at(ws, small_wt_) : nullptr;
         p.scal = (const RkStepScalars*)at(ws, small_scal_);
+        p.err = (unsigned*)at(ws, lay_->scal) + 2;
         for (int j = 0; j < 4; ++j) p.psi[j] = at(ws, lay_->psi[j]);
         return p;
     }
@@ -776,7 +782,8 @@ protected:
     int small_chunk_ = 1;
     size_t small_pack_ = 0, small_scal_ = 0, small_xs_[SMALL_MAX_L] = {0}, small_zs_[SMALL_MAX_L + 1] = {0};
     SmallMlp small_bwd_{}, small_step_{};
-    size_t small_tpart_ = 0;
+    size_t small_tpart_ = 0, small_b_[SMALL_MAX_L] = {0}, small_wt_ = 0;
+    std::vector<int> small_w_;
     const float* theta_ = nullptr;
     bool fused_ok_ = false;
     bool keep_k_ = false;
