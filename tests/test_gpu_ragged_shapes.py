@@ -79,3 +79,14 @@ def test_small_networks_at_tile_edges(batch, widths, n_steps):
         assert gpu["stats"]["fused_launches"] > 0 and gpu["stats"]["simt_contractions"] == 0
         if scaling == "dynamic":
             assert_same_log(gpu["log"], orc["log"])
+
+
+# the same in float32 (CUDA cores): one row, a block's 8 rows less and plus one, more row tiles than SMs, odd widths, 1 to 4 layers
+@pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (7, [9, 33, 65, 9], 3), (9, [64, 64], 20), (200, [72, 201, 200, 72], 2),
+                                                  (1185, [24, 40, 24], 2), (130, [16, 32, 48, 32, 16], 3)])
+def test_small_float32_networks_at_tile_edges(batch, widths, n_steps):
+    wl = inputs.mlp_block(batch=batch, n_steps=n_steps, d=widths[0], hidden=widths[1], low="f32")
+    wl.vel["n_layers"], wl.vel["widths"], wl.theta = len(widths) - 1, widths, inputs.mlp_theta(3, widths, True)
+    gpu = run_gpu(wl, low="f32")
+    assert_parity(gpu, run_oracle(wl, exact=True), TOL["f32"])
+    assert gpu["stats"]["fused_launches"] > 0
