@@ -11,7 +11,7 @@
 //              barrier), takes Alg. 2's decision from the same words, and commits its share.  The stages of the step before are
 //              recomputed while the first barrier is waited for: they do not depend on the outcome.
 // Measured (1024 samples, 128 weight sets, 128 RK4 steps, float16 with dynamic scaling): 14.3 ms per training pass with launches per
-// step, 3.7 ms with these two (forward 0.35, backward 3.25).
+// step, 3.56 ms with these two (forward 0.35, backward 3.25).
 // Rounding points and formulas are those of hyper_cnf.cu; sums run in another, fixed order.
 #include <math.h>
 
@@ -253,6 +253,10 @@ __device__ __forceinline__ int initial_exponent(float m, int pbits) {
     return e < -100 ? -100 : (e > 100 ? 100 : e);
 }
 
+constexpr int kMaxKept = 64;                                     // hidden widths up to this keep the second layer in shared memory
+// the last layer's row of entry r of weight set u (W_u, b_u, U_u)
+__device__ __forceinline__ int set_row(int u, int r, int w, int d) { return r < d ? u * d + r : (r == d ? w * d + u : w * d + w + u * d + r - d - 1); }
+
 // Device words: [0] barrier counter, [1] error, [2 .. 5] flag of attempt n in word 2 + n % 4, [6 .. 9] ||a||_inf likewise
 template <typename T, int DC>
 __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p) {
@@ -273,7 +277,9 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
     float* ob = tot + s * nv;                                    // [stages * (2 d + 1)]
     float* hb = ob + s * (2 * d + 1);                            // h2bar [stages][h], h1bar [stages][h]
     float* tred = hb + 2 * s * h;                                // [blockDim]
-    T* ua = (T*)(tred + blockDim.x);                             // [2][stages][warps][w] units
+    float* A2q = tred + blockDim.x;                              // Q16 of the second layer [h][h], where it is small
+    float* A3q = A2q + (h <= kMaxKept ? h * h : 0);              // Q16 of the last layer's rows of weight set blockIdx.x [2 d + 1][h]
+    T* ua = (T*)(A3q + (2 * d + 1) * h);                         // [2][stages][warps][w] units
     T* us = ua + (size_t)2 * s * warps * w;                      // [stages][warps][w] unit cotangents
     const T* traj = (const T*)p.traj;
     const bool dynamic = p.scaling == MPODE_SCALE_DYNAMIC, checked = p.scaling != MPODE_SCALE_NONE;
@@ -329,6 +335,10 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
         for (int q = 16; q > 0; q >>= 1) my_max = fmaxf(my_max, __shfl_xor_sync(0xffffffffu, my_max, q));
         if (lane == 0 && my_max > 0.f) atomicMax(p.words + 6 + slot, __float_as_uint(my_max));      // non-negative floats order like their bits
     };
+    if (h <= kMaxKept)
+        for (int i = threadIdx.x; i < h * h; i += blockDim.x) A2q[i] = q16<T>(p.theta[o.A2 + i]);
+    if ((int)blockIdx.x < w)
+        for (int i = threadIdx.x; i < (2 * d + 1) * h; i += blockDim.x) A3q[i] = q16<T>(p.theta[o.A3 + (long long)set_row(blockIdx.x, i / h, w, d) * h + i % h]);
     int att = 0;                                                 // attempts so far; attempt 0 is the initialisation
     load(p.n_steps - 1);
     publish(0, bad, (amax <= 3.4028234e38f) ? amax : 0.f);
@@ -470,15 +480,24 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
                     float acc[2 * DM + 2];
 #pragma unroll
                     for (int i = 0; i < 2 * DM + 2; ++i) acc[i] = 0.f;
+#pragma unroll 4
                     for (int r = 0; r < n_smp; ++r) {
                         const float a = Low<T>::to_f(ua[((size_t)(par * s + j) * warps + r) * w + u]);
                         const float sbar = Low<T>::to_f(us[((size_t)j * warps + r) * w + u]);
+                        const float* zr = zs + ((par * s + j) * warps + r) * d;
+                        const float* kr = kz + (j * warps + r) * d;
+                        if constexpr (DC == 2) {
+                            const float2 z2 = *reinterpret_cast<const float2*>(zr), k2 = *reinterpret_cast<const float2*>(kr);
+                            acc[0] = fmaf(sbar, z2.x, acc[0]); acc[1] = fmaf(sbar, z2.y, acc[1]);
+                            acc[DM + 1] = fmaf(a * inv_w, k2.x, acc[DM + 1]); acc[DM + 2] = fmaf(a * inv_w, k2.y, acc[DM + 2]);
+                        } else {
 #pragma unroll
-                        for (int i = 0; i < DM; ++i)
-                            if (i < d) {
-                                acc[i] = fmaf(sbar, zs[((par * s + j) * warps + r) * d + i], acc[i]);
-                                acc[DM + 1 + i] = fmaf(a * inv_w, kz[(j * warps + r) * d + i], acc[DM + 1 + i]);
-                            }
+                            for (int i = 0; i < DM; ++i)
+                                if (i < d) {
+                                    acc[i] = fmaf(sbar, zr[i], acc[i]);
+                                    acc[DM + 1 + i] = fmaf(a * inv_w, kr[i], acc[DM + 1 + i]);
+                                }
+                        }
                         acc[DM] += sbar;
                         acc[2 * DM + 1] = fmaf(-kl[j * warps + r] * inv_w, 1.f - a * a, acc[2 * DM + 1]);
                     }
@@ -511,7 +530,7 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
                     for (int v0 = lane; v0 < s * nv; v0 += 32) {
                         float x = 0.f;
                         const int nb = groups < G ? groups : G;   // blocks that hold samples
-#pragma unroll 8
+#pragma unroll 16
                         for (int r = warp; r < nb; r += warps) x += __ldcg(p.part + ((long long)r * w + u) * s * nv + v0);
                         red[warp * s * nv + v0] = x;
                     }
@@ -534,23 +553,21 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
                         ob[q] = v;
                     }
                     __syncthreads();
-                    // rows of the last layer that belong to weight set u: their gradient, and their part of the cotangent of h2
+                    // their part of the cotangent of h2, then the gradient of the last layer's rows that belong to weight set u
+                    const bool kept = u == (int)blockIdx.x;
+                    for (int q = threadIdx.x; q < s * h; q += blockDim.x) {
+                        const int j = q / h, k = q - j * h;
+                        float t = 0.f;
+                        for (int r = 0; r < 2 * d + 1; ++r)
+                            t = fmaf(kept ? A3q[r * h + k] : q16<T>(p.theta[o.A3 + (long long)set_row(u, r, w, d) * h + k]), ob[j * (2 * d + 1) + r], t);
+                        p.tpart[(long long)u * s * h + q] = t;
+                    }
                     for (int q = threadIdx.x; q < (2 * d + 1) * (h + 1); q += blockDim.x) {
-                        const int r = q / (h + 1), k = q - r * (h + 1);
-                        const int row = r < d ? u * d + r : (r == d ? w * d + u : w * d + w + u * d + r - d - 1);
+                        const int r = q / (h + 1), k = q - r * (h + 1), row = set_row(u, r, w, d);
                         float x = 0.f;
                         for (int j = s - 1; j >= 0; --j) x = k < h ? fmaf(ob[j * (2 * d + 1) + r], set0[j * sf + h + k], x) : x + ob[j * (2 * d + 1) + r];
                         bad2 |= q_bad<T>(q16<T>(x));
                         p.dg[k < h ? o.A3 + (long long)row * h + k : o.c3 + row] = x;
-                    }
-                    for (int q = threadIdx.x; q < s * h; q += blockDim.x) {
-                        const int j = q / h, k = q - j * h;
-                        float t = 0.f;
-                        for (int r = 0; r < 2 * d + 1; ++r) {
-                            const int row = r < d ? u * d + r : (r == d ? w * d + u : w * d + w + u * d + r - d - 1);
-                            t = fmaf(q16<T>(p.theta[o.A3 + (long long)row * h + k]), ob[j * (2 * d + 1) + r], t);
-                        }
-                        p.tpart[(long long)u * s * h + q] = t;
                     }
                     __syncthreads();
                 }
@@ -572,7 +589,7 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
                     const int q = q0 + (int)threadIdx.x % min(sh, (int)blockDim.x), pc = (int)threadIdx.x / min(sh, (int)blockDim.x);
                     float t = 0.f;
                     if (q < sh && pc < parts) {
-#pragma unroll 16
+#pragma unroll 32
                         for (int u = pc; u < w; u += parts) t += __ldcg(p.tpart + (long long)u * sh + q);
                     }
                     __syncthreads();
@@ -593,28 +610,40 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
                     const int j = q / h, l = q - j * h;
                     float t = 0.f;
 #pragma unroll 8
-                    for (int k = 0; k < h; ++k) t = fmaf(q16<T>(p.theta[o.A2 + k * h + l]), hb[j * h + k], t);
+                    for (int k = 0; k < h; ++k) t = fmaf(h <= kMaxKept ? A2q[k * h + l] : q16<T>(p.theta[o.A2 + k * h + l]), hb[j * h + k], t);
                     const float h1 = set0[j * sf + l];
                     const float v = q16<T>((1.f - h1 * h1) * t);
                     bad3 |= q_bad<T>(v);
                     hb[sh + q] = v;
                 }
                 __syncthreads();
-                // gradients of A2 | c2 | A1 | c1, stages added last to first; block 0 keeps them
-                for (int q = threadIdx.x; q < h * h + 3 * h; q += blockDim.x) {
-                    float x = 0.f;
-                    int at;
-                    if (q < h * h) {
-                        const int k = q / h, l = q - k * h;
-                        for (int j = s - 1; j >= 0; --j) x = fmaf(hb[j * h + k], set0[j * sf + l], x);
-                        at = o.A2 + q;
-                    } else {
-                        const int k = (q - h * h) % h, what = (q - h * h) / h;
-                        for (int j = s - 1; j >= 0; --j) x = what == 1 ? fmaf(hb[sh + j * h + k], sc.tau16[j], x) : x + hb[(what == 0 ? 0 : sh) + j * h + k];
-                        at = what == 0 ? o.c2 + k : (what == 1 ? o.A1 + k : o.c1 + k);
+                // Gradients of A2 | c2 | A1 | c1, stages added last to first: block 0 forms them.  Are their roundings finite?  Every entry
+                // is at most sum_j max |hbar_j| max(1, |tau_j|) (h1 and h2 lie in [-1, 1]); only if that bound does not fit the format do
+                // the other blocks look at the entries too.
+                float bound = 0.f;
+                for (int j = 0; j < s; ++j) {
+                    float m1 = 0.f;
+                    for (int k = lane; k < h; k += 32) m1 = fmaxf(m1, fmaxf(fabsf(hb[j * h + k]), fabsf(hb[sh + j * h + k])));
+#pragma unroll
+                    for (int q = 16; q > 0; q >>= 1) m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, q));
+                    bound += m1 * fmaxf(1.f, fabsf(sc.tau16[j]));
+                }
+                if (blockIdx.x == 0 || q_bad<T>(q16<T>(2.f * bound))) {
+                    for (int q = threadIdx.x; q < h * h + 3 * h; q += blockDim.x) {
+                        float x = 0.f;
+                        int at;
+                        if (q < h * h) {
+                            const int k = q / h, l = q - k * h;
+                            for (int j = s - 1; j >= 0; --j) x = fmaf(hb[j * h + k], set0[j * sf + l], x);
+                            at = o.A2 + q;
+                        } else {
+                            const int k = (q - h * h) % h, what = (q - h * h) / h;
+                            for (int j = s - 1; j >= 0; --j) x = what == 1 ? fmaf(hb[sh + j * h + k], sc.tau16[j], x) : x + hb[(what == 0 ? 0 : sh) + j * h + k];
+                            at = what == 0 ? o.c2 + k : (what == 1 ? o.A1 + k : o.c1 + k);
+                        }
+                        bad3 |= q_bad<T>(q16<T>(x));
+                        if (blockIdx.x == 0) p.dg[at] = x;
                     }
-                    bad3 |= q_bad<T>(q16<T>(x));
-                    if (blockIdx.x == 0) p.dg[at] = x;
                 }
             }
             const bool any_bad = __syncthreads_or(checked && (bad3 || *(volatile unsigned*)(p.words + 2 + slot) != 0u)) != 0;
@@ -639,7 +668,7 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
         for (int u = blockIdx.x; u < w; u += G)
             for (int q = threadIdx.x; q < (2 * d + 1) * (h + 1); q += blockDim.x) {
                 const int r = q / (h + 1), k = q - r * (h + 1);
-                const int row = r < d ? u * d + r : (r == d ? w * d + u : w * d + w + u * d + r - d - 1);
+                const int row = set_row(u, r, w, d);
                 const long long at = k < h ? o.A3 + (long long)row * h + k : o.c3 + row;
                 p.g[at] = fmaf(coef, p.dg[at], p.g[at]);
             }
@@ -666,7 +695,7 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
         for (int u = blockIdx.x; u < w; u += G)
             for (int q = threadIdx.x; q < (2 * d + 1) * (h + 1); q += blockDim.x) {
                 const int r = q / (h + 1), k = q - r * (h + 1);
-                const int row = r < d ? u * d + r : (r == d ? w * d + u : w * d + w + u * d + r - d - 1);
+                const int row = set_row(u, r, w, d);
                 p.g[k < h ? o.A3 + (long long)row * h + k : o.c3 + row] = INFINITY;
             }
         if (blockIdx.x == 0) {
@@ -679,7 +708,7 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
 
 size_t backward_smem(mpode_dtype dt, int stages, int h, int w, int d, int warps) {
     const size_t sf = hyper_stage_floats(h, w, d), s = stages, nv = 2 * d + 2;
-    const size_t fl = 2 * (s * sf + kScalarFloats) + 3 * s * warps * d + s * warps + warps * s * nv + s * nv + s * (2 * d + 1) + 2 * s * h + 32 * (size_t)warps;
+    const size_t fl = 2 * (s * sf + kScalarFloats) + 3 * s * warps * d + s * warps + warps * s * nv + s * nv + s * (2 * d + 1) + 2 * s * h + 32 * (size_t)warps + (h <= kMaxKept ? (size_t)h * h : 0) + (2 * d + 1) * (size_t)h;
     return fl * sizeof(float) + 3 * s * warps * w * low_size(dt);
 }
 constexpr size_t kSmemCap = 200 * 1024;
