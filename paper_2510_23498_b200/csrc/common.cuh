@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/mpode.h"
 
 namespace mpode {
@@ -69,6 +71,32 @@ __device__ __forceinline__ void warp_flag_or(unsigned* flag, bool bad) {
     // every lane of the warp must call this (kernels accumulate `bad` in a register and call it once at the end)
     unsigned any = __ballot_sync(0xffffffffu, bad);
     if (flag != nullptr && any != 0u && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
+}
+
+// ---------------------------------------------------------------- chained launches
+// The layer-by-layer paths are chains of kernels of a few microseconds each, and between two of them lie about 2 us of launch and
+// drain.  Every kernel of such a chain is launched with programmatic serialisation, which lets its launch be processed while its
+// predecessor runs, and starts with chain_begin(), which waits until the predecessor has finished and its writes are visible; memory
+// that others write is touched only behind it.  (Letting the successor's blocks start as soon as all of a kernel's blocks run was
+// slower: they pile up on the SMs that are free first.  Measured, ms per pass, plain launches / this / early start: flow with 63
+// features 14.3 / 10.7 / 11.8, flow with 784 features 15.4 / 13.5 / 13.9, parabolic block 14.05 / 13.56 / 14.99, convolution block
+// 24.5 / 22.4 / 23.7, its forward pass on 37 images 0.91 / 0.63 / 0.66.)
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // ---------------------------------------------------------------- dense / implicit-conv contraction (SIMT path)

@@ -176,6 +176,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *(volatile uint32_t*)tmem_holder;
+    chain_begin();                          // everything above overlaps the tail of the kernel before
 
     if (warp == 0) {
         // ------------------------------------------------------------ loads: the weights once, then one halo block per tile
@@ -382,6 +383,7 @@ conv3x3_wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *(volatile uint32_t*)tmem_holder;
+    chain_begin();                          // everything above overlaps the tail of the kernel before
 
     if (warp == 0) {
         if (lane == 0) {
@@ -486,6 +488,7 @@ __global__ void __launch_bounds__(256) conv_wgrad_halo_reduce_kernel(const float
                                                                        float beta, float sign, float* __restrict__ class_part, float tau,
                                                                        float* __restrict__ wt_out, float* __restrict__ bias_out,
                                                                        unsigned* __restrict__ counter) {
+    chain_begin();
     __shared__ float4 sm4[8 * 32];
     float* sm = reinterpret_cast<float*>(sm4);
     __shared__ bool last;
@@ -560,7 +563,7 @@ bool launch_halo(const CUtensorMap& tx, const CUtensorMap& tw, const ConvParams&
         attr_set[dev] = true;
     }
     const int grid = p.tiles < sm_count() ? p.tiles : sm_count();
-    conv3x3_halo_kernel<T><<<grid, kThreads, kSmemBytes, st>>>(tx, tw, p);
+    launch_chain(conv3x3_halo_kernel<T>, dim3(grid), dim3(kThreads), kSmemBytes, st, tx, tw, p);
     return true;
 }
 
@@ -660,10 +663,10 @@ bool launch_conv_wgrad_halo(mpode_dtype dt, const void* dz, const void* x, const
         if (e != cudaSuccess) { cudaGetLastError(); return false; }
         attr_set[dev][fi] = true;
     }
-    if (dt == MPODE_BF16) conv3x3_wgrad_halo_kernel<__nv_bfloat16><<<grid, 320, smem_bytes, st>>>(tx, tz, ti, p);
-    else conv3x3_wgrad_halo_kernel<__half><<<grid, 320, smem_bytes, st>>>(tx, tz, ti, p);
+    if (dt == MPODE_BF16) launch_chain(conv3x3_wgrad_halo_kernel<__nv_bfloat16>, dim3(grid), dim3(320), smem_bytes, st, tx, tz, ti, p);
+    else launch_chain(conv3x3_wgrad_halo_kernel<__half>, dim3(grid), dim3(320), smem_bytes, st, tx, tz, ti, p);
     if (launches) ++*launches;
-    conv_wgrad_halo_reduce_kernel<<<kWgMatrixBlocks + kWgClassBlocks, 256, 0, st>>>(partial, grid, ct, out, beta, sign, class_part, tau,
+    launch_chain(conv_wgrad_halo_reduce_kernel, dim3(kWgMatrixBlocks + kWgClassBlocks), dim3(256), 0, st, partial, grid, ct, out, beta, sign, class_part, tau,
                                                                                     ct > kC ? out : nullptr, bias_out, counter);
     if (launches) ++*launches;
     return true;

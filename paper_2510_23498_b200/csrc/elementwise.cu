@@ -32,6 +32,7 @@ inline bool aligned_to(const void* p, size_t a) { return ((uintptr_t)p % a) == 0
 template <typename T>
 __global__ void quantize_matrix_kernel(const float* __restrict__ src, long long src_ld, int rows, int cols, int rp, int cp,
                                        T* __restrict__ dst, T* __restrict__ dst_t) {
+    chain_begin();
     __shared__ float tile[32][33];
     int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -54,6 +55,7 @@ __global__ void quantize_matrix_kernel(const float* __restrict__ src, long long 
 template <typename T>
 __global__ void quantize_conv_weights_kernel(const float* __restrict__ src, int cout, int cin_total, int cin_keep,
                                              T* __restrict__ dst, T* __restrict__ dst_flip_t, float sign) {
+    chain_begin();
     long long n = (long long)cout * 9 * cin_keep;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         int c = (int)(i % cin_keep);
@@ -71,6 +73,7 @@ __global__ void quantize_conv_weights_kernel(const float* __restrict__ src, int 
 template <typename T>
 __global__ void conv_class_bias_kernel(const T* __restrict__ b, const T* __restrict__ w, int cin_total, float tau, int C,
                                        float* __restrict__ out) {
+    chain_begin();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 9 * C) return;
     int cls = i / C, co = i - cls * C, ry = cls / 3, rx = cls - ry * 3;
@@ -90,6 +93,7 @@ __global__ void conv_class_bias_kernel(const T* __restrict__ b, const T* __restr
 // tap through shared memory so that both sides are read and written in whole 128-byte lines.  C is a multiple of 32.
 __global__ void __launch_bounds__(256) conv_wgrad_reduce_kernel(const float* __restrict__ partial, int S, int C, int ct, float* __restrict__ out,
                                                                  float beta, float sign) {
+    chain_begin();
     __shared__ float tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int cin0 = blockIdx.x * 32, co0 = blockIdx.y * 32, tap = blockIdx.z;
@@ -118,6 +122,7 @@ __global__ void __launch_bounds__(256) conv_wgrad_reduce_kernel(const float* __r
 template <typename T>
 __global__ void __launch_bounds__(128, 4) conv_class_sums_kernel(const T* __restrict__ dz, long long pixels, int H, int W, int C,
                                                                 long long per_block, float* __restrict__ part) {
+    chain_begin();
     extern __shared__ float sm[];                    // [9 * 8][128]: value (class, e) of every thread
     const int groups = C / 8;                        // threads per pixel
     const int cg = threadIdx.x % groups, pl = threadIdx.x / groups, lanes = blockDim.x / groups;
@@ -189,6 +194,7 @@ __global__ void __launch_bounds__(128, 4) conv_class_sums_kernel(const T* __rest
 // gradient of that channel's weights per tap (tau times the sum over the classes in which the tap is inside the image).
 // One warp per (class, channel): the per-block sums added by the lanes in a fixed order, then a fixed shuffle tree
 __global__ void conv_class_reduce_kernel(const float* __restrict__ part, int blocks, int n, float* __restrict__ cs) {
+    chain_begin();
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n) return;
     float s = 0.f;
@@ -199,6 +205,7 @@ __global__ void conv_class_reduce_kernel(const float* __restrict__ part, int blo
 }
 __global__ void conv_class_final_kernel(const float* __restrict__ cs_in, int C, int ct, float tau, float* __restrict__ wt_out,
                                         float* __restrict__ bias_out, float beta) {
+    chain_begin();
     extern __shared__ float cs[];                    // [9][C] class sums
     for (int i = threadIdx.x; i < 9 * C; i += blockDim.x) cs[i] = cs_in[i];
     __syncthreads();
@@ -209,6 +216,7 @@ __global__ void conv_class_final_kernel(const float* __restrict__ cs_in, int C, 
 template <typename T, int V>
 __global__ void init_state_kernel(const float* __restrict__ y0, float* __restrict__ y, T* __restrict__ traj0, int B,
                                   int d, int D) {
+    chain_begin();
     long long nv = (long long)B * (d / V);
     int dv = d / V;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
@@ -230,6 +238,7 @@ __global__ void init_state_kernel(const float* __restrict__ y0, float* __restric
 // ---------------------------------------------------------------- stage input Y_j = Q16(ybar + sum_l (h a_jl) k_l)
 template <typename T, int V>
 __global__ void stage_input_kernel(const T* __restrict__ base, Terms t, T* __restrict__ out, long long nv) {
+    chain_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
         Pack<T, V> b = reinterpret_cast<const Pack<T, V>*>(base)[i];
         float acc[V];
@@ -250,6 +259,7 @@ __global__ void stage_input_kernel(const T* __restrict__ base, Terms t, T* __res
 // the same with rows of `d` in and rows of `ds` out (k too), zero behind d
 template <typename T>
 __global__ void stage_input_rows_kernel(const T* __restrict__ base, Terms t, T* __restrict__ out, int B, int d, int ds) {
+    chain_begin();
     const long long n = (long long)B * ds;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const unsigned row = (unsigned)(i / ds), col = (unsigned)(i - (long long)row * ds);
@@ -266,6 +276,7 @@ __global__ void stage_input_rows_kernel(const T* __restrict__ base, Terms t, T* 
 template <typename T, int V>
 __global__ void final_combine_kernel(float* __restrict__ y, Terms t, T* __restrict__ traj_next, int B, int d, int ds, int D,
                                      int round_increment, float h) {
+    chain_begin();
     int dv = d / V;
     long long nv = (long long)B * dv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
@@ -296,6 +307,7 @@ __global__ void final_combine_kernel(float* __restrict__ y, Terms t, T* __restri
 template <typename T>
 __global__ void column_combine_kernel(float* __restrict__ y, int D, int col, Terms t, int B, int round_increment,
                                       float h) {
+    chain_begin();
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < B; r += (long long)gridDim.x * blockDim.x) {
         float acc = 0.f;
         for (int l = 0; l < t.n; ++l) acc = fmaf(t.c[l], Low<T>::to_f(((const T*)t.p[l])[r]), acc);
@@ -323,6 +335,7 @@ __device__ __forceinline__ void block_amax_commit(float m, bool bad, float* amax
 
 __global__ void copy_amax_kernel(const float* __restrict__ src, float* __restrict__ dst, long long n,
                                  float* __restrict__ amax, unsigned* __restrict__ flag) {
+    chain_begin();
     float m = 0.f;
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -355,6 +368,7 @@ __global__ void copy_amax_kernel(const float* __restrict__ src, float* __restric
 template <typename T, int V>
 __global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ v, T* __restrict__ v_l, int B, int d, int ds,
                             int D, unsigned* __restrict__ flag, T* __restrict__ kap, float bk, const int* __restrict__ e_dev) {
+    chain_begin();
     if (e_dev != nullptr) e = *e_dev;               // the exponent lives on the device (dynamic scaling)
     int dv = d / V;
     long long nv = (long long)B * dv;
@@ -403,6 +417,7 @@ __global__ void seed_kernel(const float* __restrict__ a, int e, T* __restrict__ 
 template <typename T, int V>
 __global__ void kappa_kernel(const T* __restrict__ v, float bj, Terms t, T* __restrict__ out, long long nv,
                              unsigned* __restrict__ flag) {
+    chain_begin();
     bool bad = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
         Pack<T, V> vv = reinterpret_cast<const Pack<T, V>*>(v)[i];
@@ -430,6 +445,7 @@ template <typename T, int V>
 __global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, int B, int d, int ds, int D,
                                 float* __restrict__ amax, const unsigned* __restrict__ skip_if_set, const float* __restrict__ add,
                                 const int* __restrict__ e_dev) {
+    chain_begin();
     if (skip_if_set != nullptr && *skip_if_set != 0u) return;   // a non-finite attempt is not committed (it is repeated)
     if (e_dev != nullptr) coef = ldexpf(coef, -*e_dev);         // h / S with the device's exponent: exact
     int dv = d / V;
@@ -471,6 +487,7 @@ __global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, i
 // Alg. 2 gradient update: g <- g + (h / S) dg
 __global__ void commit_g_kernel(float* __restrict__ g, const float* __restrict__ dg, float coef, long long p,
                                 const unsigned* __restrict__ skip_if_set, const int* __restrict__ e_dev) {
+    chain_begin();
     if (skip_if_set != nullptr && *skip_if_set != 0u) return;
     if (e_dev != nullptr) coef = ldexpf(coef, -*e_dev);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p; i += (long long)gridDim.x * blockDim.x)
@@ -480,6 +497,7 @@ __global__ void commit_g_kernel(float* __restrict__ g, const float* __restrict__
 // Alg. 2 finiteness test for the parameter gradient: is Q16(dg) finite?
 template <typename T>
 __global__ void check_as_low_kernel(const float* __restrict__ x, long long n, unsigned* __restrict__ flag) {
+    chain_begin();
     bool bad = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         bad |= Low<T>::nonfinite(Low<T>::from_f(x[i]));
@@ -491,6 +509,7 @@ __global__ void check_as_low_kernel(const float* __restrict__ x, long long n, un
 // three words in mapped host memory, which the host reads without a copy once it knows the kernel has finished.
 __global__ void scale_init_kernel(unsigned* __restrict__ flag, const float* __restrict__ amax, int pbits, int e_fixed, int from_norm,
                                   int e_min, int e_max, int* __restrict__ state, volatile int* __restrict__ mirror) {
+    chain_begin();
     int e = e_fixed, bad = 0;
     const float m = *amax;
     if (*flag != 0u || !(m <= 3.4028234e38f)) {
@@ -516,6 +535,7 @@ __global__ void scale_init_kernel(unsigned* __restrict__ flag, const float* __re
 __global__ void scale_decide_kernel(const unsigned* __restrict__ flag, const float* __restrict__ amax, int* __restrict__ state,
                                     volatile int* __restrict__ mirror, int step, int k_try, int growth_rule, int pbits, int e_min,
                                     int e_max, int* __restrict__ log_exp, int* __restrict__ log_att, unsigned char* __restrict__ log_dbl) {
+    chain_begin();
     if (state[1] >= 0 || state[2] != 0) return;
     int e = state[0];
     if (*flag != 0u) {
@@ -538,15 +558,18 @@ __global__ void scale_decide_kernel(const unsigned* __restrict__ flag, const flo
 
 template <typename T>
 __global__ void fill_low_kernel(T* __restrict__ x, float v, long long n) {
+    chain_begin();
     const T q = Low<T>::from_f(v);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) x[i] = q;
 }
 
 __global__ void scale_kernel(float* __restrict__ x, float v, long long n) {
+    chain_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) x[i] *= v;
 }
 
 __global__ void fill_kernel(float* __restrict__ x, float v, long long n) {
+    chain_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         x[i] = v;
 }
@@ -561,6 +584,7 @@ template <typename T>
 __global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int ld, int rows_per_block,
                                       float* __restrict__ partial, unsigned* __restrict__ counters, float* __restrict__ dst1,
                                       long long s1, float* __restrict__ dst2, long long s2, float scale2, float beta) {
+    chain_begin();
     __shared__ float sm[kRowLanes][kColsPerBlock];
     __shared__ bool last;
     int lane = threadIdx.x & 31, rl = threadIdx.x >> 5;
@@ -619,6 +643,7 @@ __global__ void colsum_partial_kernel(const T* __restrict__ x, int M, int N, int
 
 __global__ void colsum_final_kernel(const float* __restrict__ partial, int R, int N, float* __restrict__ dst1,
                                     long long s1, float* __restrict__ dst2, long long s2, float scale2, float beta) {
+    chain_begin();
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     float s = 0.f;
@@ -630,6 +655,7 @@ __global__ void colsum_final_kernel(const float* __restrict__ partial, int R, in
 // Column sums of a low-format [M, N] matrix per group of 128 rows: out[g][n] = sum_{r in group g} x[r][n]
 template <typename T>
 __global__ void colsum_groups_kernel(const T* __restrict__ x, int M, int N, float* __restrict__ out) {
+    chain_begin();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     int g = blockIdx.y;
     if (n >= N) return;
@@ -644,6 +670,7 @@ __global__ void colsum_groups_kernel(const T* __restrict__ x, int M, int N, floa
 // lanes split the (stage, row block) terms and are combined by a fixed shuffle tree).
 constexpr int kFinishBiasBlocks = 16;
 __global__ void grad_finish_kernel(GradFinishArgs a) {
+    chain_begin();
     const GradFinishLayer& L = a.layer[blockIdx.y];
     const int wblocks = (int)gridDim.x - kFinishBiasBlocks;
     if ((int)blockIdx.x < wblocks) {
@@ -704,6 +731,7 @@ __device__ __forceinline__ float plane_sum(float v, float (*sm)[kNormCh], int pl
 // Z = Q16((S - mean) * rstd), rstd = 1 / sqrt(var + eps) per (image, channel), biased variance; rstd is kept for the backward pass
 template <typename T>
 __global__ void instnorm_fwd_kernel(const T* __restrict__ S, T* __restrict__ Z, float* __restrict__ rstd, int HW, int C, float eps) {
+    chain_begin();
     __shared__ float sm[kNormLanes][kNormCh];
     const int c = threadIdx.x % kNormCh, pl = threadIdx.x / kNormCh;
     const int ch = blockIdx.x * kNormCh + c, img = blockIdx.y;
@@ -724,6 +752,7 @@ __global__ void instnorm_fwd_kernel(const T* __restrict__ S, T* __restrict__ Z, 
 template <typename T>
 __global__ void instnorm_bwd_kernel(const T* __restrict__ dZ, const T* __restrict__ Z, const T* __restrict__ S, const float* __restrict__ rstd,
                                     T* __restrict__ dU, int HW, int C, int act, int norm, unsigned* __restrict__ flag) {
+    chain_begin();
     __shared__ float sm[kNormLanes][kNormCh];
     const int c = threadIdx.x % kNormCh, pl = threadIdx.x / kNormCh;
     const int ch = blockIdx.x * kNormCh + c, img = blockIdx.y;
@@ -773,6 +802,7 @@ __device__ __forceinline__ void plane_sum8(float (&v)[8], float (*sm)[64 + 1], i
 template <typename T>
 __global__ void __launch_bounds__(kNorm8Threads) instnorm_fwd8_kernel(const T* __restrict__ S, T* __restrict__ Z, float* __restrict__ rstd,
                                                                         int HW, int C, float eps) {
+    chain_begin();
     __shared__ float sm[kNorm8Lanes][64 + 1];
     const int cg = threadIdx.x & 7, pl = threadIdx.x >> 3;
     const int ch0 = blockIdx.x * 64 + cg * 8, img = blockIdx.y;
@@ -818,6 +848,7 @@ template <typename T>
 __global__ void __launch_bounds__(kNorm8Threads) instnorm_bwd8_kernel(const T* __restrict__ dZ, const T* __restrict__ Z, const T* __restrict__ S,
                                                                         const float* __restrict__ rstd, T* __restrict__ dU, int HW, int C, int act,
                                                                         int norm, unsigned* __restrict__ flag) {
+    chain_begin();
     __shared__ float sm[kNorm8Lanes][64 + 1];
     const int cg = threadIdx.x & 7, pl = threadIdx.x >> 3;
     const int ch0 = blockIdx.x * 64 + cg * 8, img = blockIdx.y;
@@ -879,6 +910,7 @@ __device__ __forceinline__ float block_sum_fixed(float v, float* sm) {
 
 template <typename T>
 __global__ void dot_partial_kernel(DotPairs pr, int B, int d, float* __restrict__ part) {
+    chain_begin();
     __shared__ float sm[kThreads / 32];
     const int rows_per = (B + (int)gridDim.x - 1) / (int)gridDim.x;
     const int r0 = blockIdx.x * rows_per, r1 = min(B, r0 + rows_per);
@@ -902,6 +934,7 @@ __global__ void dot_partial_kernel(DotPairs pr, int B, int d, float* __restrict_
 
 template <typename T>
 __global__ void stage_time_cot_kernel(StageTimeArgs a) {
+    chain_begin();
     __shared__ float sm[kThreads / 32];
     const T* wt = (const T*)a.wt;
     for (int j = 0; j < a.terms; ++j) {
@@ -920,6 +953,7 @@ __global__ void stage_time_cot_kernel(StageTimeArgs a) {
 template <typename T>
 __global__ void tgrad_reduce_kernel(const float* __restrict__ part_phi, const float* __restrict__ part_dh, const float* __restrict__ dtau,
                                     const float* __restrict__ c, int stages, float* __restrict__ out, unsigned* __restrict__ flag) {
+    chain_begin();
     __shared__ float sm[kThreads / 32];
     float p1 = 0.f, p2 = 0.f;
     for (int i = threadIdx.x; i < kDotBlocks; i += blockDim.x) { p1 += part_phi[i]; p2 += part_dh[i]; }
@@ -935,6 +969,7 @@ __global__ void tgrad_reduce_kernel(const float* __restrict__ part_phi, const fl
 
 __global__ void tgrad_update_kernel(float* __restrict__ tprime, int i, const float* __restrict__ vals, float coef,
                                     const unsigned* __restrict__ skip_if_set, const int* __restrict__ e_dev) {
+    chain_begin();
     if (threadIdx.x != 0 || (skip_if_set != nullptr && *skip_if_set != 0u)) return;
     if (e_dev != nullptr) coef = ldexpf(coef, -*e_dev);
     const float phi = vals[0], dt = vals[1], dh = vals[2];
@@ -947,6 +982,7 @@ __global__ void tgrad_update_kernel(float* __restrict__ tprime, int i, const flo
 template <typename T>
 __global__ void cnf_tangent_act_kernel(int act, const T* __restrict__ H, const T* __restrict__ U, T* __restrict__ G,
                                        long long n) {
+    chain_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         G[i] = Low<T>::from_f(act_deriv_from_output(act, Low<T>::to_f(H[i])) * Low<T>::to_f(U[i]));
 }
@@ -955,6 +991,7 @@ __global__ void cnf_tangent_act_kernel(int act, const T* __restrict__ H, const T
 template <typename T>
 __global__ void cnf_trace_kernel(const signed char* __restrict__ eps, const T* __restrict__ U, T* __restrict__ k_l,
                                  int B, int d, int ds) {
+    chain_begin();
     int warps_per_block = blockDim.x >> 5;
     int lane = threadIdx.x & 31;
     for (long long b = blockIdx.x * (long long)warps_per_block + (threadIdx.x >> 5); b < B;
@@ -969,6 +1006,7 @@ __global__ void cnf_trace_kernel(const signed char* __restrict__ eps, const T* _
 
 template <typename T>
 __global__ void cnf_probe_to_low_kernel(const signed char* __restrict__ eps, T* __restrict__ out, int B, int d, int ds) {
+    chain_begin();
     const long long n = (long long)B * ds;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const long long row = i / ds, col = i - row * ds;
@@ -980,6 +1018,7 @@ __global__ void cnf_probe_to_low_kernel(const signed char* __restrict__ eps, T* 
 template <typename T>
 __global__ void cnf_ubar_last_kernel(const T* __restrict__ kappa_l, const signed char* __restrict__ eps,
                                      T* __restrict__ ubar, int B, int d, int ds, unsigned* __restrict__ flag) {
+    chain_begin();
     bool bad = false;
     for (int row = blockIdx.x; row < B; row += gridDim.x) {
         const float k = Low<T>::to_f(kappa_l[row]);
@@ -1000,6 +1039,7 @@ __global__ void cnf_backprop_act_kernel(int act, const T* __restrict__ H, const 
                                         const float* __restrict__ hbar, const float* __restrict__ gbar,
                                         T* __restrict__ zeta, T* __restrict__ ubar, long long n,
                                         unsigned* __restrict__ flag) {
+    chain_begin();
     bool bad = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         float s = act_deriv_from_output(act, Low<T>::to_f(H[i]));
@@ -1023,15 +1063,14 @@ void launch_quantize_matrix(mpode_dtype dt, const float* src, long long src_ld, 
                             void* dst_t, cudaStream_t st, long long* launches, int rows_p, int cols_p) {
     const int rp = rows_p > rows ? rows_p : rows, cp = cols_p > cols ? cols_p : cols;
     dim3 grid((cp + 31) / 32, (rp + 31) / 32), block(32, 8);
-    MPODE_DISPATCH_T(dt, T, (quantize_matrix_kernel<T><<<grid, block, 0, st>>>(src, src_ld, rows, cols, rp, cp, (T*)dst, (T*)dst_t)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(quantize_matrix_kernel<T>, dim3(grid), dim3(block), 0, st, src, src_ld, rows, cols, rp, cp, (T*)dst, (T*)dst_t)));
     COUNT(launches);
 }
 
 void launch_quantize_conv_weights(mpode_dtype dt, const float* src, int cout, int cin_total, int cin_keep, void* dst,
                                   void* dst_flip_t, cudaStream_t st, long long* launches, float sign) {
     long long n = (long long)cout * 9 * cin_keep;
-    MPODE_DISPATCH_T(dt, T, (quantize_conv_weights_kernel<T><<<grid_for(n), kThreads, 0, st>>>(
-                                src, cout, cin_total, cin_keep, (T*)dst, (T*)dst_flip_t, sign)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(quantize_conv_weights_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, src, cout, cin_total, cin_keep, (T*)dst, (T*)dst_flip_t, sign)));
     COUNT(launches);
 }
 
@@ -1044,7 +1083,7 @@ static inline bool vec8_ok(int d, int D, std::initializer_list<const void*> ptrs
 
 void launch_conv_wgrad_reduce(const float* partial, int S, int C, int ct, float* out, float beta, cudaStream_t st, long long* launches,
                               float sign) {
-    conv_wgrad_reduce_kernel<<<dim3(C / 32, C / 32, 9), 256, 0, st>>>(partial, S, C, ct, out, beta, sign);
+    launch_chain(conv_wgrad_reduce_kernel, dim3(dim3(C / 32, C / 32, 9)), dim3(256), 0, st, partial, S, C, ct, out, beta, sign);
     COUNT(launches);
 }
 
@@ -1054,13 +1093,12 @@ void launch_conv_class_grads(mpode_dtype dt, const void* dz, int B, int H, int W
     int blocks = (int)((pixels + 255) / 256);        // 128-thread blocks of about 128 registers a thread: four per SM, one wave
     if (blocks > 4 * kSMs) blocks = 4 * kSMs;
     const long long per_block = (pixels + blocks - 1) / blocks;
-    MPODE_DISPATCH_T(dt, T, (conv_class_sums_kernel<T><<<blocks, 128, (size_t)72 * 128 * sizeof(float), st>>>(
-                                (const T*)dz, pixels, H, W, C, per_block, scratch)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(conv_class_sums_kernel<T>, dim3(blocks), dim3(128), (size_t)72 * 128 * sizeof(float), st, (const T*)dz, pixels, H, W, C, per_block, scratch)));
     COUNT(launches);
     float* cs = scratch + (size_t)8 * kSMs * 9 * C;   // reduced class sums behind the per-block ones
-    conv_class_reduce_kernel<<<(9 * C + 7) / 8, 256, 0, st>>>(scratch, blocks, 9 * C, cs);
+    launch_chain(conv_class_reduce_kernel, dim3((9 * C + 7) / 8), dim3(256), 0, st, scratch, blocks, 9 * C, cs);
     COUNT(launches);
-    conv_class_final_kernel<<<1, 576, (size_t)9 * C * sizeof(float), st>>>(cs, C, ct, tau, wt_out, bias_out, beta);
+    launch_chain(conv_class_final_kernel, dim3(1), dim3(576), (size_t)9 * C * sizeof(float), st, cs, C, ct, tau, wt_out, bias_out, beta);
     COUNT(launches);
 }
 
@@ -1068,6 +1106,7 @@ void launch_conv_class_grads(mpode_dtype dt, const void* dz, int B, int H, int W
 // is c, everything else 0.  As a 64-channel operand block beside the image it turns the class sums into rows of a contraction.
 template <typename T>
 __global__ void conv_class_indicator_kernel(int H, int W, T* __restrict__ out) {
+    chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= H * W * 64) return;
     const int c = i & 63, pix = i >> 6, y = pix / W, x = pix - y * W;
@@ -1076,13 +1115,13 @@ __global__ void conv_class_indicator_kernel(int H, int W, T* __restrict__ out) {
 }
 
 void launch_conv_class_indicator(mpode_dtype dt, int H, int W, void* out, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (conv_class_indicator_kernel<T><<<(H * W * 64 + 255) / 256, 256, 0, st>>>(H, W, (T*)out)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(conv_class_indicator_kernel<T>, dim3((H * W * 64 + 255) / 256), dim3(256), 0, st, H, W, (T*)out)));
     COUNT(launches);
 }
 
 void launch_conv_class_bias(mpode_dtype dt, const void* b, const void* w, int cin_total, float tau, int C, float* out,
                             cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (conv_class_bias_kernel<T><<<(9 * C + 127) / 128, 128, 0, st>>>((const T*)b, (const T*)w, cin_total, tau, C, out)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(conv_class_bias_kernel<T>, dim3((9 * C + 127) / 128), dim3(128), 0, st, (const T*)b, (const T*)w, cin_total, tau, C, out)));
     COUNT(launches);
 }
 
@@ -1098,9 +1137,9 @@ static inline bool vec16_ok(mpode_dtype dt, int d, int D, std::initializer_list<
 void launch_init_state(mpode_dtype dt, const float* y0, float* y, void* traj0, int B, int d, int D, cudaStream_t st,
                        long long* launches) {
     if (vec8_ok(d, D, {y0, y, traj0})) {
-        MPODE_DISPATCH_T(dt, T, (init_state_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(y0, y, (T*)traj0, B, d, D)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(init_state_kernel<T, 8>, dim3(grid_for((long long)B * d / 8)), dim3(kThreads), 0, st, y0, y, (T*)traj0, B, d, D)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (init_state_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(y0, y, (T*)traj0, B, d, D)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(init_state_kernel<T, 1>, dim3(grid_for((long long)B * d)), dim3(kThreads), 0, st, y0, y, (T*)traj0, B, d, D)));
     }
     COUNT(launches);
 }
@@ -1109,18 +1148,18 @@ void launch_stage_input(mpode_dtype dt, const void* base, const Terms& t, void* 
                         long long* launches) {
     const long long n = (long long)B * ds;
     if (ds != d) {
-        MPODE_DISPATCH_T(dt, T, (stage_input_rows_kernel<T><<<grid_for(n), kThreads, 0, st>>>((const T*)base, t, (T*)out, B, d, ds)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(stage_input_rows_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, (const T*)base, t, (T*)out, B, d, ds)));
         COUNT(launches);
         return;
     }
     bool v8 = (n % 8 == 0) && aligned_to(base, 32) && aligned_to(out, 32);
     for (int l = 0; l < t.n; ++l) v8 = v8 && aligned_to(t.p[l], 32);
     if (v8 && n % 16 == 0 && dt != MPODE_F32) {   // 32 bytes per operand and thread in flight: needed to fill the memory pipe
-        MPODE_DISPATCH_T(dt, T, (stage_input_kernel<T, 16><<<grid_for(n / 16), kThreads, 0, st>>>((const T*)base, t, (T*)out, n / 16)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(stage_input_kernel<T, 16>, dim3(grid_for(n / 16)), dim3(kThreads), 0, st, (const T*)base, t, (T*)out, n / 16)));
     } else if (v8) {
-        MPODE_DISPATCH_T(dt, T, (stage_input_kernel<T, 8><<<grid_for(n / 8), kThreads, 0, st>>>((const T*)base, t, (T*)out, n / 8)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(stage_input_kernel<T, 8>, dim3(grid_for(n / 8)), dim3(kThreads), 0, st, (const T*)base, t, (T*)out, n / 8)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (stage_input_kernel<T, 1><<<grid_for(n), kThreads, 0, st>>>((const T*)base, t, (T*)out, n)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(stage_input_kernel<T, 1>, dim3(grid_for(n)), dim3(kThreads), 0, st, (const T*)base, t, (T*)out, n)));
     }
     COUNT(launches);
 }
@@ -1132,40 +1171,37 @@ void launch_final_combine(mpode_dtype dt, float* y, const Terms& t, void* traj_n
     bool v16 = v8 && vec16_ok(dt, d, D, {y, traj_next});
     for (int l = 0; l < t.n; ++l) v16 = v16 && aligned_to(t.p[l], 64);
     if (v16) {
-        MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(final_combine_kernel<T, 16>, dim3(grid_for((long long)B * d / 16)), dim3(kThreads), 0, st, y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     } else if (v8) {
-        MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(final_combine_kernel<T, 8>, dim3(grid_for((long long)B * d / 8)), dim3(kThreads), 0, st, y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (final_combine_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(
-                                    y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(final_combine_kernel<T, 1>, dim3(grid_for((long long)B * d)), dim3(kThreads), 0, st, y, t, (T*)traj_next, B, d, ds, D, round_increment, h)));
     }
     COUNT(launches);
 }
 
 void launch_column_combine(mpode_dtype dt, float* y, int D, int col, const Terms& t, int B, int round_increment,
                            float h, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (column_combine_kernel<T><<<grid_for(B), kThreads, 0, st>>>(y, D, col, t, B, round_increment, h)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(column_combine_kernel<T>, dim3(grid_for(B)), dim3(kThreads), 0, st, y, D, col, t, B, round_increment, h)));
     COUNT(launches);
 }
 
 void launch_copy_amax(const float* src, float* dst, long long n, float* amax, unsigned* flag, cudaStream_t st,
                       long long* launches) {
-    copy_amax_kernel<<<grid_for(n), kThreads, 0, st>>>(src, dst, n, amax, flag);
+    launch_chain(copy_amax_kernel, dim3(grid_for(n)), dim3(kThreads), 0, st, src, dst, n, amax, flag);
     COUNT(launches);
 }
 
 void launch_seed(mpode_dtype dt, const float* a, int e, void* v, void* v_l, int B, int d, int ds, int D, unsigned* flag,
                  cudaStream_t st, long long* launches, void* kappa_last, float b_last, const int* e_dev) {
     if (vec16_ok(dt, d, D, {a, v, kappa_last})) {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(seed_kernel<T, 16>, dim3(grid_for((long long)B * d / 16)), dim3(kThreads), 0, st, a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                         (T*)kappa_last, b_last, e_dev)));
     } else if (vec8_ok(d, D, {a, v, kappa_last})) {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(seed_kernel<T, 8>, dim3(grid_for((long long)B * d / 8)), dim3(kThreads), 0, st, a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                       (T*)kappa_last, b_last, e_dev)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (seed_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(seed_kernel<T, 1>, dim3(grid_for((long long)B * d)), dim3(kThreads), 0, st, a, e, (T*)v, (T*)v_l, B, d, ds, D, flag,
                                                                                                   (T*)kappa_last, b_last, e_dev)));
     }
     COUNT(launches);
@@ -1176,11 +1212,11 @@ void launch_kappa(mpode_dtype dt, const void* v, float bj, const Terms& t, void*
     bool v8 = (n % 8 == 0) && aligned_to(v, 32) && aligned_to(out, 32);
     for (int l = 0; l < t.n; ++l) v8 = v8 && aligned_to(t.p[l], 32);
     if (v8 && n % 16 == 0 && dt != MPODE_F32) {
-        MPODE_DISPATCH_T(dt, T, (kappa_kernel<T, 16><<<grid_for(n / 16), kThreads, 0, st>>>((const T*)v, bj, t, (T*)out, n / 16, flag)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(kappa_kernel<T, 16>, dim3(grid_for(n / 16)), dim3(kThreads), 0, st, (const T*)v, bj, t, (T*)out, n / 16, flag)));
     } else if (v8) {
-        MPODE_DISPATCH_T(dt, T, (kappa_kernel<T, 8><<<grid_for(n / 8), kThreads, 0, st>>>((const T*)v, bj, t, (T*)out, n / 8, flag)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(kappa_kernel<T, 8>, dim3(grid_for(n / 8)), dim3(kThreads), 0, st, (const T*)v, bj, t, (T*)out, n / 8, flag)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (kappa_kernel<T, 1><<<grid_for(n), kThreads, 0, st>>>((const T*)v, bj, t, (T*)out, n, flag)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(kappa_kernel<T, 1>, dim3(grid_for(n)), dim3(kThreads), 0, st, (const T*)v, bj, t, (T*)out, n, flag)));
     }
     COUNT(launches);
 }
@@ -1192,53 +1228,53 @@ void launch_commit_a(mpode_dtype dt, float* a, const Terms& psis, float coef, in
     bool v16 = v8 && vec16_ok(dt, d, D, {a, add});
     for (int l = 0; l < psis.n; ++l) v16 = v16 && aligned_to(psis.p[l], 64);
     if (v16) {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 16><<<grid_for((long long)B * d / 16), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(commit_a_kernel<T, 16>, dim3(grid_for((long long)B * d / 16)), dim3(kThreads), 0, st, a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     } else if (v8) {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 8><<<grid_for((long long)B * d / 8), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(commit_a_kernel<T, 8>, dim3(grid_for((long long)B * d / 8)), dim3(kThreads), 0, st, a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (commit_a_kernel<T, 1><<<grid_for((long long)B * d), kThreads, 0, st>>>(a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(commit_a_kernel<T, 1>, dim3(grid_for((long long)B * d)), dim3(kThreads), 0, st, a, psis, coef, B, d, ds, D, amax, skip_if_set, add, e_dev)));
     }
     COUNT(launches);
 }
 
 void launch_commit_g(float* g, const float* dg, float coef, long long p, cudaStream_t st, long long* launches,
                      const unsigned* skip_if_set, const int* e_dev) {
-    commit_g_kernel<<<grid_for(p), kThreads, 0, st>>>(g, dg, coef, p, skip_if_set, e_dev);
+    launch_chain(commit_g_kernel, dim3(grid_for(p)), dim3(kThreads), 0, st, g, dg, coef, p, skip_if_set, e_dev);
     COUNT(launches);
 }
 
 void launch_scale_init(unsigned* flag, const float* amax, int pbits, int e_fixed, int from_norm, int e_min, int e_max, int* state,
                        int* mirror, cudaStream_t st, long long* launches) {
-    scale_init_kernel<<<1, 1, 0, st>>>(flag, amax, pbits, e_fixed, from_norm, e_min, e_max, state, mirror);
+    launch_chain(scale_init_kernel, dim3(1), dim3(1), 0, st, flag, amax, pbits, e_fixed, from_norm, e_min, e_max, state, mirror);
     COUNT(launches);
 }
 
 void launch_scale_decide(const unsigned* flag, const float* amax, int* state, int* mirror, int step, int k_try, int growth_rule,
                          int pbits, int e_min, int e_max, int* log_exp, int* log_att, unsigned char* log_dbl, cudaStream_t st,
                          long long* launches) {
-    scale_decide_kernel<<<1, 1, 0, st>>>(flag, amax, state, mirror, step, k_try, growth_rule, pbits, e_min, e_max, log_exp, log_att,
+    launch_chain(scale_decide_kernel, dim3(1), dim3(1), 0, st, flag, amax, state, mirror, step, k_try, growth_rule, pbits, e_min, e_max, log_exp, log_att,
                                           log_dbl);
     COUNT(launches);
 }
 
 void launch_check_as_low(mpode_dtype dt, const float* x, long long n, unsigned* flag, cudaStream_t st,
                          long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (check_as_low_kernel<T><<<grid_for(n), kThreads, 0, st>>>(x, n, flag)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(check_as_low_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, x, n, flag)));
     COUNT(launches);
 }
 
 void launch_fill_low(mpode_dtype dt, void* x, float v, long long n, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (fill_low_kernel<T><<<grid_for(n), kThreads, 0, st>>>((T*)x, v, n)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(fill_low_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, (T*)x, v, n)));
     COUNT(launches);
 }
 
 void launch_scale(float* x, float v, long long n, cudaStream_t st, long long* launches) {
-    scale_kernel<<<grid_for(n), kThreads, 0, st>>>(x, v, n);
+    launch_chain(scale_kernel, dim3(grid_for(n)), dim3(kThreads), 0, st, x, v, n);
     COUNT(launches);
 }
 
 void launch_fill(float* x, float v, long long n, cudaStream_t st, long long* launches) {
-    fill_kernel<<<grid_for(n), kThreads, 0, st>>>(x, v, n);
+    launch_chain(fill_kernel, dim3(grid_for(n)), dim3(kThreads), 0, st, x, v, n);
     COUNT(launches);
 }
 
@@ -1246,12 +1282,12 @@ void launch_instnorm_fwd(mpode_dtype dt, const void* S, void* Z, float* rstd, in
                          long long* launches) {
     if (dt != MPODE_F32 && C % 64 == 0 && aligned_to(S, 16) && aligned_to(Z, 16)) {
         dim3 grid8(C / 64, B);
-        MPODE_DISPATCH_T(dt, T, (instnorm_fwd8_kernel<T><<<grid8, kNorm8Threads, 0, st>>>((const T*)S, (T*)Z, rstd, HW, C, eps)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_fwd8_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
         COUNT(launches);
         return;
     }
     dim3 grid((C + kNormCh - 1) / kNormCh, B);
-    MPODE_DISPATCH_T(dt, T, (instnorm_fwd_kernel<T><<<grid, kThreads, 0, st>>>((const T*)S, (T*)Z, rstd, HW, C, eps)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_fwd_kernel<T>, dim3(grid), dim3(kThreads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
     COUNT(launches);
 }
 
@@ -1259,36 +1295,36 @@ void launch_instnorm_bwd(mpode_dtype dt, const void* dZ, const void* Z, const vo
                          int act, int norm, unsigned* flag, cudaStream_t st, long long* launches) {
     if (dt != MPODE_F32 && C % 64 == 0 && aligned_to(dZ, 16) && aligned_to(Z, 16) && aligned_to(S, 16) && aligned_to(dU, 16)) {
         dim3 grid8(C / 64, B);
-        MPODE_DISPATCH_T(dt, T, (instnorm_bwd8_kernel<T><<<grid8, kNorm8Threads, 0, st>>>((const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_bwd8_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU,
                                                                                             HW, C, act, norm, flag)));
         COUNT(launches);
         return;
     }
     dim3 grid((C + kNormCh - 1) / kNormCh, B);
-    MPODE_DISPATCH_T(dt, T, (instnorm_bwd_kernel<T><<<grid, kThreads, 0, st>>>((const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU, HW, C, act,
+    MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_bwd_kernel<T>, dim3(grid), dim3(kThreads), 0, st, (const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU, HW, C, act,
                                                                             norm, flag)));
     COUNT(launches);
 }
 
 void launch_dot_partial(mpode_dtype dt, const DotPairs& pr, int B, int d, float* part, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (dot_partial_kernel<T><<<kDotBlocks, kThreads, 0, st>>>(pr, B, d, part)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(dot_partial_kernel<T>, dim3(kDotBlocks), dim3(kThreads), 0, st, pr, B, d, part)));
     COUNT(launches);
 }
 
 void launch_stage_time_cot(mpode_dtype dt, const StageTimeArgs& a, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (stage_time_cot_kernel<T><<<1, kThreads, 0, st>>>(a)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(stage_time_cot_kernel<T>, dim3(1), dim3(kThreads), 0, st, a)));
     COUNT(launches);
 }
 
 void launch_tgrad_reduce(mpode_dtype dt, const float* part_phi, const float* part_dh, const float* dtau, const float* c, int stages,
                          float* out, unsigned* flag, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (tgrad_reduce_kernel<T><<<1, kThreads, 0, st>>>(part_phi, part_dh, dtau, c, stages, out, flag)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(tgrad_reduce_kernel<T>, dim3(1), dim3(kThreads), 0, st, part_phi, part_dh, dtau, c, stages, out, flag)));
     COUNT(launches);
 }
 
 void launch_tgrad_update(float* tprime, int i, const float* vals, float coef, const unsigned* skip_if_set, cudaStream_t st,
                          long long* launches, const int* e_dev) {
-    tgrad_update_kernel<<<1, 32, 0, st>>>(tprime, i, vals, coef, skip_if_set, e_dev);
+    launch_chain(tgrad_update_kernel, dim3(1), dim3(32), 0, st, tprime, i, vals, coef, skip_if_set, e_dev);
     COUNT(launches);
 }
 
@@ -1305,11 +1341,11 @@ int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* pa
     R = (M + rows_per_block - 1) / rows_per_block;
     dim3 grid(col_blocks, R);
     if (counters != nullptr && col_blocks > kColsumCounters) counters = nullptr;
-    MPODE_DISPATCH_T(dt, T, (colsum_partial_kernel<T><<<grid, kThreads, 0, st>>>((const T*)x, M, N, ld, rows_per_block, partial, counters, dst1, s1, dst2,
+    MPODE_DISPATCH_T(dt, T, (launch_chain(colsum_partial_kernel<T>, dim3(grid), dim3(kThreads), 0, st, (const T*)x, M, N, ld, rows_per_block, partial, counters, dst1, s1, dst2,
                                                                                    s2, scale2, beta)));
     COUNT(launches);
     if (counters == nullptr) {
-        colsum_final_kernel<<<(N + 127) / 128, 128, 0, st>>>(partial, R, N, dst1, s1, dst2, s2, scale2, beta);
+        launch_chain(colsum_final_kernel, dim3((N + 127) / 128), dim3(128), 0, st, partial, R, N, dst1, s1, dst2, s2, scale2, beta);
         COUNT(launches);
     }
     return R;
@@ -1317,19 +1353,19 @@ int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* pa
 
 void launch_colsum_groups(mpode_dtype dt, const void* x, int M, int N, float* out, cudaStream_t st, long long* launches) {
     dim3 grid((N + 127) / 128, (M + 127) / 128);
-    MPODE_DISPATCH_T(dt, T, (colsum_groups_kernel<T><<<grid, 128, 0, st>>>((const T*)x, M, N, out)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(colsum_groups_kernel<T>, dim3(grid), dim3(128), 0, st, (const T*)x, M, N, out)));
     COUNT(launches);
 }
 
 void launch_grad_finish(const GradFinishArgs& a, cudaStream_t st, long long* launches) {
     dim3 grid(kSMs * 2 + kFinishBiasBlocks, a.n_layers);
-    grad_finish_kernel<<<grid, kThreads, 0, st>>>(a);
+    launch_chain(grad_finish_kernel, dim3(grid), dim3(kThreads), 0, st, a);
     COUNT(launches);
 }
 
 void launch_cnf_tangent_act(mpode_dtype dt, int act, const void* H, const void* U, void* G, long long n,
                             cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_tangent_act_kernel<T><<<grid_for(n), kThreads, 0, st>>>(act, (const T*)H, (const T*)U, (T*)G, n)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(cnf_tangent_act_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, act, (const T*)H, (const T*)U, (T*)G, n)));
     COUNT(launches);
 }
 
@@ -1337,28 +1373,26 @@ void launch_cnf_trace(mpode_dtype dt, const signed char* eps, const void* U, voi
                       long long* launches) {
     int blocks = (B + 7) / 8;
     if (blocks > kSMs * 8) blocks = kSMs * 8;
-    MPODE_DISPATCH_T(dt, T, (cnf_trace_kernel<T><<<blocks, kThreads, 0, st>>>(eps, (const T*)U, (T*)k_l, B, d, ds)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(cnf_trace_kernel<T>, dim3(blocks), dim3(kThreads), 0, st, eps, (const T*)U, (T*)k_l, B, d, ds)));
     COUNT(launches);
 }
 
 void launch_cnf_probe_to_low(mpode_dtype dt, const signed char* eps, void* out, int B, int d, int ds, cudaStream_t st,
                              long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_probe_to_low_kernel<T><<<grid_for((long long)B * ds), kThreads, 0, st>>>(eps, (T*)out, B, d, ds)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(cnf_probe_to_low_kernel<T>, dim3(grid_for((long long)B * ds)), dim3(kThreads), 0, st, eps, (T*)out, B, d, ds)));
     COUNT(launches);
 }
 
 void launch_cnf_ubar_last(mpode_dtype dt, const void* kappa_l, const signed char* eps, void* ubar, int B, int d, int ds,
                           unsigned* flag, cudaStream_t st, long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_ubar_last_kernel<T><<<B < kSMs * 8 ? B : kSMs * 8, kThreads, 0, st>>>(
-                                (const T*)kappa_l, eps, (T*)ubar, B, d, ds, flag)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(cnf_ubar_last_kernel<T>, dim3(B < kSMs * 8 ? B : kSMs * 8), dim3(kThreads), 0, st, (const T*)kappa_l, eps, (T*)ubar, B, d, ds, flag)));
     COUNT(launches);
 }
 
 void launch_cnf_backprop_act(mpode_dtype dt, int act, const void* H, const void* U, const float* hbar,
                              const float* gbar, void* zeta, void* ubar, long long n, unsigned* flag, cudaStream_t st,
                              long long* launches) {
-    MPODE_DISPATCH_T(dt, T, (cnf_backprop_act_kernel<T><<<grid_for(n), kThreads, 0, st>>>(
-                                act, (const T*)H, (const T*)U, hbar, gbar, (T*)zeta, (T*)ubar, n, flag)));
+    MPODE_DISPATCH_T(dt, T, (launch_chain(cnf_backprop_act_kernel<T>, dim3(grid_for(n)), dim3(kThreads), 0, st, act, (const T*)H, (const T*)U, hbar, gbar, (T*)zeta, (T*)ubar, n, flag)));
     COUNT(launches);
 }
 

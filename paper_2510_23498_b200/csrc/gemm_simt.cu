@@ -59,6 +59,7 @@ __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, 
 
 template <typename T>
 __global__ void __launch_bounds__(kGemmThreads) gemm_simt_kernel(GemmArgs g) {
+    chain_begin();
     __shared__ float As[BK][BM + 4];
     __shared__ float Bs[BK][BN + 4];
     const T* A = (const T*)g.A;
@@ -162,6 +163,7 @@ __device__ __forceinline__ float4 load_quad(const T* __restrict__ p, long long l
 
 template <typename T, bool KFAST>
 __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, int per_slice, int vec_a, int vec_b) {
+    chain_begin();
     namespace cg = cooperative_groups;
     __shared__ __align__(16) float As[2][DK][kDenseLd];
     __shared__ __align__(16) float Bs[2][DK][kDenseLd];
@@ -314,17 +316,20 @@ bool launch_dense(const GemmArgs& g, cudaStream_t st) {
     cfg.gridDim = dim3((unsigned)tn, (unsigned)tm, (unsigned)S);
     cfg.blockDim = dim3(kDenseThreads);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = (unsigned)S;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = (unsigned)S;
     cfg.attrs = at;
-    cfg.numAttrs = S > 1 ? 1 : 0;
+    cfg.numAttrs = S > 1 ? 2 : 1;
     if (kfast) return cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, true>, g, per, vec_a, vec_b) == cudaSuccess;
     return cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, false>, g, per, vec_a, vec_b) == cudaSuccess;
 }
 
 __global__ void splitk_reduce_kernel(const float* __restrict__ partial, int S, int M, int N, float* __restrict__ out,
                                      long long ldo, float beta, int keep_m, int keep_n) {
+    chain_begin();
     long long n_el = (long long)M * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_el; i += (long long)gridDim.x * blockDim.x) {
         if (i / N >= keep_m || i % N >= keep_n) continue;
@@ -341,6 +346,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ partial, int S, i
 template <bool VEC>
 __global__ void splitk_reduce4_kernel(const float4* __restrict__ partial, int S, unsigned slice4, unsigned n4, unsigned N4, float* __restrict__ out,
                                       long long ldo, float beta, unsigned keep_n) {
+    chain_begin();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {
         float4 s = partial[i];
         for (int z = 1; z < S; ++z) {
@@ -372,13 +378,13 @@ void reduce_slices(const float* partial, int S, int M, int N, float* out, long l
         int blocks = (int)((n4 + 255) / 256);
         if (blocks > 148 * 8) blocks = 148 * 8;
         const float4* p4 = reinterpret_cast<const float4*>(partial);
-        if (keep_n == N && ldo % 4 == 0 && ((uintptr_t)out & 15) == 0) splitk_reduce4_kernel<true><<<blocks, 256, 0, st>>>(p4, S, slice4, n4, N4, out, ldo, beta, N);
-        else splitk_reduce4_kernel<false><<<blocks, 256, 0, st>>>(p4, S, slice4, n4, N4, out, ldo, beta, keep_n);
+        if (keep_n == N && ldo % 4 == 0 && ((uintptr_t)out & 15) == 0) launch_chain(splitk_reduce4_kernel<true>, dim3(blocks), dim3(256), 0, st, p4, S, slice4, n4, N4, out, ldo, beta, N);
+        else launch_chain(splitk_reduce4_kernel<false>, dim3(blocks), dim3(256), 0, st, p4, S, slice4, n4, N4, out, ldo, beta, keep_n);
         return;
     }
     int blocks = (int)((n_el + 255) / 256);
     if (blocks > 148 * 8) blocks = 148 * 8;
-    splitk_reduce_kernel<<<blocks, 256, 0, st>>>(partial, S, M, N, out, ldo, beta, keep_m, keep_n);
+    launch_chain(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, st, partial, S, M, N, out, ldo, beta, keep_m, keep_n);
 }
 
 }  // namespace
@@ -397,9 +403,9 @@ bool launch_gemm_simt(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long l
         return true;
     }
     dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.split_k > 1 ? g.split_k : 1);
-    if (dt == MPODE_BF16) gemm_simt_kernel<__nv_bfloat16><<<grid, kGemmThreads, 0, st>>>(g);
-    else if (dt == MPODE_F16) gemm_simt_kernel<__half><<<grid, kGemmThreads, 0, st>>>(g);
-    else gemm_simt_kernel<float><<<grid, kGemmThreads, 0, st>>>(g);
+    if (dt == MPODE_BF16) launch_chain(gemm_simt_kernel<__nv_bfloat16>, dim3(grid), dim3(kGemmThreads), 0, st, g);
+    else if (dt == MPODE_F16) launch_chain(gemm_simt_kernel<__half>, dim3(grid), dim3(kGemmThreads), 0, st, g);
+    else launch_chain(gemm_simt_kernel<float>, dim3(grid), dim3(kGemmThreads), 0, st, g);
     if (launches) ++*launches;
     if (g.split_k > 1) {
         reduce_slices(g.partial, g.split_k, g.M, g.N, (float*)g.out, g.ldo, g.beta, st);

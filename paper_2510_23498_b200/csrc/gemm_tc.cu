@@ -104,6 +104,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *(volatile uint32_t*)tmem_holder;
+    chain_begin();                          // everything above overlaps the tail of the kernel before
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -441,7 +442,7 @@ bool launch_tc(const CUtensorMap& ta, const CUtensorMap& tb, TcParams& p, cudaSt
     int work = p.tiles_m * p.tiles_n * p.splits;
     const int max_ctas = sm_count() * Shape<BN>::kCtasPerSm;
     int grid = work < max_ctas ? work : max_ctas;
-    gemm_tc_kernel<T, BN, WG, PAIR><<<grid, Shape<BN>::kThreads, Cfg::kSmemBytes, st>>>(ta, tb, p);
+    launch_chain(gemm_tc_kernel<T, BN, WG, PAIR>, dim3(grid), dim3(Shape<BN>::kThreads), Cfg::kSmemBytes, st, ta, tb, p);
     return true;
 }
 

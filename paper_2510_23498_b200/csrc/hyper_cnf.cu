@@ -80,6 +80,7 @@ template <typename T, int DC>
 __global__ void __launch_bounds__(256) hyper_forward_kernel(const float* __restrict__ theta, float tau16, int h, int w, int d_rt,
                                                              float* __restrict__ hyp, const T* __restrict__ Y, T* __restrict__ A,
                                                              T* __restrict__ k, T* __restrict__ k_l, int B) {
+    chain_begin();
     constexpr int DM = DC > 0 ? DC : HYPER_MAX_D;
     const int d = DC > 0 ? DC : d_rt;
     extern __shared__ float sm[];                     // h1 [h], h2 [h], W [w][d], b [w], U [w][d], c [w]
@@ -120,6 +121,7 @@ template <typename T, int DC>
 __global__ void __launch_bounds__(256) hyper_unit_cot_kernel(const float* __restrict__ hyp, int h, int w, int d_rt, const T* __restrict__ A,
                                                               const T* __restrict__ kappa, const T* __restrict__ kappa_l, T* __restrict__ Sb,
                                                               T* __restrict__ psi, int B, unsigned* __restrict__ flag) {
+    chain_begin();
     constexpr int DM = DC > 0 ? DC : HYPER_MAX_D;
     const int d = DC > 0 ? DC : d_rt;
     extern __shared__ float sm[];                     // W, b, U, c
@@ -292,6 +294,7 @@ __global__ void __launch_bounds__(256) hyper_param_cot_kernel(const float* __res
                                                                const T* __restrict__ Sb, const T* __restrict__ kappa, const T* __restrict__ kappa_l,
                                                                float* __restrict__ sums, float* __restrict__ dg, float beta, int B,
                                                                unsigned* __restrict__ flag, unsigned* __restrict__ counter) {
+    chain_begin();
     extern __shared__ float sm[];
     __shared__ bool last;
     const int j = blockIdx.x, nv = 2 * d + 2;
@@ -325,9 +328,9 @@ void launch_hyper_forward(mpode_dtype dt, const float* theta, float tau16, int h
     const size_t smem = ((size_t)2 * h + (size_t)w * (2 * d + 1) + w) * sizeof(float);
     const int blocks = (B + 255) / 256;
     if (d == 2) {
-        MPODE_DISPATCH_T(dt, T, (hyper_forward_kernel<T, 2><<<blocks, 256, smem, st>>>(theta, tau16, h, w, d, hyp, (const T*)Y, (T*)A, (T*)k, (T*)k_l, B)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(hyper_forward_kernel<T, 2>, dim3(blocks), dim3(256), smem, st, theta, tau16, h, w, d, hyp, (const T*)Y, (T*)A, (T*)k, (T*)k_l, B)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (hyper_forward_kernel<T, 0><<<blocks, 256, smem, st>>>(theta, tau16, h, w, d, hyp, (const T*)Y, (T*)A, (T*)k, (T*)k_l, B)));
+        MPODE_DISPATCH_T(dt, T, (launch_chain(hyper_forward_kernel<T, 0>, dim3(blocks), dim3(256), smem, st, theta, tau16, h, w, d, hyp, (const T*)Y, (T*)A, (T*)k, (T*)k_l, B)));
     }
     if (launches) ++*launches;
 }
@@ -340,14 +343,14 @@ void launch_hyper_vjp(mpode_dtype dt, const float* theta, float tau16, int h, in
     size_t sm_par = ((size_t)m + 2 * h + (h > 256 ? h : 256)) * sizeof(float);
     if (sm_par < (size_t)8 * nv * sizeof(float)) sm_par = (size_t)8 * nv * sizeof(float);
     if (d == 2) {
-        MPODE_DISPATCH_T(dt, T, (hyper_unit_cot_kernel<T, 2><<<blocks, 256, sm_unit, st>>>(hyp, h, w, d, (const T*)A, (const T*)kappa, (const T*)kappa_l,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(hyper_unit_cot_kernel<T, 2>, dim3(blocks), dim3(256), sm_unit, st, hyp, h, w, d, (const T*)A, (const T*)kappa, (const T*)kappa_l,
                                                                                            (T*)Sb, (T*)psi, B, flag)));
     } else {
-        MPODE_DISPATCH_T(dt, T, (hyper_unit_cot_kernel<T, 0><<<blocks, 256, sm_unit, st>>>(hyp, h, w, d, (const T*)A, (const T*)kappa, (const T*)kappa_l,
+        MPODE_DISPATCH_T(dt, T, (launch_chain(hyper_unit_cot_kernel<T, 0>, dim3(blocks), dim3(256), sm_unit, st, hyp, h, w, d, (const T*)A, (const T*)kappa, (const T*)kappa_l,
                                                                                            (T*)Sb, (T*)psi, B, flag)));
     }
     if (launches) ++*launches;
-    MPODE_DISPATCH_T(dt, T, (hyper_param_cot_kernel<T><<<w, 256, sm_par, st>>>(hyp, theta, tau16, h, w, d, (const T*)Y, (const T*)A, (const T*)Sb,
+    MPODE_DISPATCH_T(dt, T, (launch_chain(hyper_param_cot_kernel<T>, dim3(w), dim3(256), sm_par, st, hyp, theta, tau16, h, w, d, (const T*)Y, (const T*)A, (const T*)Sb,
                                                                                (const T*)kappa, (const T*)kappa_l, sums, dg, beta, B, flag, counter)));
     if (launches) ++*launches;
 }

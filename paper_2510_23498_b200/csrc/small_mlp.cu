@@ -8,8 +8,7 @@
 // Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
 // second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
 // Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.9 ms; MLP
-// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.2 ms; float32 MLP 64-256-256-64, 1024 samples, 16 RK4 steps
-// (before: a launch per layer) 10.8 -> 5.8 ms.
+// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.5 ms.
 #include "small_mlp.h"
 
 #include "profiler.h"
@@ -91,6 +90,7 @@ __host__ __device__ inline int k32(int w) { return (w + 31) / 32; }
 struct PackJob { long long first[2 * SMALL_MAX_L + 1]; };      // first 16-byte group of each (layer, direction)
 template <typename T>
 __global__ void __launch_bounds__(256) small_pack_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ PackJob job) {
+    chain_begin();
     const long long n = job.first[2 * p.L];
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         int q = 0;
@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(256) small_pack_kernel(const __grid_constant__
 
 // float32: forward [inputs][outputs], backward [outputs][inputs], zero in the padding
 __global__ void __launch_bounds__(256) small_pack_f32_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ PackJob job) {
+    chain_begin();
     const long long n = job.first[2 * p.L];
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         int q = 0;
@@ -448,6 +449,7 @@ __device__ __forceinline__ void small_stages(const SmallMlp& p, Ring& ring, cons
 
 template <typename T, int MT>
 __global__ void __launch_bounds__(kThreads + 32, 1) small_forward_kernel(const __grid_constant__ SmallMlp p) {
+    chain_begin();
     using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
     const int R = kRows<T, MT>, r0 = blockIdx.x * R;
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) small_forward_kernel(const _
 // Phi = sum_j b_j k_j, dt = sum_j dtau_j and dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>), dtau_j = <dZ_1, w_t>.
 template <typename T, int MT>
 __global__ void __launch_bounds__(kThreads + 32, 1) small_backward_kernel(const __grid_constant__ SmallMlp p) {
+    chain_begin();
     using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
     const int R = kRows<T, MT>, r0 = blockIdx.x * R;
@@ -713,6 +716,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) small_backward_kernel(const 
 // with tprime the two t' updates of Alg. 2 per step.  Q16(dt), Q16(dh) join the finiteness test.
 template <typename T>
 __global__ void __launch_bounds__(96) small_time_kernel(SmallMlp p, int blocks) {
+    chain_begin();
     __shared__ float v[3];
     const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int s = 0; s < p.count; ++s) {
@@ -744,6 +748,7 @@ constexpr int kRing = 8;
 struct WgradItems { int first[SMALL_MAX_L + 1]; };
 template <typename T, int TM, int TN>
 __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ WgradItems items) {
+    chain_begin();
     constexpr int LA = TM + 8, LB = TN + 8;                       // row lengths in shared memory: eight rows hit eight 16-byte slots
     constexpr int kStage = 16 * (LA + LB);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -905,7 +910,7 @@ bool forward_t(const SmallMlp& p, cudaStream_t st) {
     if (q.ring < 2) return false;
     const int rows = kRows<T, MT>, blocks = (p.B + rows - 1) / rows;
     const size_t smem = small_smem<T>(p, rows) + q.ring * (kUnitBytes + 16);
-    small_forward_kernel<T, MT><<<blocks, kThreads + 32, smem, st>>>(q);
+    launch_chain(small_forward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
 template <typename T, int MT>
@@ -917,7 +922,7 @@ bool backward_t(const SmallMlp& p, cudaStream_t st) {
     if (q.ring < 2) return false;
     const int rows = kRows<T, MT>, blocks = (p.B + rows - 1) / rows;
     const size_t smem = small_smem<T>(p, rows) + q.ring * (kUnitBytes + 16);
-    small_backward_kernel<T, MT><<<blocks, kThreads + 32, smem, st>>>(q);
+    launch_chain(small_backward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
 template <typename T, int TM>
@@ -925,7 +930,7 @@ bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st) {
     static bool done[kMaxDevices] = {false};
     if (!allow_smem(small_wgrad_kernel<T, TM, TM>, done)) return false;
     const size_t ring = (size_t)kWarps * kRing * 16 * 2 * (TM + 8) * sizeof(T), red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
-    small_wgrad_kernel<T, TM, TM><<<items.first[p.L], kThreads, ring > red ? ring : red, st>>>(p, items);
+    launch_chain(small_wgrad_kernel<T, TM, TM>, dim3(items.first[p.L]), dim3(kThreads), ring > red ? ring : red, st, p, items);
     return true;
 }
 WgradItems wgrad_items(const SmallMlp& p, int tm) {
@@ -969,9 +974,9 @@ void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long 
     }
     long long blocks = (job.first[2 * p.L] + 255) / 256;
     if (blocks > 148 * 4) blocks = 148 * 4;
-    if (dt == MPODE_BF16) small_pack_kernel<__nv_bfloat16><<<(int)blocks, 256, 0, st>>>(p, job);
-    else if (dt == MPODE_F16) small_pack_kernel<__half><<<(int)blocks, 256, 0, st>>>(p, job);
-    else small_pack_f32_kernel<<<(int)blocks, 256, 0, st>>>(p, job);
+    if (dt == MPODE_BF16) launch_chain(small_pack_kernel<__nv_bfloat16>, dim3((int)blocks), dim3(256), 0, st, p, job);
+    else if (dt == MPODE_F16) launch_chain(small_pack_kernel<__half>, dim3((int)blocks), dim3(256), 0, st, p, job);
+    else launch_chain(small_pack_f32_kernel, dim3((int)blocks), dim3(256), 0, st, p, job);
     if (launches) ++*launches;
 }
 
@@ -997,9 +1002,9 @@ bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, l
 
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
     const int blocks = small_blocks(dt, p.B);
-    if (dt == MPODE_BF16) small_time_kernel<__nv_bfloat16><<<1, 96, 0, st>>>(p, blocks);
-    else if (dt == MPODE_F16) small_time_kernel<__half><<<1, 96, 0, st>>>(p, blocks);
-    else small_time_kernel<float><<<1, 96, 0, st>>>(p, blocks);
+    if (dt == MPODE_BF16) launch_chain(small_time_kernel<__nv_bfloat16>, dim3(1), dim3(96), 0, st, p, blocks);
+    else if (dt == MPODE_F16) launch_chain(small_time_kernel<__half>, dim3(1), dim3(96), 0, st, p, blocks);
+    else launch_chain(small_time_kernel<float>, dim3(1), dim3(96), 0, st, p, blocks);
     if (launches) ++*launches;
 }
 
