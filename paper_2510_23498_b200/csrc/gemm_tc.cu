@@ -481,12 +481,13 @@ bool tc_eligible(mpode_dtype dt, const GemmArgs& g) {
 
 bool launch_gemm_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* launches) {
     int bn = 256;
-    // narrow outputs: smaller tiles keep more SMs busy
+    // narrow outputs: smaller tiles keep more SMs busy, paired (value, tangent) tiles too.  A tile's time hardly falls with its width below
+    // 128 columns (it is the latency of the operand loads), so 64 is taken only where 128 leaves half of the SMs without one.  Flow
+    // 63-860-860-63, 512 samples: forward layers 11.0 us each with 128 columns (56 tiles), 9.0 with 64 (112); the pass 10.75 -> 9.86 ms.
     long long tiles256 = (long long)((g.M + BM - 1) / BM) * ((g.N + 255) / 256);
     if (g.N <= 64) bn = 64;
     else if (g.N <= 128 || tiles256 < sm_count()) bn = 128;
     if (bn == 128 && g.N > 64 && (long long)((g.M + BM - 1) / BM) * ((g.N + 127) / 128) < sm_count() / 2) bn = 64;
-    if (g.cnf_pair != 0 && bn == 64) bn = 128;      // the paired tiles come 128 and 256 columns wide
     CUtensorMap ta, tb;
     if (g.conv_on == 1) {
         if (!get_tensor_map_nhwc(g.A, g.M / (g.conv_h * g.conv_w), g.conv_h, g.conv_w, g.conv_cd, 128 / g.conv_w, dt, &ta)) return false;
@@ -505,13 +506,17 @@ bool launch_gemm_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lon
     bool ok;
     if (g.cnf_pair != 0) {
         if (dt == MPODE_BF16 && g.cnf_pair == 1)
-            ok = bn == 256 ? launch_tc<__nv_bfloat16, 256, false, 1>(ta, tb, p, st) : launch_tc<__nv_bfloat16, 128, false, 1>(ta, tb, p, st);
+            ok = bn == 256 ? launch_tc<__nv_bfloat16, 256, false, 1>(ta, tb, p, st)
+               : bn == 128 ? launch_tc<__nv_bfloat16, 128, false, 1>(ta, tb, p, st) : launch_tc<__nv_bfloat16, 64, false, 1>(ta, tb, p, st);
         else if (dt == MPODE_BF16)
-            ok = bn == 256 ? launch_tc<__nv_bfloat16, 256, false, 2>(ta, tb, p, st) : launch_tc<__nv_bfloat16, 128, false, 2>(ta, tb, p, st);
+            ok = bn == 256 ? launch_tc<__nv_bfloat16, 256, false, 2>(ta, tb, p, st)
+               : bn == 128 ? launch_tc<__nv_bfloat16, 128, false, 2>(ta, tb, p, st) : launch_tc<__nv_bfloat16, 64, false, 2>(ta, tb, p, st);
         else if (g.cnf_pair == 1)
-            ok = bn == 256 ? launch_tc<__half, 256, false, 1>(ta, tb, p, st) : launch_tc<__half, 128, false, 1>(ta, tb, p, st);
+            ok = bn == 256 ? launch_tc<__half, 256, false, 1>(ta, tb, p, st)
+               : bn == 128 ? launch_tc<__half, 128, false, 1>(ta, tb, p, st) : launch_tc<__half, 64, false, 1>(ta, tb, p, st);
         else
-            ok = bn == 256 ? launch_tc<__half, 256, false, 2>(ta, tb, p, st) : launch_tc<__half, 128, false, 2>(ta, tb, p, st);
+            ok = bn == 256 ? launch_tc<__half, 256, false, 2>(ta, tb, p, st)
+               : bn == 128 ? launch_tc<__half, 128, false, 2>(ta, tb, p, st) : launch_tc<__half, 64, false, 2>(ta, tb, p, st);
     } else if (dt == MPODE_BF16) {
         ok = bn == 256 ? launch_tc<__nv_bfloat16, 256, false>(ta, tb, p, st)
            : bn == 128 ? launch_tc<__nv_bfloat16, 128, false>(ta, tb, p, st) : launch_tc<__nv_bfloat16, 64, false>(ta, tb, p, st);

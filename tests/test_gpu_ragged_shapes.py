@@ -90,3 +90,14 @@ def test_small_float32_networks_at_tile_edges(batch, widths, n_steps):
     gpu = run_gpu(wl, low="f32")
     assert_parity(gpu, run_oracle(wl, exact=True), TOL["f32"])
     assert gpu["stats"]["fused_launches"] > 0
+
+
+# paired (value, tangent) tiles of 64 columns: one tile of 64 sample pairs, several, output columns that end inside a tile, on its edge and
+# one vector past it, the smallest reduction length
+@pytest.mark.parametrize("batch,d,hidden,low", [(64, 16, 72, "bf16"), (192, 24, 200, "f16"), (128, 72, 64, "bf16"), (512, 8, 256, "f16")])
+def test_flow_with_narrow_paired_tiles(batch, d, hidden, low):
+    wl = inputs.cnf_mlp(batch=batch, n_steps=2, d=d, hidden=hidden)
+    scaling = "dynamic" if low == "f16" else "none"
+    gpu = run_gpu(wl, low=low, scaling=scaling)
+    assert_parity(gpu, run_oracle(wl, low=low, scaling=scaling), TOL[low])
+    assert gpu["stats"]["simt_contractions"] == 0
