@@ -121,6 +121,7 @@ struct GemmArgs {
     // EPI_FWD on the tensor-core convolution path: fp32 table [9][N] of bias + tau * (time-channel weights of the taps that
     // fall inside the image), one row per position class 3 * (0 top, 1 middle, 2 bottom) + (0 left, 1 middle, 2 right)
     const float* conv_tbias;
+    const float* conv_tslope;       // 64-channel kernel only: the table is conv_tbias + tau * conv_tslope, or null
     int epi;
     void* out; long long ldo;
     int crop_m, crop_n;             // EPI_WGRAD: only the first crop_m x crop_n entries are written (0 = all; the rest belongs to padding)
@@ -133,8 +134,9 @@ struct GemmArgs {
     unsigned* flag;
     unsigned* err;                  // device word that a kernel sets when a bounded wait gives up
     int split_k; float* partial;    // EPI_WGRAD only: split the K loop over gridDim.z, partial sums in `partial`
-    // EPI_DGRAD without hprev, kernels that take it only (conv_tc.cu): beside out = psi also kap_out = Q16(kap_bv * v + kap_c * psi),
-    // the cotangent of the previous stage (Eq. (vjp) through the tableau), non-finite values flagged; v, kap_out: low format [M, N]
+    // EPI_FWD, and EPI_DGRAD without hprev, kernels that take it only (conv_tc.cu): beside the output o also kap_out = Q16(kap_bv * v + kap_c * o).
+    // Forward (o = k_j, v = the state): the input of the next stage; backward (o = psi_j, v = the seed): the cotangent of the previous
+    // stage (Eq. (vjp) through the tableau), non-finite values flagged.  v, kap_out: low format [M, N]
     void* kap_out; const void* kap_v; float kap_bv, kap_c;
     // Continuous normalizing flow with a trace estimate (Sec. 6.1), tensor-core kernel only: the operand rows are m_split primal
     // rows followed by their m_split tangent rows, and a tile holds 64 primal rows and the tangent rows of the same samples.

@@ -47,9 +47,10 @@ struct ConvParams {
     int tiles;
     int epi, act;
     void* out;
-    const float* tbias;         // EPI_FWD: [9 position classes][64] fp32 bias
+    const float* tbias;         // EPI_FWD: [9 position classes][64] fp32 bias, plus tau * tslope where that is given
+    const float* tslope; float tau;
     const void* hprev;          // EPI_DGRAD: stored output of the layer whose activation derivative multiplies the result, or null
-    void* kap_out; const void* kap_v; float kap_bv, kap_c;   // EPI_DGRAD without hprev: also kap_out = Q16(kap_bv * v + kap_c * out), or null
+    void* kap_out; const void* kap_v; float kap_bv, kap_c;   // also kap_out = Q16(kap_bv * v + kap_c * out), or null (not with hprev)
     unsigned* flag;
     unsigned* err;
 };
@@ -82,14 +83,28 @@ __device__ __forceinline__ void add_neighbours(const uint32_t (&rm)[16], const u
 }
 
 // 16 columns of one output row: out = Q16(act(acc + bias))
-template <typename T, int ACT>
-__device__ __forceinline__ void store_forward(const float (&acc)[16], const float4* bv, T* orow) {
+// (NEXT, the layer without an activation: also the next stage's input Q16(y + c k) from the rounded value)
+template <typename T, int ACT, bool NEXT = false>
+__device__ __forceinline__ void store_forward(const float (&acc)[16], const float4* bv, T* orow, T* nrow = nullptr, const uint4* yv = nullptr, float c = 0.f) {
     const float* b = reinterpret_cast<const float*>(bv);
     uint32_t packed[8];
 #pragma unroll
     for (int i = 0; i < 16; i += 2) packed[i >> 1] = cvt_pack<T>(fast_act<ACT>(acc[i] + b[i]), fast_act<ACT>(acc[i + 1] + b[i + 1]));
     *reinterpret_cast<uint4*>(orow) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
     *reinterpret_cast<uint4*>(orow + 8) = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+    if (NEXT) {
+        const uint32_t* yw = reinterpret_cast<const uint32_t*>(yv);
+        uint32_t np[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float y0 = Low<T>::to_f(from_bits<T>((unsigned short)(yw[i] & 0xFFFFu))), y1 = Low<T>::to_f(from_bits<T>((unsigned short)(yw[i] >> 16)));
+            const float k0 = Low<T>::to_f(from_bits<T>((unsigned short)(packed[i] & 0xFFFFu)));
+            const float k1 = Low<T>::to_f(from_bits<T>((unsigned short)(packed[i] >> 16)));
+            np[i] = cvt_pack<T>(fmaf(c, k0, y0), fmaf(c, k1, y1));
+        }
+        *reinterpret_cast<uint4*>(nrow) = make_uint4(np[0], np[1], np[2], np[3]);
+        *reinterpret_cast<uint4*>(nrow + 8) = make_uint4(np[4], np[5], np[6], np[7]);
+    }
 }
 
 // out = Q16(act'(h) * acc) (h: the stored output of the layer, WITH_H) or Q16(acc); true if a value left the format's range
@@ -251,7 +266,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
             const int x = m & (p.W - 1);
             const bool has_left = x != 0, has_right = x != p.W - 1;
             // what the epilogue needs besides the accumulator is fetched before the wait for it
-            const float4* sb = nullptr;
+            const float4 *sb = nullptr, *sl = nullptr;
             uint4 hv[4];
             if (p.epi == EPI_FWD) {
                 // the appended time channel is zero in the padding: its contribution (a bias per position class, a table of 2.3 KB
@@ -259,11 +274,13 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                 const int y = (m >> w_shift) % p.H;
                 const int cls = 3 * (y == 0 ? 0 : (y == p.H - 1 ? 2 : 1)) + (x == 0 ? 0 : (x == p.W - 1 ? 2 : 1));
                 sb = reinterpret_cast<const float4*>(p.tbias + cls * kC + nb);
-            } else if (p.hprev != nullptr) {
+                if (p.tslope != nullptr) sl = reinterpret_cast<const float4*>(p.tslope + cls * kC + nb);
+            }
+            if (p.hprev != nullptr) {
                 const uint4* hrow = reinterpret_cast<const uint4*>((const T*)p.hprev + (long long)m * kC + nb);
 #pragma unroll
                 for (int v = 0; v < 4; ++v) hv[v] = hrow[v];
-            } else if (p.kap_out != nullptr) {      // the seed rows that enter the previous stage's cotangent
+            } else if (p.kap_out != nullptr) {      // the state's (seed's) rows that enter the next stage's input (the previous stage's cotangent)
                 const uint4* vrow = reinterpret_cast<const uint4*>((const T*)p.kap_v + (long long)m * kC + nb);
 #pragma unroll
                 for (int v = 0; v < 4; ++v) hv[v] = vrow[v];
@@ -289,7 +306,17 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                 if (p.epi == EPI_FWD) {
                     float4 bv[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) bv[u] = __ldg(sb + 4 * c + u);
+                    for (int u = 0; u < 4; ++u) {
+                        bv[u] = __ldg(sb + 4 * c + u);
+                        if (sl != nullptr) {
+                            const float4 s4 = __ldg(sl + 4 * c + u);
+                            bv[u] = make_float4(fmaf(p.tau, s4.x, bv[u].x), fmaf(p.tau, s4.y, bv[u].y), fmaf(p.tau, s4.z, bv[u].z), fmaf(p.tau, s4.w, bv[u].w));
+                        }
+                    }
+                    if (p.kap_out != nullptr) {
+                        store_forward<T, MPODE_ACT_NONE, true>(v, bv, o, (T*)p.kap_out + (long long)m * kC + nb + c * 16, hv + 2 * c, p.kap_c);
+                        continue;
+                    }
                     switch (p.act) {
                         case MPODE_ACT_SOFTPLUS: store_forward<T, MPODE_ACT_SOFTPLUS>(v, bv, o); break;
                         case MPODE_ACT_RELU: store_forward<T, MPODE_ACT_RELU>(v, bv, o); break;
@@ -579,7 +606,9 @@ bool conv_halo_eligible(mpode_dtype dt, const GemmArgs& g) {
     if (g.epi == EPI_FWD && g.conv_tbias == nullptr) return false;
     if (g.hprev != nullptr && g.ldh != kC) return false;
     if (((uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.out | (uintptr_t)g.hprev | (uintptr_t)g.kap_out | (uintptr_t)g.kap_v) & 15) return false;
-    if (g.kap_out != nullptr && (g.epi != EPI_DGRAD || g.hprev != nullptr || g.kap_v == nullptr)) return false;
+    if (g.kap_out != nullptr && (g.hprev != nullptr || g.kap_v == nullptr)) return false;
+    if (g.kap_out != nullptr && g.epi == EPI_FWD && (g.act != MPODE_ACT_NONE || g.kap_bv != 1.f)) return false;
+    if (g.conv_tslope != nullptr && ((uintptr_t)g.conv_tslope & 15)) return false;
     return g.err != nullptr;
 }
 
@@ -593,7 +622,8 @@ bool launch_conv_halo(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long l
     if (p.stages < 2) return false;
     p.tiles = g.M / BM;
     p.epi = g.epi; p.act = g.act; p.out = g.out; p.tbias = g.conv_tbias; p.hprev = g.hprev; p.flag = g.flag; p.err = g.err;
-    if (g.epi == EPI_DGRAD && g.hprev == nullptr && g.kap_out != nullptr) {
+    p.tslope = g.conv_tslope; p.tau = g.tau;
+    if (g.kap_out != nullptr) {
         p.kap_out = g.kap_out; p.kap_v = g.kap_v; p.kap_bv = g.kap_bv; p.kap_c = g.kap_c;
     }
     CUtensorMap tx, tw;

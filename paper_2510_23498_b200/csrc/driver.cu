@@ -148,9 +148,13 @@ void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes&
     const long long nBd = (long long)c->B * c->d;
     const char* traj_i = (const char*)c->traj + (size_t)i * nBd * es;
     long long* L = &c->stats.kernel_launches;
+    const bool next_input = c->v->can_write_next_input() && c->lay.ds == c->d;
+    bool ready = false;                       // the input of this stage was written with the previous stage's derivative
     for (int j = 0; j < c->stages; ++j) {
         const void* yin = traj_i;
-        if (j > 0 || c->v->needs_input_copy()) {
+        if (ready) {
+            yin = at(ws, c->lay.ybuf[j]);
+        } else if (j > 0 || c->v->needs_input_copy()) {
             Terms t{};
             t.n = 0;
             for (int l = 0; l < j; ++l) {
@@ -163,6 +167,17 @@ void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes&
             }
             launch_stage_input(dt, traj_i, t, at(ws, c->lay.ybuf[j]), c->B, c->d, c->lay.ds, st, L);
             yin = at(ws, c->lay.ybuf[j]);
+        }
+        ready = false;
+        if (next_input && j + 1 < c->stages) {      // does the next stage depend on this one alone (Euler, midpoint, Heun, RK4)?
+            bool alone = c->ta[(j + 1) * c->stages + j] != 0.0;
+            for (int l = 0; l < j; ++l) alone = alone && c->ta[(j + 1) * c->stages + l] == 0.0;
+            if (alone) {
+                KappaNext kn;
+                kn.out = at(ws, c->lay.ybuf[j + 1]); kn.v = traj_i; kn.bv = 1.f; kn.c = (float)((double)tm.h * c->ta[(j + 1) * c->stages + j]);
+                c->v->set_next_input(kn);
+                ready = true;
+            }
         }
         c->v->forward(st, ws, j, yin, tm.tau16[j], L);
     }

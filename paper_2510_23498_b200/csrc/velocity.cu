@@ -987,6 +987,8 @@ public:
         dz1_ = lay.take(pix * C_ * es);
         w1d_ = lay.take(n2_ * es);                              // first conv without the time channel: [C][9][C]
         for (int j = 0; j < 4; ++j) tb1_[j] = lay.take((size_t)9 * C_ * sizeof(float));
+        tb1b_ = lay.take((size_t)9 * C_ * sizeof(float));
+        tb1s_ = lay.take((size_t)9 * C_ * sizeof(float));
         tb2_ = lay.take((size_t)9 * C_ * sizeof(float));
         split_ = 1;
         while (split_ < 64 && (size_t)split_ * 2 * 4096 <= pix) split_ *= 2;   // >= 4096 pixels per slice
@@ -1010,6 +1012,9 @@ public:
         launch_quantize_matrix(dt_, theta + o_b1_, C_, 1, C_, at(ws, b1_), nullptr, st, L);
         launch_quantize_matrix(dt_, theta + o_b2_, C_, 1, C_, at(ws, b2_), nullptr, st, L);
         launch_conv_class_bias(dt_, at(ws, b2_), nullptr, C_, 0.f, C_, (float*)at(ws, tb2_), st, L);
+        // first convolution: bias, and the weights of the time channel summed per position class (the factor of the stage time)
+        launch_conv_class_bias(dt_, at(ws, b1_), nullptr, C_, 0.f, C_, (float*)at(ws, tb1b_), st, L);
+        launch_conv_class_bias(dt_, nullptr, at(ws, w1_), C_ + 1, 1.f, C_, (float*)at(ws, tb1s_), st, L);
     }
 
     GemmArgs conv_args(void* ws, const void* x, int ct, float tau, const void* w, int k, int epi) const {
@@ -1025,9 +1030,13 @@ public:
         // tensor-core form of the first convolution: 64 data channels per tap, the time channel folded into a bias per
         // position class; when the shape does not allow it, the general kernel takes the 65-channel form
         GemmArgs g = conv_args(ws, yin, C_, 0.f, at(ws, w1d_), 9 * C_, EPI_FWD);
-        g.conv_tbias = (const float*)at(ws, tb1_[j]);
+        g.conv_tbias = (const float*)at(ws, tb1b_); g.conv_tslope = (const float*)at(ws, tb1s_); g.tau = tau16;
         g.bias = at(ws, b1_); g.act = act_; g.out = at(ws, h1_[j]);
-        if (tc_eligible(dt_, g)) {
+        const bool halo = conv_halo_eligible(dt_, g);
+        if (!halo) { g.conv_tbias = (const float*)at(ws, tb1_[j]); g.conv_tslope = nullptr; }
+        if (halo) {
+            // the kernel puts the table together
+        } else if (tc_eligible(dt_, g)) {
             launch_conv_class_bias(dt_, at(ws, b1_), at(ws, w1_), C_ + 1, tau16, C_, (float*)at(ws, tb1_[j]), st, L);
         } else {
             g = conv_args(ws, yin, C_ + 1, tau16, at(ws, w1_), 9 * (C_ + 1), EPI_FWD);
@@ -1037,8 +1046,19 @@ public:
         g = conv_args(ws, at(ws, h1_[j]), C_, 0.f, at(ws, w2_), 9 * C_, EPI_FWD);
         g.conv_tbias = (const float*)at(ws, tb2_);
         g.bias = at(ws, b2_); g.act = MPODE_ACT_NONE; g.out = at(ws, lay_->kbuf[j]);
-        launch_contraction(dt_, g, st, L);
+        const KappaNext kn = next_in_;
+        next_in_.out = nullptr;
+        if (kn.out != nullptr) { g.kap_out = kn.out; g.kap_v = kn.v; g.kap_bv = kn.bv; g.kap_c = kn.c; }
+        if (kn.out != nullptr && !conv_halo_eligible(dt_, g)) g.kap_out = nullptr;      // (the trajectory's alignment)
+        const int path = launch_contraction(dt_, g, st, L);
+        if (kn.out != nullptr && (path != 2 || g.kap_out == nullptr)) {
+            Terms t{};
+            t.n = 1; t.p[0] = at(ws, lay_->kbuf[j]); t.c[0] = kn.c;
+            launch_stage_input(dt_, kn.v, t, kn.out, B_, H_ * W_ * C_, H_ * W_ * C_, st, L);
+        }
     }
+    bool can_write_next_input() const override { return dt_ != MPODE_F32; }
+    void set_next_input(const KappaNext& n) override { next_in_ = n; }
 
     // weight gradient of one convolution (and of its appended time channel when ct > C) plus its bias gradient
     void wgrad(cudaStream_t st, void* ws, const void* dz, const void* x, int ct, float tau, float* out, float* bias_out, float beta,
@@ -1116,8 +1136,8 @@ private:
     int act_;
     size_t n1_, n2_, o_w1_, o_b1_, o_w2_, o_b2_, p_;
     size_t w1_ = 0, w1t_ = 0, w2_ = 0, w2t_ = 0, b1_ = 0, b2_ = 0, h1_[4] = {0}, dz1_ = 0, partial_ = 0, colsum_ = 0;
-    size_t w1d_ = 0, tb1_[4] = {0}, tb2_ = 0, tws_ = 0, partial_bytes_ = 0, ind_ = 0;
-    KappaNext next_{};
+    size_t w1d_ = 0, tb1_[4] = {0}, tb1b_ = 0, tb1s_ = 0, tb2_ = 0, tws_ = 0, partial_bytes_ = 0, ind_ = 0;
+    KappaNext next_{}, next_in_{};
     int split_ = 1;
     const Layout* lay_ = nullptr;
 };

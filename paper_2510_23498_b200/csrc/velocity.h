@@ -80,6 +80,9 @@ public:
     // can_write_next_kappa(), hands the request over before vjp(), and vjp() then writes `out` whatever kernel it ends up taking.
     virtual bool can_write_next_kappa() const { return false; }
     virtual void set_next_kappa(const KappaNext&) {}
+    // The same for the next stage's input Y_{j+1} = Q16(y + c k_j) from the epilogue that produces k_j (out, v = y, c), written by forward()
+    virtual bool can_write_next_input() const { return false; }
+    virtual void set_next_input(const KappaNext&) {}
     // whether the velocity can return the cotangent of its stage times (time-grid gradient), written to dtau[j] by vjp / fused_vjp
     virtual bool supports_time_gradient() const { return false; }
     // velocities whose parameters are piecewise constant in time are told which step the following calls belong to

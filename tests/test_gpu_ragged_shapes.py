@@ -1,4 +1,5 @@
 """GPU parity at sizes where tiles, slices and padded rows end: just inside, on and just past their edges."""
+import numpy as np
 import pytest
 
 from paper_2510_23498_b200 import inputs
@@ -82,7 +83,7 @@ def test_small_networks_at_tile_edges(batch, widths, n_steps):
 
 
 # the same in float32 (CUDA cores): one row, a block's 8 rows less and plus one, more row tiles than SMs, odd widths, 1 to 4 layers
-@pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (7, [9, 33, 65, 9], 3), (9, [64, 64], 20), (200, [72, 201, 200, 72], 2),
+@pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (7, [16, 33, 65, 16], 3), (9, [64, 64], 20), (200, [72, 201, 200, 72], 2),
                                                   (1185, [24, 40, 24], 2), (130, [16, 32, 48, 32, 16], 3)])
 def test_small_float32_networks_at_tile_edges(batch, widths, n_steps):
     wl = inputs.mlp_block(batch=batch, n_steps=n_steps, d=widths[0], hidden=widths[1], low="f32")
@@ -101,3 +102,13 @@ def test_flow_with_narrow_paired_tiles(batch, d, hidden, low):
     gpu = run_gpu(wl, low=low, scaling=scaling)
     assert_parity(gpu, run_oracle(wl, low=low, scaling=scaling), TOL[low])
     assert gpu["stats"]["simt_contractions"] == 0
+
+
+# 64-channel convolutions whose second layer writes the next stage's input: solvers with such a stage everywhere (Heun, RK4, midpoint),
+# nowhere (Euler) and in some stages only (the third-order and the 3/8 tableau); time steps that differ (non-uniform grid)
+@pytest.mark.parametrize("solver", ["euler", "midpoint", "heun", "kutta3", "rk38", "rk4"])
+def test_conv_block_next_stage_input_per_solver(solver):
+    wl = inputs.conv_block(batch=3, n_steps=2, H=16, W=16, C=64, act="softplus", solver=solver)
+    wl.tgrid = np.array([0.0, 0.375, 1.0], np.float32)
+    for low, scaling in (("f16", "dynamic"), ("bf16", "none")):
+        assert_parity(run_gpu(wl, low, scaling), run_oracle(wl, low, scaling), TOL[low])
