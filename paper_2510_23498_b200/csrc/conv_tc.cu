@@ -195,7 +195,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 
     if (warp == 0) {
         // ------------------------------------------------------------ loads: the weights once, then one halo block per tile
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_arrive_expect_tx(w_bar, (uint32_t)kWeightBytes);
             for (int t = 0; t < 9; ++t) tma_load_2d(smem_u32(sW + t * kC * kC * 2), &tmW, w_bar, t * kC, 0);
             int s = 0;
@@ -213,7 +213,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = make_idesc(Fmt<T>::id, BM, kAccCols, false);
             int s = 0;
             uint32_t phase = 0;
@@ -413,7 +413,7 @@ conv3x3_wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
     chain_begin();                          // everything above overlaps the tail of the kernel before
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int s = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -432,7 +432,7 @@ conv3x3_wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = make_idesc(Fmt<T>::id, BM, kWgCols, true);
             int s = 0;
             uint32_t phase = 0;

@@ -217,7 +217,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
 
     if (warp == 0) {
         // ------------------------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int s = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -308,7 +308,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             int s = 0;
             uint32_t phase = 0;
             int k_local = 0;
@@ -381,7 +381,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
         // Releases a finished tile to the other CTAs: once all epilogue warps have issued the tile's stores it makes
         // them visible device-wide and bumps the row block's completion counter, so the epilogue warps never wait on
         // a memory fence themselves.
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             int k_local = 0;
             Sched sch(cta, G, p.chain_ctas);
@@ -418,7 +418,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
         // the stored layer output H.  H was written by the recompute launch, so it has no dependency inside this launch:
         // this thread streams it into two shared-memory units ahead of the epilogue warps (a 256-wide tile is two units of
         // 128 columns, a narrower tile one unit), bounded only by the units being free again.
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             unsigned u = 0;
             Sched sch(cta, G, p.chain_ctas);

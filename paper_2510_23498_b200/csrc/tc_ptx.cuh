@@ -44,9 +44,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 // Bounded wait: gives up after `limit_ns`, records `code` in *err and returns false.
-static __device__ __noinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned* err, unsigned code,
-                                              unsigned long long limit_ns = kWaitLimitNs) {
-    if (mbar_try_wait(bar, parity)) return true;
+static __device__ __noinline__ bool mbar_wait_long(uint64_t* bar, uint32_t parity, unsigned* err, unsigned code, unsigned long long limit_ns) {
     unsigned long long t0 = globaltimer_ns();
     unsigned it = 0;
     while (true) {
@@ -60,6 +58,17 @@ static __device__ __noinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, un
     }
 }
 
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned* err, unsigned code, unsigned long long limit_ns = kWaitLimitNs) {
+    return mbar_try_wait(bar, parity) || mbar_wait_long(bar, parity, err, code, limit_ns);
+}
+// One thread of a converged warp.  The threads that issue bulk copies and matrix instructions are chosen by this instruction, whose
+// result the compiler knows to be a single thread: those instructions take their operands from warp-uniform registers, and behind any
+// other condition (lane == 0) every operand is moved there in a loop over the threads that might be active.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t yes;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(yes));
+    return yes != 0u;
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* tmap, uint64_t* bar, int x, int y) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
