@@ -112,3 +112,11 @@ def test_conv_block_next_stage_input_per_solver(solver):
     wl.tgrid = np.array([0.0, 0.375, 1.0], np.float32)
     for low, scaling in (("f16", "dynamic"), ("bf16", "none")):
         assert_parity(run_gpu(wl, low, scaling), run_oracle(wl, low, scaling), TOL[low])
+
+
+# 64-channel convolutions: tiles in and out through shared memory.  Every image-row width, fewer tiles than SMs, and more than four per SM
+# (the buffers of operand tiles wrap around)
+@pytest.mark.parametrize("batch,H,W", [(1, 16, 8), (3, 8, 16), (2, 4, 32), (75, 32, 32)])
+def test_conv_block_tile_buffers(batch, H, W):
+    wl = inputs.conv_block(batch=batch, n_steps=1, H=H, W=W, C=64, act="softplus", solver="heun")
+    assert_parity(run_gpu(wl, "f16", "dynamic"), run_oracle(wl, "f16", "dynamic"), TOL["f16"])
