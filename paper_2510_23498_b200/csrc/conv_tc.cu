@@ -102,11 +102,9 @@ __device__ __forceinline__ void forward_chunk(const float (&acc)[16], const floa
     }
 }
 
-// out = Q16(act'(h) * acc) (h: the stored output of the layer, WITH_H) or Q16(acc); true if a value left the format's range
+// out = Q16(act'(h) * acc) (h: the stored output of the layer, WITH_H) or Q16(acc); values outside the format's range are noted in `bad`
 template <typename T, int ACT, bool WITH_H>
-__device__ __forceinline__ bool backward_chunk(const float (&acc)[16], const uint32_t* hw, uint32_t (&packed)[8]) {
-    const float lim = OverflowLimit<T>::value();
-    bool bad = false;
+__device__ __forceinline__ void backward_chunk(const float (&acc)[16], const uint32_t* hw, uint32_t (&packed)[8], uint32_t& bad) {
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
         float v0 = acc[i], v1 = acc[i + 1];
@@ -115,22 +113,20 @@ __device__ __forceinline__ bool backward_chunk(const float (&acc)[16], const uin
             v0 *= fast_act_deriv<ACT>(Low<T>::to_f(from_bits<T>((unsigned short)(w & 0xFFFFu))));
             v1 *= fast_act_deriv<ACT>(Low<T>::to_f(from_bits<T>((unsigned short)(w >> 16))));
         }
-        bad |= !(fabsf(v0) < lim) | !(fabsf(v1) < lim);
         packed[i >> 1] = cvt_pack<T>(v0, v1);
+        note_nonfinite<T>(packed[i >> 1], bad);
     }
-    return bad;
 }
 
 // Input gradient without an activation (the stage's psi): out = Q16(acc), and optionally the previous stage's cotangent from
-// the rounded value, kappa = Q16(bv * v + c * psi), 16 columns; true if a value left the format's range
+// the rounded value, kappa = Q16(bv * v + c * psi), 16 columns; values outside the format's range are noted in `bad`
 template <typename T>
-__device__ __forceinline__ bool psi_kappa_chunk(const float (&acc)[16], bool with_kap, const uint32_t* vw, float bv, float c, uint32_t (&packed)[8], uint32_t (&kp)[8]) {
-    const float lim = OverflowLimit<T>::value();
-    bool bad = false;
+__device__ __forceinline__ void psi_kappa_chunk(const float (&acc)[16], bool with_kap, const uint32_t* vw, float bv, float c, uint32_t (&packed)[8], uint32_t (&kp)[8],
+                                                uint32_t& bad) {
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        bad |= !(fabsf(acc[i]) < lim) | !(fabsf(acc[i + 1]) < lim);
         packed[i >> 1] = cvt_pack<T>(acc[i], acc[i + 1]);
+        note_nonfinite<T>(packed[i >> 1], bad);
     }
     if (with_kap) {
 #pragma unroll
@@ -139,11 +135,10 @@ __device__ __forceinline__ bool psi_kappa_chunk(const float (&acc)[16], bool wit
             const float q0 = Low<T>::to_f(from_bits<T>((unsigned short)(packed[i] & 0xFFFFu)));
             const float q1 = Low<T>::to_f(from_bits<T>((unsigned short)(packed[i] >> 16)));
             const T k0 = Low<T>::from_f(fmaf(c, q0, bv * v0)), k1 = Low<T>::from_f(fmaf(c, q1, bv * v1));
-            bad |= Low<T>::nonfinite(k0) | Low<T>::nonfinite(k1);
             kp[i] = pack2<T>(k0, k1);
+            note_nonfinite<T>(kp[i], bad);
         }
     }
-    return bad;
 }
 
 template <typename T>
@@ -260,7 +255,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         const int nb = (((warp - 2) >> 2) & 1) * 32;
         const int w_shift = 31 - __clz(p.W);                    // W is a power of two
         const bool leader = (warp - 2) % (kEpiWarps / 2) == 0 && elect_one();      // issues the group's tile stores
-        bool bad = false;
+        uint32_t bad = 0u;
         bool ok = true;
         int it = 0;
         for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x, ++it) {
@@ -332,13 +327,13 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                         }
                     }
                 } else if (!p.with_h) {
-                    bad |= psi_kappa_chunk<T>(v, p.with_kap != 0, vw, p.kap_bv, p.kap_c, o, k2);
+                    psi_kappa_chunk<T>(v, p.with_kap != 0, vw, p.kap_bv, p.kap_c, o, k2, bad);
                 } else {
                     switch (p.act) {
-                        case MPODE_ACT_SOFTPLUS: bad |= backward_chunk<T, MPODE_ACT_SOFTPLUS, true>(v, vw, o); break;
-                        case MPODE_ACT_RELU: bad |= backward_chunk<T, MPODE_ACT_RELU, true>(v, vw, o); break;
-                        case MPODE_ACT_TANH: bad |= backward_chunk<T, MPODE_ACT_TANH, true>(v, vw, o); break;
-                        default: bad |= backward_chunk<T, MPODE_ACT_NONE, true>(v, vw, o); break;
+                        case MPODE_ACT_SOFTPLUS: backward_chunk<T, MPODE_ACT_SOFTPLUS, true>(v, vw, o, bad); break;
+                        case MPODE_ACT_RELU: backward_chunk<T, MPODE_ACT_RELU, true>(v, vw, o, bad); break;
+                        case MPODE_ACT_TANH: backward_chunk<T, MPODE_ACT_TANH, true>(v, vw, o, bad); break;
+                        default: backward_chunk<T, MPODE_ACT_NONE, true>(v, vw, o, bad); break;
                     }
                 }
                 sts128(swizzled(otile, row, j0), o[0], o[1], o[2], o[3]);
@@ -358,7 +353,7 @@ conv3x3_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         }
         if (leader) bulk_wait();
         __syncwarp();
-        if (p.epi == EPI_DGRAD) warp_flag_or(p.flag, bad);
+        if (p.epi == EPI_DGRAD) warp_flag_or(p.flag, any_nonfinite(bad));
     }
 
     tc_fence_before_sync();

@@ -208,7 +208,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int half = (warp - 2) >> 2;
         constexpr int kColsPerWarp = BN / (Shape<BN>::kEpiWarps / 4);
         float* sb_warp = sbias + (warp - 2) * kColsPerWarp;   // this warp's slice of the effective bias b + tau * w_t
-        bool bad = false;
+        uint32_t bad = 0u;
         bool ok = true;
         int it = 0;
         for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++it) {
@@ -415,7 +415,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty_bar[acc]);
         }
-        if (!WG && p.epi == EPI_DGRAD) warp_flag_or(p.flag, bad);
+        if (!WG && p.epi == EPI_DGRAD) warp_flag_or(p.flag, any_nonfinite(bad));
     }
 
     tc_fence_before_sync();

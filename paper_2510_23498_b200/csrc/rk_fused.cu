@@ -155,20 +155,16 @@ __device__ __forceinline__ void hidden_chunk(const uint32_t (&r)[16], const floa
 }
 
 template <typename T, int ACT>
-__device__ __forceinline__ bool dgrad_chunk(const uint32_t (&r)[16], const uint32_t (&hw)[8], T* orow, int nb, int N,
-                                            uint32_t (&packed)[8]) {
-    const float lim = OverflowLimit<T>::value();
-    bool bad = false;
+__device__ __forceinline__ void dgrad_chunk(const uint32_t (&r)[16], const uint32_t (&hw)[8], T* orow, int nb, int N,
+                                            uint32_t (&packed)[8], uint32_t& bad) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         float v0 = __uint_as_float(r[2 * i]) * fast_act_deriv<ACT>(lo_f<T>(hw[i]));
         float v1 = __uint_as_float(r[2 * i + 1]) * fast_act_deriv<ACT>(hi_f<T>(hw[i]));
-        bad |= (nb + 2 * i < N) && !(fabsf(v0) < lim);
-        bad |= (nb + 2 * i + 1 < N) && !(fabsf(v1) < lim);
         packed[i] = cvt_pack<T>(v0, v1);
+        note_nonfinite<T>(packed[i], bad);      // (columns past N hold zeros)
     }
     store16<T>(orow, nb, N, packed);
-    return bad;
 }
 
 // BWD = false: programs of hidden-layer and stage-output phases (forward loop, recompute); BWD = true: programs of
@@ -455,7 +451,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
         const int q4 = warp & 3;                 // TMEM lane quadrant this warp may read
         const int cg = ew >> 2;                  // which half of the tile's columns (of each unit, for two-unit tiles)
         float* sb_warp = sbias + ew * kStrip;
-        bool bad = false;
+        uint32_t bad = 0u;
         bool ok = true;
         int k_local = 0;
         unsigned u_local = 0;                    // units of stored layer outputs consumed so far (same count as the loader's)
@@ -561,10 +557,10 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
                                 T* orow = (T*)p.dzslab[ph.layer] + (long long)ph.out_slot * p.dz_slot_stride[ph.layer] + (long long)m * ph.N;
                                 uint32_t out[8];
                                 switch (ph.act) {
-                                    case MPODE_ACT_SOFTPLUS: bad |= dgrad_chunk<T, MPODE_ACT_SOFTPLUS>(r, hw, orow, nb, ph.N, out); break;
-                                    case MPODE_ACT_RELU: bad |= dgrad_chunk<T, MPODE_ACT_RELU>(r, hw, orow, nb, ph.N, out); break;
-                                    case MPODE_ACT_TANH: bad |= dgrad_chunk<T, MPODE_ACT_TANH>(r, hw, orow, nb, ph.N, out); break;
-                                    default: bad |= dgrad_chunk<T, MPODE_ACT_NONE>(r, hw, orow, nb, ph.N, out); break;
+                                    case MPODE_ACT_SOFTPLUS: dgrad_chunk<T, MPODE_ACT_SOFTPLUS>(r, hw, orow, nb, ph.N, out, bad); break;
+                                    case MPODE_ACT_RELU: dgrad_chunk<T, MPODE_ACT_RELU>(r, hw, orow, nb, ph.N, out, bad); break;
+                                    case MPODE_ACT_TANH: dgrad_chunk<T, MPODE_ACT_TANH>(r, hw, orow, nb, ph.N, out, bad); break;
+                                    default: dgrad_chunk<T, MPODE_ACT_NONE>(r, hw, orow, nb, ph.N, out, bad); break;
                                 }
                             }
                             if ((c % per_unit) == per_unit - 1) {      // this warp is done with the unit
@@ -652,17 +648,14 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
                         } else if (BWD) {   // RK_EPI_PSI
                             const int j = ph.stage, d = p.d;
                             const long long slab = (long long)p.B * d, roff = (long long)m * d;
-                            const float lim = OverflowLimit<T>::value();
                             // operands of the stage cotangent below, requested together
                             uint32_t pre[8];
                             if (j > 0) load16_cg<T>((const T*)p.v + roff, nb, d, pre);
                             uint32_t pq[8], w[8];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
-                                const float v0 = __uint_as_float(r[2 * i]), v1 = __uint_as_float(r[2 * i + 1]);
-                                bad |= (nb + 2 * i < d) && !(fabsf(v0) < lim);
-                                bad |= (nb + 2 * i + 1 < d) && !(fabsf(v1) < lim);
-                                pq[i] = cvt_pack<T>(v0, v1);
+                                pq[i] = cvt_pack<T>(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+                                note_nonfinite<T>(pq[i], bad);
                             }
                             store16<T>((T*)p.psislab + j * slab + roff, nb, d, pq);
                             if (j > 0) {
@@ -681,9 +674,8 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
                                 }
 #pragma unroll
                                 for (int i = 0; i < 8; ++i) {
-                                    bad |= (nb + 2 * i < d) && !(fabsf(a[2 * i]) < lim);
-                                    bad |= (nb + 2 * i + 1 < d) && !(fabsf(a[2 * i + 1]) < lim);
                                     w[i] = cvt_pack<T>(a[2 * i], a[2 * i + 1]);
+                                    note_nonfinite<T>(w[i], bad);
                                 }
                                 store16<T>((T*)p.kappaslab + (long long)((j - 1) % 3) * slab + roff, nb, d, w);
                             }
@@ -710,7 +702,7 @@ rk_fused_kernel(const __grid_constant__ RkMaps maps, const RkParams p) {
                 }
             }
         }
-        warp_flag_or(p.flag, bad);
+        warp_flag_or(p.flag, any_nonfinite(bad));
     }
 
     tc_fence_before_sync();

@@ -37,10 +37,10 @@ __device__ __forceinline__ void store_chunk(T* orow, int nb, int N, const uint32
 // One 32-column chunk of one accumulator row: epilogue math, rounding, stores.  `hv`: load_h_chunk's result when
 // `with_h` (input gradient through an activation).
 template <typename T, int ACT, bool FWD>
-__device__ __forceinline__ bool epilogue_chunk(const uint32_t (&r)[32], const float* sb, bool plain, bool with_h, const uint4 (&hv)[4],
-                                               T* orow, int nb, int N, uint32_t* keep = nullptr) {
+__device__ __forceinline__ uint32_t epilogue_chunk(const uint32_t (&r)[32], const float* sb, bool plain, bool with_h, const uint4 (&hv)[4],
+                                                   T* orow, int nb, int N, uint32_t* keep = nullptr) {
     uint32_t packed[16];
-    bool bad = false;
+    uint32_t bad = 0u;         // note_nonfinite's sum (columns past N hold zeros)
     if (FWD) {
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
@@ -53,7 +53,6 @@ __device__ __forceinline__ bool epilogue_chunk(const uint32_t (&r)[32], const fl
         }
     } else {
         const uint32_t* hw = reinterpret_cast<const uint32_t*>(hv);
-        const float lim = OverflowLimit<T>::value();
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
             float v0 = __uint_as_float(r[i]), v1 = __uint_as_float(r[i + 1]);
@@ -62,9 +61,8 @@ __device__ __forceinline__ bool epilogue_chunk(const uint32_t (&r)[32], const fl
                 v0 *= fast_act_deriv<ACT>(Low<T>::to_f(from_bits<T>((unsigned short)(w & 0xFFFFu))));
                 v1 *= fast_act_deriv<ACT>(Low<T>::to_f(from_bits<T>((unsigned short)(w >> 16))));
             }
-            bad |= (nb + i < N) && !(fabsf(v0) < lim);
-            bad |= (nb + i + 1 < N) && !(fabsf(v1) < lim);
             packed[i >> 1] = cvt_pack<T>(v0, v1);
+            note_nonfinite<T>(packed[i >> 1], bad);
         }
     }
     store_chunk<T>(orow, nb, N, packed);
@@ -137,12 +135,11 @@ __device__ __forceinline__ void tangent_chunk(const uint32_t (&r)[32], const uin
 // Backward pass of the same flow through one activation, 16 columns: s = act'(H); the tangent rows give ubar = Q16(s gbar), the
 // primal rows zeta = Q16(s hbar + s (1 - s) U gbar) (softplus: act'' = s (1 - s)).  `acc`: 16 of this row's accumulators (gbar or
 // hbar), `gb`: gbar of the sample (primal rows only), `hw` / `uw`: 8 packed words of H and U, `out`: 8 packed results.
-// Returns whether a rounded value is not finite.
+// Returns note_nonfinite's sum over the rounded values.
 template <typename T, int ACT, int HF>
-__device__ __forceinline__ bool cnf_backward_half(const uint32_t (&r)[32], bool tangent, const float (&gb)[16], const uint4 (&hv)[4],
+__device__ __forceinline__ uint32_t cnf_backward_half(const uint32_t (&r)[32], bool tangent, const float (&gb)[16], const uint4 (&hv)[4],
                                                   const uint4 (&uv)[4], uint32_t (&packed)[16], int nb, int N) {
-    const float lim = OverflowLimit<T>::value();
-    bool bad = false;
+    uint32_t bad = 0u;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
         const int word = 8 * HF + (i >> 1);       // packed word of the chunk: uint4 number word / 4, component word % 4
@@ -159,9 +156,8 @@ __device__ __forceinline__ bool cnf_backward_half(const uint32_t (&r)[32], bool 
             v0 = s0 * v0 + s0 * (1.f - s0) * Low<T>::to_f(from_bits<T>((unsigned short)(u & 0xFFFFu))) * gb[i];
             v1 = s1 * v1 + s1 * (1.f - s1) * Low<T>::to_f(from_bits<T>((unsigned short)(u >> 16))) * gb[i + 1];
         }
-        bad |= (nb + 16 * HF + i < N) && !(fabsf(v0) < lim);
-        bad |= (nb + 16 * HF + i + 1 < N) && !(fabsf(v1) < lim);
         packed[word] = cvt_pack<T>(v0, v1);
+        note_nonfinite<T>(packed[word], bad);
     }
     return bad;
 }

@@ -231,6 +231,17 @@ template <typename T> struct OverflowLimit;
 template <> struct OverflowLimit<__half> { static __device__ __forceinline__ float value() { return 65520.f; } };
 template <> struct OverflowLimit<__nv_bfloat16> { static __device__ __forceinline__ float value() { return __uint_as_float(0x7F7F8000u); } };
 
+// Whether a rounded value is not finite, noted for two values at once: 0 * Inf and 0 * NaN are NaN, which the sum keeps.  (Comparing
+// every value with the limit, a chain of predicates, was a third of the instructions of an input gradient's epilogue.)
+template <typename T> __device__ __forceinline__ void note_nonfinite(uint32_t packed, uint32_t& acc);
+template <> __device__ __forceinline__ void note_nonfinite<__half>(uint32_t packed, uint32_t& acc) {
+    asm("fma.rn.f16x2 %0, %1, %2, %0;" : "+r"(acc) : "r"(packed), "r"(0u));
+}
+template <> __device__ __forceinline__ void note_nonfinite<__nv_bfloat16>(uint32_t packed, uint32_t& acc) {
+    asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(acc) : "r"(packed), "r"(0u));
+}
+__device__ __forceinline__ bool any_nonfinite(uint32_t acc) { return (acc & 0x7FFF7FFFu) != 0u; }
+
 // Activations for the tensor-core epilogue: one MUFU (ex2) per element plus a short FMA-pipe polynomial.  The results
 // are rounded to a 16-bit format next (unit roundoff 2^-8 or 2^-11), so a relative error near 1e-5 is invisible.
 //   softplus(z) = max(z, 0) + log1p(t), t = exp(-|z|) in (0, 1]; log1p(t) = t * P5(t), |rel. err| < 9e-6

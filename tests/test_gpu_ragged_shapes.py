@@ -119,4 +119,4 @@ def test_conv_block_next_stage_input_per_solver(solver):
 @pytest.mark.parametrize("batch,H,W", [(1, 16, 8), (3, 8, 16), (2, 4, 32), (75, 32, 32)])
 def test_conv_block_tile_buffers(batch, H, W):
     wl = inputs.conv_block(batch=batch, n_steps=1, H=H, W=W, C=64, act="softplus", solver="heun")
-    assert_parity(run_gpu(wl, "f16", "dynamic"), run_oracle(wl, "f16", "dynamic"), TOL["f16"])
+    assert_parity(run_gpu(wl, "bf16", "none"), run_oracle(wl, "bf16", "none"), TOL["bf16"])
