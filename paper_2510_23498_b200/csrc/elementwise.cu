@@ -452,17 +452,23 @@ __global__ void commit_a_kernel(float* __restrict__ a, Terms psis, float coef, i
     long long nv = (long long)B * dv;
     float m = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
-        long long row = i / dv;
-        int col = (int)(i % dv) * V;
+        long long row = nv <= 0x7fffffffLL ? (unsigned)i / (unsigned)dv : i / dv;
+        int col = (int)(i - row * dv) * V;
+        // every operand is requested before the first is used: one trip to memory, not one per stage (8192 x 256, four stages: 15.6 -> 13.4 us)
+        Pack<float, V> aa = *reinterpret_cast<Pack<float, V>*>(a + row * D + col);
+        Pack<T, V> pp[4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+            if (l < psis.n) pp[l] = *reinterpret_cast<const Pack<T, V>*>((const T*)psis.p[l] + row * ds + col);
         float da[V];
 #pragma unroll
         for (int k = 0; k < V; ++k) da[k] = 0.f;
-        for (int l = 0; l < psis.n; ++l) {
-            Pack<T, V> pp = *reinterpret_cast<const Pack<T, V>*>((const T*)psis.p[l] + row * ds + col);
 #pragma unroll
-            for (int k = 0; k < V; ++k) da[k] += Low<T>::to_f(pp.v[k]);
-        }
-        Pack<float, V> aa = *reinterpret_cast<Pack<float, V>*>(a + row * D + col);
+        for (int l = 0; l < 4; ++l)
+            if (l < psis.n) {
+#pragma unroll
+                for (int k = 0; k < V; ++k) da[k] += Low<T>::to_f(pp[l].v[k]);
+            }
 #pragma unroll
         for (int k = 0; k < V; ++k) aa.v[k] = fmaf(coef, da[k], aa.v[k]);
         if (add != nullptr) {
@@ -674,13 +680,30 @@ __global__ void grad_finish_kernel(GradFinishArgs a) {
     const GradFinishLayer& L = a.layer[blockIdx.y];
     const int wblocks = (int)gridDim.x - kFinishBiasBlocks;
     if ((int)blockIdx.x < wblocks) {
-        const long long n_el = (long long)L.Mp * L.Np;
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_el; i += (long long)wblocks * blockDim.x) {
-            if (i / L.Np >= L.M || i % L.Np >= L.N) continue;
-            float s = 0.f;
-            for (int z = 0; z < L.splits; ++z) s += L.partial[(long long)z * n_el + i];
-            float* o = a.out + L.w_off + (i / L.Np) * L.ldo + (i % L.Np);
-            *o = (a.beta != 0.f ? a.beta * *o : 0.f) + a.coef * s;
+        // four elements of a thread at a time, all their slices and old values requested before the sums (one element: 27.7 us, four: 15.5, for
+        // 1.57M weights in 3 slices, bound by the trips to L2 one after the other)
+        constexpr int kEl = 4;
+        const unsigned n_el = (unsigned)L.Mp * (unsigned)L.Np, Np = (unsigned)L.Np;
+        for (unsigned i0 = blockIdx.x * (unsigned)kEl * blockDim.x + threadIdx.x; i0 < n_el; i0 += (unsigned)wblocks * kEl * blockDim.x) {
+            float s[kEl], old[kEl];
+            float* o[kEl];
+#pragma unroll
+            for (int k = 0; k < kEl; ++k) {
+                const unsigned i = i0 + (unsigned)k * blockDim.x, m = i / Np, c = i - m * Np;
+                const bool on = i < n_el && (int)m < L.M && (int)c < L.N;
+                o[k] = on ? a.out + L.w_off + (long long)m * L.ldo + c : nullptr;
+                s[k] = 0.f;
+                old[k] = on && a.beta != 0.f ? *o[k] : 0.f;
+            }
+            for (int z = 0; z < L.splits; ++z) {
+                const float* part = L.partial + (long long)z * n_el + i0;
+#pragma unroll
+                for (int k = 0; k < kEl; ++k)
+                    if (o[k] != nullptr) s[k] += part[k * blockDim.x];
+            }
+#pragma unroll
+            for (int k = 0; k < kEl; ++k)
+                if (o[k] != nullptr) *o[k] = a.beta * old[k] + a.coef * s[k];
         }
     } else if (L.bias_off >= 0 || L.time_off >= 0) {
         const int lane = threadIdx.x & 31;
