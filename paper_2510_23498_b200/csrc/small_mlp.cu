@@ -957,8 +957,14 @@ bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp) {
     long long elems = 0;
     for (int l = 0; l <= L; ++l) { p.wp[l] = p.wr[l] = wp[l]; if (l < L) elems += (long long)wp[l] * wp[l + 1]; }
     if (dt == MPODE_F32) return ring_buffers<float>(p, 16) >= 3 && elems <= 256 * 1024 && B <= 16 * sm_count();
-    return ring_buffers<__half>(p, 32) >= 3 && elems <= 160 * 1024 && B <= 8192;
+    return ring_buffers<__half>(p, 32) >= 3 && elems <= 160 * 1024 && B <= 32 * sm_count();
 }
+
+// The 16-bit backward pass stops at one row tile per SM: its weight gradients grow with the batch and run on the slower matrix
+// instructions.  Training pass of 8 RK4 steps, bf16, ms here / tensor-core program (rk_fused.cu): 64-128-64 0.66 / 1.21 at 1000 samples,
+// 0.97 / 1.23 at 2300, 1.50 / 1.24 at 4000; 112-336-112 1.46 / 1.52 at 2300, 2.28 / 1.70 at 4000; 128-256-256-128 1.54 / 1.90 at 2300,
+// 2.45 / 2.02 at 4000.  The forward pass alone at 4000: 0.16 / 0.37, 0.33 / 0.46, 0.36 / 0.56; at 8000 0.29 / 0.37, 0.62 / 0.47, 0.69 / 0.64.
+bool small_backward_supported(mpode_dtype dt, int B) { return dt == MPODE_F32 || rows_tiles(dt, B) == 1; }
 
 int small_blocks(mpode_dtype dt, int B) {
     const int r = (dt == MPODE_F32 ? 8 : 16) * rows_tiles(dt, B);
@@ -991,10 +997,9 @@ bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, lo
 }
 
 bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    const bool one = rows_tiles(dt, p.B) == 1;
-    const bool ok = dt == MPODE_BF16 ? (one ? backward_t<__nv_bfloat16, 1>(p, st) : backward_t<__nv_bfloat16, 2>(p, st))
-                  : dt == MPODE_F16  ? (one ? backward_t<__half, 1>(p, st) : backward_t<__half, 2>(p, st))
-                                     : (one ? backward_t<float, 1>(p, st) : backward_t<float, 2>(p, st));
+    const bool ok = dt == MPODE_BF16 ? backward_t<__nv_bfloat16, 1>(p, st)
+                  : dt == MPODE_F16  ? backward_t<__half, 1>(p, st)
+                                     : (rows_tiles(dt, p.B) == 1 ? backward_t<float, 1>(p, st) : backward_t<float, 2>(p, st));
     if (ok && launches) ++*launches;
     if (ok && tl_counters) ++tl_counters->fused;
     return ok;

@@ -39,6 +39,7 @@ constexpr int SMALL_MAX_CHUNK = 16;
 size_t small_pack_elems(mpode_dtype dt, int n, int k);      // of one layer and direction: n columns, reduction of k
 size_t small_pack_bytes(mpode_dtype dt, int L, const int* wp);
 bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp);
+bool small_backward_supported(mpode_dtype dt, int B);       // of a network that small_mlp_supported takes
 
 void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);

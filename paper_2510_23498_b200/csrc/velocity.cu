@@ -159,6 +159,7 @@ public:
         for (int w : w_) small_w_.push_back((w + 7) / 8 * 8);
         // (the float32 buffers of the other paths are not padded: the state's rows have to agree)
         small_ok_ = !tiny_ok_ && (dt_ != MPODE_F32 || w_[0] % 8 == 0) && small_mlp_supported(dt_, B_, L_, small_w_.data());
+        small_bwd_ok_ = small_ok_ && small_backward_supported(dt_, B_);
         if (!small_ok_) return;
         const size_t es = low_size(dt_);
         size_t per_step = 0;
@@ -171,11 +172,11 @@ public:
         for (int l = 0; l < L_; ++l) small_b_[l] = lay.take((size_t)small_w_[l + 1] * es);
         small_wt_ = lay.take((size_t)small_w_[1] * es);
         small_scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
-        for (int l = 0; l < L_; ++l) {
+        for (int l = 0; l < L_ && small_bwd_ok_; ++l) {
             small_xs_[l] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
             small_zs_[l + 1] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
         }
-        if (lay.time_gradient) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
+        if (lay.time_gradient && small_bwd_ok_) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
     }
     SmallMlp small_params(void* ws) const {
         SmallMlp p{};
@@ -469,7 +470,7 @@ public:
     // ---- fused backward: per step one launch that recomputes the stages (keeping every layer output) and one launch
     // per attempt for the vector-Jacobian products and weight gradients.  begin() builds both phase tables.
     bool fused_backward_begin(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
-        b_small_ = small_usable(fs);
+        b_small_ = small_bwd_ok_ && small_usable(fs);
         if (b_small_) {
             small_bwd_ = small_solve(st, ws, fs);
             b_stages_ = fs.stages;
@@ -778,7 +779,7 @@ protected:
     size_t f_scalars_ = 0, f_phases_[3] = {0, 0, 0}, f_cnt_ = 0, kappaslab_ = 0;
     size_t tiny_scal_ = 0, tiny_log_ = 0;
     bool tiny_ok_ = false;
-    bool small_ok_ = false, b_small_ = false, quantized_ = false;
+    bool small_ok_ = false, small_bwd_ok_ = false, b_small_ = false, quantized_ = false;
     int small_chunk_ = 1;
     size_t small_pack_ = 0, small_scal_ = 0, small_xs_[SMALL_MAX_L] = {0}, small_zs_[SMALL_MAX_L + 1] = {0};
     SmallMlp small_bwd_{}, small_step_{};
