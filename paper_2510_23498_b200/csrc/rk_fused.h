@@ -45,7 +45,6 @@ struct RkPhase {
     // RK_EPI_WGRAD only
     int tiles_m, splits, kb_per_split;          // output tiles along M, batch slices, k-blocks per slice
     int accumulate;            // 1: add to the partial sums already there (a later stage of the same step)
-    int pack2;                 // 1: 64-column items whose ring stages hold two k-blocks each (the ones-products)
     long long part_off;        // element offset of this phase's [splits][M][N] partial sums in the fp32 scratch
     int M;                     // output rows (wgrad); batch rows otherwise come from RkParams::B
 };

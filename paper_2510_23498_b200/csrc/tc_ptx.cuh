@@ -43,6 +43,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// has the phase completed (never suspends)?
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0u;
+}
 // Bounded wait: gives up after `limit_ns`, records `code` in *err and returns false.
 static __device__ __noinline__ bool mbar_wait_long(uint64_t* bar, uint32_t parity, unsigned* err, unsigned code, unsigned long long limit_ns) {
     unsigned long long t0 = globaltimer_ns();

@@ -580,7 +580,7 @@ public:
                         b.b_map = m_ones; b.b_slot = 0;
                         b.N = kOnesKeep; b.bn = 64; b.tiles_n = 1;
                         b.part_off = (long long)(wg_part_elems_) + col_off_[j][l + 1];
-                        b.accumulate = 0; b.dep_phase = -1; b.pack2 = 1;
+                        b.accumulate = 0; b.dep_phase = -1;
                         wg_items += b.tiles_m * b.splits;
                         ph.push_back(b);
                     }
