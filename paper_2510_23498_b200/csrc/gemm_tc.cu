@@ -24,6 +24,13 @@ namespace mpode {
 using namespace tc;
 namespace {
 
+// 32 bytes, 32-byte aligned
+__device__ __forceinline__ void st_v8(float* dst, const uint32_t* r) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
+                 "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+
 // Widest tiles (BN = 256): one CTA per SM, eight epilogue warps (two per TMEM lane quadrant, each half of the columns).
 // Narrower tiles (BN <= 128: the convolutions, thin layers): half the shared memory, four epilogue warps and a small register
 // footprint, so that two CTAs share an SM and one's loads and epilogue hide behind the other's MMAs.
@@ -295,9 +302,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (row_ok && nb < p.N) {
                         float* prow = p.partial + ((long long)z * p.M + m) * p.N + nb;
 #pragma unroll
-                        for (int v = 0; v < 8; ++v)
-                            if (nb + v * 4 < p.N)   // N is a multiple of 8
-                                *reinterpret_cast<uint4*>(prow + v * 4) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+                        for (int v = 0; v < 4; ++v)
+                            if (nb + v * 8 < p.N)   // N is a multiple of 8; whole sectors (a lane holds a row: an instruction touches 32 lines)
+                                st_v8(prow + v * 8, r + 8 * v);
                     }
                 } else if (pair) {
                     // The warp that produces what its partner needs writes one of two sets of exchange rows and the two meet at
