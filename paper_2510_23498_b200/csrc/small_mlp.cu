@@ -7,7 +7,7 @@
 // float32 runs the same program on the CUDA cores, 8 rows to a block, bound by the weights' way from L2 (about 64 bytes a cycle).
 // Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
 // second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
-// Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.9 ms; MLP
+// Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.75 ms; MLP
 // 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.5 ms.
 #include "small_mlp.h"
 
