@@ -120,3 +120,11 @@ def test_conv_block_next_stage_input_per_solver(solver):
 def test_conv_block_tile_buffers(batch, H, W):
     wl = inputs.conv_block(batch=batch, n_steps=1, H=H, W=W, C=64, act="softplus", solver="heun")
     assert_parity(run_gpu(wl, "bf16", "none"), run_oracle(wl, "bf16", "none"), TOL["bf16"])
+
+
+# column sums (bias and time-column gradients of the flow): batches of one row chunk, of chunks that end early, the largest that the
+# cluster kernel takes and the next that it does not
+@pytest.mark.parametrize("batch", [3, 130, 2048, 2112])
+def test_flow_column_sums_at_chunk_edges(batch):
+    wl = inputs.cnf_mlp(batch=batch, n_steps=1, d=16, hidden=72)
+    assert_parity(run_gpu(wl, low="bf16"), run_oracle(wl, low="bf16"), TOL["bf16"])
