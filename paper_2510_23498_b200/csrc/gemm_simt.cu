@@ -32,7 +32,8 @@ __device__ __forceinline__ float load_operand(const T* __restrict__ p, long long
     return Low<T>::to_f(p[((long long)pixel + (long long)dy * W + dx) * Cd + c]);
 }
 
-// The layer epilogue of one output element; returns whether the rounded value of an input gradient is not finite.
+// The layer epilogue of one output element; returns whether the rounded value of an input gradient (with a flag: of a weight gradient)
+// is not finite.
 template <typename T>
 __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, float v) {
     if (g.epi == EPI_FWD) {
@@ -51,6 +52,7 @@ __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, 
     } else if (g.epi == EPI_WGRAD) {
         float* o = (float*)g.out + (long long)m * g.ldo + n;
         *o = fmaf(g.alpha != 0.f ? g.alpha : 1.f, v, g.beta != 0.f ? *o : 0.f);
+        return g.flag != nullptr && Low<T>::nonfinite(Low<T>::from_f(v));
     } else {
         ((float*)g.out)[(long long)m * g.ldo + n] = v;
     }
@@ -244,15 +246,20 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     }
 
     const float alpha = g.alpha != 0.f ? g.alpha : 1.f;
+    bool bad = false;
     auto put_row_sum = [&](int m, float s, float st) {
-        if (g.row_sum != nullptr) g.row_sum[m] = fmaf(alpha, s, g.beta != 0.f ? g.row_sum[m] : 0.f);
+        if (g.row_sum != nullptr) {
+            g.row_sum[m] = fmaf(alpha, s, g.beta != 0.f ? g.row_sum[m] : 0.f);
+            bad |= Low<T>::nonfinite(Low<T>::from_f(s));
+        }
         if (g.row_sum_time != nullptr) {
             float* o = g.row_sum_time + (long long)m * g.ldo;
-            *o = fmaf(alpha, g.k_tau != nullptr ? st : g.tau * s, g.beta != 0.f ? *o : 0.f);
+            const float v = g.k_tau != nullptr ? st : g.tau * s;
+            *o = fmaf(alpha, v, g.beta != 0.f ? *o : 0.f);
+            bad |= Low<T>::nonfinite(Low<T>::from_f(v));
         }
         if (g.row_sum_raw != nullptr) g.row_sum_raw[m] = s;
     };
-    bool bad = false;
     const int S = (int)gridDim.z;
     if (S == 1) {
 #pragma unroll
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
         }
         cl.sync();      // no block leaves while another reads its shared memory
     }
-    if (g.epi == EPI_DGRAD) warp_flag_or(g.flag, bad);
+    if (g.epi == EPI_DGRAD || g.epi == EPI_WGRAD) warp_flag_or(g.flag, bad);
 }
 
 // Blocks of a cluster share a reduction of at least 64: as many (up to 8) as it takes to give every SM a block.

@@ -744,9 +744,12 @@ __global__ void __launch_bounds__(96) small_time_kernel(SmallMlp p, int blocks) 
 // of stages * B rows; warp w takes the groups of 16 rows w, w + 8, ... through its own ring of asynchronous copies, so that no barrier
 // stands in the loop; the eight sums meet in shared memory in ascending order.  The bias gradient and the time column are two more
 // columns (ones, stage times) of the pieces in the first column of pieces.
+// CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of the step's gradient
+// that does not fit the format raises the flag.
 constexpr int kRing = 8;
 struct WgradItems { int first[SMALL_MAX_L + 1]; };
-template <typename T, int TM, int TN>
+template <typename T, int TM> constexpr size_t kWgradRingBytes = (size_t)kWarps * kRing * 16 * 2 * (TM + 8) * sizeof(T);
+template <typename T, int TM, int TN, bool CHECK>
 __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ WgradItems items) {
     chain_begin();
     constexpr int LA = TM + 8, LB = TN + 8;                       // row lengths in shared memory: eight rows hit eight 16-byte slots
@@ -784,6 +787,36 @@ __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_cons
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     float tot[TM / 16][TN / 8][4], acc[TM / 16][TN / 8][4], stot[TM / 16][4], sacc[TM / 16][4];
+    constexpr int LR = TN + 3;                                    // row of sums: TN columns, bias, time (odd stride)
+    float* red = (float*)(smem + (CHECK ? kWgradRingBytes<T, TM> : 0));      // [warps][TM][LR]
+    auto put_sums = [&](const float (&w)[TM / 16][TN / 8][4], const float (&ws)[TM / 16][4]) {
+#pragma unroll
+        for (int m = 0; m < TM / 16; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = m * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
+                float* row = red + ((size_t)warp * TM + r) * LR;
+#pragma unroll
+                for (int q = 0; q < TN / 8; ++q) row[q * 8 + c] = w[m][q][i];
+                if (c < 2) row[TN + c] = ws[m][i];
+            }
+    };
+    // the parameter that entry (r, c) of the piece belongs to, or -1; and the warps' sum
+    const int in_full = p.wr[l] + (time ? 1 : 0);
+    auto param_of = [&](int r, int c) -> long long {
+        const int m = m0 + r, n = n0 + c;
+        if (m >= p.wr[l + 1]) return -1;
+        if (c < TN) return n < p.wr[l] ? p.woff[l] + (long long)m * in_full + n : -1;
+        if (c == TN) return sums && p.bias ? p.boff[l] + m : -1;
+        return sums && time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1;
+    };
+    auto warps_sum = [&](int r, int c) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) v += red[((size_t)w * TM + r) * LR + c];
+        return v;
+    };
+    bool bad = false;
 #pragma unroll
     for (int m = 0; m < TM / 16; ++m)
 #pragma unroll
@@ -832,6 +865,15 @@ __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_cons
         fetch(it + kRing - 1);
         if (gi == per - 1) {      // the step is complete
             const float cf = p.coef[s];
+            if (CHECK) {
+                put_sums(acc, sacc);
+                __syncthreads();
+                for (int i = threadIdx.x; i < TM * (TN + 2); i += kThreads) {
+                    const int r = i / (TN + 2), c = i - r * (TN + 2);
+                    if (param_of(r, c) >= 0) bad |= Low<T>::nonfinite(Low<T>::from_f(warps_sum(r, c)));
+                }
+                __syncthreads();
+            }
 #pragma unroll
             for (int m = 0; m < TM / 16; ++m)
 #pragma unroll
@@ -844,39 +886,14 @@ __global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_cons
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    constexpr int LR = TN + 3;                                    // row of sums: TN columns, bias, time (odd stride)
-    float* red = (float*)smem;                                    // [warps][TM][LR]
-#pragma unroll
-    for (int m = 0; m < TM / 16; ++m)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = m * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
-            float* row = red + ((size_t)warp * TM + r) * LR;
-#pragma unroll
-            for (int q = 0; q < TN / 8; ++q) row[q * 8 + c] = tot[m][q][i];
-            if (c < 2) row[TN + c] = stot[m][i];
-        }
+    put_sums(tot, stot);
     __syncthreads();
-    const int in_full = p.wr[l] + (time ? 1 : 0);
     for (int i = threadIdx.x; i < TM * (TN + 2); i += kThreads) {
-        const int r = i / (TN + 2), c = i - r * (TN + 2), m = m0 + r, n = n0 + c;
-        if (m >= p.wr[l + 1]) continue;
-        long long at;
-        if (c < TN) {
-            if (n >= p.wr[l]) continue;
-            at = p.woff[l] + (long long)m * in_full + n;
-        } else if (c == TN) {
-            if (!sums || !p.bias) continue;
-            at = p.boff[l] + m;
-        } else {
-            if (!sums || !time) continue;
-            at = p.woff[l] + (long long)m * in_full + p.wr[l];
-        }
-        float v = 0.f;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) v += red[((size_t)w * TM + r) * LR + c];
-        p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + v;
+        const int r = i / (TN + 2), c = i - r * (TN + 2);
+        const long long at = param_of(r, c);
+        if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + warps_sum(r, c);
     }
+    if (CHECK) warp_flag_or(p.flag, bad);
 }
 
 constexpr int kSmemCap = 220 * 1024;
@@ -925,13 +942,18 @@ bool backward_t(const SmallMlp& p, cudaStream_t st) {
     launch_chain(small_backward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
-template <typename T, int TM>
+template <typename T, int TM, bool CHECK>
 bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st) {
     static bool done[kMaxDevices] = {false};
-    if (!allow_smem(small_wgrad_kernel<T, TM, TM>, done)) return false;
-    const size_t ring = (size_t)kWarps * kRing * 16 * 2 * (TM + 8) * sizeof(T), red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
-    launch_chain(small_wgrad_kernel<T, TM, TM>, dim3(items.first[p.L]), dim3(kThreads), ring > red ? ring : red, st, p, items);
+    if (!allow_smem(small_wgrad_kernel<T, TM, TM, CHECK>, done)) return false;
+    const size_t ring = kWgradRingBytes<T, TM>, red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
+    launch_chain(small_wgrad_kernel<T, TM, TM, CHECK>, dim3(items.first[p.L]), dim3(kThreads), CHECK ? ring + red : (ring > red ? ring : red), st, p, items);
     return true;
+}
+template <typename T>
+bool wgrad_t(const SmallMlp& p, const WgradItems& items, bool wide, cudaStream_t st) {
+    if (p.flag != nullptr) return wide ? wgrad_t<T, 32, true>(p, items, st) : wgrad_t<T, 16, true>(p, items, st);
+    return wide ? wgrad_t<T, 32, false>(p, items, st) : wgrad_t<T, 16, false>(p, items, st);
 }
 WgradItems wgrad_items(const SmallMlp& p, int tm) {
     WgradItems it{};
@@ -1025,7 +1047,7 @@ static bool small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launc
             g.B = (const float*)p.xs[l] + s * rows * p.wp[l]; g.b_rs = 1; g.b_ks = p.wp[l];
             g.M = p.wr[l + 1]; g.N = p.wr[l]; g.K = (int)rows;
             g.epi = EPI_WGRAD; g.out = p.out + p.woff[l]; g.ldo = p.wr[l] + (time ? 1 : 0); g.beta = s == 0 ? p.beta : 1.f; g.alpha = p.coef[s];
-            g.split_k = 1;
+            g.split_k = 1; g.flag = p.flag;
             g.row_sum = p.bias ? p.out + p.boff[l] : nullptr;
             if (time) { g.row_sum_time = p.out + p.woff[l] + p.wr[l]; g.k_tau = p.scal[0].tau16 + (size_t)(p.step_hi - s) * (sizeof(RkStepScalars) / 4); g.k_per = p.B; }
             if (!launch_gemm_simt(MPODE_F32, g, st, launches)) return false;
@@ -1041,8 +1063,7 @@ bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long
     WgradItems items = wgrad_items(p, 32);
     const bool wide = items.first[p.L] >= sm_count() / 2;
     if (!wide) items = wgrad_items(p, 16);
-    const bool ok = dt == MPODE_BF16 ? (wide ? wgrad_t<__nv_bfloat16, 32>(p, items, st) : wgrad_t<__nv_bfloat16, 16>(p, items, st))
-                                     : (wide ? wgrad_t<__half, 32>(p, items, st) : wgrad_t<__half, 16>(p, items, st));
+    const bool ok = dt == MPODE_BF16 ? wgrad_t<__nv_bfloat16>(p, items, wide, st) : wgrad_t<__half>(p, items, wide, st);
     if (ok && launches) ++*launches;
     if (ok && tl_counters) ++tl_counters->fused;
     return ok;

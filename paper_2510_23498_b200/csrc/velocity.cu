@@ -691,8 +691,9 @@ public:
             p.step_hi = step; p.count = 1; p.vjp = 1; p.flag = flag;
             if (lay_->time_gradient) { p.recompute = 1; p.tpart = (float*)at(ws, small_tpart_); }
             small_step_ = p;
-            p.out = out; p.beta = beta; p.coef[0] = coef;
-            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, p, st, L); });
+            SmallMlp w = p;
+            w.out = out; w.beta = beta; w.coef[0] = coef; w.flag = nullptr;      // (the driver tests the step's gradient)
+            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, w, st, L); });
             if (after_kernel != nullptr) cudaEventRecord(after_kernel, st);
             if (st_finish != nullptr && after_kernel != nullptr) cudaStreamWaitEvent(st_finish, after_kernel, 0);
             return;

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2510_23498_b200 import inputs
-from _harness import TOL, assert_parity, assert_same_log, run_gpu, run_oracle
+from _harness import TOL, assert_parity, assert_same_log, rel_l2, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -91,6 +91,32 @@ def test_small_float32_networks_at_tile_edges(batch, widths, n_steps):
     gpu = run_gpu(wl, low="f32")
     assert_parity(gpu, run_oracle(wl, exact=True), TOL["f32"])
     assert gpu["stats"]["fused_launches"] > 0
+
+
+# unscaled-safe passes of small dense networks: the step's parameter gradient alone leaves the format (its sums run over the batch; the
+# cotangents and the adjoint stay finite), on both sizes of gradient pieces, in one chunk of steps and across chunks, in all formats
+@pytest.mark.parametrize("low,batch,widths,n_steps,size", [("f16", 1000, [64, 128, 64], 2, 100.0), ("f16", 1000, [64, 64], 20, 200.0), ("f16", 700, [72, 200, 200, 72], 2, 300.0),
+                                                           ("bf16", 1000, [64, 128, 64], 2, 5e36), ("f32", 1000, [64, 128, 64], 2, 5e36)])
+def test_small_networks_report_a_parameter_gradient_that_overflows(low, batch, widths, n_steps, size):
+    from oracle import BY_NAME, Policy, make_velocity, odeint_backward, odeint_forward
+    wl = inputs.mlp_block(batch=batch, n_steps=n_steps, d=widths[0], hidden=widths[1])
+    wl.vel["n_layers"], wl.vel["widths"], wl.theta = len(widths) - 1, widths, inputs.mlp_theta(3, widths, True)
+    dl = np.full((batch, widths[0]), size)
+    gpu = run_gpu(wl, low, "none_safe", dLdyT=dl)
+    assert gpu["stats"]["fused_launches"] > 0                                     # the row-local kernels
+    assert gpu["status"] == 8 and np.all(np.isposinf(gpu["g"])) and np.all(np.isposinf(gpu["a0"]))
+    vel, pol = make_velocity(wl.vel), Policy(low=low, scaling="none_safe")
+    traj, _ = odeint_forward(vel, wl.theta, wl.y0, wl.tgrid, BY_NAME["rk4"], pol)
+    _, _, log = odeint_backward(vel, wl.theta, traj, wl.tgrid, BY_NAME["rk4"], pol, dl)
+    assert log.overflowed
+    # the cotangents alone are finite: without the batch sum (one row) nothing overflows, on either side
+    one = inputs.mlp_block(batch=1, n_steps=n_steps, d=widths[0], hidden=widths[1])
+    one.vel, one.theta, one.y0 = wl.vel, wl.theta, wl.y0[:1]
+    gpu = run_gpu(one, low, "none_safe", dLdyT=dl[:1])
+    _, g, log = odeint_backward(vel, wl.theta, traj[:, :1], wl.tgrid, BY_NAME["rk4"], pol, dl[:1])
+    assert gpu["status"] == 0 and not log.overflowed
+    if low != "f32":
+        assert rel_l2(gpu["g"], g) <= TOL[low]
 
 
 # paired (value, tangent) tiles of 64 columns: one tile of 64 sample pairs, several, output columns that end inside a tile, on its edge and
