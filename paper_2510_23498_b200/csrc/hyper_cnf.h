@@ -43,6 +43,7 @@ struct HyperSolve {
     float* a_new;                       // [B][d + 1] the adjoint the attempt would leave
     unsigned* words;                    // 16 device words, zero at launch
     unsigned long long wait_ns;         // limit of a grid barrier
+    int starve;                         // test of that limit: the last block's last barrier waits for one arrival too many
     int *log_exp, *log_attempts, *log_doubled, *status;     // device [n_steps] each; status [4], zero at launch
 };
 bool hyper_solve_shape_ok(mpode_dtype dt, int h, int w, int d, int stages);

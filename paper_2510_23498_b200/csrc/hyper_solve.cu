@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(256) hyper_solve_forward_kernel(HyperSolve p) 
 
 // ---------------------------------------------------------------- grid barrier (cooperative launch), in two halves
 // Everything the block wrote before arrive() is visible to every block that has passed wait().  Bounded: a wait that gives up raises
-// the error word and returns false, and so does every later one.
+// the error word and returns false, and so does every later one.  Its block leaves without committing; the others may have passed (it had
+// arrived), so it is the error word that says whether the pass is good.
 __device__ __forceinline__ void grid_arrive(unsigned* counter) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -575,7 +576,8 @@ __global__ void __launch_bounds__(512) hyper_solve_backward_kernel(HyperSolve p)
             }
             grid_arrive(counter);
             ++arrived;
-            alive = grid_wait(counter, arrived * G, err, p.wait_ns) && alive;
+            const unsigned extra = p.starve && n == 0 && (int)blockIdx.x == G - 1 ? 1u : 0u;      // test: an arrival that never comes
+            alive = grid_wait(counter, arrived * G + extra, err, p.wait_ns) && alive;
             if (!alive) {
                 if (blockIdx.x == 0 && threadIdx.x == 0) p.status[0] = MPODE_ERR_CUDA;
                 return;

@@ -1411,15 +1411,17 @@ public:
         int* logs = (int*)at(ws, log_);
         p.log_exp = logs; p.log_attempts = logs + N; p.log_doubled = logs + 2 * N; p.status = logs + 3 * N; p.words = (unsigned*)(logs + 3 * N + 4);
         p.wait_ns = fs.wait_ns;
-        const size_t ints = (size_t)3 * N + 4;
-        cudaMemsetAsync(logs, 0, (ints + 16) * sizeof(int), st);
+        p.starve = fs.starve;
+        const size_t ints = (size_t)3 * N + 6;          // scale log, status [4], barrier counter, error word of the bounded waits
+        cudaMemsetAsync(logs, 0, ((size_t)3 * N + 4 + 16) * sizeof(int), st);
         if (!launch_hyper_solve_backward(dt_, p, st, L)) return false;
         if (tl_counters) ++tl_counters->whole;
         std::vector<int> hl(ints);
         cudaMemcpyAsync(hl.data(), logs, ints * sizeof(int), cudaMemcpyDeviceToHost, st);
         cudaStreamSynchronize(st);
         const int* stp = hl.data() + 3 * N;
-        wb.status = stp[0]; wb.first_failed_step = wb.status == MPODE_ERR_SCALE_FAILED ? stp[1] : -1; wb.retries = stp[2];
+        wb.status = stp[5] != 0 ? (int)MPODE_ERR_CUDA : stp[0];      // (a block that gave up may have been behind the one that writes stp[0])
+        wb.first_failed_step = wb.status == MPODE_ERR_SCALE_FAILED ? stp[1] : -1; wb.retries = stp[2];
         for (int i = 0; i < N; ++i) {
             if (wb.exp_used) wb.exp_used[i] = hl[i];
             if (wb.attempts) wb.attempts[i] = hl[N + i];

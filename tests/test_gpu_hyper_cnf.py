@@ -76,3 +76,26 @@ def test_hyper_cnf_full_size():
     assert gpu["status"] == 0
     assert_parity(gpu, orc, TOL[wl.low])
     assert_same_log(gpu["log"], orc["log"])
+
+
+def test_hyper_cnf_a_grid_barrier_that_gives_up_in_any_block_is_reported():
+    # The cooperative backward kernel's barriers never wait without a limit (set to 20 ms here).  The last block's last barrier waits for
+    # an arrival that never comes, while every other block passes it and finishes: the pass lacks that block's updates and must not be
+    # reported as good.  Nothing faults or hangs; afterwards the same context gives the usual result.
+    import torch
+    from paper_2510_23498_b200 import binding
+    wl = inputs.hyper_cnf(batch=300, n_steps=3, hidden=16, w=40)
+    ref = run_gpu(wl)
+    ctx = binding.Context(wl.vel, wl.batch, wl.n_steps, low=wl.low, scaling=wl.scaling)
+    theta, y0 = torch.from_numpy(wl.theta).to(ctx.device), torch.from_numpy(wl.y0).to(ctx.device)
+    dl = torch.from_numpy(np.ascontiguousarray(ref["dLdyT"], dtype=np.float32)).to(ctx.device)
+    ctx.forward(theta, y0, wl.tgrid, wl.solver)
+    ctx.debug_waits(20_000_000, True)
+    with pytest.raises(binding.MpodeError) as ei:
+        ctx.backward(dl)
+    assert ei.value.status == binding.ERR_CUDA and "wait timed out" in str(ei.value)
+    ctx.debug_waits(0, False)
+    ctx.forward(theta, y0, wl.tgrid, wl.solver)
+    a0, g, _, st = ctx.backward(dl)
+    assert st == 0 and np.array_equal(a0.cpu().numpy(), ref["a0"]) and np.array_equal(g.cpu().numpy(), ref["g"])
+    ctx.close()
