@@ -368,11 +368,13 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
     long long* L = &c->stats.kernel_launches;
 
     cudaMemsetAsync(at(ws, c->lay.scal), 0, 256, st);
-    {   // very small velocities: the whole loop in one launch of one CTA
+    {   // very small networks and hypernetwork flows: the whole loop in one launch
         FusedSolve whole = fused_solve(c, yT_dev);
-        if (c->v->whole_forward(st, ws, whole, theta_dev, y0_dev, yT_dev, L)) {
+        const Whole w = c->v->whole_forward(st, ws, whole, theta_dev, y0_dev, yT_dev, L);
+        if (w != Whole::kNo) {
             mpode_status ws_ = check_cuda(c, "mpode_forward");
             if (ws_ != MPODE_OK) return ws_;
+            if (w == Whole::kRefused) return fail(c, MPODE_ERR_CUDA, "mpode_forward: the whole-solve kernel could not be launched");
             c->have_forward = true;
             return MPODE_OK;
         }
@@ -442,7 +444,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     c->stats.host_syncs = 0;
     c->stats.step_waits = 0;
 
-    {   // very small velocities: Alg. 2 with its scale decisions in one launch of one CTA
+    {   // very small networks and hypernetwork flows: Alg. 2 with its scale decisions in one launch
         WholeBackward wb;
         wb.theta = c->theta; wb.dLdyT = dL_dyT_dev; wb.a = a; wb.g = g; wb.accumulate = accumulate_dtheta;
         wb.scaling = (int)c->pol.scaling; wb.k_max = c->pol.k_max; wb.growth_rule = c->pol.growth_rule; wb.pbits = precision_bits(dt);
@@ -455,11 +457,13 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         if (log) { wb.exp_used = log->exp_used; wb.attempts = log->attempts; wb.doubled = log->doubled; }
         wb.cot = cot; wb.dt_host = dt_host;
         FusedSolve whole = fused_solve(c, nullptr);
-        if (c->v->whole_backward(st, ws, whole, wb, L)) {
-            ++c->stats.host_syncs;
+        const Whole w = c->v->whole_backward(st, ws, whole, wb, L);
+        if (w != Whole::kNo) {
+            if (w == Whole::kDone) ++c->stats.host_syncs;
             c->stats.retries = wb.retries;
             mpode_status cs = check_cuda(c, "mpode_backward");
             if (cs != MPODE_OK) return cs;
+            if (w == Whole::kRefused) return fail(c, MPODE_ERR_CUDA, "mpode_backward: the whole-solve kernel could not be launched");
             if (wb.status == MPODE_ERR_CUDA) return fail(c, MPODE_ERR_CUDA, "a device-side wait timed out");
             if (wb.status == MPODE_ERR_NONFINITE_INPUT) return fail(c, MPODE_ERR_NONFINITE_INPUT, "dL/dy_T is not finite");
             if (wb.status == MPODE_ERR_SCALE_FAILED) {

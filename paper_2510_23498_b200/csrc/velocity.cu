@@ -341,18 +341,18 @@ public:
         t.round_increment = fs.round_increment;
         return t;
     }
-    bool whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
+    Whole whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
                        long long* L) override {
-        if (!tiny_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
+        if (!tiny_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return Whole::kNo;
         cudaMemcpyAsync(at(ws, tiny_scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         TinyParams t = tiny_params(ws, fs, theta);
         t.y0 = y0; t.yT = yT;
-        if (!launch_tiny_forward(dt_, t, st, L)) return false;
+        if (!launch_tiny_forward(dt_, t, st, L)) return Whole::kNo;
         if (tl_counters) ++tl_counters->whole;
-        return true;
+        return Whole::kDone;
     }
-    bool whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
-        if (!tiny_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
+    Whole whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
+        if (!tiny_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return Whole::kNo;
         const int N = fs.n_steps;
         cudaMemcpyAsync(at(ws, tiny_scal_), fs.scalars.data(), (size_t)N * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         int* logs = (int*)at(ws, tiny_log_);
@@ -364,7 +364,7 @@ public:
         t.log_exp = logs; t.log_attempts = logs + max_steps_; t.log_doubled = logs + 2 * max_steps_; t.status = logs + 3 * max_steps_;
         t.cot = wb.cot;
         t.tprime = wb.dt_host != nullptr ? (float*)(logs + 3 * max_steps_ + 4) : nullptr;
-        if (!launch_tiny_backward(dt_, t, st, L)) return false;
+        if (!launch_tiny_backward(dt_, t, st, L)) return Whole::kNo;
         if (tl_counters) ++tl_counters->whole;
         std::vector<int> h((size_t)3 * max_steps_ + 4);
         cudaMemcpyAsync(h.data(), logs, h.size() * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -377,7 +377,7 @@ public:
             if (wb.attempts) wb.attempts[i] = h[max_steps_ + i];
             if (wb.doubled) wb.doubled[i] = (unsigned char)h[2 * max_steps_ + i];
         }
-        return true;
+        return Whole::kDone;
     }
 
     // ---- fused Runge-Kutta path (16-bit formats, state width a multiple of 8; hidden widths are padded to one)
@@ -1305,16 +1305,16 @@ public:
         t.round_increment = fs.round_increment;
         return t;
     }
-    bool whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
+    Whole whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
                        long long* L) override {
         cudaMemcpyAsync(at(ws, scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         TinyParams t = params(ws, fs, theta);
         t.y0 = y0; t.yT = yT;
-        launch_tiny_forward(dt_, t, st, L);
+        if (!launch_tiny_forward(dt_, t, st, L)) return Whole::kRefused;
         if (tl_counters) ++tl_counters->whole;
-        return true;
+        return Whole::kDone;
     }
-    bool whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
+    Whole whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
         const int N = fs.n_steps;
         cudaMemcpyAsync(at(ws, scal_), fs.scalars.data(), (size_t)N * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         int* logs = (int*)at(ws, log_);
@@ -1326,7 +1326,7 @@ public:
         t.log_exp = logs; t.log_attempts = logs + max_steps_; t.log_doubled = logs + 2 * max_steps_; t.status = logs + 3 * max_steps_;
         t.cot = wb.cot;
         t.tprime = wb.dt_host != nullptr ? (float*)(logs + 3 * max_steps_ + 4) : nullptr;
-        launch_tiny_backward(dt_, t, st, L);
+        if (!launch_tiny_backward(dt_, t, st, L)) return Whole::kRefused;
         if (tl_counters) ++tl_counters->whole;
         std::vector<int> h((size_t)3 * max_steps_ + 4);
         cudaMemcpyAsync(h.data(), logs, h.size() * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1339,7 +1339,7 @@ public:
             if (wb.attempts) wb.attempts[i] = h[max_steps_ + i];
             if (wb.doubled) wb.doubled[i] = (unsigned char)h[2 * max_steps_ + i];
         }
-        return true;
+        return Whole::kDone;
     }
     void bind(const Layout* lay) { lay_ = lay; }
 
@@ -1391,17 +1391,17 @@ public:
         launch_hyper_table(dt_, theta, p.scal, fs.n_steps, fs.stages, h_, w_, d_, (float*)at(ws, table_), st, L);
         return p;
     }
-    bool whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
+    Whole whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
                        long long* L) override {
-        if (!whole_ || fs.n_steps > max_steps_) return false;
+        if (!whole_) return Whole::kNo;
         HyperSolve p = solve_params(st, ws, fs, theta, L);
         p.y0 = y0; p.yT = yT;
-        if (!launch_hyper_solve_forward(dt_, p, st, L)) return false;
+        if (!launch_hyper_solve_forward(dt_, p, st, L)) return Whole::kRefused;
         if (tl_counters) ++tl_counters->whole;
-        return true;
+        return Whole::kDone;
     }
-    bool whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
-        if (!whole_ || fs.n_steps > max_steps_) return false;
+    Whole whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) override {
+        if (!whole_) return Whole::kNo;
         const int N = fs.n_steps;
         HyperSolve p = solve_params(st, ws, fs, wb.theta, L);
         p.dLdyT = wb.dLdyT; p.a = wb.a; p.g = wb.g; p.accumulate = wb.accumulate; p.cot = wb.cot;
@@ -1414,7 +1414,7 @@ public:
         p.starve = fs.starve;
         const size_t ints = (size_t)3 * N + 6;          // scale log, status [4], barrier counter, error word of the bounded waits
         cudaMemsetAsync(logs, 0, ((size_t)3 * N + 4 + 16) * sizeof(int), st);
-        if (!launch_hyper_solve_backward(dt_, p, st, L)) return false;
+        if (!launch_hyper_solve_backward(dt_, p, st, L)) return Whole::kRefused;
         if (tl_counters) ++tl_counters->whole;
         std::vector<int> hl(ints);
         cudaMemcpyAsync(hl.data(), logs, ints * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1427,7 +1427,7 @@ public:
             if (wb.attempts) wb.attempts[i] = hl[N + i];
             if (wb.doubled) wb.doubled[i] = (unsigned char)hl[2 * N + i];
         }
-        return true;
+        return Whole::kDone;
     }
     void forward(cudaStream_t st, void* ws, int j, const void* yin, float tau16, long long* L) override {
         launch_hyper_forward(dt_, theta_, tau16, h_, w_, d_, (float*)at(ws, hyp_[j]), yin, at(ws, units_[j]), at(ws, lay_->kbuf[j]),

@@ -60,6 +60,10 @@ struct Layout {
     }
 };
 
+// What became of a whole-solve launch: the velocity has none for this pass, it ran, or the runtime refused it and the workspace holds nothing
+// that another path could run in (the call has to fail)
+enum class Whole { kNo, kDone, kRefused };
+
 // kappa_{j-1} = Q16(bv * v + c * psi_j): the previous stage's cotangent when the tableau couples it to stage j alone
 struct KappaNext { void* out = nullptr; const void* v = nullptr; float bv = 0.f, c = 0.f; };
 
@@ -94,10 +98,10 @@ public:
     // velocity / format / shape, the caller then runs the layer-by-layer path.
     virtual bool fused_forward(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) { return false; }
     // Velocities with whole-solve kernels: the whole forward pass (Alg. 1) or backward pass (Alg. 2, including the scale decisions) in one
-    // launch; false = not available.  whole_backward synchronises the stream to read back the status and the scale log.
-    virtual bool whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
-                               long long* L) { return false; }
-    virtual bool whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) { return false; }
+    // launch.  whole_backward synchronises the stream to read back the status and the scale log.
+    virtual Whole whole_forward(cudaStream_t st, void* ws, const FusedSolve& fs, const float* theta, const float* y0, float* yT,
+                                long long* L) { return Whole::kNo; }
+    virtual Whole whole_backward(cudaStream_t st, void* ws, const FusedSolve& fs, WholeBackward& wb, long long* L) { return Whole::kNo; }
     // Fused backward: begin() prepares the phase tables of one solve (false = not available); then per step one
     // recompute launch (keeps every layer output of every stage) and, per attempt, one launch for all stage
     // vector-Jacobian products and weight gradients.  fused_vjp reads the seed from the layout's v buffer, writes

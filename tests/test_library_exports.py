@@ -61,6 +61,31 @@ def test_host_only_calls_work_without_a_device():
     assert lib.mpode_create(C.byref(h), C.byref(bad), 8, 4, C.byref(pol)) == 1
 
 
+def test_a_refused_whole_solve_launch_fails_the_call_and_nothing_else_runs():
+    # The hypernetwork flow plans its workspace for the whole-solve kernels alone: where the runtime refuses their launch (here every
+    # launch, there is no device) the call fails with a status, and no kernel of another path is queued, for which no buffers exist.
+    # Without a device no address is followed, so made-up ones do.
+    import ctypes as C
+    import pytest
+    import torch
+    from paper_2510_23498_b200 import binding
+    if torch.cuda.is_available():
+        pytest.skip("needs a machine whose launches are refused")
+    lib = binding.load_library()
+    widths = (C.c_int * 2)(16, 32)
+    desc = binding.VelocityDesc(binding.KINDS["cnf_hyper"], 2, 1, C.cast(widths, C.POINTER(C.c_int)), 0, 0, 0, 0, 0, 0, 0, 0)
+    pol = binding.Policy(1, 0, 0, 0, 0, binding.NO_OVERRIDE)
+    h = C.c_void_p()
+    assert lib.mpode_create(C.byref(h), C.byref(desc), 100, 2, C.byref(pol)) == 0
+    t = (C.c_float * 3)(0.0, 0.5, 1.0)
+    at = [(1 << 40) + (i << 30) for i in range(5)]
+    assert lib.mpode_forward(h, None, at[0], at[1], t, 2, lib.mpode_tableau_rk4(), None, at[2], at[3], at[4], lib.mpode_workspace_bytes(h)) == binding.ERR_CUDA
+    stats = binding.Stats()
+    lib.mpode_get_stats(h, C.byref(stats))
+    assert stats.kernel_launches <= 1 and stats.whole_solve_launches <= 1          # the table of weight sets at most
+    lib.mpode_destroy(h)
+
+
 def test_cnf_workspace_has_no_float32_cotangent_scratch_where_the_epilogue_takes_the_activation_step():
     # c5 (2048 x 784, 785 -> 2048 -> 2048 -> 784): with a batch that is a multiple of 64 and widths of at least 64 the backward
     # step through an activation runs in the tensor-core epilogue, so mixed mode plans no [2 B, 2048] float32 buffer (33.5 MB);
