@@ -930,36 +930,42 @@ bool forward_t(const SmallMlp& p, cudaStream_t st) {
     launch_chain(small_forward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
+// (st null, `ready`: only makes the kernel ready for its launch)
 template <typename T, int MT>
-bool backward_t(const SmallMlp& p, cudaStream_t st) {
+bool backward_t(const SmallMlp& p, cudaStream_t st, bool ready = false) {
     static bool done[kMaxDevices] = {false};
     if (!allow_smem(small_backward_kernel<T, MT>, done)) return false;
     SmallMlp q = p;
     q.ring = ring_buffers<T>(p, kRows<T, MT>);
     if (q.ring < 2) return false;
+    if (ready) return true;
     const int rows = kRows<T, MT>, blocks = (p.B + rows - 1) / rows;
     const size_t smem = small_smem<T>(p, rows) + q.ring * (kUnitBytes + 16);
     launch_chain(small_backward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
 template <typename T, int TM, bool CHECK>
-bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st) {
+bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st, bool ready) {
     static bool done[kMaxDevices] = {false};
     if (!allow_smem(small_wgrad_kernel<T, TM, TM, CHECK>, done)) return false;
+    if (ready) return true;
     const size_t ring = kWgradRingBytes<T, TM>, red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
     launch_chain(small_wgrad_kernel<T, TM, TM, CHECK>, dim3(items.first[p.L]), dim3(kThreads), CHECK ? ring + red : (ring > red ? ring : red), st, p, items);
     return true;
 }
 template <typename T>
-bool wgrad_t(const SmallMlp& p, const WgradItems& items, bool wide, cudaStream_t st) {
-    if (p.flag != nullptr) return wide ? wgrad_t<T, 32, true>(p, items, st) : wgrad_t<T, 16, true>(p, items, st);
-    return wide ? wgrad_t<T, 32, false>(p, items, st) : wgrad_t<T, 16, false>(p, items, st);
+bool wgrad_t(const SmallMlp& p, const WgradItems& items, bool wide, bool check, cudaStream_t st, bool ready = false) {
+    if (check) return wide ? wgrad_t<T, 32, true>(p, items, st, ready) : wgrad_t<T, 16, true>(p, items, st, ready);
+    return wide ? wgrad_t<T, 32, false>(p, items, st, ready) : wgrad_t<T, 16, false>(p, items, st, ready);
 }
 WgradItems wgrad_items(const SmallMlp& p, int tm) {
     WgradItems it{};
     for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + tm - 1) / tm) * ((p.wp[l] + tm - 1) / tm);
     return it;
 }
+// 32 x 32 pieces where there are enough of them to occupy half the SMs, else 16 x 16 (each block reads its operands from L2: a smaller
+// piece reads more in total but less per block)
+bool wide_pieces(const SmallMlp& p) { return wgrad_items(p, 32).first[p.L] >= sm_count() / 2; }
 
 }  // namespace
 
@@ -1018,13 +1024,22 @@ bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, lo
     return ok;
 }
 
-bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    const bool ok = dt == MPODE_BF16 ? backward_t<__nv_bfloat16, 1>(p, st)
-                  : dt == MPODE_F16  ? backward_t<__half, 1>(p, st)
-                                     : (rows_tiles(dt, p.B) == 1 ? backward_t<float, 1>(p, st) : backward_t<float, 2>(p, st));
-    if (ok && launches) ++*launches;
-    if (ok && tl_counters) ++tl_counters->fused;
-    return ok;
+bool small_backward_ready(mpode_dtype dt, const SmallMlp& p) {
+    if (dt == MPODE_F32) return rows_tiles(dt, p.B) == 1 ? backward_t<float, 1>(p, nullptr, true) : backward_t<float, 2>(p, nullptr, true);
+    const bool wide = wide_pieces(p);
+    for (int check = 0; check < 2; ++check)
+        if (!(dt == MPODE_BF16 ? wgrad_t<__nv_bfloat16>(p, WgradItems{}, wide, check != 0, nullptr, true)
+                               : wgrad_t<__half>(p, WgradItems{}, wide, check != 0, nullptr, true))) return false;
+    return dt == MPODE_BF16 ? backward_t<__nv_bfloat16, 1>(p, nullptr, true) : backward_t<__half, 1>(p, nullptr, true);
+}
+
+void launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    if (dt == MPODE_BF16) backward_t<__nv_bfloat16, 1>(p, st);
+    else if (dt == MPODE_F16) backward_t<__half, 1>(p, st);
+    else if (rows_tiles(dt, p.B) == 1) backward_t<float, 1>(p, st);
+    else backward_t<float, 2>(p, st);
+    if (launches) ++*launches;
+    if (tl_counters) ++tl_counters->fused;
 }
 
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
@@ -1037,7 +1052,7 @@ void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long 
 
 // float32: the CUDA-core contraction per layer and step (the rows of all stages are its reduction range; it takes the bias and the time
 // column along)
-static bool small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launches) {
+static void small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launches) {
     for (int s = 0; s < p.count; ++s)
         for (int l = 0; l < p.L; ++l) {
             const bool time = p.time && l == 0;
@@ -1050,23 +1065,20 @@ static bool small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launc
             g.split_k = 1; g.flag = p.flag;
             g.row_sum = p.bias ? p.out + p.boff[l] : nullptr;
             if (time) { g.row_sum_time = p.out + p.woff[l] + p.wr[l]; g.k_tau = p.scal[0].tau16 + (size_t)(p.step_hi - s) * (sizeof(RkStepScalars) / 4); g.k_per = p.B; }
-            if (!launch_gemm_simt(MPODE_F32, g, st, launches)) return false;
+            // (the general kernel, which runs where this one cannot be launched, takes no sums along: the pass is not good)
+            if (!launch_gemm_simt(MPODE_F32, g, st, launches)) cudaMemsetAsync(p.err, 0xff, sizeof(unsigned), st);
             if (tl_counters) ++tl_counters->simt;
         }
-    return true;
 }
 
-bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    if (dt == MPODE_F32) return small_wgrad_f32(p, st, launches);
-    // 32 x 32 pieces where there are enough of them to occupy half the SMs, else 16 x 16 (each block reads its operands from L2: a
-    // smaller piece reads more in total but less per block)
-    WgradItems items = wgrad_items(p, 32);
-    const bool wide = items.first[p.L] >= sm_count() / 2;
-    if (!wide) items = wgrad_items(p, 16);
-    const bool ok = dt == MPODE_BF16 ? wgrad_t<__nv_bfloat16>(p, items, wide, st) : wgrad_t<__half>(p, items, wide, st);
-    if (ok && launches) ++*launches;
-    if (ok && tl_counters) ++tl_counters->fused;
-    return ok;
+void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    if (dt == MPODE_F32) { small_wgrad_f32(p, st, launches); return; }
+    const bool wide = wide_pieces(p);
+    const WgradItems items = wgrad_items(p, wide ? 32 : 16);
+    if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, items, wide, p.flag != nullptr, st);
+    else wgrad_t<__half>(p, items, wide, p.flag != nullptr, st);
+    if (launches) ++*launches;
+    if (tl_counters) ++tl_counters->fused;
 }
 
 }  // namespace mpode

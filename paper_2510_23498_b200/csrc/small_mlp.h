@@ -43,9 +43,12 @@ bool small_backward_supported(mpode_dtype dt, int B);       // of a network that
 
 void launch_small_pack(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
-bool launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
+// Whether the backward kernels can be launched.  Asked before the first of them: a pass that has committed steps cannot change its path
+// (a launch that the runtime refuses after that leaves its error for the driver)
+bool small_backward_ready(mpode_dtype dt, const SmallMlp& p);
+void launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 int small_blocks(mpode_dtype dt, int B);                               // blocks of the forward and backward kernels
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
-bool launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
+void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 
 }  // namespace mpode

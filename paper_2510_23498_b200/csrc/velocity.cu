@@ -473,6 +473,9 @@ public:
         b_small_ = small_bwd_ok_ && small_usable(fs);
         if (b_small_) {
             small_bwd_ = small_solve(st, ws, fs);
+            b_small_ = small_backward_ready(dt_, small_bwd_);
+        }
+        if (b_small_) {
             b_stages_ = fs.stages;
             scal_host_ = fs.scalars;
             return true;
@@ -648,7 +651,7 @@ public:
             p.count = hi + 1 < small_chunk_ ? hi + 1 : small_chunk_;
             for (int s = 0; s < p.count; ++s) p.coef[s] = ldexpf(fs.scalars[hi - s].h, -e);
             const double f = (double)p.count * fs.stages * layer_flops();
-            if (!small_timed(3, 3.0 * f, st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, p, st, L); })) return false;
+            small_timed(3, 3.0 * f, st, [&] { launch_small_backward(dt_, p, st, L); launch_small_wgrad(dt_, p, st, L); return true; });
             if (tprime != nullptr) launch_small_time(dt_, p, st, L);
         }
         return true;
@@ -659,7 +662,7 @@ public:
             if (lay_->time_gradient) return;          // the product wants the stage derivatives too: it recomputes them itself
             SmallMlp p = small_bwd_;
             p.step_hi = step; p.count = 1; p.recompute = 1;
-            small_timed(0, b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L); });
+            small_timed(0, b_stages_ * layer_flops(), st, [&] { launch_small_backward(dt_, p, st, L); return true; });
             return;
         }
         const size_t es = low_size(dt_);
@@ -693,7 +696,7 @@ public:
             small_step_ = p;
             SmallMlp w = p;
             w.out = out; w.beta = beta; w.coef[0] = coef; w.flag = nullptr;      // (the driver tests the step's gradient)
-            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { return launch_small_backward(dt_, p, st, L) && launch_small_wgrad(dt_, w, st, L); });
+            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { launch_small_backward(dt_, p, st, L); launch_small_wgrad(dt_, w, st, L); return true; });
             if (after_kernel != nullptr) cudaEventRecord(after_kernel, st);
             if (st_finish != nullptr && after_kernel != nullptr) cudaStreamWaitEvent(st_finish, after_kernel, 0);
             return;
