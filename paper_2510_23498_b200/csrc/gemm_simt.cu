@@ -330,8 +330,10 @@ bool launch_dense(const GemmArgs& g, cudaStream_t st) {
     at[1].val.clusterDim.x = 1; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = (unsigned)S;
     cfg.attrs = at;
     cfg.numAttrs = S > 1 ? 2 : 1;
-    if (kfast) return cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, true>, g, per, vec_a, vec_b) == cudaSuccess;
-    return cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, false>, g, per, vec_a, vec_b) == cudaSuccess;
+    const bool clean = cudaPeekAtLastError() == cudaSuccess;
+    const cudaError_t e = kfast ? cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, true>, g, per, vec_a, vec_b) : cudaLaunchKernelEx(&cfg, gemm_dense_kernel<T, false>, g, per, vec_a, vec_b);
+    if (e != cudaSuccess && clean) cudaGetLastError();      // the general kernel runs instead: this error is dealt with (an earlier one is not)
+    return e == cudaSuccess;
 }
 
 __global__ void splitk_reduce_kernel(const float* __restrict__ partial, int S, int M, int N, float* __restrict__ out,

@@ -557,10 +557,8 @@ bool backward_t(const TinyParams& p, cudaStream_t st) {
     const int dev = current_device();
     if (!attr[dev]) {
         if (cudaFuncSetAttribute(tiny_backward_kernel<T, UH, DM, POLY, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(tiny_backward_kernel<T, UH, DM, POLY, THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            cudaGetLastError();
+            cudaFuncSetAttribute(tiny_backward_kernel<T, UH, DM, POLY, THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return false;
-        }
         attr[dev] = true;
     }
     cudaLaunchConfig_t cfg{};

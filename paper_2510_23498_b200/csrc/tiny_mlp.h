@@ -34,7 +34,7 @@ struct TinyParams {
 };
 
 bool tiny_mlp_supported(int B, int d, int h, int n_layers, int p);
-// return false when the launch is refused (nothing has run then)
+// return false when the launch is refused: nothing has run then, and the runtime's error is still to be taken by who has another way
 bool launch_tiny_forward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
 bool launch_tiny_backward(mpode_dtype dt, const TinyParams& p, cudaStream_t st, long long* launches);
 

@@ -347,7 +347,7 @@ public:
         cudaMemcpyAsync(at(ws, tiny_scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         TinyParams t = tiny_params(ws, fs, theta);
         t.y0 = y0; t.yT = yT;
-        if (!launch_tiny_forward(dt_, t, st, L)) return Whole::kNo;
+        if (!launch_tiny_forward(dt_, t, st, L)) { cudaGetLastError(); return Whole::kNo; }      // (the other paths take over)
         if (tl_counters) ++tl_counters->whole;
         return Whole::kDone;
     }
@@ -364,7 +364,7 @@ public:
         t.log_exp = logs; t.log_attempts = logs + max_steps_; t.log_doubled = logs + 2 * max_steps_; t.status = logs + 3 * max_steps_;
         t.cot = wb.cot;
         t.tprime = wb.dt_host != nullptr ? (float*)(logs + 3 * max_steps_ + 4) : nullptr;
-        if (!launch_tiny_backward(dt_, t, st, L)) return Whole::kNo;
+        if (!launch_tiny_backward(dt_, t, st, L)) { cudaGetLastError(); return Whole::kNo; }
         if (tl_counters) ++tl_counters->whole;
         std::vector<int> h((size_t)3 * max_steps_ + 4);
         cudaMemcpyAsync(h.data(), logs, h.size() * sizeof(int), cudaMemcpyDeviceToHost, st);
