@@ -11,8 +11,10 @@ thread_local Profiler* tl_profiler = nullptr;
 thread_local PathCounters* tl_counters = nullptr;
 
 // returns which kernel ran: 0 the general CUDA-core kernel, 1 the general tensor-core kernel, 2 the 64-channel convolution kernel,
-// 3 the CUDA-core kernel of plain operands (which also took GemmArgs::row_sum)
-int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* L) {
+// 3 the CUDA-core kernel of plain operands (which also took GemmArgs::row_sum); -1: none, with `tensor_only` when no tensor-core kernel takes
+// the arguments (a convolution whose time channel sits in the bias table means something else to the CUDA-core kernel, and with a
+// slope beside the table to the general tensor-core kernel too)
+int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* L, bool tensor_only) {
     Profiler* pr = tl_profiler;
     int klass = g.epi == EPI_FWD ? 0 : (g.epi == EPI_WGRAD ? 2 : 1);
     if (pr && pr->enabled) pr->begin(klass, 2.0 * g.M * g.N * (double)g.K, st);
@@ -20,7 +22,11 @@ int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long 
     if (g.epi == EPI_WGRAD) done = wgrad_tc_eligible(dt, g) && launch_wgrad_tc(dt, g, st, L);
     else {
         done = halo = conv_halo_eligible(dt, g) && launch_conv_halo(dt, g, st, L);
-        if (!done) done = tc_eligible(dt, g) && launch_gemm_tc(dt, g, st, L);
+        if (!done) done = g.conv_tslope == nullptr && tc_eligible(dt, g) && launch_gemm_tc(dt, g, st, L);
+    }
+    if (!done && (tensor_only || g.conv_tslope != nullptr)) {
+        if (pr && pr->enabled) pr->cancel();
+        return -1;
     }
     if (tl_counters) ++(done ? tl_counters->tc : tl_counters->simt);
     if (!done) {

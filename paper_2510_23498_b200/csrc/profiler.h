@@ -25,6 +25,7 @@ struct Profiler {
         recs.push_back(r);
     }
     void end(cudaStream_t st) { cudaEventRecord(recs.back().b, st); }
+    void cancel() { pool.push_back(recs.back().a); pool.push_back(recs.back().b); recs.pop_back(); }      // nothing was launched
     // sums and clears the records; the stream must be idle
     void collect(double* ms, long long* launches, double* flops) {
         for (int k = 0; k < kClasses; ++k) { ms[k] = 0; launches[k] = 0; flops[k] = 0; }

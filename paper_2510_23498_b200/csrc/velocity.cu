@@ -12,7 +12,7 @@
 
 namespace mpode {
 
-int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* L);   // dispatch.cu: returns the kernel taken
+int launch_contraction(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long long* L, bool tensor_only = false);   // dispatch.cu: returns the kernel taken
 
 namespace {
 
@@ -1037,17 +1037,18 @@ public:
         GemmArgs g = conv_args(ws, yin, C_, 0.f, at(ws, w1d_), 9 * C_, EPI_FWD);
         g.conv_tbias = (const float*)at(ws, tb1b_); g.conv_tslope = (const float*)at(ws, tb1s_); g.tau = tau16;
         g.bias = at(ws, b1_); g.act = act_; g.out = at(ws, h1_[j]);
-        const bool halo = conv_halo_eligible(dt_, g);
-        if (!halo) { g.conv_tbias = (const float*)at(ws, tb1_[j]); g.conv_tslope = nullptr; }
-        if (halo) {
-            // the kernel puts the table together
-        } else if (tc_eligible(dt_, g)) {
+        // (the 64-channel kernel puts the table together itself)
+        bool done = conv_halo_eligible(dt_, g) && launch_contraction(dt_, g, st, L, true) >= 0;
+        g.conv_tbias = (const float*)at(ws, tb1_[j]); g.conv_tslope = nullptr;
+        if (!done && tc_eligible(dt_, g)) {
             launch_conv_class_bias(dt_, at(ws, b1_), at(ws, w1_), C_ + 1, tau16, C_, (float*)at(ws, tb1_[j]), st, L);
-        } else {
+            done = launch_contraction(dt_, g, st, L, true) >= 0;
+        }
+        if (!done) {
             g = conv_args(ws, yin, C_ + 1, tau16, at(ws, w1_), 9 * (C_ + 1), EPI_FWD);
             g.bias = at(ws, b1_); g.act = act_; g.out = at(ws, h1_[j]);
+            launch_contraction(dt_, g, st, L);
         }
-        launch_contraction(dt_, g, st, L);
         g = conv_args(ws, at(ws, h1_[j]), C_, 0.f, at(ws, w2_), 9 * C_, EPI_FWD);
         g.conv_tbias = (const float*)at(ws, tb2_);
         g.bias = at(ws, b2_); g.act = MPODE_ACT_NONE; g.out = at(ws, lay_->kbuf[j]);

@@ -38,3 +38,21 @@ def test_the_row_local_backward_path_is_declined_before_its_first_step(tmp_path)
         printf("%d\\n", (int)v->fused_backward_begin(nullptr, (void*)(1ull << 41), fs, &launches));
     }""")
     assert out == ["0", "0", "0"]
+
+
+def test_the_convolution_keeps_its_time_channel_where_the_64_channel_kernel_is_declined(tmp_path):
+    # The 64-channel kernel adds tau times a slope to its bias table, which no other kernel reads.  Declined although the shape is its
+    # own (16-pixel rows), the first convolution has to take the steps of a shape that is not (64-pixel rows): the table with the time
+    # channel for the general tensor-core kernel, and where that is declined too the 65-channel form.
+    out = _run(tmp_path, """
+    for (int side : {16, 64}) {
+        mpode_velocity_desc d{};
+        d.kind = MPODE_VEL_CONV3X3_2; d.d = side * side * 64; d.H = d.W = side; d.C = 64; d.act = MPODE_ACT_RELU; d.append_time = 1;
+        Velocity* v = make_velocity(d, 4, MPODE_BF16, 1);
+        Layout lay;
+        v->plan(lay);
+        long long launches = 0;
+        v->forward(nullptr, (void*)(1ull << 41), 0, (const void*)(1ull << 40), 0.5f, &launches);
+        printf("%lld\\n", launches);
+    }""")
+    assert out == ["3", "3"]
