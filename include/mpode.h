@@ -270,7 +270,8 @@ void mpode_get_stats(const mpode_ctx* ctx, mpode_stats* out);
  * that next synchronises returns MPODE_ERR_CUDA ("a device-side wait timed out").  wait_limit_ns > 0 replaces the default
  * limit of 2 s for later calls on this context (0 restores it); starve_forward != 0 makes the second phase of the fused
  * forward program wait for a tile count one higher than is ever published, so that the limit is reached by construction, and
- * the last block of the cooperative backward kernel (hypernetwork flow) for an arrival that never comes.
+ * the last block of the cooperative backward kernel (hypernetwork flow) for an arrival, and the row-local backward kernel (small dense
+ * networks) for weights that never come.
  * Nothing faults or hangs: the context and the device stay usable.
  */
 void mpode_debug_waits(mpode_ctx* ctx, unsigned long long wait_limit_ns, int starve_forward);

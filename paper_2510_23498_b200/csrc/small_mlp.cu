@@ -156,33 +156,39 @@ __global__ void __launch_bounds__(256) small_pack_f32_kernel(const __grid_consta
 // The order in which a block needs the weights is fixed, so one thread streams them ahead of the arithmetic: bulk copies of at most
 // 16 KB (32 of the reduction for up to 32 column tiles; in float32 16 rows of up to 256 columns) through a ring of buffers, across layer
 // and stage boundaries.  (Loaded by the warps themselves, even 16 loads ahead, each unit cost an L2 round trip of half a microsecond.)
-// Every wait is bounded; after one has given up the block runs on without waiting and the error word tells the host.
+// Every wait is bounded.  A thread whose wait has given up waits no more (the producer issues no more) and runs on to its end, the error
+// word tells the host, and the producer leaves last: a block does not end while copies into its shared memory are on their way.
 struct Ring {
     uint64_t *full, *empty;
     unsigned char* buf;
     int n, s;
     uint32_t phase;
+    bool lost;
     unsigned* err;
-    __device__ __forceinline__ void next() { if (++s == n) { s = 0; phase ^= 1u; } }
+    unsigned long long wait_ns;
+    bool laps;                 // whether every buffer has been used
+    __device__ __forceinline__ void next() { if (++s == n) { s = 0; phase ^= 1u; laps = true; } }
     __device__ __forceinline__ unsigned char* stage() const { return buf + s * kUnitBytes; }
 };
 __device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }      // the working warps
 
-__device__ __forceinline__ void ring_wait(const Ring& r) {
-    if (!mbar_try_wait(&r.full[r.s], r.phase)) mbar_wait(&r.full[r.s], r.phase, r.err, 4u);
+__device__ __forceinline__ void ring_wait(Ring& r) {
+    if (!mbar_try_wait(&r.full[r.s], r.phase) && !r.lost) r.lost = !mbar_wait_long(&r.full[r.s], r.phase, r.err, 4u, r.wait_ns);
 }
 __device__ __forceinline__ void stream_units(Ring& r, const unsigned char* src, int bytes) {
-    if (r.n == 0) return;
-    if (!mbar_wait(&r.empty[r.s], r.phase ^ 1u, r.err, 1u)) {      // gave up: nothing more is issued, what is in flight lands first
-        const unsigned long long t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-        r.n = 0;
-        return;
-    }
+    if (!r.lost) r.lost = !mbar_wait(&r.empty[r.s], r.phase ^ 1u, r.err, 1u, r.wait_ns);
+    if (r.lost) return;
     mbar_arrive_expect_tx(&r.full[r.s], (uint32_t)bytes);
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(r.stage())), "l"(src), "r"(bytes),
                  "r"(smem_u32(&r.full[r.s])) : "memory");
     r.next();
+}
+// the producer's last act: what it has issued lands (the last fill of every buffer that has been filled)
+__device__ __forceinline__ void ring_drain(const Ring& r) {
+    for (int q = 0; q < r.n; ++q) {
+        const bool this_lap = q < r.s;
+        if (this_lap || r.laps) mbar_wait(&r.full[q], this_lap ? r.phase : r.phase ^ 1u, r.err, 2u, r.wait_ns);
+    }
 }
 // one contraction's weights: reduction K, N columns
 template <typename T> __device__ __forceinline__ void stream_layer(Ring& r, const uint4* W, int K, int N) {
@@ -295,9 +301,9 @@ template <typename T> size_t small_smem(const SmallMlp& p, int rows) {
            (sizeof(T) == 4 ? (size_t)kThreads * rows * 4 : 0);
 }
 // the ring behind the block's own shared memory: `n` buffers, then the barriers
-__device__ __forceinline__ Ring make_ring(unsigned char* base, int n, unsigned* err) {
+__device__ __forceinline__ Ring make_ring(unsigned char* base, int n, unsigned* err, unsigned long long wait_ns) {
     Ring r;
-    r.buf = base; r.n = n; r.s = 0; r.phase = 0; r.err = err;
+    r.buf = base; r.n = n; r.s = 0; r.phase = 0; r.lost = r.laps = false; r.err = err; r.wait_ns = wait_ns;
     r.full = (uint64_t*)(base + n * kUnitBytes);
     r.empty = r.full + n;
     if (threadIdx.x == 0) {
@@ -453,11 +459,13 @@ __global__ void __launch_bounds__(kThreads + 32, 1) small_forward_kernel(const _
     using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
     const int R = kRows<T, MT>, r0 = blockIdx.x * R;
-    Ring ring = make_ring(smem, p.ring, p.err);
+    Ring ring = make_ring(smem, p.ring, p.err, p.wait_ns);
     if (threadIdx.x >= kThreads) {
-        if (threadIdx.x == kThreads)
+        if (threadIdx.x == kThreads) {
             for (int n = 0; n < p.n_steps * p.stages; ++n)
                 for (int l = 0; l < p.L; ++l) stream_layer<T>(ring, p.wf[l], p.wp[l], p.wp[l + 1]);
+            ring_drain(ring);
+        }
         return;
     }
     const SmallSmem<T> sm(p, smem + p.ring * (kUnitBytes + 16), R);
@@ -526,18 +534,22 @@ __global__ void __launch_bounds__(kThreads + 32, 1) small_backward_kernel(const 
     using W = typename Pair<T>::W;
     extern __shared__ __align__(16) unsigned char smem[];
     const int R = kRows<T, MT>, r0 = blockIdx.x * R;
-    Ring ring = make_ring(smem, p.ring, p.err);
+    Ring ring = make_ring(smem, p.ring, p.err, p.wait_ns);
     if (threadIdx.x >= kThreads) {
-        if (threadIdx.x == kThreads)
+        if (threadIdx.x == kThreads) {
             for (int s = 0; s < p.count; ++s) {
                 if (p.recompute)
                     for (int j = 0; j < p.stages; ++j)
                         for (int l = 0; l < p.L; ++l)      // (the last stage's derivative only for the time terms)
                             if (!(l == p.L - 1 && j == p.stages - 1 && p.tpart == nullptr)) stream_layer<T>(ring, p.wf[l], p.wp[l], p.wp[l + 1]);
                 if (p.vjp)
-                    for (int j = 0; j < p.stages; ++j)
+                    for (int j = 0; j < p.stages; ++j) {
                         for (int l = p.L - 1; l >= 0; --l) stream_layer<T>(ring, p.wb[l], p.wp[l + 1], p.wp[l]);
+                        ring.lost |= p.starve != 0;      // test of the waits: the rest of the weights never comes
+                    }
             }
+            ring_drain(ring);
+        }
         return;
     }
     const SmallSmem<T> sm(p, smem + p.ring * (kUnitBytes + 16), R);

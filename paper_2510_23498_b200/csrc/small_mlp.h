@@ -27,6 +27,7 @@ struct SmallMlp {
     void* psi[4];                                      // without commit: psi_j, low [B][wp_0]
     unsigned* flag;
     unsigned* err;                                     // a bounded wait that gave up
+    unsigned long long wait_ns; int starve;            // limit of every wait; test of it: the backward kernel's weights stop coming
     int ring;                                          // buffers of the weight stream (set by the launch)
     // time-grid gradient (null: not wanted): [slot][blocks][3] shares; results of the last step [3]; t' [n + 1], updated per step
     float *tpart, *tvals, *tprime;

@@ -201,11 +201,11 @@ public:
         cudaMemcpyAsync(at(ws, small_scal_), fs.scalars.data(), (size_t)fs.n_steps * sizeof(RkStepScalars), cudaMemcpyHostToDevice, st);
         SmallMlp p = small_params(ws);
         p.stages = fs.stages; p.n_steps = fs.n_steps; p.round_increment = fs.round_increment; p.traj = const_cast<void*>(fs.traj);
+        p.wait_ns = fs.wait_ns; p.starve = fs.starve;
         return p;
     }
-    // the test of the bounded waits (starve) is about the kernel that has them
     bool small_usable(const FusedSolve& fs) const {
-        return small_ok_ && !fs.starve && fs.stages <= RK_MAX_STAGES && fs.n_steps <= max_steps_ && ((uintptr_t)fs.traj & 31) == 0;
+        return small_ok_ && fs.stages <= RK_MAX_STAGES && fs.n_steps <= max_steps_ && ((uintptr_t)fs.traj & 31) == 0;
     }
     template <typename F> bool small_timed(int klass, double flops, cudaStream_t st, F&& launch) {
         Profiler* pr = tl_profiler;
@@ -401,7 +401,7 @@ public:
     }
 
     bool fused_forward(cudaStream_t st, void* ws, const FusedSolve& fs, long long* L) override {
-        if (small_usable(fs)) {
+        if (small_usable(fs) && !fs.starve) {      // (the test of the bounded waits is about the fused program here)
             SmallMlp p = small_solve(st, ws, fs);
             p.y0 = p.yT = fs.y;                       // the driver has put y_0 there
             if (small_timed(0, (double)fs.n_steps * fs.stages * layer_flops(), st, [&] { return launch_small_forward(dt_, p, st, L); })) return true;

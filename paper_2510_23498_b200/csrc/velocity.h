@@ -25,8 +25,9 @@ struct WholeBackward {
 struct FusedSolve {
     int n_steps = 0, stages = 0, round_increment = 0;
     unsigned long long wait_ns = 2000000000ull; // limit of every device-side wait
-    int starve = 0;                             // test of the bounded waits: the fused forward program's second phase, or the last
-                                                // barrier of the cooperative backward kernel, waits for a count that is never reached
+    int starve = 0;                             // test of the bounded waits: the fused forward program's second phase or the last
+                                                // barrier of the cooperative backward kernel waits for a count that is never reached,
+                                                // the row-local backward kernel for weights that never come
     const void* traj = nullptr;                 // low [(n_steps+1), B, d]
     float* y = nullptr;                         // fp32 running state [B, D]
     std::vector<RkStepScalars> scalars;         // one entry per step

@@ -119,6 +119,33 @@ def test_small_networks_report_a_parameter_gradient_that_overflows(low, batch, w
         assert rel_l2(gpu["g"], g) <= TOL[low]
 
 
+# The row-local kernels wait for their weights with a limit (20 ms here).  The weights stop after the first stage: every block gives up, waits
+# no more, runs to its end and leaves no copy in flight; the call reports it, and the same context then gives the usual result.
+@pytest.mark.parametrize("low,scaling", [("bf16", "none"), ("f16", "dynamic"), ("f32", "none")])
+def test_row_local_waits_that_run_out_are_reported(low, scaling):
+    import time
+    import torch
+    from paper_2510_23498_b200 import binding
+    wl = inputs.mlp_block(batch=300, n_steps=24, d=64, hidden=160)
+    ref = run_gpu(wl, low, scaling)
+    ctx = binding.Context(wl.vel, wl.batch, wl.n_steps, low=low, scaling=scaling)
+    theta, y0 = torch.from_numpy(wl.theta).cuda(), torch.from_numpy(wl.y0).cuda()
+    dl = torch.from_numpy(np.ascontiguousarray(ref["dLdyT"], dtype=np.float32)).cuda()
+    ctx.forward(theta, y0, wl.tgrid, wl.solver)
+    torch.cuda.synchronize()
+    ctx.debug_waits(20_000_000, True)
+    t0 = time.perf_counter()
+    with pytest.raises(binding.MpodeError) as ei:
+        ctx.backward(dl)
+    assert ei.value.status == binding.ERR_CUDA and "wait timed out" in str(ei.value)
+    assert time.perf_counter() - t0 < 2.0
+    ctx.debug_waits(0, False)
+    ctx.forward(theta, y0, wl.tgrid, wl.solver)
+    a0, g, _, st = ctx.backward(dl)
+    assert st == 0 and np.array_equal(a0.cpu().numpy(), ref["a0"]) and np.array_equal(g.cpu().numpy(), ref["g"])
+    ctx.close()
+
+
 # paired (value, tangent) tiles of 64 columns: one tile of 64 sample pairs, several, output columns that end inside a tile, on its edge and
 # one vector past it, the smallest reduction length
 @pytest.mark.parametrize("batch,d,hidden,low", [(64, 16, 72, "bf16"), (192, 24, 200, "f16"), (128, 72, 64, "bf16"), (512, 8, 256, "f16")])
