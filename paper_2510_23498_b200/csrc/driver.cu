@@ -256,6 +256,7 @@ mpode_status mpode_create(mpode_ctx** out, const mpode_velocity_desc* vel, int b
         if (!c->v->supports_time_gradient() || c->pol.round_increment) { delete c->v; delete c; return MPODE_ERR_UNSUPPORTED; }
         c->lay.time_gradient = true;
     }
+    c->lay.stepwise = c->pol.scaling == MPODE_SCALE_DYNAMIC;
     c->v->plan(c->lay);
     if (c->pol.scaling == MPODE_SCALE_DYNAMIC)      // the device-side scale log: exponent, attempts (int each), doubled (byte) per step
         c->lay.slog = c->lay.take((size_t)c->max_steps * 9);

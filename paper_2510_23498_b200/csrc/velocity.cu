@@ -25,7 +25,9 @@ void plan_common(Layout& lay, int B, int d, bool wide, size_t p, mpode_dtype dt,
     lay.ds = d;
     // one slab per family, stage slots back to back (the fused kernels address a slot through a 3-D tensor map)
     const size_t slot = (size_t)B * d * es;
-    const size_t k0 = lay.take(4 * slot), y0 = lay.take(4 * ybuf_rows_factor * slot), p0 = lay.take(4 * slot);
+    const size_t p0 = lay.take(4 * slot);
+    lay.dg = lay.take(p * sizeof(float));
+    const size_t k0 = lay.take(4 * slot), y0 = lay.take(4 * ybuf_rows_factor * slot);
     for (int j = 0; j < 4; ++j) {
         lay.kbuf[j] = k0 + j * slot;
         lay.ybuf[j] = y0 + j * ybuf_rows_factor * slot;
@@ -38,7 +40,6 @@ void plan_common(Layout& lay, int B, int d, bool wide, size_t p, mpode_dtype dt,
         lay.vl = lay.take((size_t)B * es);
         lay.kappal = lay.take((size_t)B * es);
     }
-    lay.dg = lay.take(p * sizeof(float));
 }
 
 // words 24 .. 55 of the scalar slice: the last-block counters of the one-launch column sums
@@ -152,8 +153,12 @@ public:
         plan_small(lay);
     }
 
-    // Row-local kernels (small_mlp.cu): packed weights, and the layer inputs and cotangents of a few steps at a time (8 MB at most, or
-    // one step's)
+    // Row-local kernels (small_mlp.cu): packed weights, and the layer inputs and cotangents of a few steps at a time.  They lie over the
+    // buffers of the other paths (all but psi and dg where the pass goes step by step): a call runs one path or the other, and one that
+    // has packed the weights and then takes another path forms that path's operands afterwards.  As many steps at a time as those bytes
+    // hold (8 MB at most: they should stay in the L2), and one step at least, which alone can make the workspace larger than the other
+    // path's.  A launch pair costs about 6 us besides its steps.  Training pass, ms with 1 / 2 / 4 / 8 steps a pair: linear equation 64 wide,
+    // 1024 samples, 100 RK4 steps 3.30 / 3.01 / 2.87 / 2.77; 24-40-24, 512 samples, 64 steps 3.25 / 3.06 / 2.98 / 2.94 (other path 8.6, 8.2).
     void plan_small(Layout& lay) {
         small_w_.clear();
         for (int w : w_) small_w_.push_back((w + 7) / 8 * 8);
@@ -162,21 +167,28 @@ public:
         small_bwd_ok_ = small_ok_ && small_backward_supported(dt_, B_);
         if (!small_ok_) return;
         const size_t es = low_size(dt_);
-        size_t per_step = 0;
-        for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
-        small_chunk_ = (int)(((size_t)8 << 20) / per_step);
-        if (small_chunk_ < 1) small_chunk_ = 1;
-        if (small_chunk_ > SMALL_MAX_CHUNK) small_chunk_ = SMALL_MAX_CHUNK;
-        if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
-        small_pack_ = lay.take(small_pack_bytes(dt_, L_, small_w_.data()));
-        for (int l = 0; l < L_; ++l) small_b_[l] = lay.take((size_t)small_w_[l + 1] * es);
-        small_wt_ = lay.take((size_t)small_w_[1] * es);
-        small_scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
-        for (int l = 0; l < L_ && small_bwd_ok_; ++l) {
-            small_xs_[l] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
-            small_zs_[l + 1] = lay.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
+        Layout own;
+        own.total = lay.stepwise ? lay.kbuf[0] : lay.psi[0];
+        small_pack_ = own.take(small_pack_bytes(dt_, L_, small_w_.data()));
+        for (int l = 0; l < L_; ++l) small_b_[l] = own.take((size_t)small_w_[l + 1] * es);
+        small_wt_ = own.take((size_t)small_w_[1] * es);
+        small_scal_ = own.take((size_t)max_steps_ * sizeof(RkStepScalars));
+        if (small_bwd_ok_) {
+            size_t per_step = lay.time_gradient ? (size_t)small_blocks(dt_, B_) * 3 * sizeof(float) : 0;
+            for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
+            const size_t slack = (size_t)(2 * L_ + 1) * 256, used = own.total + slack;      // (every slab starts on 256 bytes)
+            size_t room = used < lay.total ? lay.total - used : 0;
+            if (room > (size_t)8 << 20) room = (size_t)8 << 20;
+            const size_t steps = lay.stepwise ? 1 : room / per_step;
+            small_chunk_ = steps < 1 ? 1 : (steps > SMALL_MAX_CHUNK ? SMALL_MAX_CHUNK : (int)steps);
+            if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
+            for (int l = 0; l < L_; ++l) {
+                small_xs_[l] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
+                small_zs_[l + 1] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
+            }
+            if (lay.time_gradient) small_tpart_ = own.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
         }
-        if (lay.time_gradient && small_bwd_ok_) small_tpart_ = lay.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
+        if (own.total > lay.total) lay.total = own.total;
     }
     SmallMlp small_params(void* ws) const {
         SmallMlp p{};

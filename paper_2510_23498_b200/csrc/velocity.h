@@ -53,6 +53,7 @@ struct Layout {
     // time-grid gradient (policy.time_gradient): t' fp32 [max_steps + 1]; scratch floats: partial sums of Phi^T a [148], of the
     // <psi_j, k_l> terms [148], dtau_j [4], c_j [4], {Phi^T a, dt, dh} [4]
     bool time_gradient = false;
+    bool stepwise = false;    // dynamic scaling: a pass goes step by step through psi and dg, whatever its path
     size_t tprime = 0, tdots = 0;
     size_t take(size_t bytes) {
         size_t o = total;

@@ -86,6 +86,27 @@ def test_a_refused_whole_solve_launch_fails_the_call_and_nothing_else_runs():
     lib.mpode_destroy(h)
 
 
+def test_row_local_kernels_lie_over_the_buffers_of_the_other_path():
+    # Small dense networks run row-local kernels in place of the fused or layer-by-layer path, never both in a call: their packed weights,
+    # layer inputs and cotangents take no bytes of their own.  Bounds: what the other path alone needs (MB, rounded up), and for the
+    # float32 network the layer inputs and cotangents of one RK4 step, 2 * 4 * 1024 * (64 + 256 + 256) * 4 = 18.9 MB, and its weights.
+    import ctypes as C
+    from paper_2510_23498_b200 import binding
+    lib = binding.load_library()
+    for widths, batch, steps, low, scaling, most in (([64, 64], 1024, 100, "bf16", "none", 2.5), ([24, 40, 24], 512, 64, "bf16", "none_safe", 0.8),
+                                                     ([64, 128, 64], 1000, 64, "f16", "none", 4.1), ([72, 200, 200, 72], 1000, 16, "f16", "dynamic", 8.9),
+                                                     ([64, 256, 256, 64], 2048, 64, "bf16", "none", 20.7), ([64, 256, 256, 64], 1024, 16, "f32", "none", 19.8)):
+        arr = (C.c_int * len(widths))(*widths)
+        linear = len(widths) == 2
+        desc = binding.VelocityDesc(binding.KINDS["mlp"], widths[0], len(widths) - 1, C.cast(arr, C.POINTER(C.c_int)),
+                                    binding.ACTS["none" if linear else "softplus"], 0 if linear else 1, 0 if linear else 1, 0, 0, 0, 0, 0)
+        pol = binding.Policy(binding.DTYPES[low], binding.SCALINGS[scaling], 0, 0, 0, binding.NO_OVERRIDE)
+        h = C.c_void_p()
+        assert lib.mpode_create(C.byref(h), C.byref(desc), batch, steps, C.byref(pol)) == 0
+        assert lib.mpode_workspace_bytes(h) <= most * 1e6, (widths, batch, low, lib.mpode_workspace_bytes(h))
+        lib.mpode_destroy(h)
+
+
 def test_cnf_workspace_has_no_float32_cotangent_scratch_where_the_epilogue_takes_the_activation_step():
     # c5 (2048 x 784, 785 -> 2048 -> 2048 -> 784): with a batch that is a multiple of 64 and widths of at least 64 the backward
     # step through an activation runs in the tensor-core epilogue, so mixed mode plans no [2 B, 2048] float32 buffer (33.5 MB);
