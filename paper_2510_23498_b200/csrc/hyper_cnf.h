@@ -47,7 +47,7 @@ struct HyperSolve {
     int *log_exp, *log_attempts, *log_doubled, *status;     // device [n_steps] each; status [4], zero at launch
 };
 bool hyper_solve_shape_ok(mpode_dtype dt, int h, int w, int d, int stages);
-size_t hyper_solve_part_floats(int w, int d);
+size_t hyper_solve_part_floats(mpode_dtype dt, int B, int h, int w, int d);
 size_t hyper_solve_tpart_floats(int h, int w);
 void launch_hyper_table(mpode_dtype dt, const float* theta, const RkStepScalars* scal, int n_steps, int stages, int h, int w, int d, float* table,
                         cudaStream_t st, long long* launches);

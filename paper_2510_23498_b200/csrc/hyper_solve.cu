@@ -728,7 +728,11 @@ int backward_warps(mpode_dtype dt, int B, int stages, int h, int w, int d) {
 bool hyper_solve_shape_ok(mpode_dtype dt, int h, int w, int d, int stages) {
     return hyper_shape_ok(h, w, d) && stages >= 1 && stages <= RK_MAX_STAGES && backward_smem(dt, stages, h, w, d, 1) <= kSmemCap;
 }
-size_t hyper_solve_part_floats(int w, int d) { return (size_t)sm_count() * w * RK_MAX_STAGES * (2 * d + 2); }
+// a row of partial sums for every block that holds samples (the fewer samples a block takes, the more of them: four stages need the most room)
+size_t hyper_solve_part_floats(mpode_dtype dt, int B, int h, int w, int d) {
+    const int warps = backward_warps(dt, B, RK_MAX_STAGES, h, w, d), groups = (B + warps - 1) / warps;
+    return (size_t)(groups < sm_count() ? groups : sm_count()) * w * RK_MAX_STAGES * (2 * d + 2);
+}
 size_t hyper_solve_tpart_floats(int h, int w) { return (size_t)w * RK_MAX_STAGES * h; }
 
 void launch_hyper_table(mpode_dtype dt, const float* theta, const RkStepScalars* scal, int n_steps, int stages, int h, int w, int d, float* table,

@@ -1385,7 +1385,7 @@ public:
             table_ = lay.take((size_t)max_steps_ * RK_MAX_STAGES * hyper_stage_floats(h_, w_, d_) * sizeof(float));
             scal_ = lay.take((size_t)max_steps_ * sizeof(RkStepScalars));
             log_ = lay.take(((size_t)3 * max_steps_ + 4 + 16) * sizeof(int));       // scale log, status [4], words [16]
-            part_ = lay.take(hyper_solve_part_floats(w_, d_) * sizeof(float));
+            part_ = lay.take(hyper_solve_part_floats(dt_, B_, h_, w_, d_) * sizeof(float));
             tpart_ = lay.take(hyper_solve_tpart_floats(h_, w_) * sizeof(float));
             return;
         }

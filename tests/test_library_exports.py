@@ -107,6 +107,26 @@ def test_row_local_kernels_lie_over_the_buffers_of_the_other_path():
         lib.mpode_destroy(h)
 
 
+def test_hypernetwork_flow_plans_partial_sums_for_the_blocks_that_hold_samples():
+    # Five samples are one block: one row of the 287 weight sets' sums (18 floats for each of four stages, 83 KB) and not one for each of the
+    # 148 SMs (12 MB); 100 000 samples use every SM
+    import ctypes as C
+    from paper_2510_23498_b200 import binding
+    lib = binding.load_library()
+
+    def size(batch):
+        widths = (C.c_int * 2)(15, 287)
+        desc = binding.VelocityDesc(binding.KINDS["cnf_hyper"], 8, 1, C.cast(widths, C.POINTER(C.c_int)), 0, 0, 0, 0, 0, 0, 0, 0)
+        pol = binding.Policy(1, 0, 0, 0, 0, binding.NO_OVERRIDE)
+        h = C.c_void_p()
+        assert lib.mpode_create(C.byref(h), C.byref(desc), batch, 5, C.byref(pol)) == 0
+        out = lib.mpode_workspace_bytes(h)
+        lib.mpode_destroy(h)
+        return out
+
+    assert size(5) < 2.4e6 and size(100000) > 12e6
+
+
 def test_cnf_workspace_has_no_float32_cotangent_scratch_where_the_epilogue_takes_the_activation_step():
     # c5 (2048 x 784, 785 -> 2048 -> 2048 -> 784): with a batch that is a multiple of 64 and widths of at least 64 the backward
     # step through an activation runs in the tensor-core epilogue, so mixed mode plans no [2 B, 2048] float32 buffer (33.5 MB);
