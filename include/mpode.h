@@ -243,12 +243,13 @@ mpode_status mpode_backward_host(mpode_ctx* ctx, void* cuda_stream, const float*
  * the process exits.  Inputs and outputs are still the caller's: dL_dyT_dev, dL_dy0_dev, dL_dtheta_dev and log mean
  * what they mean for mpode_backward, and the trajectory, parameters and time grid are those of the last
  * mpode_forward on this context (which keeps using the caller's workspace).
- *   - Returns MPODE_ERR_WORKSPACE_TOO_SMALL, with a message in mpode_last_error, when
- *     mpode_workspace_bytes(ctx) > MPODE_STATIC_WORKSPACE_BYTES; nothing is launched then.
+ *   - A context with mpode_workspace_bytes(ctx) <= MPODE_STATIC_WORKSPACE_BYTES runs here what it runs in mpode_backward.  A larger one
+ *     runs the general, slower kernels, which need less (no padded rows, nothing kept on the chip for whole steps), if those fit;
+ *     otherwise MPODE_ERR_WORKSPACE_TOO_SMALL with a message in mpode_last_error, and nothing is launched.
  *   - The first call on a device looks up the array's device address (no allocation, but a runtime query): make that
  *     first call before any stream capture begins.
  *   - The CUDA runtime may load a kernel's code the first time that kernel is launched in a process, and that can allocate.
- *     A caller with a no-allocation region therefore runs one forward / backward pair of each configuration once, as a
+ *     A caller with a no-allocation region therefore runs a forward pass and this call once for each configuration, as a
  *     warm-up, before entering that region; from then on the call launches only kernels that are already resident.
  *   - The context, its buffers and the array must live on the current device: a dL_dyT_dev that belongs to another device
  *     is refused with MPODE_ERR_INVALID_ARG.  Arguments are checked before anything is queued on the stream.

@@ -49,6 +49,9 @@ struct mpode_ctx {
     mpode_policy pol{};
     Velocity* v = nullptr;
     Layout lay;
+    // contexts whose workspace does not fit the static one: the same velocity without the paths that ask for more room, where that fits
+    Velocity* v_compact = nullptr;
+    Layout lay_compact;
     // record of the last forward
     bool have_forward = false;
     const float* theta = nullptr;
@@ -141,32 +144,44 @@ FusedSolve fused_solve(const mpode_ctx* c, float* y) {
     return fs;
 }
 
+void plan_workspace(const mpode_ctx* c, Velocity* v, Layout& lay) {
+    lay.time_gradient = c->pol.time_gradient != 0;
+    lay.stepwise = c->pol.scaling == MPODE_SCALE_DYNAMIC;
+    v->plan(lay);
+    if (c->pol.scaling == MPODE_SCALE_DYNAMIC)      // the device-side scale log: exponent, attempts (int each), doubled (byte) per step
+        lay.slog = lay.take((size_t)c->max_steps * 9);
+    if (c->pol.time_gradient) {
+        lay.tprime = lay.take(((size_t)c->max_steps + 1) * sizeof(float));
+        lay.tdots = lay.take(((size_t)2 * kDotBlocks + 12) * sizeof(float));
+    }
+}
+
 // Evaluate all stages of step i from the stored state traj[i] (increment of Alg. 1 / recompute of Alg. 2).
-void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes& tm) {
+void run_stages(mpode_ctx* c, Velocity* v, const Layout& lay, cudaStream_t st, void* ws, int i, const StepTimes& tm) {
     const mpode_dtype dt = c->pol.low;
     const size_t es = low_size(dt);
     const long long nBd = (long long)c->B * c->d;
     const char* traj_i = (const char*)c->traj + (size_t)i * nBd * es;
     long long* L = &c->stats.kernel_launches;
-    const bool next_input = c->v->can_write_next_input() && c->lay.ds == c->d;
+    const bool next_input = v->can_write_next_input() && lay.ds == c->d;
     bool ready = false;                       // the input of this stage was written with the previous stage's derivative
     for (int j = 0; j < c->stages; ++j) {
         const void* yin = traj_i;
         if (ready) {
-            yin = at(ws, c->lay.ybuf[j]);
-        } else if (j > 0 || c->v->needs_input_copy()) {
+            yin = at(ws, lay.ybuf[j]);
+        } else if (j > 0 || v->needs_input_copy()) {
             Terms t{};
             t.n = 0;
             for (int l = 0; l < j; ++l) {
                 double a = c->ta[j * c->stages + l];
                 if (a != 0.0) {
-                    t.p[t.n] = at(ws, c->lay.kbuf[l]);
+                    t.p[t.n] = at(ws, lay.kbuf[l]);
                     t.c[t.n] = (float)((double)tm.h * a);
                     ++t.n;
                 }
             }
-            launch_stage_input(dt, traj_i, t, at(ws, c->lay.ybuf[j]), c->B, c->d, c->lay.ds, st, L);
-            yin = at(ws, c->lay.ybuf[j]);
+            launch_stage_input(dt, traj_i, t, at(ws, lay.ybuf[j]), c->B, c->d, lay.ds, st, L);
+            yin = at(ws, lay.ybuf[j]);
         }
         ready = false;
         if (next_input && j + 1 < c->stages) {      // does the next stage depend on this one alone (Euler, midpoint, Heun, RK4)?
@@ -174,12 +189,12 @@ void run_stages(mpode_ctx* c, cudaStream_t st, void* ws, int i, const StepTimes&
             for (int l = 0; l < j; ++l) alone = alone && c->ta[(j + 1) * c->stages + l] == 0.0;
             if (alone) {
                 KappaNext kn;
-                kn.out = at(ws, c->lay.ybuf[j + 1]); kn.v = traj_i; kn.bv = 1.f; kn.c = (float)((double)tm.h * c->ta[(j + 1) * c->stages + j]);
-                c->v->set_next_input(kn);
+                kn.out = at(ws, lay.ybuf[j + 1]); kn.v = traj_i; kn.bv = 1.f; kn.c = (float)((double)tm.h * c->ta[(j + 1) * c->stages + j]);
+                v->set_next_input(kn);
                 ready = true;
             }
         }
-        c->v->forward(st, ws, j, yin, tm.tau16[j], L);
+        v->forward(st, ws, j, yin, tm.tau16[j], L);
     }
 }
 
@@ -254,15 +269,12 @@ mpode_status mpode_create(mpode_ctx** out, const mpode_velocity_desc* vel, int b
     if (c->pol.time_gradient) {
         // the rounded increment (round_increment = 1) would need Q16 of the combined stage derivatives inside Phi^T a
         if (!c->v->supports_time_gradient() || c->pol.round_increment) { delete c->v; delete c; return MPODE_ERR_UNSUPPORTED; }
-        c->lay.time_gradient = true;
     }
-    c->lay.stepwise = c->pol.scaling == MPODE_SCALE_DYNAMIC;
-    c->v->plan(c->lay);
-    if (c->pol.scaling == MPODE_SCALE_DYNAMIC)      // the device-side scale log: exponent, attempts (int each), doubled (byte) per step
-        c->lay.slog = c->lay.take((size_t)c->max_steps * 9);
-    if (c->pol.time_gradient) {
-        c->lay.tprime = c->lay.take(((size_t)c->max_steps + 1) * sizeof(float));
-        c->lay.tdots = c->lay.take(((size_t)2 * kDotBlocks + 12) * sizeof(float));
+    plan_workspace(c, c->v, c->lay);
+    if (c->lay.total > (size_t)MPODE_STATIC_WORKSPACE_BYTES) {
+        c->v_compact = make_velocity(c->vel, c->B, c->pol.low, c->max_steps, true);
+        plan_workspace(c, c->v_compact, c->lay_compact);
+        if (c->lay_compact.total > (size_t)MPODE_STATIC_WORKSPACE_BYTES) { delete c->v_compact; c->v_compact = nullptr; }
     }
     *out = c;
     return MPODE_OK;
@@ -279,6 +291,7 @@ void mpode_destroy(mpode_ctx* ctx) {
         cudaEventDestroy(ctx->ev_step[0]); cudaEventDestroy(ctx->ev_step[1]);
     }
     delete ctx->v;
+    delete ctx->v_compact;
     delete ctx;
 }
 
@@ -388,7 +401,7 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
     for (int i = 0; i < n_steps && !fused; ++i) {
         StepTimes tm = step_times(c, i);
         c->v->set_step(i, n_steps);
-        run_stages(c, st, ws, i, tm);
+        run_stages(c, c->v, c->lay, st, ws, i, tm);
         Terms t{};
         t.n = c->stages;
         for (int j = 0; j < c->stages; ++j) {
@@ -408,20 +421,15 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
     return MPODE_OK;
 }
 
-mpode_status mpode_backward(mpode_ctx* c, void* cuda_stream, const float* dL_dyT_dev, float* a, float* g,
-                            int accumulate_dtheta, mpode_scale_log* log, void* ws, size_t ws_bytes) {
-    return mpode_backward_ex(c, cuda_stream, dL_dyT_dev, nullptr, a, g, accumulate_dtheta, nullptr, log, ws, ws_bytes);
-}
-
-mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_dyT_dev, const float* cot, float* a, float* g,
-                               int accumulate_dtheta, float* dt_host, mpode_scale_log* log, void* ws, size_t ws_bytes) {
-    if (!c) return MPODE_ERR_INVALID_ARG;
+// Alg. 2 with velocity `v` of the context and its workspace layout
+static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, void* cuda_stream, const float* dL_dyT_dev, const float* cot, float* a, float* g,
+                                 int accumulate_dtheta, float* dt_host, mpode_scale_log* log, void* ws, size_t ws_bytes) {
     if (!c->have_forward) return fail(c, MPODE_ERR_BAD_STATE, "mpode_backward needs a preceding mpode_forward");
     if (!dL_dyT_dev || !a || !g || !ws) return fail(c, MPODE_ERR_INVALID_ARG, "null pointer argument");
     if (dt_host != nullptr && !c->pol.time_gradient)
         return fail(c, MPODE_ERR_INVALID_ARG, "dL/dt needs a context created with policy.time_gradient = 1");
     if (cot != nullptr && ((uintptr_t)cot & 15)) return fail(c, MPODE_ERR_INVALID_ARG, "misaligned device pointer");
-    if (ws_bytes < c->lay.total) return fail(c, MPODE_ERR_WORKSPACE_TOO_SMALL, "workspace too small");
+    if (ws_bytes < lay.total) return fail(c, MPODE_ERR_WORKSPACE_TOO_SMALL, "workspace too small");
     if (((uintptr_t)ws & 255) || ((uintptr_t)a & 15) || ((uintptr_t)g & 15) || ((uintptr_t)dL_dyT_dev & 15))
         return fail(c, MPODE_ERR_INVALID_ARG, "misaligned device pointer");
     const int N = c->n_steps, s = c->stages;
@@ -436,7 +444,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     const mpode_dtype dt = c->pol.low;
     const size_t es = low_size(dt);
     const long long nBd = (long long)c->B * c->d;
-    const long long p = (long long)c->v->param_count();
+    const long long p = (long long)v->param_count();
     const bool dynamic = c->pol.scaling == MPODE_SCALE_DYNAMIC;
     const bool checked = c->pol.scaling != MPODE_SCALE_NONE;
     long long launches0 = c->stats.kernel_launches;
@@ -458,7 +466,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         if (log) { wb.exp_used = log->exp_used; wb.attempts = log->attempts; wb.doubled = log->doubled; }
         wb.cot = cot; wb.dt_host = dt_host;
         FusedSolve whole = fused_solve(c, nullptr);
-        const Whole w = c->v->whole_backward(st, ws, whole, wb, L);
+        const Whole w = v->whole_backward(st, ws, whole, wb, L);
         if (w != Whole::kNo) {
             if (w == Whole::kDone) ++c->stats.host_syncs;
             c->stats.retries = wb.retries;
@@ -475,14 +483,14 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
             return MPODE_OK;
         }
     }
-    unsigned* flag = (unsigned*)at(ws, c->lay.scal);
-    float* amax = (float*)at(ws, c->lay.scal) + 1;
+    unsigned* flag = (unsigned*)at(ws, lay.scal);
+    float* amax = (float*)at(ws, lay.scal) + 1;
     unsigned* vjp_flag = checked ? flag : nullptr;
-    float* dg = (float*)at(ws, c->lay.dg);
+    float* dg = (float*)at(ws, lay.dg);
     // time-grid gradient: t' and its scratch (partial sums of Phi^T a, of the <psi_j, k_l> terms, dtau_j, c_j, {Phi^T a, dt, dh})
     const bool tg = dt_host != nullptr;
-    float* tprime = tg ? (float*)at(ws, c->lay.tprime) : nullptr;
-    float* part_phi = tg ? (float*)at(ws, c->lay.tdots) : nullptr;
+    float* tprime = tg ? (float*)at(ws, lay.tprime) : nullptr;
+    float* part_phi = tg ? (float*)at(ws, lay.tdots) : nullptr;
     float* part_dh = tg ? part_phi + kDotBlocks : nullptr;
     float* dtau = tg ? part_phi + 2 * kDotBlocks : nullptr;
     float* cvec = tg ? dtau + 4 : nullptr;
@@ -496,8 +504,8 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     // dynamic scaling: log2 S, the first failed step and the bad-input mark live on the device (words 8..10 of the scalar slice);
     // the seed and the updates read the exponent there, one-thread kernels take Alg. 2's decisions, and the host reads the state
     // once, after the last step (again after every retry)
-    int* sstate = (int*)at(ws, c->lay.scal) + 8;
-    int* slog_exp = dynamic ? (int*)at(ws, c->lay.slog) : nullptr;
+    int* sstate = (int*)at(ws, lay.scal) + 8;
+    int* slog_exp = dynamic ? (int*)at(ws, lay.slog) : nullptr;
     int* slog_att = dynamic ? slog_exp + c->max_steps : nullptr;
     unsigned char* slog_dbl = dynamic ? (unsigned char*)(slog_att + c->max_steps) : nullptr;
     const int* e_dev = dynamic ? sstate : nullptr;
@@ -521,7 +529,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     volatile int* mirror_h = c->mirror_host;
 
     // Alg. 2 initialisation: a <- dL/dy_N, g <- 0 (or the caller's partial), then the initial scale
-    if (ws != c->ws_forward) cudaMemsetAsync(at(ws, c->lay.scal), 0, 256, st);     // a workspace no forward pass has prepared
+    if (ws != c->ws_forward) cudaMemsetAsync(at(ws, lay.scal), 0, 256, st);     // a workspace no forward pass has prepared
     cudaMemsetAsync(flag, 0, 8, st);
     launch_copy_amax(dL_dyT_dev, a, (long long)c->B * c->D, amax, flag, st, L);
     if (!accumulate_dtheta) launch_fill(g, 0.f, p, st, L);
@@ -535,15 +543,15 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         launch_scale_init(flag, amax, precision_bits(dt), e, c->pol.init_scale_exp_override == MPODE_NO_OVERRIDE ? 1 : 0, kExpMin, kExpMax,
                           sstate, mirror, st, L);
     }
-    c->v->prepare(st, ws, c->theta, c->probe, L);                                            // weights in low precision
+    v->prepare(st, ws, c->theta, c->probe, L);                                            // weights in low precision
     // fused kernels (one recompute launch per step, one VJP launch per attempt) where the velocity has them
     FusedSolve fs = fused_solve(c, nullptr);
-    const bool fused = c->v->fused_backward_begin(st, ws, fs, L);
+    const bool fused = v->fused_backward_begin(st, ws, fs, L);
     // Without finiteness decisions nothing of step i - 1's recompute depends on step i's adjoint.  The two fused launches of
     // every step then follow each other on the caller's stream (recompute of step i - 1 right behind the VJP launch of
     // step i, whose layer outputs it overwrites), and the small kernels between them (gradient finish, adjoint commit,
     // next seed) run beside the recompute on a second stream.
-    const bool all_done = fused && !dynamic && c->v->fused_backward_all(st, ws, fs, a, g, cot, e, vjp_flag, tprime, L);
+    const bool all_done = fused && !dynamic && v->fused_backward_all(st, ws, fs, a, g, cot, e, vjp_flag, tprime, L);
     if (all_done && log)
         for (int i = 0; i < N; ++i) { log->attempts[i] = 1; log->exp_used[i] = e; log->doubled[i] = 0; }
     bool overlap = fused && !checked && c->allow_side && !tg && !all_done;
@@ -562,7 +570,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         cudaEventRecord(c->ev_ready, st);
         cudaStreamWaitEvent(c->side, c->ev_ready, 0);
         sr = c->side;
-        c->v->fused_recompute(st, ws, fs, N - 1, L);
+        v->fused_recompute(st, ws, fs, N - 1, L);
     }
 
     int start = N - 1;                          // first step of this round of queueing (dynamic scaling: the step to repeat)
@@ -573,16 +581,16 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     // the stages of step i again (Alg. 2, recompute), and what else depends on them but not on the attempt
     auto queue_recompute = [&](int i) {
         StepTimes tm = step_times(c, i);
-        c->v->set_step(i, N);
+        v->set_step(i, N);
         recomputed = i;
         if (overlap) { /* queued on the second stream */ }
-        else if (fused) c->v->fused_recompute(st, ws, fs, i, L);
-        else run_stages(c, st, ws, i, tm);
-        if (tg && !(fused && c->v->fused_has_time_terms())) {      // Phi^T a_{i+1} with Phi = sum_j b_j k_j from the recomputed stages and the adjoint before its update
+        else if (fused) v->fused_recompute(st, ws, fs, i, L);
+        else run_stages(c, v, lay, st, ws, i, tm);
+        if (tg && !(fused && v->fused_has_time_terms())) {      // Phi^T a_{i+1} with Phi = sum_j b_j k_j from the recomputed stages and the adjoint before its update
             DotPairs pr{};
             pr.n = s;
             for (int j = 0; j < s; ++j) {
-                pr.x[j] = at(ws, c->lay.kbuf[j]); pr.ldx[j] = c->lay.ds; pr.y[j] = a; pr.y_f32[j] = 1; pr.ldy[j] = c->D; pr.coef[j] = (float)c->tb[j];
+                pr.x[j] = at(ws, lay.kbuf[j]); pr.ldx[j] = lay.ds; pr.y[j] = a; pr.y_f32[j] = 1; pr.ldy[j] = c->D; pr.coef[j] = (float)c->tb[j];
             }
             launch_dot_partial(dt, pr, c->B, c->d, part_phi, st, L);
         }
@@ -591,25 +599,25 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     for (int i = start; i >= 0 && !all_done; --i) {
         if (recomputed != i) queue_recompute(i);     // a repeated attempt finds its step's stages still in place
         StepTimes tm = step_times(c, i);
-        c->v->set_step(i, N);
+        v->set_step(i, N);
         const char* traj_i = (const char*)c->traj + (size_t)i * nBd * es;
         {
             if (tg) cudaMemsetAsync(dtau, 0, 4 * sizeof(float), st);
             // velocities that write kappa_{j-1} from their own epilogues (state without extra columns) get kappa_s from the seed
-            const bool kappa_in_vjp = !fused && c->D == c->d && c->v->can_write_next_kappa();
+            const bool kappa_in_vjp = !fused && c->D == c->d && v->can_write_next_kappa();
             const bool seeded_kappa = kappa_in_vjp;
-            if (!(fused && c->v->fused_seeds_itself(a, e, e_dev)))
-                launch_seed(dt, a, e, at(ws, c->lay.v), c->D > c->d ? at(ws, c->lay.vl) : nullptr, c->B, c->d, c->lay.ds, c->D,
-                        vjp_flag, sr, L, fused ? c->v->fused_kappa_last(ws) : (seeded_kappa ? at(ws, c->v->kappa_offset(c->lay)) : nullptr),
+            if (!(fused && v->fused_seeds_itself(a, e, e_dev)))
+                launch_seed(dt, a, e, at(ws, lay.v), c->D > c->d ? at(ws, lay.vl) : nullptr, c->B, c->d, lay.ds, c->D,
+                        vjp_flag, sr, L, fused ? v->fused_kappa_last(ws) : (seeded_kappa ? at(ws, v->kappa_offset(lay)) : nullptr),
                         (float)c->tb[s - 1], e_dev);                                             // seed Q16(S a)
             // without a finiteness decision the step gradient goes straight into g <- g + (h / S) dg
             if (overlap) {
                 cudaEventRecord(c->ev_rec, sr);                    // the seed of this step is ready
                 cudaStreamWaitEvent(st, c->ev_rec, 0);
-                c->v->fused_vjp(st, ws, fs, i, g, 1.f, (float)((double)tm.h * ldexp(1.0, -e)), vjp_flag, L, c->ev_vjp, sr);
-                if (i > 0) c->v->fused_recompute(st, ws, fs, i - 1, L);
-            } else if (fused && !checked) c->v->fused_vjp(st, ws, fs, i, g, 1.f, (float)((double)tm.h * ldexp(1.0, -e)), vjp_flag, L);
-            else if (fused) c->v->fused_vjp(st, ws, fs, i, dg, 0.f, 1.f, vjp_flag, L);
+                v->fused_vjp(st, ws, fs, i, g, 1.f, (float)((double)tm.h * ldexp(1.0, -e)), vjp_flag, L, c->ev_vjp, sr);
+                if (i > 0) v->fused_recompute(st, ws, fs, i - 1, L);
+            } else if (fused && !checked) v->fused_vjp(st, ws, fs, i, g, 1.f, (float)((double)tm.h * ldexp(1.0, -e)), vjp_flag, L);
+            else if (fused) v->fused_vjp(st, ws, fs, i, dg, 0.f, 1.f, vjp_flag, L);
             bool kappa_ready = seeded_kappa;          // stage s - 1: kappa = Q16(b_s v), written by the seed kernel
             for (int j = s - 1; j >= 0 && !fused; --j) {
                 Terms t{};
@@ -617,13 +625,13 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
                 for (int l = j + 1; l < s; ++l) {
                     double alj = c->ta[l * s + j];
                     if (alj != 0.0) {
-                        t.p[t.n] = at(ws, c->lay.psi[l]);
+                        t.p[t.n] = at(ws, lay.psi[l]);
                         t.c[t.n] = (float)((double)tm.h * alj);
                         ++t.n;
                     }
                 }
-                void* kappa = at(ws, c->v->kappa_offset(c->lay));
-                if (!kappa_ready) launch_kappa(dt, at(ws, c->lay.v), (float)c->tb[j], t, kappa, (long long)c->B * c->lay.ds, vjp_flag, st, L);
+                void* kappa = at(ws, v->kappa_offset(lay));
+                if (!kappa_ready) launch_kappa(dt, at(ws, lay.v), (float)c->tb[j], t, kappa, (long long)c->B * lay.ds, vjp_flag, st, L);
                 // can this stage's vector-Jacobian product also write kappa_{j-1}?  Yes when the tableau couples stage j - 1 to
                 // stage j alone (a_lj = 0 for l > j: Euler, midpoint, RK4, ...)
                 kappa_ready = false;
@@ -632,25 +640,25 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
                     for (int l = j; l < s; ++l) terms += c->ta[l * s + (j - 1)] != 0.0 ? 1 : 0;
                     if (terms == 1 && c->ta[j * s + (j - 1)] != 0.0) {
                         KappaNext kn;
-                        kn.out = kappa; kn.v = at(ws, c->lay.v); kn.bv = (float)c->tb[j - 1]; kn.c = (float)((double)tm.h * c->ta[j * s + (j - 1)]);
-                        c->v->set_next_kappa(kn);
+                        kn.out = kappa; kn.v = at(ws, lay.v); kn.bv = (float)c->tb[j - 1]; kn.c = (float)((double)tm.h * c->ta[j * s + (j - 1)]);
+                        v->set_next_kappa(kn);
                         kappa_ready = true;
                     }
                 }
                 if (c->D > c->d) {
                     Terms none{};
-                    launch_kappa(dt, at(ws, c->lay.vl), (float)c->tb[j], none, at(ws, c->lay.kappal), c->B, vjp_flag, st, L);
+                    launch_kappa(dt, at(ws, lay.vl), (float)c->tb[j], none, at(ws, lay.kappal), c->B, vjp_flag, st, L);
                 }
-                const void* yin = (j > 0 || c->v->needs_input_copy()) ? (const void*)at(ws, c->lay.ybuf[j]) : (const void*)traj_i;
-                c->v->vjp(st, ws, j, yin, tm.tau16[j], at(ws, c->lay.psi[j]), dg, j == s - 1 ? 0.f : 1.f, vjp_flag, L);
+                const void* yin = (j > 0 || v->needs_input_copy()) ? (const void*)at(ws, lay.ybuf[j]) : (const void*)traj_i;
+                v->vjp(st, ws, j, yin, tm.tau16[j], at(ws, lay.psi[j]), dg, j == s - 1 ? 0.f : 1.f, vjp_flag, L);
             }
-            if (tg && !(fused && c->v->fused_time_terms(st, tvals, vjp_flag, L))) {      // dt = sum_j dtau_j, dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>); Q16(dt), Q16(dh) join the test
+            if (tg && !(fused && v->fused_time_terms(st, tvals, vjp_flag, L))) {      // dt = sum_j dtau_j, dh = sum_j (c_j dtau_j + sum_{l<j} a_jl <psi_j, k_l>); Q16(dt), Q16(dh) join the test
                 DotPairs pr{};
                 for (int j = 1; j < s; ++j)
                     for (int l = 0; l < j; ++l)
                         if (c->ta[j * s + l] != 0.0 && pr.n < 8) {
                             const int q = pr.n++;
-                            pr.x[q] = at(ws, c->lay.psi[j]); pr.ldx[q] = c->lay.ds; pr.y[q] = at(ws, c->lay.kbuf[l]); pr.y_f32[q] = 0; pr.ldy[q] = c->lay.ds;
+                            pr.x[q] = at(ws, lay.psi[j]); pr.ldx[q] = lay.ds; pr.y[q] = at(ws, lay.kbuf[l]); pr.y_f32[q] = 0; pr.ldy[q] = lay.ds;
                             pr.coef[q] = (float)c->ta[j * s + l];
                         }
                 launch_dot_partial(dt, pr, c->B, c->d, part_dh, st, L);
@@ -661,14 +669,14 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         // high-precision updates of a and g with h / S (exact in fp32: a power-of-two scaling of h)
         Terms ps{};
         ps.n = s;
-        for (int j = 0; j < s; ++j) { ps.p[j] = at(ws, c->lay.psi[s - 1 - j]); ps.c[j] = 1.f; }
+        for (int j = 0; j < s; ++j) { ps.p[j] = at(ws, lay.psi[s - 1 - j]); ps.c[j] = 1.f; }
         const float* cot_i = cot ? cot + (size_t)i * c->B * c->D : nullptr;
         if (dynamic) {
             // queued at once: they skip themselves while the flag is raised, take 2^-e from the device, and the decision kernel
             // behind them records the attempt (growth test on the new ||a||_inf) or the failure
             cudaMemsetAsync(amax, 0, 4, st);
             if (tg) launch_tgrad_update(tprime, i, tvals, tm.h, flag, st, L, e_dev);        // before a changes: it holds Phi^T a_{i+1} already
-            launch_commit_a(dt, a, ps, tm.h, c->B, c->d, c->lay.ds, c->D, amax, st, L, flag, cot_i, e_dev);
+            launch_commit_a(dt, a, ps, tm.h, c->B, c->d, lay.ds, c->D, amax, st, L, flag, cot_i, e_dev);
             launch_commit_g(g, dg, tm.h, p, st, L, flag, e_dev);
             launch_scale_decide(flag, amax, sstate, mirror, i, i == fail_step ? fail_count + 1 : 1, c->pol.growth_rule, precision_bits(dt),
                                 kExpMin, kExpMax, slog_exp, slog_att, slog_dbl, st, L);
@@ -696,7 +704,7 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
         } else {
             float coef = (float)((double)tm.h * ldexp(1.0, -e));
             if (tg) launch_tgrad_update(tprime, i, tvals, coef, nullptr, st, L);
-            launch_commit_a(dt, a, ps, coef, c->B, c->d, c->lay.ds, c->D, nullptr, sr, L, nullptr, cot_i);
+            launch_commit_a(dt, a, ps, coef, c->B, c->d, lay.ds, c->D, nullptr, sr, L, nullptr, cot_i);
             if (!(fused && !checked)) launch_commit_g(g, dg, coef, p, st, L);
             if (log) { log->attempts[i] = 1; log->exp_used[i] = e; log->doubled[i] = 0; }
         }
@@ -770,6 +778,17 @@ mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_
     dev_err |= fwd_err;
     if (dev_err != 0u) return fail(c, MPODE_ERR_CUDA, "a device-side wait timed out (code " + std::to_string(dev_err) + ")");
     return rs;
+}
+
+mpode_status mpode_backward(mpode_ctx* c, void* cuda_stream, const float* dL_dyT_dev, float* a, float* g,
+                            int accumulate_dtheta, mpode_scale_log* log, void* ws, size_t ws_bytes) {
+    return mpode_backward_ex(c, cuda_stream, dL_dyT_dev, nullptr, a, g, accumulate_dtheta, nullptr, log, ws, ws_bytes);
+}
+
+mpode_status mpode_backward_ex(mpode_ctx* c, void* cuda_stream, const float* dL_dyT_dev, const float* cot, float* a, float* g,
+                               int accumulate_dtheta, float* dt_host, mpode_scale_log* log, void* ws, size_t ws_bytes) {
+    if (!c) return MPODE_ERR_INVALID_ARG;
+    return run_backward(c, c->v, c->lay, cuda_stream, dL_dyT_dev, cot, a, g, accumulate_dtheta, dt_host, log, ws, ws_bytes);
 }
 
 mpode_status mpode_forward_host(mpode_ctx* c, void* cuda_stream, const float* theta_host, const float* y0_host,
@@ -850,9 +869,11 @@ mpode_status static_workspace_address(mpode_ctx* c, int dev, void** out) {
 mpode_status mpode_backward_static_workspace(mpode_ctx* c, void* cuda_stream, const float* dL_dyT_dev, float* dL_dy0_dev,
                                              float* dL_dtheta_dev, int accumulate_dtheta, mpode_scale_log* log) {
     if (!c) return MPODE_ERR_INVALID_ARG;
-    if (c->lay.total > (size_t)MPODE_STATIC_WORKSPACE_BYTES)
+    Velocity* v = c->v_compact != nullptr ? c->v_compact : c->v;
+    const Layout& lay = c->v_compact != nullptr ? c->lay_compact : c->lay;
+    if (lay.total > (size_t)MPODE_STATIC_WORKSPACE_BYTES)
         return fail(c, MPODE_ERR_WORKSPACE_TOO_SMALL,
-                    "this context needs " + std::to_string(c->lay.total) + " bytes of workspace, the static workspace holds " +
+                    "this context needs " + std::to_string(lay.total) + " bytes of workspace, the static workspace holds " +
                         std::to_string((size_t)MPODE_STATIC_WORKSPACE_BYTES));
     // everything mpode_backward would refuse is refused here first, so that an invalid call queues nothing on the stream
     if (!c->have_forward) return fail(c, MPODE_ERR_BAD_STATE, "mpode_backward needs a preceding mpode_forward");
@@ -874,9 +895,9 @@ mpode_status mpode_backward_static_workspace(mpode_ctx* c, void* cuda_stream, co
     if (s != MPODE_OK) return s;
     // the array keeps the previous call's contents: the scalar words (non-finite flag, norm, device error word) must
     // start at zero; every other slice is written by the backward pass before it is read
-    cudaMemsetAsync((char*)ws + c->lay.scal, 0, 256, (cudaStream_t)cuda_stream);
+    cudaMemsetAsync((char*)ws + lay.scal, 0, 256, (cudaStream_t)cuda_stream);
     c->allow_side = false;      // no second stream here: creating one may allocate
-    s = mpode_backward(c, cuda_stream, dL_dyT_dev, dL_dy0_dev, dL_dtheta_dev, accumulate_dtheta, log, ws, c->lay.total);
+    s = run_backward(c, v, lay, cuda_stream, dL_dyT_dev, nullptr, dL_dy0_dev, dL_dtheta_dev, accumulate_dtheta, nullptr, log, ws, lay.total);
     c->allow_side = true;
     return s;
 }

@@ -55,7 +55,7 @@ GemmArgs base_args(void* ws, const Layout* lay) {
 // ---------------------------------------------------------------------------------------------------- MLP
 class MlpVelocity : public Velocity {
 public:
-    MlpVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps) : B_(B), dt_(dt), act_(v.act),
+    MlpVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps, bool compact) : B_(B), dt_(dt), compact_(compact), act_(v.act),
         time_(v.append_time != 0), bias_(v.has_bias != 0), L_(v.n_layers), max_steps_(max_steps),
         w_(v.widths, v.widths + v.n_layers + 1) {
         size_t off = 0;
@@ -69,7 +69,7 @@ public:
         p_ = off;
         // 16-bit formats: every internal row length is rounded up to 8 elements (16 bytes, what a bulk tensor copy needs); the pad
         // columns of weights, biases, states and cotangents are zero, so that they add nothing to any sum
-        for (int w : w_) wp_.push_back(dt_ == MPODE_F32 ? w : (w + 7) / 8 * 8);
+        for (int w : w_) wp_.push_back(dt_ == MPODE_F32 || compact_ ? w : (w + 7) / 8 * 8);
     }
     size_t param_count() const override { return p_; }
 
@@ -163,7 +163,7 @@ public:
         small_w_.clear();
         for (int w : w_) small_w_.push_back((w + 7) / 8 * 8);
         // (the float32 buffers of the other paths are not padded: the state's rows have to agree)
-        small_ok_ = !tiny_ok_ && (dt_ != MPODE_F32 || w_[0] % 8 == 0) && small_mlp_supported(dt_, B_, L_, small_w_.data());
+        small_ok_ = !compact_ && !tiny_ok_ && (dt_ != MPODE_F32 || w_[0] % 8 == 0) && small_mlp_supported(dt_, B_, L_, small_w_.data());
         small_bwd_ok_ = small_ok_ && small_backward_supported(dt_, B_);
         if (!small_ok_) return;
         const size_t es = low_size(dt_);
@@ -395,6 +395,7 @@ public:
     // ---- fused Runge-Kutta path (16-bit formats, state width a multiple of 8; hidden widths are padded to one)
     virtual bool fused_shape_ok() const {
         if (dt_ != MPODE_BF16 && dt_ != MPODE_F16) return false;
+        for (int w : wp_) if (w % 8 != 0) return false;
         return L_ <= 4 && w_[0] % 8 == 0;
     }
     // output-tile width of a contraction with N columns: wide tiles for the tensor pipe, narrower ones when that
@@ -782,6 +783,7 @@ public:
 protected:
     int B_;
     mpode_dtype dt_;
+    bool compact_;
     int act_;
     bool time_, bias_;
     int L_;
@@ -823,7 +825,7 @@ protected:
 // rows [0, B) carry the state, rows [B, 2B) the forward-mode tangent started at the probe (Sec. 6.1).
 class CnfVelocity : public MlpVelocity {
 public:
-    CnfVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps) : MlpVelocity(v, B, dt, max_steps) {}
+    CnfVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps, bool compact) : MlpVelocity(v, B, dt, max_steps, compact) {}
     bool fused_shape_ok() const override { return false; }
     bool tiny_shape_ok() const override { return false; }
     bool supports_time_gradient() const override { return false; }
@@ -1373,13 +1375,13 @@ private:
 // (hyper_cnf.cu) where the weight sets do not fit shared memory.
 class HyperCnfVelocity : public Velocity {
 public:
-    HyperCnfVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps) : B_(B), dt_(dt), d_(v.d), h_(v.widths[0]),
-        w_(v.widths[1]), max_steps_(max_steps) {}
+    HyperCnfVelocity(const mpode_velocity_desc& v, int B, mpode_dtype dt, int max_steps, bool compact) : B_(B), dt_(dt), d_(v.d), h_(v.widths[0]),
+        w_(v.widths[1]), max_steps_(max_steps), compact_(compact) {}
     size_t param_count() const override { return hyper_param_count(h_, w_, d_); }
     void plan(Layout& lay) override {
         const size_t es = low_size(dt_);
         plan_common(lay, B_, d_, true, param_count(), dt_, 1);
-        whole_ = hyper_solve_shape_ok(dt_, h_, w_, d_, RK_MAX_STAGES);
+        whole_ = !compact_ && hyper_solve_shape_ok(dt_, h_, w_, d_, RK_MAX_STAGES);
         if (whole_) {
             // the hypernetwork's layers and weight sets for every stage time of a solve; per-step scalars; scratch of the backward pass
             table_ = lay.take((size_t)max_steps_ * RK_MAX_STAGES * hyper_stage_floats(h_, w_, d_) * sizeof(float));
@@ -1462,6 +1464,7 @@ private:
     mpode_dtype dt_;
     int d_, h_, w_;
     int max_steps_;
+    bool compact_;
     bool whole_ = false;                   // whole-solve kernels
     size_t hyp_[4] = {0}, units_[4] = {0}, sbar_ = 0, part_ = 0, tpart_ = 0, table_ = 0, scal_ = 0, log_ = 0;
     const float* theta_ = nullptr;
@@ -1481,14 +1484,14 @@ public:
 
 }  // namespace
 
-Velocity* make_velocity(const mpode_velocity_desc& desc, int batch, mpode_dtype low, int max_steps) {
+Velocity* make_velocity(const mpode_velocity_desc& desc, int batch, mpode_dtype low, int max_steps, bool compact) {
     switch (desc.kind) {
-        case MPODE_VEL_MLP: return new Bound<MlpVelocity>(desc, batch, low, max_steps);
-        case MPODE_VEL_CNF_MLP: return new Bound<CnfVelocity>(desc, batch, low, max_steps);
+        case MPODE_VEL_MLP: return new Bound<MlpVelocity>(desc, batch, low, max_steps, compact);
+        case MPODE_VEL_CNF_MLP: return new Bound<CnfVelocity>(desc, batch, low, max_steps, compact);
         case MPODE_VEL_CONV3X3_2: return new Bound<ConvVelocity>(desc, batch, low, max_steps);
         case MPODE_VEL_PARABOLIC_CONV: return new Bound<ParabolicVelocity>(desc, batch, low, max_steps);
         case MPODE_VEL_SCALAR_POLY: return batch <= TINY_MAX_B ? new Bound<ScalarPolyVelocity>(desc, batch, low, max_steps) : nullptr;
-        case MPODE_VEL_CNF_HYPER: return new Bound<HyperCnfVelocity>(desc, batch, low, max_steps);
+        case MPODE_VEL_CNF_HYPER: return new Bound<HyperCnfVelocity>(desc, batch, low, max_steps, compact);
     }
     return nullptr;
 }

@@ -130,6 +130,7 @@ public:
     virtual void* fused_kappa_last(void* ws) const { return nullptr; }
 };
 
-Velocity* make_velocity(const mpode_velocity_desc& desc, int batch, mpode_dtype low, int max_steps);
+// compact: without what asks for more workspace than the general paths do (padded rows, row-local kernels, whole-solve kernels of the flows)
+Velocity* make_velocity(const mpode_velocity_desc& desc, int batch, mpode_dtype low, int max_steps, bool compact = false);
 
 }  // namespace mpode

@@ -118,6 +118,31 @@ def test_static_workspace_dynamic_scaling_without_the_mapped_state_words():
     assert st_ref["step_waits"] > 0 and st_s["step_waits"] == 0 and st_s["host_syncs"] >= wl.n_steps + st_s["retries"]
 
 
+@pytest.mark.parametrize("kind,batch,d,hidden,low", [("mlp", 1800, 64, 256, "f32"), ("mlp", 4350, 9, 301, "bf16"), ("cnf", 3650, 9, 121, "f16")])
+def test_static_workspace_takes_contexts_whose_general_paths_fit(kind, batch, d, hidden, low):
+    # The paths a context usually takes (layer inputs and cotangents of a whole step on the chip, padded rows) need more than the static
+    # workspace holds, the general ones do not: the entry point runs those, and gives what mpode_backward gives
+    import torch
+    from paper_2510_23498_b200 import binding
+    wl = inputs.mlp_block(batch=batch, n_steps=2, d=d, hidden=hidden) if kind == "mlp" else inputs.cnf_mlp(batch=batch, n_steps=2, d=d, hidden=hidden)
+    ctx = binding.Context(wl.vel, wl.batch, wl.n_steps, low=low, scaling="dynamic" if low == "f16" else "none")
+    assert ctx.workspace_bytes > binding.STATIC_WORKSPACE_BYTES
+    theta, y0 = torch.from_numpy(wl.theta).to(ctx.device), torch.from_numpy(wl.y0).to(ctx.device)
+    probe = None if wl.probe is None else torch.from_numpy(wl.probe).to(ctx.device)
+    _, yT = ctx.forward(theta, y0, wl.tgrid, wl.solver, probe)
+    _, dl = wl.loss(yT.cpu().numpy().astype(np.float64))
+    dl = torch.from_numpy(dl.astype(np.float32)).to(ctx.device)
+    a_ref, g_ref, _, _ = ctx.backward(dl)
+    for _ in range(2):
+        a0, g, st = ctx.backward_static_workspace(dl)
+        torch.cuda.synchronize()
+        assert st == 0
+        assert rel_l2(a0.cpu().numpy(), a_ref.cpu().numpy()) <= TOL[low] and rel_l2(g.cpu().numpy(), g_ref.cpu().numpy()) <= TOL[low]
+    a1, g1, _, _ = ctx.backward(dl)                     # and the context's own path is as before
+    assert torch.equal(a1, a_ref) and torch.equal(g1, g_ref)
+    ctx.close()
+
+
 def test_static_workspace_refuses_invalid_calls_before_queueing_work():
     import torch
     from paper_2510_23498_b200 import binding
