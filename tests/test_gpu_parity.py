@@ -88,7 +88,8 @@ def test_c3_mlp_block_reduced_batch_bf16(batch, n_steps):
 
 @pytest.mark.parametrize("batch", [127, 129, 255, 300, 513])
 def test_fused_kernels_on_ragged_row_blocks(batch):
-    # batches around multiples of the 128-row tile; widths that leave ragged column tiles (200 = 3 x 64 + 8, 72 = 64 + 8)
+    # batches around multiples of the 128-row tile; widths that leave ragged column tiles (200 = 3 x 64 + 8, 72 = 64 + 8).  The row-local
+    # kernels run these; the fused program's are in test_gpu_fused_path.py
     _check(inputs.mlp_block(batch=batch, n_steps=2, d=72, hidden=200))
 
 
@@ -209,7 +210,8 @@ def test_forced_overflow_gives_identical_retry_sequence():
 
 
 def test_forced_overflow_on_the_fused_tensor_core_path():
-    # same state machine, but the finiteness flags now come from the fused kernel's epilogues and the retries relaunch it
+    # same state machine, but the finiteness flags come from the row-local kernels' epilogues and the retries relaunch them (the fused
+    # program and the layer-by-layer path: test_gpu_fused_path.py)
     wl = inputs.mlp_block(batch=96, n_steps=3, d=64, hidden=160)
     gpu, orc, _ = _check(wl, "f16", "dynamic", k_max=60, init_scale_exp_override=40)
     assert max(gpu["log"]["attempts"]) > 1 and gpu["stats"]["retries"] == sum(k - 1 for k in gpu["log"]["attempts"])
@@ -218,7 +220,7 @@ def test_forced_overflow_on_the_fused_tensor_core_path():
 
 
 def test_dynamic_scaling_decisions_are_taken_on_the_device():
-    # layer-by-layer / fused path (not the whole-solve kernel): the scale, the accept / halve / double decisions and the log live
+    # row-local kernels (not the whole-solve kernel; the other paths are in test_gpu_fused_path.py): the scale, the accept / halve / double decisions and the log live
     # on the device; a pass without overflow drains the stream once, every overflowing attempt costs one more drain
     wl = inputs.mlp_block(batch=130, n_steps=4, d=72, hidden=200)
     gpu, _, _ = _check(wl, "f16", "dynamic", init_scale_exp_override=0)
@@ -246,7 +248,7 @@ def test_scale_failure_is_a_status_not_a_trap():
 
 
 def test_scale_failure_on_the_layer_path_reports_the_step_and_leaves_the_context_usable():
-    # not the whole-solve kernel: the device-side state machine halves k_max times at the first step, the host gives up there
+    # row-local kernels, not the whole-solve kernel: the device-side state machine halves k_max times at the first step, the host gives up there
     wl = inputs.mlp_block(batch=130, n_steps=3, d=72, hidden=200)
     gpu = run_gpu(wl, "f16", "dynamic", k_max=3, init_scale_exp_override=40)
     orc = run_oracle(wl, "f16", "dynamic", k_max=3, init_scale_exp_override=40)
@@ -442,7 +444,7 @@ def test_trajectory_aligned_to_16_bytes_only_takes_the_layer_by_layer_path_at_pa
     gpu = dict(yT=yT.cpu().numpy(), traj=traj.float().cpu().numpy(), a0=a0.cpu().numpy(), g=g.cpu().numpy())
     assert_parity(gpu, orc, TOL[wl.low])
     ctx.close()
-    # the same workload with an aligned trajectory runs fused
+    # the same workload with an aligned trajectory runs the row-local kernels
     ref = run_gpu(wl)
     assert ref["stats"]["fused_launches"] > 0 and ref["stats"]["tc_contractions"] == 0 and ref["stats"]["simt_contractions"] == 0
 

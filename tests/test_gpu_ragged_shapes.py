@@ -29,6 +29,7 @@ def test_flow_with_odd_widths_runs_on_the_tensor_cores(batch, d, hidden, low):
     assert gpu["stats"]["simt_contractions"] == 0 and gpu["stats"]["tc_contractions"] > 0
 
 
+# the same for MLPs (of these sizes on the row-local kernels; the padded fused program and layer-by-layer path are in test_gpu_fused_path.py)
 @pytest.mark.parametrize("batch,d,hidden,low", [(200, 64, 137, "bf16"), (130, 33, 100, "bf16"), (257, 71, 65, "f16"), (128, 9, 72, "f16")])
 def test_mlp_with_odd_widths_runs_on_the_tensor_cores(batch, d, hidden, low):
     wl = inputs.mlp_block(batch=batch, n_steps=2, d=d, hidden=hidden)

@@ -62,10 +62,10 @@ def test_mlp_block_fused_path_time_gradient_and_running_cost(batch, d, hidden, n
 
 def test_mlp_block_layer_by_layer_paths_time_gradient():
     wl = inputs.mlp_block(batch=96, n_steps=3, d=64, hidden=160)
-    _check(wl, "f16", "dynamic")                       # fused kernels, finiteness test extended by Q16(dt), Q16(dh)
+    _check(wl, "f16", "dynamic")                       # row-local kernels, finiteness test extended by Q16(dt), Q16(dh)
     wl.solver = "kutta3"
     wl.tgrid = np.array([0.0, 0.2, 0.55, 1.0], dtype=np.float32)
-    _check(wl, "f32", "none", exact=True)              # CUDA-core float32 path, another tableau, non-uniform grid
+    _check(wl, "f32", "none", exact=True)              # the same in float32, another tableau, non-uniform grid
 
 
 def test_scalar_example_time_gradient_matches_oracle_and_the_analytic_end_point_derivative():

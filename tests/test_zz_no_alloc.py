@@ -34,7 +34,7 @@ def _forward_and_reference(wl):
 def test_static_workspace_backward_matches_backward_on_two_calls_in_a_row():
     import torch
     from paper_2510_23498_b200 import binding
-    wl = inputs.mlp_block(batch=200, n_steps=3, d=64, hidden=128)                    # fused tensor-core path, bf16
+    wl = inputs.mlp_block(batch=200, n_steps=3, d=64, hidden=128)                    # row-local kernels, bf16
     wl2 = inputs.toy_mlp(batch=64, n_steps=4, hidden=16)                             # fp16, dynamic adjoint scaling
     ctx, dl, a_ref, g_ref, keep = _forward_and_reference(wl)
     ctx2, dl2, a_ref2, g_ref2, keep2 = _forward_and_reference(wl2)
@@ -59,7 +59,7 @@ def test_static_workspace_backward_allocates_no_device_memory_and_keeps_the_scal
     import ctypes as C
     import torch
     wl = inputs.toy_mlp(batch=64, n_steps=4, hidden=16)                              # fp16, dynamic adjoint scaling
-    wl2 = inputs.mlp_block(batch=200, n_steps=3, d=64, hidden=128)                   # fused tensor-core path, bf16
+    wl2 = inputs.mlp_block(batch=200, n_steps=3, d=64, hidden=128)                   # row-local kernels, bf16
     for w in (wl, wl2):
         ctx, dl, a_ref, g_ref, keep = _forward_and_reference(w)
         _, _, log_ref, _ = ctx.backward(dl)
@@ -85,7 +85,7 @@ def test_static_workspace_backward_allocates_no_device_memory_and_keeps_the_scal
 
 
 def test_static_workspace_dynamic_scaling_without_the_mapped_state_words():
-    # Fused / layer-by-layer kernels (not the whole-solve kernel) under dynamic scaling with overflowing attempts.  A context
+    # Row-local kernels (not the whole-solve kernel) under dynamic scaling with overflowing attempts.  A context
     # whose only backward calls go through this entry point has no mapped copy of the device's scale state (creating it would
     # allocate) and reads the decisions back after every step; the result and the scale log are those of mpode_backward.
     import ctypes as C
