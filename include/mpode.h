@@ -17,11 +17,12 @@
  *     "high" is float32.  All rounding is round-to-nearest-even.
  *   - The device never traps: numerical failures are reported as status codes.
  *   - Dense velocities in the 16-bit formats run as persistent kernels with one thread block per SM whose blocks hand tiles
- *     to each other through counters in the workspace.  They expect the GPU to themselves for the duration of a call: if
+ *     to each other through counters in the workspace (small networks excepted, whose blocks are independent), and the backward pass of
+ *     a hypernetwork flow is one cooperative kernel with grid barriers.  They expect the GPU to themselves for the duration of a call: if
  *     other work keeps some SMs occupied for seconds, a block's bounded wait (2 s) gives up and the call returns
  *     MPODE_ERR_CUDA with "a device-side wait timed out" instead of hanging.  mpode_backward may use a second, internal
  *     stream for part of its work; everything is joined to `cuda_stream` before the call returns.
- *   - These kernels move 32-byte pieces of trajectory rows: with a trajectory pointer that is only 16-byte aligned the
+ *   - The kernels of dense velocities move 32-byte pieces of trajectory rows: with a trajectory pointer that is only 16-byte aligned the
  *     library silently takes its layer-by-layer path.
  */
 #ifndef MPODE_H_
@@ -151,8 +152,9 @@ typedef struct {
     long long host_syncs;          /* times the last call waited for its stream to drain */
     long long tc_contractions;     /* layer-by-layer contractions that ran on the tensor-core kernels */
     long long simt_contractions;   /* layer-by-layer contractions that ran on the CUDA-core kernel (float32 mode, odd shapes) */
-    long long fused_launches;      /* launches of the fused Runge-Kutta kernel (whole steps on the tensor cores) */
-    long long whole_solve_launches;/* launches of the whole-solve kernels for very small networks */
+    long long fused_launches;      /* launches of the fused Runge-Kutta kernel (whole steps on the tensor cores) and of the row-local kernels
+                                      of small dense networks */
+    long long whole_solve_launches;/* launches of the whole-solve kernels for very small networks and hypernetwork flows */
     long long step_waits;          /* dynamic scaling: waits for the decision of a step, taken on the device, while the recompute of the
                                       next step is already queued (the stream keeps work) */
 } mpode_stats;

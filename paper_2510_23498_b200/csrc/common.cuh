@@ -275,8 +275,6 @@ void launch_fill_low(mpode_dtype dt, void* x, float v, long long n, cudaStream_t
 constexpr int kColsumCounters = 32;   // column blocks a one-launch column sum can count (words of the caller's `counters`)
 int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* partial, float* dst1, long long s1, float* dst2,
                   long long s2, float scale2, float beta, cudaStream_t st, long long* launches, unsigned* counters = nullptr);
-// column sums of a low-format [M, N] matrix per group of 128 rows (the layout the fused backward kernel also writes)
-void launch_colsum_groups(mpode_dtype dt, const void* x, int M, int N, float* out, cudaStream_t st, long long* launches);
 // out[m * ldo + n] = (beta ? out : 0) + sum_z partial[z][m][n], z in ascending order
 void launch_splitk_reduce(const float* partial, int S, int M, int N, float* out, long long ldo, float beta, cudaStream_t st,
                           long long* launches, int crop_m = 0, int crop_n = 0);

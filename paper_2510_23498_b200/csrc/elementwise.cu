@@ -715,19 +715,6 @@ __global__ void colsum_final_kernel(const float* __restrict__ partial, int R, in
     if (dst2 != nullptr) dst2[c * s2] = (beta != 0.f ? dst2[c * s2] : 0.f) + scale2 * s;
 }
 
-// Column sums of a low-format [M, N] matrix per group of 128 rows: out[g][n] = sum_{r in group g} x[r][n]
-template <typename T>
-__global__ void colsum_groups_kernel(const T* __restrict__ x, int M, int N, float* __restrict__ out) {
-    chain_begin();
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    int g = blockIdx.y;
-    if (n >= N) return;
-    int r0 = g * 128, r1 = min(M, r0 + 128);
-    float s = 0.f;
-    for (int r = r0; r < r1; ++r) s += Low<T>::to_f(x[(long long)r * N + n]);
-    out[(long long)g * N + n] = s;
-}
-
 // Step parameter gradient from the fused kernel's scratch (see GradFinishArgs): blockIdx.y = layer; the first
 // blocks of a layer walk its weight elements, the last ones its bias / time-column entries (one warp per entry,
 // lanes split the (stage, row block) terms and are combined by a fixed shuffle tree).
@@ -1411,9 +1398,10 @@ void launch_tgrad_update(float* tprime, int i, const float* vals, float coef, co
 int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* partial, float* dst1, long long s1, float* dst2,
                   long long s2, float scale2, float beta, cudaStream_t st, long long* launches, unsigned* counters) {
     int col_blocks = (N + kColsPerBlock - 1) / kColsPerBlock;
-    // Beyond kClusterRows a warp's rows are more than four trips to memory and more chunks are the better use of the SMs: training pass of
-    // flows, this / chunks, 63-1024-1024-63 with 512 samples 4.24 / 4.39 ms, 784-2048-2048-784 with 2048 6.45 / 6.50, 64-256-256-64 with
-    // 4096 4.53 / 4.29 and with 8192 5.84 / 5.22.
+    // Beyond kClusterRows a warp's rows are more than four trips to memory and more chunks are the better use of the SMs.  Training passes, ms
+    // this / chunks at 512, 1024, 2048, 3072, 4096 and 8192 samples: flow 63-256-256-63 (4 RK4 steps) 1.68 / 1.74, 1.82 / 1.88, 1.87 / 1.85, 2.27 / 2.22,
+    // 2.43 / 2.30, 3.08 / 2.76; flow 63-1024-1024-63 2.20 / 2.28, 2.76 / 2.81, 2.92 / 2.90, 3.87 / 3.84, 4.11 / 4.05, 6.49 / 6.20; MLP 33-500-500-33 (8 steps)
+    // 3.47 / 3.62, 3.75 / 3.86, 4.04 / 3.99, 4.59 / 4.43, 4.86 / 4.55, 6.40 / 5.56; flow 784-2048-2048-784 at 2048 6.47 / 6.52.
     if (M <= kClusterRows) {
         const int rows = (M + kColsumCluster - 1) / kColsumCluster;
         MPODE_DISPATCH_T(dt, T, (launch_chain(colsum_cluster_kernel<T>, dim3(col_blocks, kColsumCluster), dim3(kThreads), 0, st, (const T*)x, M, N, ld, rows, partial, dst1, s1, dst2,
@@ -1439,12 +1427,6 @@ int launch_colsum(mpode_dtype dt, const void* x, int M, int N, int ld, float* pa
         COUNT(launches);
     }
     return R;
-}
-
-void launch_colsum_groups(mpode_dtype dt, const void* x, int M, int N, float* out, cudaStream_t st, long long* launches) {
-    dim3 grid((N + 127) / 128, (M + 127) / 128);
-    MPODE_DISPATCH_T(dt, T, (launch_chain(colsum_groups_kernel<T>, dim3(grid), dim3(128), 0, st, (const T*)x, M, N, out)));
-    COUNT(launches);
 }
 
 void launch_grad_finish(const GradFinishArgs& a, cudaStream_t st, long long* launches) {

@@ -51,8 +51,8 @@ extern thread_local Profiler* tl_profiler;
 struct PathCounters {
     long long tc = 0;      // layer-by-layer contractions on the tensor-core kernels
     long long simt = 0;    // layer-by-layer contractions on the CUDA-core kernel
-    long long fused = 0;   // launches of the fused Runge-Kutta kernel
-    long long whole = 0;   // launches of the whole-solve kernels for very small networks
+    long long fused = 0;   // launches of the fused Runge-Kutta kernel and of the row-local kernels
+    long long whole = 0;   // launches of the whole-solve kernels (very small networks, hypernetwork flows)
 };
 extern thread_local PathCounters* tl_counters;
 

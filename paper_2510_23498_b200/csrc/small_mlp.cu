@@ -1,14 +1,14 @@
 // Row-local kernels for small dense velocities.  Samples are independent through the time loop, so a block
 // takes 16 (or 32) of them through the whole forward solve, or through the backward chain of several steps, without talking to any
-// other block: a layer is one contraction [16 x K] x [K x N] whose operands never leave the SM (activations in shared memory, weights
-// through L1), and the next layer starts after a block barrier.  What bounds this is the chain of layers, not bytes or tensor rate:
+// other block: a layer is one contraction [16 x K] x [K x N] whose activations never leave the SM (the weights come from L2 through a
+// ring of buffers in shared memory), and the next layer starts after a block barrier.  What bounds this is the chain of layers, not bytes or tensor rate:
 // a tcgen05 tile needs 128 rows (64 at half rate) and a hand-over between its epilogue and the next tile's operands, about 8 us per
 // layer in rk_fused.cu, while mma.sync fragments of 16 rows spread the batch over the SMs and hand over in registers and shared memory.
 // float32 runs the same program on the CUDA cores, 8 rows to a block, bound by the weights' way from L2 (about 64 bytes a cycle).
 // Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
 // second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
-// Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.5 -> 2.75 ms; MLP
-// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.7 -> 5.5 ms.
+// Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.6 -> 2.96 ms; MLP
+// 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.6 -> 4.77 ms.
 #include "small_mlp.h"
 
 #include "profiler.h"
@@ -990,6 +990,14 @@ size_t small_pack_bytes(mpode_dtype dt, int L, const int* wp) {
     return n * low_size(dt);
 }
 
+// Shared memory draws the first line: a block's rows and three ring buffers have to fit (32-512-512-32 does; a state width of 256 or a hidden width of 1024 does not).  Then the
+// weights, since every block streams all of them: training pass of 8 RK4 steps, ms here / other path (fused program; float32: layer by
+// layer), bf16 at 200, 1000 and 2300 samples: 128-256-256-128 (128 K weights) 1.03 / 1.65, 1.24 / 1.71, 1.54 / 1.80; 64-384-384-64 (192 K)
+// 1.47 / 1.71, 1.66 / 1.77, 1.97 / 1.92; 32-512-512-32 (288 K) 1.77 / 1.74, 2.03 / 1.79, 2.41 / 1.97.  float32 at 64, 500, 1024 and 2300: 64-256-256-64
+// (96 K) 2.19 / 3.88, 2.50 / 4.16, 2.90 / 4.45, 5.06 / 6.35; 128-384-384-128 (240 K) 4.42 / 4.47, 4.80 / 5.12, 5.25 / 6.54, 8.93 / 10.5 (the forward pass
+// of 64 samples alone 1.39 / 1.15, of 2300 2.17 / 2.75); 64-512-512-64 (320 K) 5.52 / 3.83, 5.98 / 5.15, 6.53 / 7.02, 11.3 / 11.2.  And the batch,
+// at one block of two row tiles per SM: with a second round of blocks at 3000 samples, float32, 8.62 / 8.26 (96 K), 16.2 / 11.9 (240 K),
+// 20.5 / 14.8 (320 K); the 16-bit forward pass at 4700 0.36 / 0.59 (128 K), 0.54 / 0.61 (192 K), at 8000 see below.
 bool small_mlp_supported(mpode_dtype dt, int B, int L, const int* wp) {
     if (L < 1 || L > SMALL_MAX_L) return false;
     SmallMlp p{};

@@ -855,7 +855,7 @@ public:
         cot_.assign(L_ + 1, 0);
         for (int l = 1; l <= L_; ++l) cot_[l] = lay.take((size_t)2 * B_ * wp_[l] * es);   // [zeta_l; ubar_l]
         // fp32 [hbar; gbar] of the backward step through an activation: not needed where the tensor-core epilogue takes that
-        // step (tiles of sample pairs; every such contraction is eligible when the widths are multiples of 8 and at least 64)
+        // step (tiles of sample pairs; every such contraction is eligible when the row lengths are multiples of 8)
         pair_bwd_ = pair_tiles();
         for (int l = 1; l <= L_; ++l) pair_bwd_ = pair_bwd_ && wp_[l] % 8 == 0;
         wide_ = pair_bwd_ ? 0 : lay.take((size_t)2 * B_ * maxw * sizeof(float));
@@ -1301,8 +1301,8 @@ private:
 };
 
 // ---------------------------------------------------------------------------------------------------- scalar example
-// Example 1 of the paper: one state component, three parameters.  Both passes run as whole-solve kernels (one CTA, one thread
-// per sample); there is no layer-by-layer form.
+// Example 1 of the paper: one state component, three parameters.  Both passes run as whole-solve kernels (one thread
+// per sample, the backward pass as one cluster); there is no layer-by-layer form.
 class ScalarPolyVelocity : public Velocity {
 public:
     ScalarPolyVelocity(const mpode_velocity_desc&, int B, mpode_dtype dt, int max_steps) : B_(B), dt_(dt), max_steps_(max_steps) {}

@@ -59,7 +59,7 @@ def test_c1_toy_mlp_full_size_fp16_dynamic():
 
 @pytest.mark.parametrize("low,scaling", [("f16", "dynamic"), ("bf16", "none"), ("f32", "none")])
 def test_c1_toy_mlp_ragged_batch_whole_solve_kernels(low, scaling):
-    # 37 samples (one full warp and a ragged one), 20 hidden units: the single-CTA whole-solve kernels
+    # 37 samples (one full warp and a ragged one), 20 hidden units: the whole-solve kernels
     wl = inputs.toy_mlp(batch=37, n_steps=5, hidden=20)
     if low == "f32":
         assert_parity(run_gpu(wl, "f32", "none"), run_oracle(wl, exact=True), TOL["f32"])
