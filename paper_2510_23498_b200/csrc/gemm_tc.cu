@@ -627,6 +627,7 @@ static void conv_wgrad_plan(long long pixels, int C, int* splits, int* per) {
     if (s > kb_total / 8) s = kb_total / 8;
     if (s < 1) s = 1;
     *per = (kb_total + s - 1) / s;
+    if (*per < 1) *per = 1;                // fewer than 64 pixels: not a shape of this kernel
     *splits = (kb_total + *per - 1) / *per;
 }
 

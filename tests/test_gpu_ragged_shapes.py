@@ -176,6 +176,12 @@ def test_conv_block_tile_buffers(batch, H, W):
     assert_parity(run_gpu(wl, "bf16", "none"), run_oracle(wl, "bf16", "none"), TOL["bf16"])
 
 
+# 64 channels, fewer pixels in all than one k-block of the tensor-core weight gradient
+def test_conv_block_of_few_pixels():
+    wl = inputs.conv_block(batch=1, n_steps=2, H=7, W=7, C=64, act="softplus")
+    assert_parity(run_gpu(wl, "bf16", "none"), run_oracle(wl, "bf16", "none"), TOL["bf16"])
+
+
 # column sums (bias and time-column gradients of the flow): batches of one row chunk, of chunks that end early, the largest that the
 # cluster kernel takes and the next that it does not
 @pytest.mark.parametrize("batch", [3, 130, 2048, 2112])

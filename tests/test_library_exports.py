@@ -61,6 +61,20 @@ def test_host_only_calls_work_without_a_device():
     assert lib.mpode_create(C.byref(h), C.byref(bad), 8, 4, C.byref(pol)) == 1
 
 
+def test_convolutions_of_few_pixels_can_be_created():
+    # fewer than 64 pixels in all, channels that the tensor-core weight gradient would take: its slice plan must not divide by zero
+    import ctypes as C
+    from paper_2510_23498_b200 import binding
+    lib = binding.load_library()
+    for kind, side, channels in (("conv", 7, 64), ("conv", 1, 64), ("parabolic", 3, 128)):
+        desc = binding.VelocityDesc(binding.KINDS[kind], side * side * channels, 0, None, binding.ACTS["relu"], 1, 1, side, side, channels, 1, 1)
+        pol = binding.Policy(binding.DTYPES["f16"], 0, 0, 0, 0, binding.NO_OVERRIDE)
+        h = C.c_void_p()
+        assert lib.mpode_create(C.byref(h), C.byref(desc), 1, 2, C.byref(pol)) == 0
+        assert lib.mpode_workspace_bytes(h) > 0
+        lib.mpode_destroy(h)
+
+
 def test_a_refused_whole_solve_launch_fails_the_call_and_nothing_else_runs():
     # The hypernetwork flow plans its workspace for the whole-solve kernels alone: where the runtime refuses their launch (here every
     # launch, there is no device) the call fails with a status, and no kernel of another path is queued, for which no buffers exist.
