@@ -174,9 +174,10 @@ public:
         small_wt_ = own.take((size_t)small_w_[1] * es);
         small_scal_ = own.take((size_t)max_steps_ * sizeof(RkStepScalars));
         if (small_bwd_ok_) {
-            size_t per_step = lay.time_gradient ? (size_t)small_blocks(dt_, B_) * 3 * sizeof(float) : 0;
+            if (lay.time_gradient) small_tpart_ = own.take((size_t)SMALL_MAX_CHUNK * small_blocks(dt_, B_) * 3 * sizeof(float));
+            size_t per_step = 0;
             for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
-            const size_t slack = (size_t)(2 * L_ + 1) * 256, used = own.total + slack;      // (every slab starts on 256 bytes)
+            const size_t slack = (size_t)2 * L_ * 256, used = own.total + slack;      // (every slab starts on 256 bytes)
             size_t room = used < lay.total ? lay.total - used : 0;
             if (room > (size_t)8 << 20) room = (size_t)8 << 20;
             const size_t steps = lay.stepwise ? 1 : room / per_step;
@@ -186,7 +187,6 @@ public:
                 small_xs_[l] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
                 small_zs_[l + 1] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
             }
-            if (lay.time_gradient) small_tpart_ = own.take((size_t)small_chunk_ * small_blocks(dt_, B_) * 3 * sizeof(float));
         }
         if (own.total > lay.total) lay.total = own.total;
     }
@@ -659,9 +659,12 @@ public:
         p.a = a; p.cot = cot; p.e = e; p.e_dev = nullptr; p.flag = flag; p.recompute = p.vjp = p.commit = 1;
         p.out = g; p.beta = 1.f;
         if (tprime != nullptr) { p.tpart = (float*)at(ws, small_tpart_); p.tprime = tprime; }
-        for (int hi = fs.n_steps - 1; hi >= 0; hi -= small_chunk_) {
+        // the slabs hold small_chunk_ steps of four stages: more steps of a tableau with fewer
+        int chunk = small_chunk_ * RK_MAX_STAGES / fs.stages;
+        if (chunk > SMALL_MAX_CHUNK) chunk = SMALL_MAX_CHUNK;
+        for (int hi = fs.n_steps - 1; hi >= 0; hi -= chunk) {
             p.step_hi = hi;
-            p.count = hi + 1 < small_chunk_ ? hi + 1 : small_chunk_;
+            p.count = hi + 1 < chunk ? hi + 1 : chunk;
             for (int s = 0; s < p.count; ++s) p.coef[s] = ldexpf(fs.scalars[hi - s].h, -e);
             const double f = (double)p.count * fs.stages * layer_flops();
             small_timed(3, 3.0 * f, st, [&] { launch_small_backward(dt_, p, st, L); launch_small_wgrad(dt_, p, st, L); return true; });

@@ -83,6 +83,23 @@ def test_small_networks_at_tile_edges(batch, widths, n_steps):
             assert_same_log(gpu["log"], orc["log"])
 
 
+# tableaux with fewer than four stages: the buffers hold more of their steps (chunks of steps that end early, the longest chunk of 16), with
+# the time terms of every step of a chunk
+@pytest.mark.parametrize("solver,n_steps", [("euler", 37), ("midpoint", 21), ("kutta3", 9)])
+@pytest.mark.parametrize("low", ["bf16", "f32"])
+def test_small_networks_chunks_of_steps_per_tableau(solver, n_steps, low):
+    wl = inputs.mlp_block(batch=300, n_steps=n_steps, d=40, hidden=72)
+    wl.vel["n_layers"], wl.vel["widths"], wl.theta = 2, [40, 72, 40], inputs.mlp_theta(3, [40, 72, 40], True)
+    wl.solver = solver
+    gpu = run_gpu(wl, low, "none", want_dt=True)
+    orc = run_oracle(wl, exact=True, want_dt=True) if low == "f32" else run_oracle(wl, low, "none", want_dt=True)
+    assert_parity(gpu, orc, TOL[low])
+    assert rel_l2(gpu["dL_dt"], orc["dL_dt"]) <= TOL[low]
+    plain = run_gpu(wl, low, "none")
+    assert np.array_equal(plain["a0"], gpu["a0"]) and plain["stats"]["fused_launches"] > 0
+    assert rel_l2(plain["g"], gpu["g"]) <= 2.2e-6        # (steps may be grouped otherwise: float32 sums over at most 37 of them, 37 * 2^-24)
+
+
 # the same in float32 (CUDA cores): one row, a block's 8 rows less and plus one, more row tiles than SMs, odd widths, 1 to 4 layers
 @pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (7, [16, 33, 65, 16], 3), (9, [64, 64], 20), (200, [72, 201, 200, 72], 2),
                                                   (1185, [24, 40, 24], 2), (130, [16, 32, 48, 32, 16], 3)])
