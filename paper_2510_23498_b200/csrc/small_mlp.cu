@@ -1062,8 +1062,7 @@ void launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, l
     if (tl_counters) ++tl_counters->fused;
 }
 
-void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    const int blocks = small_blocks(dt, p.B);
+void launch_small_time(mpode_dtype dt, const SmallMlp& p, int blocks, cudaStream_t st, long long* launches) {
     if (dt == MPODE_BF16) launch_chain(small_time_kernel<__nv_bfloat16>, dim3(1), dim3(96), 0, st, p, blocks);
     else if (dt == MPODE_F16) launch_chain(small_time_kernel<__half>, dim3(1), dim3(96), 0, st, p, blocks);
     else launch_chain(small_time_kernel<float>, dim3(1), dim3(96), 0, st, p, blocks);

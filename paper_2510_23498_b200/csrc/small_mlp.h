@@ -49,7 +49,7 @@ bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, lo
 bool small_backward_ready(mpode_dtype dt, const SmallMlp& p);
 void launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 int small_blocks(mpode_dtype dt, int B);                               // blocks of the forward and backward kernels
-void launch_small_time(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
+void launch_small_time(mpode_dtype dt, const SmallMlp& p, int blocks, cudaStream_t st, long long* launches);
 void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 
 }  // namespace mpode

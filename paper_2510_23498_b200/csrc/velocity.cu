@@ -6,6 +6,7 @@
 #include "hyper_cnf.h"
 #include "profiler.h"
 #include "small_mlp.h"
+#include "resident_mlp.h"
 #include "tensormap.h"
 #include "tiny_mlp.h"
 #include "velocity.h"
@@ -169,12 +170,20 @@ public:
         const size_t es = low_size(dt_);
         Layout own;
         own.total = lay.stepwise ? lay.kbuf[0] : lay.psi[0];
-        small_pack_ = own.take(small_pack_bytes(dt_, L_, small_w_.data()));
+        res_ = plan_resident(dt_, B_, L_, small_w_.data(), bias_, time_);
+        res_.params = (long long)p_;
+        {   // one form of the weights at a time
+            const size_t pack = small_pack_bytes(dt_, L_, small_w_.data());
+            small_pack_ = own.take((size_t)res_.image_bytes > pack ? (size_t)res_.image_bytes : pack);
+        }
         for (int l = 0; l < L_; ++l) small_b_[l] = own.take((size_t)small_w_[l + 1] * es);
         small_wt_ = own.take((size_t)small_w_[1] * es);
         small_scal_ = own.take((size_t)max_steps_ * sizeof(RkStepScalars));
         if (small_bwd_ok_) {
-            if (lay.time_gradient) small_tpart_ = own.take((size_t)SMALL_MAX_CHUNK * small_blocks(dt_, B_) * 3 * sizeof(float));
+            if (lay.time_gradient) {
+                const int blocks = small_blocks(dt_, B_);
+                small_tpart_ = own.take((size_t)SMALL_MAX_CHUNK * (blocks > res_.blocks_b ? blocks : res_.blocks_b) * 3 * sizeof(float));
+            }
             size_t per_step = 0;
             for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
             const size_t slack = (size_t)2 * L_ * 256, used = own.total + slack;      // (every slab starts on 256 bytes)
@@ -183,10 +192,15 @@ public:
             const size_t steps = lay.stepwise ? 1 : room / per_step;
             small_chunk_ = steps < 1 ? 1 : (steps > SMALL_MAX_CHUNK ? SMALL_MAX_CHUNK : (int)steps);
             if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
+            // (the blocks' parameter gradients, in passes that form them without the slabs)
+            const size_t partial = res_.backward && res_.pieces > 0 ? (size_t)res_.blocks_b * p_ * sizeof(float) : 0;
+            Layout sums = own;
+            small_partial_ = sums.take(partial);
             for (int l = 0; l < L_; ++l) {
                 small_xs_[l] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l] * es);
                 small_zs_[l + 1] = own.take((size_t)small_chunk_ * RK_MAX_STAGES * B_ * small_w_[l + 1] * es);
             }
+            if (sums.total > own.total) own.total = sums.total;
         }
         if (own.total > lay.total) lay.total = own.total;
     }
@@ -256,8 +270,22 @@ public:
     void prepare(cudaStream_t st, void* ws, const float* theta, const signed char*, long long* L) override {
         theta_ = theta;
         quantized_ = false;
-        if (small_ok_) launch_small_pack(dt_, small_params(ws), st, L);      // the other forms only if a pass turns out to need them
-        else quantize(st, ws, L);
+        packed_ = 0;
+        if (!small_ok_) quantize(st, ws, L);      // (the row-local kernels' form when they run, this one only if a pass turns out to need it)
+    }
+    // the weights as the row-local kernels read them: 1 streamed, 2 resident
+    void pack(int form, const SmallMlp& p, cudaStream_t st, long long* L) {
+        if (packed_ == form) return;
+        packed_ = form;
+        if (form == 1) launch_small_pack(dt_, p, st, L);
+        else launch_resident_pack(dt_, resident(p), st, L);
+    }
+    ResidentMlp resident(const SmallMlp& p, bool sums = false) const {
+        ResidentMlp r;
+        r.s = p; r.g = res_;
+        r.image = (unsigned char*)p.wf[0];
+        if (sums) r.partial = (float*)((char*)p.wf[0] - small_pack_ + small_partial_);
+        return r;
     }
     // Q16(theta) in the layouts of the tensor-core and CUDA-core contractions, once per pass
     void quantize(cudaStream_t st, void* ws, long long* L) {
@@ -417,7 +445,14 @@ public:
         if (small_usable(fs) && !fs.starve) {      // (the test of the bounded waits is about the fused program here)
             SmallMlp p = small_solve(st, ws, fs);
             p.y0 = p.yT = fs.y;                       // the driver has put y_0 there
-            if (small_timed(0, (double)fs.n_steps * fs.stages * layer_flops(), st, [&] { return launch_small_forward(dt_, p, st, L); })) return true;
+            const double f = (double)fs.n_steps * fs.stages * layer_flops();
+            if (res_.forward) {
+                pack(2, p, st, L);
+                if (small_timed(0, f, st, [&] { return launch_resident_forward(dt_, resident(p), st, L); })) return true;
+                cudaGetLastError();                   // (the other kernels take over)
+            }
+            pack(1, p, st, L);
+            if (small_timed(0, f, st, [&] { return launch_small_forward(dt_, p, st, L); })) return true;
         }
         quantize(st, ws, L);
         if (!fused_ok_ || fs.stages > RK_MAX_STAGES || fs.n_steps > max_steps_) return false;
@@ -487,8 +522,12 @@ public:
         if (b_small_) {
             small_bwd_ = small_solve(st, ws, fs);
             b_small_ = small_backward_ready(dt_, small_bwd_);
+            // (the test of the bounded waits is about the kernel that has some)
+            b_res_ = b_small_ && res_.backward && !fs.starve && resident_backward_ready(dt_, resident(small_bwd_)) &&
+                     (res_.pieces == 0 || resident_backward_ready(dt_, resident(small_bwd_, true)));
         }
         if (b_small_) {
+            pack(b_res_ ? 2 : 1, small_bwd_, st, L);
             b_stages_ = fs.stages;
             scal_host_ = fs.scalars;
             return true;
@@ -642,12 +681,18 @@ public:
         return true;
     }
 
+    void small_backward(const SmallMlp& p, cudaStream_t st, long long* L) {
+        if (b_res_) launch_resident_backward(dt_, resident(p), st, L);
+        else launch_small_backward(dt_, p, st, L);
+    }
+    int small_time_blocks() const { return b_res_ ? res_.blocks_b : small_blocks(dt_, B_); }
+
     bool fused_has_time_terms() const override { return b_small_; }
     bool fused_time_terms(cudaStream_t st, float* tvals, unsigned* flag, long long* L) override {
         if (!b_small_) return false;
         SmallMlp p = small_step_;
         p.tvals = tvals; p.flag = flag;
-        launch_small_time(dt_, p, st, L);
+        launch_small_time(dt_, p, small_time_blocks(), st, L);
         return true;
     }
 
@@ -662,13 +707,25 @@ public:
         // the slabs hold small_chunk_ steps of four stages: more steps of a tableau with fewer
         int chunk = small_chunk_ * RK_MAX_STAGES / fs.stages;
         if (chunk > SMALL_MAX_CHUNK) chunk = SMALL_MAX_CHUNK;
+        // parameter gradients in registers: no slabs, so all steps at once (the time terms are kept for a chunk of steps)
+        const bool sums = b_res_ && res_.pieces > 0 && flag == nullptr;
+        if (sums) chunk = tprime != nullptr ? SMALL_MAX_CHUNK : fs.n_steps;
         for (int hi = fs.n_steps - 1; hi >= 0; hi -= chunk) {
             p.step_hi = hi;
             p.count = hi + 1 < chunk ? hi + 1 : chunk;
-            for (int s = 0; s < p.count; ++s) p.coef[s] = ldexpf(fs.scalars[hi - s].h, -e);
+            for (int s = 0; s < p.count && s < SMALL_MAX_CHUNK; ++s) p.coef[s] = ldexpf(fs.scalars[hi - s].h, -e);
             const double f = (double)p.count * fs.stages * layer_flops();
-            small_timed(3, 3.0 * f, st, [&] { launch_small_backward(dt_, p, st, L); launch_small_wgrad(dt_, p, st, L); return true; });
-            if (tprime != nullptr) launch_small_time(dt_, p, st, L);
+            small_timed(3, 3.0 * f, st, [&] {
+                if (sums) {
+                    launch_resident_backward(dt_, resident(p, true), st, L);
+                    launch_resident_reduce(resident(p, true), st, L);
+                } else {
+                    small_backward(p, st, L);
+                    launch_small_wgrad(dt_, p, st, L);
+                }
+                return true;
+            });
+            if (tprime != nullptr) launch_small_time(dt_, p, small_time_blocks(), st, L);
         }
         return true;
     }
@@ -678,7 +735,7 @@ public:
             if (lay_->time_gradient) return;          // the product wants the stage derivatives too: it recomputes them itself
             SmallMlp p = small_bwd_;
             p.step_hi = step; p.count = 1; p.recompute = 1;
-            small_timed(0, b_stages_ * layer_flops(), st, [&] { launch_small_backward(dt_, p, st, L); return true; });
+            small_timed(0, b_stages_ * layer_flops(), st, [&] { small_backward(p, st, L); return true; });
             return;
         }
         const size_t es = low_size(dt_);
@@ -712,7 +769,7 @@ public:
             small_step_ = p;
             SmallMlp w = p;
             w.out = out; w.beta = beta; w.coef[0] = coef; w.flag = nullptr;      // (the driver tests the step's gradient)
-            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { launch_small_backward(dt_, p, st, L); launch_small_wgrad(dt_, w, st, L); return true; });
+            small_timed(3, 2.0 * b_stages_ * layer_flops(), st, [&] { small_backward(p, st, L); launch_small_wgrad(dt_, w, st, L); return true; });
             if (after_kernel != nullptr) cudaEventRecord(after_kernel, st);
             if (st_finish != nullptr && after_kernel != nullptr) cudaStreamWaitEvent(st_finish, after_kernel, 0);
             return;
@@ -800,8 +857,10 @@ protected:
     size_t f_scalars_ = 0, f_phases_[3] = {0, 0, 0}, f_cnt_ = 0, kappaslab_ = 0;
     size_t tiny_scal_ = 0, tiny_log_ = 0;
     bool tiny_ok_ = false;
-    bool small_ok_ = false, small_bwd_ok_ = false, b_small_ = false, quantized_ = false;
-    int small_chunk_ = 1;
+    bool small_ok_ = false, small_bwd_ok_ = false, b_small_ = false, b_res_ = false, quantized_ = false;
+    int small_chunk_ = 1, packed_ = 0;
+    ResidentPlan res_;
+    size_t small_partial_ = 0;
     size_t small_pack_ = 0, small_scal_ = 0, small_xs_[SMALL_MAX_L] = {0}, small_zs_[SMALL_MAX_L + 1] = {0};
     SmallMlp small_bwd_{}, small_step_{};
     size_t small_tpart_ = 0, small_b_[SMALL_MAX_L] = {0}, small_wt_ = 0;
