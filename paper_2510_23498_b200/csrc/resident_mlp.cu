@@ -23,6 +23,8 @@ constexpr int kPieceWarps = 8;
 constexpr int kScalarWords = sizeof(RkStepScalars) / sizeof(float);
 
 __host__ __device__ inline int up16(int w) { return (w + 15) / 16 * 16; }
+// rows and columns of a layer's weights in the image: whole reduction steps, of a single layer an even number of them
+__host__ __device__ inline int image_width(int L, int w) { return L == 1 ? (w + 31) / 32 * 32 : up16(w); }
 // warps that carry the chain: 16 features each, one tile per warp up to 256 features
 inline int chain_warps(int L, const int* wp) {
     int m = 0;
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(256) resident_pack_kernel(const __grid_constan
     const SmallMlp& s = p.s;
     const int step = (int)(gridDim.x * blockDim.x), first = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     for (int l = 0; l < s.L; ++l) {
-        const int ld = p.g.sw[l], n = up16(s.wp[l + 1]) * ld, in_full = s.wr[l] + ((s.time && l == 0) ? 1 : 0);
+        const int ld = p.g.sw[l], n = image_width(s.L, s.wp[l + 1]) * ld, in_full = s.wr[l] + ((s.time && l == 0) ? 1 : 0);
         T* dst = (T*)p.image + p.g.w_at[l];
         for (int i = first; i < n; i += step) {
             const int out = i / ld, in = i - out * ld;
@@ -132,53 +134,91 @@ inline ResidentBufs plan_bufs(const ResidentPlan& g, int L, int stages, int R, b
 }
 // pieces of 8 inputs in a layer's parameter gradient; the bias and time columns are one more
 __host__ __device__ inline int piece_columns(int inputs, bool sums) { return inputs / 8 + (sums ? 1 : 0); }
-// [image][buffers][slots: `slots` words for each of the state tiles' threads][scalars of two steps][sums of the time terms]
+// [image][buffers][slots: words of the state tiles' threads: k_j; forward y; backward psi_j, seed, adjoint][scalars of two steps][sums of the time terms]
 inline size_t resident_smem(const ResidentPlan& g, int L, int wp0, int stages, int mt, bool back) {
     const int owners = up16(wp0) / 16 * 32;
-    return plan_bufs(g, L, stages, 8 * mt, back).slots + (size_t)(back ? 2 : 1) * stages * 2 * mt * owners * 4 + 2 * kScalarWords * 4 + 3 * 16 * 4 + 16;
+    const int words = (back ? 4 * RK_MAX_STAGES + 6 : 2 * RK_MAX_STAGES + 4) * mt;
+    return plan_bufs(g, L, stages, 8 * mt, back).slots + (size_t)words * owners * 4 + 2 * kScalarWords * 4 + 3 * 16 * 4 + 16;
 }
 
 // One tile of 16 features for the block's 8 MT rows: acc[m][0, 1] = feature g of rows 2t, 2t + 1 (g = lane / 4, t = lane % 4), acc[m][2, 3]
-// feature g + 8.  `w`: this lane's address in the weights, advanced by wstep per 16 of the reduction; `x`: in the rows' buffer.
+// feature g + 8.  `w`: this lane's address in the weights, advanced by wstep per 16 of the reduction; `x`: in the rows' buffer.  The operands
+// of a group of kAhead reduction steps are requested while the group before is multiplied; the weights of the first group depend on nothing
+// and are requested before the barrier that the rows are waited for with.  (Without the second set of registers a 208-long reduction took
+// 918 cycles, 270 of them matrix instructions.)
+constexpr int kAhead = 2;
+template <int MT> struct Ops { uint32_t a[kAhead][4], b[MT][4]; };
+template <int MT, bool BACK, int N = kAhead>
+__device__ __forceinline__ void load_weights(Ops<MT>& o, uint32_t w, uint32_t wstep) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) { if (BACK) ldm4_t(w + q * wstep, o.a[q]); else ldm4(w + q * wstep, o.a[q]); }
+}
+template <int MT>
+__device__ __forceinline__ void load_rows(Ops<MT>& o, uint32_t x, uint32_t xrow8) {
+#pragma unroll
+    for (int m = 0; m < MT; ++m) ldm4(x + m * xrow8, o.b[m]);
+}
+template <typename T, int MT, int N = kAhead>
+__device__ __forceinline__ void multiply(float (&acc)[MT][4], const Ops<MT>& o) {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+#pragma unroll
+        for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m], o.a[q], o.b[m][2 * q], o.b[m][2 * q + 1]);
+}
+// Where a warp's product of a phase finds its operands.  Formed for the next phase at the start of this one, beside the matrix
+// instructions: everything that belongs to a layer comes from the constant bank at an index.
+struct Phase { uint32_t w, wstep, x, xrow8; int ks; bool on; };
+template <int MT, bool BACK>
+__device__ __forceinline__ void request_weights(Ops<MT>& o, const Phase& ph) {      // the first group's
+    load_weights<MT, BACK, 1>(o, ph.w, ph.wstep);
+    if (ph.ks > 1) { if (BACK) ldm4_t(ph.w + ph.wstep, o.a[1]); else ldm4(ph.w + ph.wstep, o.a[1]); }
+}
+// KS reduction steps as straight-line code: a branch costs as much as a matrix instruction here, where each scheduler has one or two warps
+template <typename T, int MT, bool BACK, int KS>
+__device__ __forceinline__ void product_steps(float (&acc)[MT][4], Ops<MT>& o, const Phase& ph) {
+    load_rows<MT>(o, ph.x, ph.xrow8);
+#pragma unroll
+    for (int k = 0; k < KS; k += kAhead) {
+        Ops<MT> nx;
+        const uint32_t w = ph.w + (uint32_t)(k + kAhead) * ph.wstep, x = ph.x + (uint32_t)(k + kAhead) * 32u;
+        if (k + 2 * kAhead <= KS) { load_weights<MT, BACK>(nx, w, ph.wstep); load_rows<MT>(nx, x, ph.xrow8); }
+        else if (k + kAhead < KS) { load_weights<MT, BACK, 1>(nx, w, ph.wstep); load_rows<MT>(nx, x, ph.xrow8); }
+        if (k + kAhead <= KS) multiply<T, MT>(acc, o); else multiply<T, MT, 1>(acc, o);
+        if (k + kAhead < KS) o = nx;
+    }
+}
 template <typename T, int MT, bool BACK>
-__device__ __forceinline__ void tile_product(float (&acc)[MT][4], uint32_t w, uint32_t wstep, uint32_t x, uint32_t xrow8, int ks) {
+__device__ __forceinline__ void tail_product(float (&acc)[MT][4], Ops<MT>& o, Phase q) {      // up to 16 steps, two at a time
+#pragma unroll 1
+    for (;;) {
+        load_rows<MT>(o, q.x, q.xrow8);
+        if (q.ks == 1) { multiply<T, MT, 1>(acc, o); return; }
+        multiply<T, MT>(acc, o);
+        if ((q.ks -= 2) <= 0) return;
+        q.w += 2u * q.wstep; q.x += 64u;
+        request_weights<MT, BACK>(o, q);
+    }
+}
+template <typename T, int MT, bool BACK>
+__device__ __forceinline__ void tile_product(float (&acc)[MT][4], Ops<MT>& o, const Phase& ph) {
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[m][i] = 0.f;
-    int k = 0;
-    constexpr int G = MT <= 2 ? 4 : 2;      // reduction steps whose operands are requested together
-#pragma unroll 1
-    for (; k + G <= ks; k += G) {
-        uint32_t a[G][4], b[G / 2][MT][4];
-#pragma unroll
-        for (int q = 0; q < G; ++q) {
-            if (BACK) ldm4_t(w + q * wstep, a[q]); else ldm4(w + q * wstep, a[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < G / 2; ++q)
-#pragma unroll
-            for (int m = 0; m < MT; ++m) ldm4(x + q * 64 + m * xrow8, b[q][m]);
-        w += G * wstep; x += G * 32;
-#pragma unroll
-        for (int q = 0; q < G; ++q)
-#pragma unroll
-            for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m], a[q], b[q >> 1][m][2 * (q & 1)], b[q >> 1][m][2 * (q & 1) + 1]);
+    switch (ph.ks) {
+#define MPODE_STEPS(K) case K: product_steps<T, MT, BACK, K>(acc, o, ph); return;
+        MPODE_STEPS(1) MPODE_STEPS(2) MPODE_STEPS(3) MPODE_STEPS(4) MPODE_STEPS(5) MPODE_STEPS(6) MPODE_STEPS(7) MPODE_STEPS(8)
+        MPODE_STEPS(9) MPODE_STEPS(10) MPODE_STEPS(11) MPODE_STEPS(12) MPODE_STEPS(13) MPODE_STEPS(14) MPODE_STEPS(15) MPODE_STEPS(16)
+#undef MPODE_STEPS
+        default: break;
     }
+    Phase q = ph;
 #pragma unroll 1
-    for (; k < ks; k += 2) {
-        uint32_t a[2][4], b[MT][4];
-#pragma unroll
-        for (int m = 0; m < MT; ++m) ldm4(x + m * xrow8, b[m]);
-        if (BACK) ldm4_t(w, a[0]); else ldm4(w, a[0]);
-        if (k + 1 < ks) { if (BACK) ldm4_t(w + wstep, a[1]); else ldm4(w + wstep, a[1]); }
-        w += 2 * wstep; x += 64;
-#pragma unroll
-        for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m], a[0], b[m][0], b[m][1]);
-        if (k + 1 < ks) {
-#pragma unroll
-            for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m], a[1], b[m][2], b[m][3]);
-        }
+    for (;;) {      // (wider than 256: 16 steps at a time)
+        if (q.ks <= 16) { tail_product<T, MT, BACK>(acc, o, q); return; }
+        product_steps<T, MT, BACK, 16>(acc, o, q);
+        q.w += 16u * q.wstep; q.x += 512u; q.ks -= 16;
+        request_weights<MT, BACK>(o, q);
     }
 }
 
@@ -186,7 +226,6 @@ __device__ __forceinline__ void tile_product(float (&acc)[MT][4], uint32_t w, ui
 template <typename T, int MT>
 struct Lane {
     int warp, lane, g, t;
-    uint32_t xo8, xoff;                // lane's row and column offsets of matrix loads: rows' operand
     __device__ Lane() {
         warp = threadIdx.x >> 5; lane = threadIdx.x & 31; g = lane >> 2; t = lane & 3;
     }
@@ -259,30 +298,400 @@ __device__ __forceinline__ void copy_scalars(float* dst, const RkStepScalars* sr
     if (tid < kScalarWords) dst[tid] = ((const float*)src)[tid];
 }
 
-// A hidden layer: H = Q16(act(W x + b + tau w_t)) of the block's rows
+// the phase of layer l on the rows in `in`: the layer itself, or its input gradient
+template <typename T, int MT>
+__device__ __forceinline__ Phase forward_phase(const ResidentMlp& p, const Lane<T, MT>& ln, uint32_t base, int l, uint32_t in) {
+    const int sw = p.g.sw[l], f0 = ln.warp * 16;
+    return Phase{ln.w_fwd(base + (uint32_t)p.g.w_at[l] * 2u, sw, f0), 32u, ln.x_at(in, sw), (uint32_t)(16 * sw), up16(p.s.wp[l]) / 16, f0 < p.s.wp[l + 1]};
+}
+template <typename T, int MT>
+__device__ __forceinline__ Phase backward_phase(const ResidentMlp& p, const Lane<T, MT>& ln, uint32_t base, int l, uint32_t in) {
+    const int sw = p.g.sw[l], sz = p.g.sw[l + 1], f0 = ln.warp * 16;
+    return Phase{ln.w_bwd(base + (uint32_t)p.g.w_at[l] * 2u, sw, f0), (uint32_t)(32 * sw), ln.x_at(in, sz), (uint32_t)(16 * sz), up16(p.s.wp[l + 1]) / 16, f0 < p.s.wp[l]};
+}
+
+// A hidden layer: H = Q16(act(W x + b + tau w_t)) of the block's rows.
 template <typename T, int MT, int NW>
-__device__ __forceinline__ void hidden_layer(const ResidentMlp& p, const Lane<T, MT>& ln, uint32_t wimg, const float* fl, int l, float tau, uint32_t in, uint32_t out) {
+__device__ __forceinline__ void hidden_layer(const ResidentMlp& p, const Lane<T, MT>& ln, const float* fl, int l, float tau, uint32_t out, Phase ph, Ops<MT>& ahead) {
     const SmallMlp& s = p.s;
-    const int K = up16(s.wp[l]) / 16, N = s.wp[l + 1], sx = p.g.sw[l];
-    const uint32_t w = wimg + (uint32_t)p.g.w_at[l] * 2u, x = ln.x_at(in, sx);
-    const bool time = s.time && l == 0;
+    const int N = s.wp[l + 1], so = p.g.sw[l + 1], b = p.g.b_at[l];
+#pragma unroll 1
     for (int f0 = ln.warp * 16; f0 < N; f0 += NW * 16) {
-        float bA = fl[p.g.b_at[l] + f0 + ln.g], bB = fl[p.g.b_at[l] + f0 + 8 + ln.g];
-        if (time) { bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], bA); bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], bB); }
+        float bA = fl[b + f0 + ln.g], bB = fl[b + f0 + 8 + ln.g];
+        if (s.time && l == 0) { bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], bA); bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], bB); }
+        if (f0 >= NW * 16) {
+            ph.w += NW * 2 * ph.xrow8;       // (a row's features further by the rows of one tile per warp: 16 NW rows of 2 sw bytes)
+            request_weights<MT, false>(ahead, ph);
+        }
         float acc[MT][4];
-        tile_product<T, MT, false>(acc, ln.w_fwd(w, p.g.sw[l], f0), 32u, x, (uint32_t)(16 * sx), K);
+        tile_product<T, MT, false>(acc, ahead, ph);
         uint32_t v[MT][2];
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
             v[m][0] = cvt_pack<T>(act16<T>(s.act, acc[m][0] + bA), act16<T>(s.act, acc[m][1] + bA));
             v[m][1] = cvt_pack<T>(act16<T>(s.act, acc[m][2] + bB), act16<T>(s.act, acc[m][3] + bB));
         }
-        put_tile<MT>(ln, out, p.g.sw[l + 1], f0, N, v);
+        put_tile<MT>(ln, out, so, f0, N, v);
     }
 }
 
+// What the last layer's epilogue of stage j needs besides the product: the terms of the next stage's input (or, after the last stage, of the
+// increment) that do not depend on this stage, and this stage's coefficient.
+template <typename T, int MT>
+struct StageTerms {
+    float v[MT][4], c, bA, bB;
+    bool on;
+    // row: h a_{j+1, .} or h b_.; from the state or from zero
+    __device__ __forceinline__ void start(const float* row, int j, bool sum, const uint32_t (&yb)[MT][2], const uint32_t* ks, int owners) {
+        const float4 r = *reinterpret_cast<const float4*>(row);
+        const float cq[RK_MAX_STAGES - 1] = {r.x, r.y, r.z};
+        c = row[j];
+        on = sum || c != 0.f;
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v0 = sum ? 0.f : lo_of<T>(yb[m][h]), v1 = sum ? 0.f : hi_of<T>(yb[m][h]);
+#pragma unroll
+                for (int q = 0; q < RK_MAX_STAGES - 1; ++q) {      // (no branches: a slot that is not wanted is read all the same)
+                    const bool use = q < j && (sum || cq[q] != 0.f);
+                    const uint32_t k = ks[((q * MT + m) * 2 + h) * owners];
+                    const float w0 = fmaf(cq[q], lo_of<T>(k), v0), w1 = fmaf(cq[q], hi_of<T>(k), v1);
+                    v0 = use ? w0 : v0;
+                    v1 = use ? w1 : v1;
+                }
+                v[m][2 * h] = v0; v[m][2 * h + 1] = v1;
+            }
+    }
+    // k_j of pair (m, h), rounded once; the terms with it
+    __device__ __forceinline__ uint32_t stage(const float (&acc)[MT][4], int m, int h) {
+        const float b = h ? bB : bA;
+        const uint32_t k = cvt_pack<T>(acc[m][2 * h] + b, acc[m][2 * h + 1] + b);
+        const float w0 = fmaf(c, lo_of<T>(k), v[m][2 * h]), w1 = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
+        v[m][2 * h] = on ? w0 : v[m][2 * h];
+        v[m][2 * h + 1] = on ? w1 : v[m][2 * h + 1];
+        return k;
+    }
+};
+
+// ---------------------------------------------------------------- one layer
+// A velocity of a single layer is the shortest chain: every phase is one product of up to 128 x 128 and the elementwise step behind it.  With
+// one warp to a scheduler a phase is the sum of its instructions' latencies (the general code's 150 instructions: 1000 cycles), so the
+// weights of a warp's tile stay in registers, for both directions, and nothing is left in a phase but matrix loads, matrix
+// instructions, the epilogue and the barrier.  KS1: reduction steps, a multiple of two (the image is padded with zeros to it).
+template <typename T, int MT, int KS1>
+struct Linear {
+    uint32_t w[KS1][4];
+    template <bool BACK> __device__ __forceinline__ void load(uint32_t at, uint32_t wstep) {
+#pragma unroll
+        for (int k = 0; k < KS1; ++k) { if (BACK) ldm4_t(at + k * wstep, w[k]); else ldm4(at + k * wstep, w[k]); }
+    }
+    __device__ __forceinline__ void product(float (&acc)[MT][4], uint32_t x, uint32_t xrow8) const {
+        uint32_t b[KS1 / 2][MT][4];
+#pragma unroll
+        for (int k = 0; k < KS1 / 2; ++k)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) ldm4(x + k * 64 + m * xrow8, b[k][m]);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[m][i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < KS1; ++k)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m], w[k], b[k >> 1][m][2 * (k & 1)], b[k >> 1][m][2 * (k & 1) + 1]);
+    }
+};
+// Y_{j+1} = Q16(ybar + sum_{l <= j} (h a_{j+1,l}) k_l): the terms with l < j, where the tableau has any
+template <typename T, int MT>
+__device__ __forceinline__ void earlier_terms(float (&v)[MT][4], const float* row, int j, const uint32_t* ks, int owners) {
+    for (int q = 0; q < j; ++q) {
+        const float c = row[q];
+        if (c == 0.f) continue;
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t k = ks[((q * MT + m) * 2 + h) * owners];
+                v[m][2 * h] = fmaf(c, lo_of<T>(k), v[m][2 * h]);
+                v[m][2 * h + 1] = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
+            }
+    }
+}
+
+template <typename T, int MT, int KS1>
+__device__ __forceinline__ void linear_forward(const ResidentMlp& p, uint32_t base, uint32_t* ks, const float* scal, const float* fl, int r0) {
+    const SmallMlp& s = p.s;
+    const Lane<T, MT> ln;
+    const int d = s.wr[0], S = s.stages, sx = p.g.sw[0], tiles0 = up16(s.wp[0]) / 16, owners = tiles0 * 32, f0 = ln.warp * 16;
+    const bool owner = ln.warp < tiles0, upper = f0 + 8 < s.wp[0], time = s.time != 0, alone = s.alone != 0;
+    const uint32_t xrow8 = (uint32_t)(16 * sx), z0 = base + (uint32_t)p.b.z0;
+    float y[MT][4], u[MT][4];
+    uint32_t yb[MT][2];
+    if (owner) {
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                y[m][i] = r < s.B && c < d ? s.y0[(long long)r * d + c] : 0.f;
+                u[m][i] = 0.f;
+            }
+            yb[m][0] = cvt_pack<T>(y[m][0], y[m][1]);
+            yb[m][1] = cvt_pack<T>(y[m][2], y[m][3]);
+        }
+        put_tile<MT>(ln, z0, sx, f0, s.wp[0], yb);
+    }
+    copies_done();
+    __syncthreads();
+    Linear<T, MT, KS1> W;
+    float b0 = 0.f, b1 = 0.f, t0 = 0.f, t1 = 0.f;
+    if (owner) {
+        W.template load<false>(ln.w_fwd(base, sx, f0), 32u);
+        b0 = fl[f0 + ln.g]; b1 = fl[f0 + 8 + ln.g];
+        t0 = fl[p.g.t_at + f0 + ln.g]; t1 = fl[p.g.t_at + f0 + 8 + ln.g];
+    }
+    const uint32_t x0 = ln.x_at(z0, sx), o0 = ln.frag_at(z0, sx, f0, 0);
+    uint32_t cur = 0;      // offset of the buffer that holds the stage input
+    for (int n = 0; n < s.n_steps; ++n) {
+        const RkStepScalars& sc = *(const RkStepScalars*)(scal + (n & 1) * kScalarWords);
+#pragma unroll
+        for (int j = 0; j < RK_MAX_STAGES; ++j) {
+            if (j >= S) break;
+            const uint32_t nxt = (uint32_t)p.b.state - cur;
+            if (owner) {
+                const bool last = j + 1 == S;
+                const float hb = sc.hb[j], c = sc.ha[j + 1 < RK_MAX_STAGES ? j + 1 : j][j];
+                float acc[MT][4];
+                W.product(acc, x0 + cur, xrow8);
+                const float bA = time ? fmaf(sc.tau16[j], t0, b0) : b0, bB = time ? fmaf(sc.tau16[j], t1, b1) : b1;
+                float v[MT][4];
+                uint32_t k[MT][2];
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        k[m][h] = cvt_pack<T>(acc[m][2 * h] + (h ? bB : bA), acc[m][2 * h + 1] + (h ? bB : bA));
+                        u[m][2 * h] = fmaf(hb, lo_of<T>(k[m][h]), u[m][2 * h]);
+                        u[m][2 * h + 1] = fmaf(hb, hi_of<T>(k[m][h]), u[m][2 * h + 1]);
+                        v[m][2 * h] = lo_of<T>(yb[m][h]);
+                        v[m][2 * h + 1] = hi_of<T>(yb[m][h]);
+                    }
+                if (!last) {
+                    if (!alone) {
+                        earlier_terms<T, MT>(v, sc.ha[j + 1 < RK_MAX_STAGES ? j + 1 : j], j, ks, owners);
+#pragma unroll
+                        for (int m = 0; m < MT; ++m) { ks[((j * MT + m) * 2) * owners] = k[m][0]; ks[((j * MT + m) * 2 + 1) * owners] = k[m][1]; }
+                    }
+                    if (alone || c != 0.f) {
+#pragma unroll
+                        for (int m = 0; m < MT; ++m)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) v[m][i] = fmaf(c, (i & 1) ? hi_of<T>(k[m][i >> 1]) : lo_of<T>(k[m][i >> 1]), v[m][i]);
+                    }
+                } else {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            y[m][i] += s.round_increment ? sc.h * Low<T>::to_f(Low<T>::from_f(u[m][i])) : u[m][i];
+                            v[m][i] = y[m][i];
+                            u[m][i] = 0.f;
+                        }
+                }
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    const uint32_t q0 = cvt_pack<T>(v[m][0], v[m][1]), q1 = cvt_pack<T>(v[m][2], v[m][3]);
+                    if (last) { yb[m][0] = q0; yb[m][1] = q1; }
+                    stm2_t(o0 + nxt + m * xrow8, q0, upper ? q1 : 0u);
+                }
+            }
+            __syncthreads();
+            cur = nxt;
+        }
+    }
+    if (owner) {
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                if (r < s.B && c < d) s.yT[(long long)r * d + c] = y[m][i];
+            }
+    }
+}
+
+// (no time terms: the general code has them)
+template <typename T, int MT, int KS1>
+__device__ __forceinline__ void linear_backward(const ResidentMlp& p, uint32_t base, uint32_t* ks, const float* scal, const float* fl, int r0) {
+    const SmallMlp& s = p.s;
+    const Lane<T, MT> ln;
+    const int d = s.wr[0], S = s.stages, B = s.B, sx = p.g.sw[0], tiles0 = up16(s.wp[0]) / 16, owners = tiles0 * 32, f0 = ln.warp * 16;
+    const bool owner = ln.warp < tiles0, upper = f0 + 8 < s.wp[0], time = s.time != 0, alone = s.alone != 0;
+    const uint32_t xrow8 = (uint32_t)(16 * sx);
+    uint32_t* ps = ks + RK_MAX_STAGES * 2 * MT * owners;
+    const int e = s.e_dev != nullptr ? *s.e_dev : s.e;
+    const float scale = ldexpf(1.f, e), unscale = ldexpf(1.f, -e);      // (|e| <= 100: products with them are what ldexp gives)
+    uint32_t bad = 0u;
+    Linear<T, MT, KS1> F, Bk;
+    float b0 = 0.f, b1 = 0.f, t0 = 0.f, t1 = 0.f, a[MT][4];
+    if (owner) {
+        F.template load<false>(ln.w_fwd(base, sx, f0), 32u);
+        Bk.template load<true>(ln.w_bwd(base, sx, f0), (uint32_t)(32 * sx));
+        b0 = fl[f0 + ln.g]; b1 = fl[f0 + 8 + ln.g];
+        t0 = fl[p.g.t_at + f0 + ln.g]; t1 = fl[p.g.t_at + f0 + 8 + ln.g];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                a[m][i] = s.vjp && r < B && c < d ? s.a[(long long)r * d + c] : 0.f;
+            }
+    }
+    const uint32_t xl = ln.x_at(base, sx), ol = ln.frag_at(base, sx, f0, 0);      // + the buffer's offset
+    for (int st = 0; st < s.count; ++st) {
+        const int n = s.step_hi - st;
+        const RkStepScalars& sc = *(const RkStepScalars*)(scal + (st & 1) * kScalarWords);
+        const uint32_t x00 = (uint32_t)(p.b.x00 + (st & 1) * p.b.state);
+        uint32_t vv[MT][2];
+        if (s.vjp && owner) {              // seed Q16(S a); the last stage's cotangent Q16(b v)
+            const float bj = sc.b[S - 1];
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                uint32_t o[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    vv[m][h] = cvt_pack<T>(a[m][2 * h] * scale, a[m][2 * h + 1] * scale);
+                    note_nonfinite<T>(vv[m][h], bad);
+                    o[h] = cvt_pack<T>(bj * lo_of<T>(vv[m][h]), bj * hi_of<T>(vv[m][h]));
+                    note_nonfinite<T>(o[h], bad);
+                }
+                stm2_t(ol + (uint32_t)p.b.z0 + m * xrow8, o[0], upper ? o[1] : 0u);
+            }
+        }
+        __syncthreads();
+        if (s.recompute) {
+            uint32_t yb[MT][2];
+            if (owner) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m) ldm2_t(ol + x00 + m * xrow8, yb[m][0], yb[m][1]);
+            }
+#pragma unroll
+            for (int j = 0; j + 1 < RK_MAX_STAGES; ++j) {
+                if (j + 1 >= S) break;
+                if (owner) {
+                    const float c = sc.ha[j + 1][j];
+                    float acc[MT][4];
+                    F.product(acc, xl + (j == 0 ? x00 : (uint32_t)(p.b.keep + j * p.b.keep_stage)), xrow8);
+                    const float bA = time ? fmaf(sc.tau16[j], t0, b0) : b0, bB = time ? fmaf(sc.tau16[j], t1, b1) : b1;
+                    float v[MT][4];
+                    uint32_t k[MT][2];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            k[m][h] = cvt_pack<T>(acc[m][2 * h] + (h ? bB : bA), acc[m][2 * h + 1] + (h ? bB : bA));
+                            v[m][2 * h] = lo_of<T>(yb[m][h]);
+                            v[m][2 * h + 1] = hi_of<T>(yb[m][h]);
+                        }
+                    if (!alone) {
+                        earlier_terms<T, MT>(v, sc.ha[j + 1], j, ks, owners);
+#pragma unroll
+                        for (int m = 0; m < MT; ++m) { ks[((j * MT + m) * 2) * owners] = k[m][0]; ks[((j * MT + m) * 2 + 1) * owners] = k[m][1]; }
+                    }
+                    if (alone || c != 0.f) {
+#pragma unroll
+                        for (int m = 0; m < MT; ++m)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) v[m][i] = fmaf(c, (i & 1) ? hi_of<T>(k[m][i >> 1]) : lo_of<T>(k[m][i >> 1]), v[m][i]);
+                    }
+#pragma unroll
+                    for (int m = 0; m < MT; ++m)
+                        stm2_t(ol + (uint32_t)(p.b.keep + (j + 1) * p.b.keep_stage) + m * xrow8, cvt_pack<T>(v[m][0], v[m][1]), upper ? cvt_pack<T>(v[m][2], v[m][3]) : 0u);
+                }
+                __syncthreads();
+            }
+        }
+        if (!s.vjp) continue;
+        float sum[MT][4];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[m][i] = 0.f;
+        uint32_t z = (uint32_t)p.b.z0, zn = z + (uint32_t)p.b.state;
+#pragma unroll
+        for (int j = RK_MAX_STAGES - 1; j >= 0; --j) {
+            if (j >= S) continue;
+            if (owner) {
+                const int jp = j > 0 ? j - 1 : 0;
+                const float bj = sc.b[jp], cj = sc.ha[j][jp];
+                float acc[MT][4];
+                Bk.product(acc, xl + z, xrow8);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    uint32_t o[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t q = cvt_pack<T>(acc[m][2 * h], acc[m][2 * h + 1]);
+                        note_nonfinite<T>(q, bad);
+                        sum[m][2 * h] += lo_of<T>(q);
+                        sum[m][2 * h + 1] += hi_of<T>(q);
+                        if (!alone) ps[((j * MT + m) * 2 + h) * owners] = q;
+                        if (!s.commit) {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                const int r = r0 + m * 8 + 2 * ln.t + i, c = f0 + ln.g + h * 8;
+                                if (r < B && c < s.wp[0]) reinterpret_cast<unsigned short*>(s.psi[j])[(long long)r * s.wp[0] + c] = (unsigned short)(i ? q >> 16 : q & 0xFFFFu);
+                            }
+                        }
+                        if (j > 0) {
+                            float v0 = bj * lo_of<T>(vv[m][h]), v1 = bj * hi_of<T>(vv[m][h]);
+                            if (alone || cj != 0.f) { v0 = fmaf(cj, lo_of<T>(q), v0); v1 = fmaf(cj, hi_of<T>(q), v1); }
+                            if (!alone) {
+                                for (int l = j + 1; l < S; ++l) {
+                                    const float c = sc.ha[l][jp];
+                                    if (c == 0.f) continue;
+                                    const uint32_t w = ps[((l * MT + m) * 2 + h) * owners];
+                                    v0 = fmaf(c, lo_of<T>(w), v0);
+                                    v1 = fmaf(c, hi_of<T>(w), v1);
+                                }
+                            }
+                            o[h] = cvt_pack<T>(v0, v1);
+                            note_nonfinite<T>(o[h], bad);
+                        }
+                    }
+                    if (j > 0) stm2_t(ol + zn + m * xrow8, o[0], upper ? o[1] : 0u);
+                }
+            }
+            __syncthreads();
+            const uint32_t w = z; z = zn; zn = w;
+        }
+        if (s.commit && owner) {      // a <- a + (h / S) sum_j psi_j (+ running cost)
+            const float coef = sc.h * unscale;
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    a[m][i] = fmaf(coef, sum[m][i], a[m][i]);
+                    const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                    if (s.cot != nullptr && r < B && c < d) a[m][i] += s.cot[((long long)n * B + r) * d + c];
+                }
+        }
+    }
+    if (s.vjp && s.commit && owner) {
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                if (r < B && c < d) s.a[(long long)r * d + c] = a[m][i];
+            }
+    }
+    warp_flag_or(s.flag, any_nonfinite(bad));
+}
+
 // ---------------------------------------------------------------- forward
-template <typename T, int MT, int NW>
+template <typename T, int MT, int NW, int KS1>
 __global__ void __launch_bounds__(NW * 32 + 64, 1) resident_forward_kernel(const __grid_constant__ ResidentMlp p) {
     chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -294,7 +703,7 @@ __global__ void __launch_bounds__(NW * 32 + 64, 1) resident_forward_kernel(const
     auto z_at = [&](int l) -> uint32_t { return base + (uint32_t)p.b.z[l]; };
     const int tiles0 = up16(s.wp[0]) / 16, owners = tiles0 * 32;
     uint32_t* slots = (uint32_t*)(smem + p.b.slots);
-    float* scal = (float*)(slots + S * 2 * MT * owners);
+    float* scal = (float*)(slots + (2 * RK_MAX_STAGES + 4) * MT * owners);
     const float* fl = (const float*)(smem + (size_t)p.g.w_elems * sizeof(T));
     load_image(p, smem);
     copy_scalars(scal, s.scal, threadIdx.x);
@@ -316,85 +725,79 @@ __global__ void __launch_bounds__(NW * 32 + 64, 1) resident_forward_kernel(const
         state_out<T>(z0_at(cur), p.g.sw[0], traj + (long long)s.n_steps * s.B * d, d, R, r0, s.B, tid, 64);
         return;
     }
+    if constexpr (KS1 > 0) { linear_forward<T, MT, KS1>(p, base, slots + threadIdx.x, scal, fl, r0); return; }
     const Lane<T, MT> ln;
     const bool owner = ln.warp < tiles0;
     const int f0 = ln.warp * 16;
     uint32_t* ks = slots + threadIdx.x;            // k_j of this thread's values: word (2 MT j + 2 m + h) * owners
-    float y[MT][4];
+    float* ys = (float*)(ks + RK_MAX_STAGES * 2 * MT * owners);      // y: word (4 m + i) * owners
     uint32_t yb[MT][2];
     if (owner) {
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
+            float y[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
-                y[m][i] = r < s.B && c < d ? s.y0[(long long)r * d + c] : 0.f;
+                y[i] = r < s.B && c < d ? s.y0[(long long)r * d + c] : 0.f;
+                ys[(4 * m + i) * owners] = y[i];
             }
-            yb[m][0] = cvt_pack<T>(y[m][0], y[m][1]);
-            yb[m][1] = cvt_pack<T>(y[m][2], y[m][3]);
+            yb[m][0] = cvt_pack<T>(y[0], y[1]);
+            yb[m][1] = cvt_pack<T>(y[2], y[3]);
         }
         put_tile<MT>(ln, z0_at(0), p.g.sw[0], f0, s.wp[0], yb);
     }
     copies_done();
     __syncthreads();
     int cur = 0;
+    Ops<MT> ahead;
+    const float bias0 = owner ? fl[p.g.b_at[L - 1] + f0 + ln.g] : 0.f, bias1 = owner ? fl[p.g.b_at[L - 1] + f0 + 8 + ln.g] : 0.f;
+    Phase ph = forward_phase(p, ln, base, 0, z0_at(0));
+    if (ph.on) request_weights<MT, false>(ahead, ph);
     for (int n = 0; n < s.n_steps; ++n) {
         const RkStepScalars& sc = *(const RkStepScalars*)(scal + (n & 1) * kScalarWords);
+#pragma unroll 1
         for (int j = 0; j < S; ++j) {
             const float tau = sc.tau16[j];
+#pragma unroll 1
             for (int l = 0; l + 1 < L; ++l) {
-                hidden_layer<T, MT, NW>(p, ln, base, fl, l, tau, l == 0 ? z0_at(cur) : z_at(l), z_at(l + 1));
+                const Phase nx = forward_phase(p, ln, base, l + 1, z_at(l + 1));
+                hidden_layer<T, MT, NW>(p, ln, fl, l, tau, z_at(l + 1), ph, ahead);
+                ph = nx;
+                if (ph.on) request_weights<MT, false>(ahead, ph);
                 __syncthreads();
             }
+            const Phase nx = forward_phase(p, ln, base, 0, z0_at(cur ^ 1));
             if (owner) {
-                const int l = L - 1, K = up16(s.wp[l]) / 16, sx = p.g.sw[l];
                 const bool last = j + 1 == S;
-                // the terms of what follows that do not depend on this stage
-                float v[MT][4];
+                StageTerms<T, MT> w;
+                w.start(last ? sc.hb : sc.ha[j + 1], j, last, yb, ks, owners);
+                w.bA = bias0; w.bB = bias1;
+                if (s.time && L == 1) { w.bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], w.bA); w.bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], w.bB); }
+                float acc[MT][4];
+                tile_product<T, MT, false>(acc, ahead, ph);
+                uint32_t o[MT][2];
 #pragma unroll
                 for (int m = 0; m < MT; ++m)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) v[m][i] = last ? 0.f : ((i & 1) ? hi_of<T>(yb[m][i >> 1]) : lo_of<T>(yb[m][i >> 1]));
-                for (int q = 0; q < j; ++q) {
-                    const float c = last ? sc.hb[q] : sc.ha[j + 1][q];
-                    if (!last && c == 0.f) continue;
-#pragma unroll
-                    for (int m = 0; m < MT; ++m)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const uint32_t k = ks[((q * MT + m) * 2 + h) * owners];
-                            v[m][2 * h] = fmaf(c, lo_of<T>(k), v[m][2 * h]);
-                            v[m][2 * h + 1] = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
-                        }
-                }
-                float bA = fl[p.g.b_at[l] + f0 + ln.g], bB = fl[p.g.b_at[l] + f0 + 8 + ln.g];
-                if (s.time && l == 0) { bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], bA); bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], bB); }
-                const float c = last ? sc.hb[j] : sc.ha[j + 1][j];
-                float acc[MT][4];
-                tile_product<T, MT, false>(acc, ln.w_fwd(base + (uint32_t)p.g.w_at[l] * 2u, p.g.sw[l], f0), 32u, ln.x_at(l == 0 ? z0_at(cur) : z_at(l), sx),
-                                           (uint32_t)(16 * sx), K);
-                uint32_t o[MT][2];
-#pragma unroll
-                for (int m = 0; m < MT; ++m) {
-#pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const float b = h ? bB : bA;
-                        const uint32_t k = cvt_pack<T>(acc[m][2 * h] + b, acc[m][2 * h + 1] + b);
-                        ks[((j * MT + m) * 2 + h) * owners] = k;
-                        if (last || c != 0.f) {
-                            v[m][2 * h] = fmaf(c, lo_of<T>(k), v[m][2 * h]);
-                            v[m][2 * h + 1] = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
-                        }
-                        if (last) {
+                        const uint32_t k = w.stage(acc, m, h);
+                        if (!last) {
+                            ks[((j * MT + m) * 2 + h) * owners] = k;
+                        } else {
 #pragma unroll
-                            for (int i = 2 * h; i < 2 * h + 2; ++i) y[m][i] += s.round_increment ? sc.h * Low<T>::to_f(Low<T>::from_f(v[m][i])) : v[m][i];
-                            yb[m][h] = cvt_pack<T>(y[m][2 * h], y[m][2 * h + 1]);
+                            for (int i = 2 * h; i < 2 * h + 2; ++i) {
+                                const float y = ys[(4 * m + i) * owners] + (s.round_increment ? sc.h * Low<T>::to_f(Low<T>::from_f(w.v[m][i])) : w.v[m][i]);
+                                ys[(4 * m + i) * owners] = w.v[m][i] = y;
+                            }
                         }
-                        o[m][h] = last ? yb[m][h] : cvt_pack<T>(v[m][2 * h], v[m][2 * h + 1]);
+                        o[m][h] = cvt_pack<T>(w.v[m][2 * h], w.v[m][2 * h + 1]);
+                        if (last) yb[m][h] = o[m][h];
                     }
-                }
                 put_tile<MT>(ln, z0_at(cur ^ 1), p.g.sw[0], f0, s.wp[0], o);
             }
+            ph = nx;
+            if (ph.on) request_weights<MT, false>(ahead, ph);
             __syncthreads();
             cur ^= 1;
         }
@@ -405,7 +808,7 @@ __global__ void __launch_bounds__(NW * 32 + 64, 1) resident_forward_kernel(const
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
-                if (r < s.B && c < d) s.yT[(long long)r * d + c] = y[m][i];
+                if (r < s.B && c < d) s.yT[(long long)r * d + c] = ys[(4 * m + i) * owners];
             }
     }
 }
@@ -414,7 +817,7 @@ __global__ void __launch_bounds__(NW * 32 + 64, 1) resident_forward_kernel(const
 // The chain of `count` steps (recompute, seed, stage and layer cotangents, with commit the adjoint update), as small_backward_kernel
 // describes it; with REG the parameter gradient of the block's rows beside it, in the registers of eight warps, pieces of 16 x 8: a step's
 // sums first, then g += (h / S) dg in float32.
-template <typename T, int MT, int NW, bool REG>
+template <typename T, int MT, int NW, bool REG, int KS1>
 __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) resident_backward_kernel(const __grid_constant__ ResidentMlp p) {
     chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -428,7 +831,7 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
     auto keep_at = [&](int j, int l) -> uint32_t { return base + (uint32_t)(p.b.keep + j * p.b.keep_stage + p.b.keep_at[l]); };
     const int tiles0 = up16(s.wp[0]) / 16, owners = tiles0 * 32;
     uint32_t* slots = (uint32_t*)(smem + p.b.slots);
-    float* scal = (float*)(slots + 2 * S * 2 * MT * owners);
+    float* scal = (float*)(slots + (4 * RK_MAX_STAGES + 6) * MT * owners);
     float* red = scal + 2 * kScalarWords;
     const float* fl = (const float*)(smem + (size_t)p.g.w_elems * sizeof(T));
     const T* traj = (const T*)s.traj;
@@ -453,6 +856,7 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
         auto pl = [&](int i) { return piece[i] >> 20; };
         auto pm = [&](int i) { return piece[i] >> 10 & 0x3FF; };
         auto pn = [&](int i) { return (piece[i] & 0x3FF) == 0x3FF ? -1 : piece[i] & 0x3FF; };
+        uint32_t off[kPieces], off2[kPieces];      // this lane's offsets in the rows' buffers of outputs and inputs
         float acc[kPieces][4], tot[kPieces][4];
         if (REG) {
 #pragma unroll
@@ -464,6 +868,10 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
                     if (id < tm * tn) piece[i] = l << 20 | (id / tn * 16) << 10 | (id % tn * 8 < s.wp[l] ? id % tn * 8 : 0x3FF);
                     id -= tm * tn;
                 }
+                const int l = piece[i] < 0 ? 0 : pl(i), m0 = pm(i), n0 = piece[i] < 0 || pn(i) < 0 ? 0 : pn(i), sz = p.g.sw[l + 1], sx = p.g.sw[l];
+                off[i] = (uint32_t)(MT == 1 ? ((lane >> 4) == 0 ? (lane & 7) * sz + m0 + (lane >> 3) * 8 : (lane & 7) * sx + n0)
+                                            : ((lane & 7) + (lane >> 4) * 8) * sz + m0 + ((lane >> 3) & 1) * 8) * 2u;
+                off2[i] = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * sx + n0) * 2u;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) acc[i][q] = tot[i][q] = 0.f;
             }
@@ -495,25 +903,24 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
                         rows_out<T>(z, sz, (T*)s.zs[l + 1] + (long long)(st * S + j) * B * s.wp[l + 1], s.wp[l + 1], R, r0, B, tid, threads);
                     } else {
                         const uint32_t x = x_of(st, j, l);
-                        const int sx = p.g.sw[l];
                         uint32_t ones = 0u;      // column 0: ones, column 1: the rounded stage time
                         if ((lane >> 2) == 0) ones = cvt_pack<T>(1.f, 1.f);
                         else if ((lane >> 2) == 1 && s.time && l == 0) ones = cvt_pack<T>(sc.tau16[j], sc.tau16[j]);
+                        const uint32_t at = MT == 2 || (lane >> 4) == 0 ? z : x;
 #pragma unroll
                         for (int i = 0; i < kPieces; ++i) {
                             if (pl(i) != l) continue;
-                            const int n0 = pn(i) < 0 ? 0 : pn(i);
+                            const bool cols = pn(i) >= 0;
                             if constexpr (MT == 1) {
                                 uint32_t f[4];      // both halves of the outputs, then the inputs (twice)
-                                const int q = lane >> 3;
-                                ldm4_t(q < 2 ? z + (uint32_t)(((lane & 7) * sz + pm(i) + q * 8) * 2) : x + (uint32_t)(((lane & 7) * sx + n0) * 2), f);
-                                mma_k8<T>(acc[i], f[0], f[1], pn(i) < 0 ? ones : f[2]);
+                                ldm4_t(at + off[i], f);
+                                mma_k8<T>(acc[i], f[0], f[1], cols ? f[2] : ones);
                             } else {
                                 static_assert(!REG || MT <= 2, "16 rows at most");
                                 uint32_t a[4], b0, b1;
-                                ldm4_t(z + (uint32_t)((((lane & 7) + (lane >> 4) * 8) * sz + pm(i) + ((lane >> 3) & 1) * 8) * 2), a);
-                                ldm2_t(x + (uint32_t)((((lane & 7) + ((lane >> 3) & 1) * 8) * sx + n0) * 2), b0, b1);
-                                mma_k16<T>(acc[i], a, pn(i) < 0 ? ones : b0, pn(i) < 0 ? ones : b1);
+                                ldm4_t(at + off[i], a);
+                                ldm2_t(x + off2[i], b0, b1);
+                                mma_k16<T>(acc[i], a, cols ? b0 : ones, cols ? b1 : ones);
                             }
                         }
                     }
@@ -548,126 +955,109 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
         }
         return;
     }
+    if constexpr (KS1 > 0) { linear_backward<T, MT, KS1>(p, base, slots + threadIdx.x, scal, fl, r0); return; }
     // ---- the chain
     const Lane<T, MT> ln;
     const bool owner = ln.warp < tiles0;
     const int f0 = ln.warp * 16;
     uint32_t* ks = slots + threadIdx.x;                                // k_j and psi_j of this thread's values
-    uint32_t* ps = ks + S * 2 * MT * owners;
-    const float lim = OverflowLimit<T>::value();
+    uint32_t* ps = ks + RK_MAX_STAGES * 2 * MT * owners;
+    uint32_t* vs = ps + RK_MAX_STAGES * 2 * MT * owners;                           // seed: word (2 m + h) * owners
+    float* as = (float*)(vs + 2 * MT * owners);                        // adjoint: word (4 m + i) * owners
     const int e = s.e_dev != nullptr ? *s.e_dev : s.e;
-    bool bad = false;
-    auto note = [&](float x, float yv) { bad |= !(fabsf(x) < lim) | !(fabsf(yv) < lim); };
-    float a[MT][4];
+    const float scale = ldexpf(1.f, e), unscale = ldexpf(1.f, -e);      // (|e| <= 100: products with them are what ldexp gives)
+    uint32_t bad = 0u;
+    if (owner && s.vjp) {
 #pragma unroll
-    for (int m = 0; m < MT; ++m)
+        for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
-            a[m][i] = owner && s.vjp && r < B && c < d ? s.a[(long long)r * d + c] : 0.f;
-        }
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
+                as[(4 * m + i) * owners] = r < B && c < d ? s.a[(long long)r * d + c] : 0.f;
+            }
+    }
+    Ops<MT> ahead;
+    const float bias0 = owner ? fl[p.g.b_at[L - 1] + f0 + ln.g] : 0.f, bias1 = owner ? fl[p.g.b_at[L - 1] + f0 + 8 + ln.g] : 0.f;
+    Phase ph;
+    // what follows a phase: the operands' place is settled at its start, the weights are requested at its end
+    auto first_back = [&](int par) { return backward_phase(p, ln, base, L - 1, z0_at(par)); };
+    auto take = [&](const Phase& nx, bool back) {
+        ph = nx;
+        if (ph.on) { if (back) request_weights<MT, true>(ahead, ph); else request_weights<MT, false>(ahead, ph); }
+    };
+    const bool evaluates = s.recompute && (S > 1 || L > 1 || want_t);      // whether anything is evaluated before the vector-Jacobian product
     for (int st = 0; st < s.count; ++st) {
         const int n = s.step_hi - st;
         const RkStepScalars& sc = *(const RkStepScalars*)(scal + (st & 1) * kScalarWords);
-        uint32_t vv[MT][2];
         float t_phi = 0.f, t_dt = 0.f, t_dh = 0.f;
-        // seed Q16(S a); kappa_j = Q16(b_j v + sum_{l > j} (h a_lj) psi_l), into the rows' buffer of its parity
-        auto put_kappa = [&](int j, int par, float& dtau) {
-            float ha[RK_MAX_STAGES];
+        float dtau_k = 0.f;                // (one layer: of the stage cotangent in the buffer)
+        auto put_kappa = [&](int par, uint32_t (&o)[MT][2]) {
+            if (want_t && L == 1 && s.time) {
+                const float wA = fl[p.g.t_at + f0 + ln.g], wB = fl[p.g.t_at + f0 + 8 + ln.g];
 #pragma unroll
-            for (int l = 1; l < RK_MAX_STAGES; ++l) ha[l] = l > j && l < S ? sc.ha[l][j] : 0.f;
-            const float bj = sc.b[j];
-            float wA = 0.f, wB = 0.f;
-            if (want_t && L == 1 && s.time) { wA = fl[p.g.t_at + f0 + ln.g]; wB = fl[p.g.t_at + f0 + 8 + ln.g]; }
-            uint32_t o[MT][2];
+                for (int m = 0; m < MT; ++m)
 #pragma unroll
-            for (int m = 0; m < MT; ++m)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float v0 = bj * lo_of<T>(vv[m][h]), v1 = bj * hi_of<T>(vv[m][h]);
-#pragma unroll
-                    for (int l = 1; l < RK_MAX_STAGES; ++l)
-                        if (ha[l] != 0.f) {
-                            const uint32_t q = ps[((l * MT + m) * 2 + h) * owners];
-                            v0 = fmaf(ha[l], lo_of<T>(q), v0);
-                            v1 = fmaf(ha[l], hi_of<T>(q), v1);
-                        }
-                    note(v0, v1);
-                    o[m][h] = cvt_pack<T>(v0, v1);
-                    const float wt = h ? wB : wA;
-                    dtau = fmaf(lo_of<T>(o[m][h]), wt, fmaf(hi_of<T>(o[m][h]), wt, dtau));
-                }
+                    for (int h = 0; h < 2; ++h) dtau_k = fmaf(lo_of<T>(o[m][h]), h ? wB : wA, fmaf(hi_of<T>(o[m][h]), h ? wB : wA, dtau_k));
+            }
             put_tile<MT>(ln, z0_at(par), p.g.sw[0], f0, s.wp[0], o);
         };
-        float dtau_k = 0.f;                // (one layer: of the cotangent in the buffer)
-        if (s.vjp && owner) {
+        if (s.vjp && owner) {              // seed Q16(S a); the last stage's cotangent Q16(b v)
+            uint32_t o[MT][2];
+            const float bj = sc.b[S - 1];
 #pragma unroll
             for (int m = 0; m < MT; ++m)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const float v0 = ldexpf(a[m][2 * h], e), v1 = ldexpf(a[m][2 * h + 1], e);
-                    note(v0, v1);
-                    vv[m][h] = cvt_pack<T>(v0, v1);
+                    const uint32_t v = cvt_pack<T>(as[(4 * m + 2 * h) * owners] * scale, as[(4 * m + 2 * h + 1) * owners] * scale);
+                    note_nonfinite<T>(v, bad);
+                    vs[(2 * m + h) * owners] = v;
+                    const float k0 = bj * lo_of<T>(v), k1 = bj * hi_of<T>(v);
+                    o[m][h] = cvt_pack<T>(k0, k1);
+                    note_nonfinite<T>(o[m][h], bad);
                 }
-            put_kappa(S - 1, 0, dtau_k);
+            put_kappa(0, o);
         }
+        if (evaluates) take(forward_phase(p, ln, base, 0, x00_at(st & 1)), false); else take(first_back(0), true);
         __syncthreads();
         if (s.recompute) {
-            uint32_t yb[MT][2];
-            if (owner) {
-#pragma unroll
-                for (int m = 0; m < MT; ++m) ldm2_t(ln.frag_at(x00_at(st & 1), p.g.sw[0], f0, m), yb[m][0], yb[m][1]);
-            }
+#pragma unroll 1
             for (int j = 0; j < S; ++j) {
                 const float tau = sc.tau16[j];
-                for (int l = 0; l < L; ++l) {
-                    const bool last = l == L - 1;
-                    if (last && j == S - 1 && !want_t) break;
-                    if (!last) {
-                        hidden_layer<T, MT, NW>(p, ln, base, fl, l, tau, x_of(st, j, l), x_of(st, j, l + 1));
-                    } else if (owner) {
-                        const int K = up16(s.wp[l]) / 16, sx = p.g.sw[l];
-                        const bool next = j + 1 < S;
-                        float v[MT][4];
-#pragma unroll
-                        for (int m = 0; m < MT; ++m)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) v[m][i] = (i & 1) ? hi_of<T>(yb[m][i >> 1]) : lo_of<T>(yb[m][i >> 1]);
-                        for (int q = 0; q < j && next; ++q) {
-                            const float c = sc.ha[j + 1][q];
-                            if (c == 0.f) continue;
-#pragma unroll
-                            for (int m = 0; m < MT; ++m)
-#pragma unroll
-                                for (int h = 0; h < 2; ++h) {
-                                    const uint32_t k = ks[((q * MT + m) * 2 + h) * owners];
-                                    v[m][2 * h] = fmaf(c, lo_of<T>(k), v[m][2 * h]);
-                                    v[m][2 * h + 1] = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
-                                }
-                        }
-                        float bA = fl[p.g.b_at[l] + f0 + ln.g], bB = fl[p.g.b_at[l] + f0 + 8 + ln.g];
-                        if (s.time && l == 0) { bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], bA); bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], bB); }
-                        const float c = next ? sc.ha[j + 1][j] : 0.f;
-                        float acc[MT][4];
-                        tile_product<T, MT, false>(acc, ln.w_fwd(base + (uint32_t)p.g.w_at[l] * 2u, p.g.sw[l], f0), 32u, ln.x_at(x_of(st, j, l), sx), (uint32_t)(16 * sx), K);
-                        uint32_t o[MT][2];
-#pragma unroll
-                        for (int m = 0; m < MT; ++m)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const float b = h ? bB : bA;
-                                const uint32_t k = cvt_pack<T>(acc[m][2 * h] + b, acc[m][2 * h + 1] + b);
-                                ks[((j * MT + m) * 2 + h) * owners] = k;
-                                if (c != 0.f) {
-                                    v[m][2 * h] = fmaf(c, lo_of<T>(k), v[m][2 * h]);
-                                    v[m][2 * h + 1] = fmaf(c, hi_of<T>(k), v[m][2 * h + 1]);
-                                }
-                                o[m][h] = cvt_pack<T>(v[m][2 * h], v[m][2 * h + 1]);
-                            }
-                        if (next) put_tile<MT>(ln, x0_of(st, j + 1), p.g.sw[0], f0, s.wp[0], o);
-                    }
+                const bool next = j + 1 < S, eval = next || want_t;      // (the last stage's derivative is wanted for the time terms alone)
+#pragma unroll 1
+                for (int l = 0; l + 1 < L; ++l) {
+                    const bool back = l + 2 == L && !eval;
+                    const Phase nx = back ? first_back(0) : forward_phase(p, ln, base, l + 1, keep_at(j, l + 1));
+                    hidden_layer<T, MT, NW>(p, ln, fl, l, tau, keep_at(j, l + 1), ph, ahead);
+                    take(nx, back);
                     __syncthreads();
                 }
+                if (!eval) break;
+                // with one layer nothing of the last stage is evaluated
+                const bool back = !next || (L == 1 && j + 2 == S && !want_t);
+                const Phase nx = back ? first_back(0) : forward_phase(p, ln, base, 0, keep_at(j + 1, 0));
+                if (owner) {
+                    StageTerms<T, MT> w;
+                    uint32_t yb[MT][2];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) ldm2_t(ln.frag_at(x00_at(st & 1), p.g.sw[0], f0, m), yb[m][0], yb[m][1]);
+                    w.start(next ? sc.ha[j + 1] : sc.hb, j, false, yb, ks, owners);
+                    w.bA = bias0; w.bB = bias1;
+                    if (s.time && L == 1) { w.bA = fmaf(tau, fl[p.g.t_at + f0 + ln.g], w.bA); w.bB = fmaf(tau, fl[p.g.t_at + f0 + 8 + ln.g], w.bB); }
+                    float acc[MT][4];
+                    tile_product<T, MT, false>(acc, ahead, ph);
+                    uint32_t o[MT][2];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            ks[((j * MT + m) * 2 + h) * owners] = w.stage(acc, m, h);
+                            o[m][h] = cvt_pack<T>(w.v[m][2 * h], w.v[m][2 * h + 1]);
+                        }
+                    if (next) put_tile<MT>(ln, keep_at(j + 1, 0), p.g.sw[0], f0, s.wp[0], o);
+                }
+                take(nx, back);
+                __syncthreads();
             }
         }
         if (!s.vjp) continue;
@@ -682,63 +1072,96 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
                         p0 = fmaf(sc.b[j], lo_of<T>(k), p0);
                         p1 = fmaf(sc.b[j], hi_of<T>(k), p1);
                     }
-                    t_phi = fmaf(p0, a[m][2 * h], fmaf(p1, a[m][2 * h + 1], t_phi));
+                    t_phi = fmaf(p0, as[(4 * m + 2 * h) * owners], fmaf(p1, as[(4 * m + 2 * h + 1) * owners], t_phi));
                 }
         }
-        int par = 0;
-        for (int j = S - 1; j >= 0; --j, par ^= 1) {
+#pragma unroll 1
+        for (int j = S - 1; j >= 0; --j) {
+            const int par = (S - 1 - j) & 1;
             float dtau = dtau_k;
             dtau_k = 0.f;
-            for (int l = L - 1; l >= 0; --l) {
-                const uint32_t z = l == L - 1 ? z0_at(par) : z_at(l + 1);
-                const int K = up16(s.wp[l + 1]) / 16, sz = p.g.sw[l + 1], sw = p.g.sw[l];
-                const uint32_t w = base + (uint32_t)p.g.w_at[l] * 2u, zx = ln.x_at(z, sz);
-                if (l > 0) {
-                    const int N = s.wp[l];
-                    const uint32_t H = x_of(st, j, l);
-                    for (int n0 = ln.warp * 16; n0 < N; n0 += NW * 16) {
-                        uint32_t hv[MT][2];
-#pragma unroll
-                        for (int m = 0; m < MT; ++m) ldm2_t(ln.frag_at(H, sw, n0, m), hv[m][0], hv[m][1]);
-                        float acc[MT][4];
-                        tile_product<T, MT, true>(acc, ln.w_bwd(w, sw, n0), (uint32_t)(32 * sw), zx, (uint32_t)(16 * sz), K);
-                        float wA = 0.f, wB = 0.f;
-                        if (want_t && l == 1 && s.time) { wA = fl[p.g.t_at + n0 + ln.g]; wB = fl[p.g.t_at + n0 + 8 + ln.g]; }
-                        uint32_t o[MT][2];
-#pragma unroll
-                        for (int m = 0; m < MT; ++m)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const float v0 = acc[m][2 * h] * act16_d<T>(s.act, lo_of<T>(hv[m][h])), v1 = acc[m][2 * h + 1] * act16_d<T>(s.act, hi_of<T>(hv[m][h]));
-                                note(v0, v1);
-                                o[m][h] = cvt_pack<T>(v0, v1);
-                                const float wt = h ? wB : wA;
-                                if (want_t) dtau = fmaf(lo_of<T>(o[m][h]), wt, fmaf(hi_of<T>(o[m][h]), wt, dtau));
-                            }
-                        put_tile<MT>(ln, z_at(l), sw, n0, N, o);
+#pragma unroll 1
+            for (int l = L - 1; l >= 1; --l) {
+                const Phase nx = backward_phase(p, ln, base, l - 1, z_at(l));
+                const int N = s.wp[l], sw = p.g.sw[l];
+                const uint32_t H = keep_at(j, l);
+#pragma unroll 1
+                for (int n0 = ln.warp * 16; n0 < N; n0 += NW * 16) {
+                    if (n0 >= NW * 16) {
+                        ph.w += NW * 32;
+                        request_weights<MT, true>(ahead, ph);
                     }
-                } else if (owner) {
+                    uint32_t hv[MT][2];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) ldm2_t(ln.frag_at(H, sw, n0, m), hv[m][0], hv[m][1]);
                     float acc[MT][4];
-                    tile_product<T, MT, true>(acc, ln.w_bwd(w, sw, f0), (uint32_t)(32 * sw), zx, (uint32_t)(16 * sz), K);
+                    tile_product<T, MT, true>(acc, ahead, ph);
+                    uint32_t o[MT][2];
 #pragma unroll
                     for (int m = 0; m < MT; ++m)
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            note(acc[m][2 * h], acc[m][2 * h + 1]);
-                            const uint32_t q = cvt_pack<T>(acc[m][2 * h], acc[m][2 * h + 1]);
-                            ps[((j * MT + m) * 2 + h) * owners] = q;
-                            if (!s.commit) {
-#pragma unroll
-                                for (int i = 0; i < 2; ++i) {
-                                    const int r = r0 + m * 8 + 2 * ln.t + i, c = f0 + ln.g + h * 8;
-                                    if (r < B && c < s.wp[0]) reinterpret_cast<unsigned short*>(s.psi[j])[(long long)r * s.wp[0] + c] = (unsigned short)(i ? q >> 16 : q & 0xFFFFu);
-                                }
-                            }
+                            const float v0 = acc[m][2 * h] * act16_d<T>(s.act, lo_of<T>(hv[m][h])), v1 = acc[m][2 * h + 1] * act16_d<T>(s.act, hi_of<T>(hv[m][h]));
+                            o[m][h] = cvt_pack<T>(v0, v1);
+                            note_nonfinite<T>(o[m][h], bad);
                         }
-                    if (j > 0) put_kappa(j - 1, par ^ 1, dtau_k);
+                    if (want_t && l == 1 && s.time) {
+                        const float wA = fl[p.g.t_at + n0 + ln.g], wB = fl[p.g.t_at + n0 + 8 + ln.g];
+#pragma unroll
+                        for (int m = 0; m < MT; ++m)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) dtau = fmaf(lo_of<T>(o[m][h]), h ? wB : wA, fmaf(hi_of<T>(o[m][h]), h ? wB : wA, dtau));
+                    }
+                    put_tile<MT>(ln, z_at(l), sw, n0, N, o);
                 }
+                take(nx, true);
                 __syncthreads();
             }
+            const Phase nx = first_back(par ^ 1);
+            if (owner) {
+                // psi_j; then kappa_{j-1} = Q16(b_{j-1} v + sum_{l >= j} (h a_{l,j-1}) psi_l)
+                float cl[RK_MAX_STAGES], bj = 0.f, cj = 0.f;
+#pragma unroll
+                for (int l = 2; l < RK_MAX_STAGES; ++l) cl[l] = j > 0 && l > j && l < S ? sc.ha[l][j - 1] : 0.f;
+                if (j > 0) { bj = sc.b[j - 1]; cj = sc.ha[j][j - 1]; }
+                float acc[MT][4];
+                tile_product<T, MT, true>(acc, ahead, ph);
+                uint32_t o[MT][2];
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t q = cvt_pack<T>(acc[m][2 * h], acc[m][2 * h + 1]);
+                        note_nonfinite<T>(q, bad);
+                        ps[((j * MT + m) * 2 + h) * owners] = q;
+                        if (!s.commit) {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                const int r = r0 + m * 8 + 2 * ln.t + i, c = f0 + ln.g + h * 8;
+                                if (r < B && c < s.wp[0]) reinterpret_cast<unsigned short*>(s.psi[j])[(long long)r * s.wp[0] + c] = (unsigned short)(i ? q >> 16 : q & 0xFFFFu);
+                            }
+                        }
+                        if (j > 0) {
+                            const uint32_t v = vs[(2 * m + h) * owners];
+                            float v0 = bj * lo_of<T>(v), v1 = bj * hi_of<T>(v);
+                            const float u0 = fmaf(cj, lo_of<T>(q), v0), u1 = fmaf(cj, hi_of<T>(q), v1);
+                            v0 = cj != 0.f ? u0 : v0;
+                            v1 = cj != 0.f ? u1 : v1;
+#pragma unroll
+                            for (int l = 2; l < RK_MAX_STAGES; ++l) {
+                                const uint32_t u = ps[((l * MT + m) * 2 + h) * owners];
+                                const float w0 = fmaf(cl[l], lo_of<T>(u), v0), w1 = fmaf(cl[l], hi_of<T>(u), v1);
+                                v0 = cl[l] != 0.f ? w0 : v0;
+                                v1 = cl[l] != 0.f ? w1 : v1;
+                            }
+                            o[m][h] = cvt_pack<T>(v0, v1);
+                            note_nonfinite<T>(o[m][h], bad);
+                        }
+                    }
+                if (j > 0) put_kappa(par ^ 1, o);
+            }
+            if (j > 0) take(nx, true);
+            __syncthreads();
             if (want_t) {
                 t_dt += dtau;
                 t_dh = fmaf(sc.c[j], dtau, t_dh);
@@ -759,7 +1182,7 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
             }
         }
         if (s.commit && owner) {      // a <- a + (h / S) sum_j psi_j (+ running cost)
-            const float coef = ldexpf(sc.h, -e);
+            const float coef = sc.h * unscale;
 #pragma unroll
             for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -772,14 +1195,12 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
                             d0 += lo_of<T>(q);
                             d1 += hi_of<T>(q);
                         }
-                    a[m][2 * h] = fmaf(coef, d0, a[m][2 * h]);
-                    a[m][2 * h + 1] = fmaf(coef, d1, a[m][2 * h + 1]);
-                    if (s.cot != nullptr) {
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {
-                            const int r = r0 + m * 8 + 2 * ln.t + i, c = f0 + ln.g + h * 8;
-                            if (r < B && c < d) a[m][2 * h + i] += s.cot[((long long)n * B + r) * d + c];
-                        }
+                    for (int i = 0; i < 2; ++i) {
+                        float v = fmaf(coef, i ? d1 : d0, as[(4 * m + 2 * h + i) * owners]);
+                        const int r = r0 + m * 8 + 2 * ln.t + i, c = f0 + ln.g + h * 8;
+                        if (s.cot != nullptr && r < B && c < d) v += s.cot[((long long)n * B + r) * d + c];
+                        as[(4 * m + 2 * h + i) * owners] = v;
                     }
                 }
         }
@@ -805,10 +1226,10 @@ __global__ void __launch_bounds__(NW * 32 + (REG ? kPieceWarps * 32 : 128), 1) r
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = r0 + m * 8 + 2 * ln.t + (i & 1), c = f0 + ln.g + (i >> 1) * 8;
-                if (r < B && c < d) s.a[(long long)r * d + c] = a[m][i];
+                if (r < B && c < d) s.a[(long long)r * d + c] = as[(4 * m + i) * owners];
             }
     }
-    warp_flag_or(s.flag, bad);
+    warp_flag_or(s.flag, any_nonfinite(bad));
 }
 
 // out = beta out + the blocks' gradients, in ascending order
@@ -831,38 +1252,58 @@ bool allow_cap(K kernel, bool (&done)[kMaxDevices]) {
     }
     return true;
 }
-template <typename T, int MT, int NW>
+template <typename T, int MT, int NW, int KS1>
 bool forward_t(const ResidentMlp& p, cudaStream_t st) {
     static bool done[kMaxDevices] = {false};
-    if (!allow_cap(resident_forward_kernel<T, MT, NW>, done)) return false;
+    if (!allow_cap(resident_forward_kernel<T, MT, NW, KS1>, done)) return false;
     ResidentMlp q = p;
     q.b = plan_bufs(p.g, p.s.L, p.s.stages, 8 * MT, false);
-    return launch_chain(resident_forward_kernel<T, MT, NW>, dim3(p.g.blocks_f), dim3(NW * 32 + 64), resident_smem(p.g, p.s.L, p.s.wp[0], p.s.stages, MT, false), st, q) == cudaSuccess;
+    return launch_chain(resident_forward_kernel<T, MT, NW, KS1>, dim3(p.g.blocks_f), dim3(NW * 32 + 64), resident_smem(p.g, p.s.L, p.s.wp[0], p.s.stages, MT, false), st, q) ==
+           cudaSuccess;
 }
 template <typename T, int MT>
 bool forward_t(const ResidentMlp& p, cudaStream_t st) {
-    return chain_warps(p.s.L, p.s.wp) == 8 ? forward_t<T, MT, 8>(p, st) : forward_t<T, MT, 16>(p, st);
+    if (p.s.L == 1 && p.s.wp[0] <= 128) {
+        const int w = image_width(1, p.s.wp[0]);
+        return w == 32 ? forward_t<T, MT, 8, 2>(p, st) : w == 64 ? forward_t<T, MT, 8, 4>(p, st) : w == 96 ? forward_t<T, MT, 8, 6>(p, st) : forward_t<T, MT, 8, 8>(p, st);
+    }
+    if (chain_warps(p.s.L, p.s.wp) == 8) return forward_t<T, MT, 8, 0>(p, st);
+    if constexpr (MT <= 2) return forward_t<T, MT, 16, 0>(p, st); else return false;
 }
 template <typename T>
 bool forward_t(const ResidentMlp& p, cudaStream_t st) {
     return p.g.mt_f == 1 ? forward_t<T, 1>(p, st) : p.g.mt_f == 2 ? forward_t<T, 2>(p, st) : forward_t<T, 4>(p, st);
 }
 // (`ready`: only makes the kernel ready for its launch)
-template <typename T, int MT, int NW, bool REG>
+template <typename T, int MT, int NW, bool REG, int KS1>
 bool backward_t(const ResidentMlp& p, cudaStream_t st, bool ready) {
     static bool done[kMaxDevices] = {false};
-    if (!allow_cap(resident_backward_kernel<T, MT, NW, REG>, done)) return false;
+    if (!allow_cap(resident_backward_kernel<T, MT, NW, REG, KS1>, done)) return false;
     if (ready) return true;
     ResidentMlp q = p;
     q.b = plan_bufs(p.g, p.s.L, p.s.stages, 8 * MT, true);
-    return launch_chain(resident_backward_kernel<T, MT, NW, REG>, dim3(p.g.blocks_b), dim3(NW * 32 + (REG ? kPieceWarps * 32 : 128)),
+    return launch_chain(resident_backward_kernel<T, MT, NW, REG, KS1>, dim3(p.g.blocks_b), dim3(NW * 32 + (REG ? kPieceWarps * 32 : 128)),
                         resident_smem(p.g, p.s.L, p.s.wp[0], p.s.stages, MT, true), st, q) == cudaSuccess;
+}
+template <typename T, int MT, bool REG>
+bool backward_t(const ResidentMlp& p, cudaStream_t st, bool ready) {
+    if (p.s.L == 1 && p.s.wp[0] <= 128) {
+        const int w = image_width(1, p.s.wp[0]);
+        bool ok = true;
+        if (p.s.tpart == nullptr)
+            ok = w == 32 ? backward_t<T, MT, 8, REG, 2>(p, st, ready) : w == 64 ? backward_t<T, MT, 8, REG, 4>(p, st, ready)
+               : w == 96 ? backward_t<T, MT, 8, REG, 6>(p, st, ready) : backward_t<T, MT, 8, REG, 8>(p, st, ready);
+        if (p.s.tpart == nullptr && !ready) return ok;
+        return ok && backward_t<T, MT, 8, REG, 0>(p, st, ready);      // the time terms are in the general code
+    }
+    if constexpr (!REG)
+        if (chain_warps(p.s.L, p.s.wp) != 8) return backward_t<T, MT, 16, false, 0>(p, st, ready);
+    return backward_t<T, MT, 8, REG, 0>(p, st, ready);
 }
 template <typename T>
 bool backward_t(const ResidentMlp& p, cudaStream_t st, bool ready) {
-    const bool narrow = chain_warps(p.s.L, p.s.wp) == 8, reg = p.partial != nullptr;
-    if (p.g.mt_b == 1) return !narrow ? backward_t<T, 1, 16, false>(p, st, ready) : reg ? backward_t<T, 1, 8, true>(p, st, ready) : backward_t<T, 1, 8, false>(p, st, ready);
-    return !narrow ? backward_t<T, 2, 16, false>(p, st, ready) : reg ? backward_t<T, 2, 8, true>(p, st, ready) : backward_t<T, 2, 8, false>(p, st, ready);
+    if (p.g.mt_b == 1) return p.partial != nullptr ? backward_t<T, 1, true>(p, st, ready) : backward_t<T, 1, false>(p, st, ready);
+    return p.partial != nullptr ? backward_t<T, 2, true>(p, st, ready) : backward_t<T, 2, false>(p, st, ready);
 }
 
 }  // namespace
@@ -873,11 +1314,11 @@ ResidentPlan plan_resident(mpode_dtype dt, int B, int L, const int* wp, bool bia
     int floats = 0;
     for (int l = 0; l <= L; ++l) {
         if (wp[l] > 1000) return g;
-        g.sw[l] = up16(wp[l]) + 8;
+        g.sw[l] = image_width(L, wp[l]) + 8;
     }
     for (int l = 0; l < L; ++l) {
         g.w_at[l] = g.w_elems;
-        g.w_elems += up16(wp[l + 1]) * g.sw[l];
+        g.w_elems += image_width(L, wp[l + 1]) * g.sw[l];
         g.b_at[l] = floats;
         floats += up16(wp[l + 1]);
     }
@@ -886,7 +1327,7 @@ ResidentPlan plan_resident(mpode_dtype dt, int B, int L, const int* wp, bool bia
     g.image_bytes = (g.w_elems * 2 + floats * 4 + 15) / 16 * 16;
     const int sms = sm_count();
     auto tiles = [&](int most) { int mt = 1; while (mt < most && (B + 8 * mt - 1) / (8 * mt) > sms) mt *= 2; return mt; };
-    g.mt_f = tiles(4); g.blocks_f = (B + 8 * g.mt_f - 1) / (8 * g.mt_f);
+    g.mt_f = tiles(chain_warps(L, wp) == 8 ? 4 : 2); g.blocks_f = (B + 8 * g.mt_f - 1) / (8 * g.mt_f);
     g.mt_b = tiles(2); g.blocks_b = (B + 8 * g.mt_b - 1) / (8 * g.mt_b);
     g.forward = g.blocks_f <= sms && resident_smem(g, L, wp[0], RK_MAX_STAGES, g.mt_f, false) <= (size_t)kCap;
     g.backward = g.blocks_b <= sms && resident_smem(g, L, wp[0], RK_MAX_STAGES, g.mt_b, true) <= (size_t)kCap;

@@ -6,7 +6,7 @@
 // layer in rk_fused.cu, while mma.sync fragments of 16 rows spread the batch over the SMs and hand over in registers and shared memory.
 // float32 runs the same program on the CUDA cores, 8 rows to a block, bound by the weights' way from L2 (about 64 bytes a cycle).
 // Weight gradients reduce over the whole batch: the chain keeps every layer input and cotangent of its steps in memory (L2), and a
-// second launch forms them, one block per 32 x 32 (or 16 x 16) piece of a layer's gradient, the reduction split over its warps.
+// second launch forms them (small_wgrad.cu).
 // Measured (training pass, before: rk_fused.cu): linear equation 64 wide, 1024 samples, 100 RK4 steps, bf16 8.6 -> 2.96 ms; MLP
 // 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 7.6 -> 4.77 ms.
 #include "small_mlp.h"
@@ -57,12 +57,6 @@ template <> __device__ __forceinline__ void mma16816<__nv_bfloat16>(float (&d)[4
 }
 __device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool on) {      // off: 16 zero bytes
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
 }
 
 template <typename T> __device__ __forceinline__ float act_f(int act, float z) {
@@ -323,55 +317,102 @@ __device__ __forceinline__ void fetch_scalars(const SmallMlp& p, const SmallSmem
 }
 __device__ __forceinline__ void scalars_ready() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// float32 on the CUDA cores: a thread has one column of the pass and all the block's rows, and where the pass has fewer than 256 columns
-// a share of each unit's 16 reduction steps; activations are broadcast from shared memory four reduction steps at a time.  The shares
-// meet in shared memory, added in order.
+// float32 on the CUDA cores: a lane has four columns and all the block's rows, and a quarter of each unit's 16 reduction steps (8 lanes side
+// by side share a quarter): 12 shared-memory reads of 16 bytes for 128 multiply-adds (16 rows: 20 for 256).  (One column a thread was 12 reads,
+// 8 of 16 bytes, for 32, and bound by them.)  A warp covers 32 columns; where the pass has fewer than 256 the warps that are left
+// share out the units.  The quarters meet by shuffles, each lane keeping a quarter of the rows, the warps' shares in shared memory; sums are
+// added in a fixed order.
 template <int MT, typename P, typename F>
 __device__ __forceinline__ void rows_gemm_f32(Ring& ring, const SmallSmem<float>& sm, const float* A, int K, int N, P&& pre, F&& epi) {
-    constexpr int R = kRows<float, MT>;
-    const int lane = threadIdx.x & 31;
+    constexpr int R = kRows<float, MT>, Q = R / 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, kg = lane >> 3;
     for (int c0 = 0; c0 < N; c0 += kPassCols) {
         const int cols = min(kPassCols, N - c0);
-        int ct = 64;
-        while (ct < cols) ct *= 2;
-        const int kg = threadIdx.x / ct, tc = threadIdx.x % ct, KG = kThreads / ct, rows = 16 / KG;
-        const bool on = tc < cols;
-        float acc[R];
+        int cw = 1;                                               // warps side by side; the others of the 8 take other units
+        while (cw * 32 < cols) cw *= 2;
+        const int kw = kWarps / cw, mine = warp / cw, col = (warp % cw) * 32 + (lane & 7) * 4;
+        const bool on = col < cols;                               // (widths are multiples of 8)
+        const int row0 = (kg >> 1) * (R / 2) + (kg & 1) * Q;      // the rows this lane keeps
+        if (kw == 1 && on) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = 0.f;
+            for (int g = 0; g < 2; ++g)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) pre(g, q, row0 + q, c0 + col + 2 * g);
+        }
+        float acc[R][4];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
+        int turn = 0;
         for (int k = 0; k < K; k += 16) {
             ring_wait(ring);
-            const float* w = (const float*)ring.stage() + tc;
-            const int ke = min(16, K - k);                        // a multiple of 8
-            for (int i = kg * rows; i < kg * rows + rows && i < ke; i += 4) {
-                float wb[4];
+            if (turn == mine && on && k + 4 * kg < K) {           // (K is a multiple of 8)
+                const float* w = (const float*)ring.stage() + (size_t)(4 * kg) * cols + col;
+                float4 wv[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) wb[q] = on ? w[(i + q) * cols] : 0.f;
+                for (int q = 0; q < 4; ++q) wv[q] = *reinterpret_cast<const float4*>(w + (size_t)q * cols);
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const float4 a = *reinterpret_cast<const float4*>(A + r * sm.lda + k + i);
-                    acc[r] = fmaf(a.w, wb[3], fmaf(a.z, wb[2], fmaf(a.y, wb[1], fmaf(a.x, wb[0], acc[r]))));
+                    const float4 a = *reinterpret_cast<const float4*>(A + r * sm.lda + k + 4 * kg);
+                    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        acc[r][0] = fmaf(av[q], wv[q].x, acc[r][0]);
+                        acc[r][1] = fmaf(av[q], wv[q].y, acc[r][1]);
+                        acc[r][2] = fmaf(av[q], wv[q].z, acc[r][2]);
+                        acc[r][3] = fmaf(av[q], wv[q].w, acc[r][3]);
+                    }
                 }
             }
+            if (++turn == kw) turn = 0;
             __syncwarp();
             if (lane == 0) mbar_arrive(&ring.empty[ring.s]);
             ring.next();
         }
+        float v[Q][4];
+        {
+            float h[R / 2][4];
+#pragma unroll
+            for (int r = 0; r < R / 2; ++r)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float send = (kg & 2) ? acc[r][i] : acc[r + R / 2][i];
+                    h[r][i] = ((kg & 2) ? acc[r + R / 2][i] : acc[r][i]) + __shfl_xor_sync(0xffffffffu, send, 16);
+                }
+#pragma unroll
+            for (int r = 0; r < Q; ++r)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float send = (kg & 1) ? h[r][i] : h[r + Q][i];
+                    v[r][i] = ((kg & 1) ? h[r + Q][i] : h[r][i]) + __shfl_xor_sync(0xffffffffu, send, 8);
+                }
+        }
+        if (kw == 1) {
+            if (on) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g)
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) epi(g, q, row0 + q, c0 + col + 2 * g, v[q][2 * g], v[q][2 * g + 1]);
+            }
+            continue;
+        }
+        const int ct = cw * 32;
         if (c0 > 0) work_sync();
 #pragma unroll
-        for (int r = 0; r < R; ++r) sm.scratch[(kg * R + r) * ct + tc] = acc[r];
+        for (int q = 0; q < Q; ++q) *reinterpret_cast<float4*>(sm.scratch + ((size_t)(mine * R + row0 + q) * ct + col)) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
         work_sync();
         const int hc = ct / 2;
         for (int i = threadIdx.x; i < R * hc; i += kThreads) {
             const int r = i / hc, c = 2 * (i - r * hc);
             if (c >= cols) continue;
             pre(0, 0, r, c0 + c);
-            float2 v = make_float2(0.f, 0.f);
-            for (int q = 0; q < KG; ++q) {
-                const float2 x = *reinterpret_cast<const float2*>(sm.scratch + (q * R + r) * ct + c);
-                v.x += x.x; v.y += x.y;
+            float2 u = make_float2(0.f, 0.f);
+            for (int q = 0; q < kw; ++q) {
+                const float2 x = *reinterpret_cast<const float2*>(sm.scratch + (size_t)(q * R + r) * ct + c);
+                u.x += x.x; u.y += x.y;
             }
-            epi(0, 0, r, c0 + c, v.x, v.y);
+            epi(0, 0, r, c0 + c, u.x, u.y);
         }
     }
 }
@@ -751,163 +792,6 @@ __global__ void __launch_bounds__(96) small_time_kernel(SmallMlp p, int blocks) 
     }
 }
 
-// ---------------------------------------------------------------- weight, bias and time-column gradients
-// One block per TM x TN piece of a layer's dW_l = sum over the rows of dZ_{l+1}^T X_l.  The rows of all stages of a step are one matrix
-// of stages * B rows; warp w takes the groups of 16 rows w, w + 8, ... through its own ring of asynchronous copies, so that no barrier
-// stands in the loop; the eight sums meet in shared memory in ascending order.  The bias gradient and the time column are two more
-// columns (ones, stage times) of the pieces in the first column of pieces.
-// CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of the step's gradient
-// that does not fit the format raises the flag.
-constexpr int kRing = 8;
-struct WgradItems { int first[SMALL_MAX_L + 1]; };
-template <typename T, int TM> constexpr size_t kWgradRingBytes = (size_t)kWarps * kRing * 16 * 2 * (TM + 8) * sizeof(T);
-template <typename T, int TM, int TN, bool CHECK>
-__global__ void __launch_bounds__(kThreads) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ WgradItems items) {
-    chain_begin();
-    constexpr int LA = TM + 8, LB = TN + 8;                       // row lengths in shared memory: eight rows hit eight 16-byte slots
-    constexpr int kStage = 16 * (LA + LB);
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T* ring = (T*)smem + (size_t)warp * kRing * kStage;
-    int l = 0;
-    while ((int)blockIdx.x >= items.first[l + 1]) ++l;
-    const int M = p.wp[l + 1], N = p.wp[l], tn = (N + TN - 1) / TN;
-    const int tile = (int)blockIdx.x - items.first[l], m0 = (tile / tn) * TM, n0 = (tile % tn) * TN;
-    const bool time = p.time && l == 0, sums = n0 == 0 && (p.bias || time);
-    const int KR = p.stages * p.B;
-    const int groups = (KR + 15) / 16, per = (groups + kWarps - 1) / kWarps;      // groups of this step for each warp
-    const int total = per * p.count;
-    const T* Z = (const T*)p.zs[l + 1];
-    const T* X = (const T*)p.xs[l];
-    auto fetch = [&](int it) {
-        if (it < total) {
-            const int s = it / per, g = (it - s * per) * kWarps + warp;
-            T* dst = ring + (it % kRing) * kStage;
-            const T* zs = Z + (long long)s * KR * M;
-            const T* xs = X + (long long)s * KR * N;
-            constexpr int PA = TM / 8, PB = TN / 8;
-#pragma unroll
-            for (int q = lane; q < 16 * (PA + PB); q += 32) {
-                const bool isA = q < 16 * PA;
-                const int r = isA ? q / PA : (q - 16 * PA) / PB, c = 8 * (isA ? q % PA : (q - 16 * PA) % PB);
-                const int row = g * 16 + r;
-                const bool on = row < KR && (isA ? m0 + c < M : n0 + c < N);
-                const T* src = isA ? zs + (long long)row * M + m0 + c : xs + (long long)row * N + n0 + c;
-                cp_async16(smem_u32(dst + (isA ? r * LA : 16 * LA + r * LB) + c), on ? src : (isA ? Z : X), on);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    float tot[TM / 16][TN / 8][4], acc[TM / 16][TN / 8][4], stot[TM / 16][4], sacc[TM / 16][4];
-    constexpr int LR = TN + 3;                                    // row of sums: TN columns, bias, time (odd stride)
-    float* red = (float*)(smem + (CHECK ? kWgradRingBytes<T, TM> : 0));      // [warps][TM][LR]
-    auto put_sums = [&](const float (&w)[TM / 16][TN / 8][4], const float (&ws)[TM / 16][4]) {
-#pragma unroll
-        for (int m = 0; m < TM / 16; ++m)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = m * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
-                float* row = red + ((size_t)warp * TM + r) * LR;
-#pragma unroll
-                for (int q = 0; q < TN / 8; ++q) row[q * 8 + c] = w[m][q][i];
-                if (c < 2) row[TN + c] = ws[m][i];
-            }
-    };
-    // the parameter that entry (r, c) of the piece belongs to, or -1; and the warps' sum
-    const int in_full = p.wr[l] + (time ? 1 : 0);
-    auto param_of = [&](int r, int c) -> long long {
-        const int m = m0 + r, n = n0 + c;
-        if (m >= p.wr[l + 1]) return -1;
-        if (c < TN) return n < p.wr[l] ? p.woff[l] + (long long)m * in_full + n : -1;
-        if (c == TN) return sums && p.bias ? p.boff[l] + m : -1;
-        return sums && time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1;
-    };
-    auto warps_sum = [&](int r, int c) {
-        float v = 0.f;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) v += red[((size_t)w * TM + r) * LR + c];
-        return v;
-    };
-    bool bad = false;
-#pragma unroll
-    for (int m = 0; m < TM / 16; ++m)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            stot[m][i] = sacc[m][i] = 0.f;
-#pragma unroll
-            for (int q = 0; q < TN / 8; ++q) tot[m][q][i] = acc[m][q][i] = 0.f;
-        }
-#pragma unroll
-    for (int k = 0; k < kRing - 1; ++k) fetch(k);
-    for (int it = 0; it < total; ++it) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
-        __syncwarp();
-        const T* buf = ring + (it % kRing) * kStage;
-        const int s = it / per, gi = it - s * per;
-        // fragments of dZ^T (rows = columns of dZ) and X from [16 rows][columns] blocks: transposing loads
-        uint32_t a[TM / 16][4], b[TN / 16][4];
-        const int r8 = lane & 7, id = lane >> 3;
-#pragma unroll
-        for (int m = 0; m < TM / 16; ++m) ldmatrix4_trans(smem_u32(buf + (r8 + (id >> 1) * 8) * LA + m * 16 + (id & 1) * 8), a[m]);
-#pragma unroll
-        for (int q = 0; q < TN / 16; ++q) ldmatrix4_trans(smem_u32(buf + 16 * LA + (r8 + (id & 1) * 8) * LB + q * 16 + (id >> 1) * 8), b[q]);
-#pragma unroll
-        for (int m = 0; m < TM / 16; ++m)
-#pragma unroll
-            for (int q = 0; q < TN / 8; ++q) mma16816<T>(acc[m][q], a[m], b[q >> 1][2 * (q & 1)], b[q >> 1][2 * (q & 1) + 1]);
-        if (sums) {      // column 0: ones, column 1: the rounded stage time of the row
-            uint32_t o0 = 0u, o1 = 0u;
-            const int c = lane >> 2;
-            if (c == 0) o0 = o1 = cvt_pack<T>(1.f, 1.f);
-            else if (c == 1 && time) {
-                const RkStepScalars& sc = p.scal[p.step_hi - s];
-                float t[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int row = (gi * kWarps + warp) * 16 + 2 * (lane & 3) + (i & 1) + (i >> 1) * 8;
-                    t[i] = row < KR ? sc.tau16[row / p.B] : 0.f;
-                }
-                o0 = cvt_pack<T>(t[0], t[1]);
-                o1 = cvt_pack<T>(t[2], t[3]);
-            }
-#pragma unroll
-            for (int m = 0; m < TM / 16; ++m) mma16816<T>(sacc[m], a[m], o0, o1);
-        }
-        __syncwarp();
-        fetch(it + kRing - 1);
-        if (gi == per - 1) {      // the step is complete
-            const float cf = p.coef[s];
-            if (CHECK) {
-                put_sums(acc, sacc);
-                __syncthreads();
-                for (int i = threadIdx.x; i < TM * (TN + 2); i += kThreads) {
-                    const int r = i / (TN + 2), c = i - r * (TN + 2);
-                    if (param_of(r, c) >= 0) bad |= Low<T>::nonfinite(Low<T>::from_f(warps_sum(r, c)));
-                }
-                __syncthreads();
-            }
-#pragma unroll
-            for (int m = 0; m < TM / 16; ++m)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    stot[m][i] = fmaf(cf, sacc[m][i], stot[m][i]); sacc[m][i] = 0.f;
-#pragma unroll
-                    for (int q = 0; q < TN / 8; ++q) { tot[m][q][i] = fmaf(cf, acc[m][q][i], tot[m][q][i]); acc[m][q][i] = 0.f; }
-                }
-        }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    put_sums(tot, stot);
-    __syncthreads();
-    for (int i = threadIdx.x; i < TM * (TN + 2); i += kThreads) {
-        const int r = i / (TN + 2), c = i - r * (TN + 2);
-        const long long at = param_of(r, c);
-        if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + warps_sum(r, c);
-    }
-    if (CHECK) warp_flag_or(p.flag, bad);
-}
-
 constexpr int kSmemCap = 220 * 1024;
 // ring buffers that fit beside the block's own shared memory: eight (128 KB ahead) at most, two at least
 template <typename T> int ring_buffers(const SmallMlp& p, int rows) {
@@ -956,29 +840,6 @@ bool backward_t(const SmallMlp& p, cudaStream_t st, bool ready = false) {
     launch_chain(small_backward_kernel<T, MT>, dim3(blocks), dim3(kThreads + 32), smem, st, q);
     return true;
 }
-template <typename T, int TM, bool CHECK>
-bool wgrad_t(const SmallMlp& p, const WgradItems& items, cudaStream_t st, bool ready) {
-    static bool done[kMaxDevices] = {false};
-    if (!allow_smem(small_wgrad_kernel<T, TM, TM, CHECK>, done)) return false;
-    if (ready) return true;
-    const size_t ring = kWgradRingBytes<T, TM>, red = (size_t)kWarps * TM * (TM + 3) * sizeof(float);
-    launch_chain(small_wgrad_kernel<T, TM, TM, CHECK>, dim3(items.first[p.L]), dim3(kThreads), CHECK ? ring + red : (ring > red ? ring : red), st, p, items);
-    return true;
-}
-template <typename T>
-bool wgrad_t(const SmallMlp& p, const WgradItems& items, bool wide, bool check, cudaStream_t st, bool ready = false) {
-    if (check) return wide ? wgrad_t<T, 32, true>(p, items, st, ready) : wgrad_t<T, 16, true>(p, items, st, ready);
-    return wide ? wgrad_t<T, 32, false>(p, items, st, ready) : wgrad_t<T, 16, false>(p, items, st, ready);
-}
-WgradItems wgrad_items(const SmallMlp& p, int tm) {
-    WgradItems it{};
-    for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + tm - 1) / tm) * ((p.wp[l] + tm - 1) / tm);
-    return it;
-}
-// 32 x 32 pieces where there are enough of them to occupy half the SMs, else 16 x 16 (each block reads its operands from L2: a smaller
-// piece reads more in total but less per block)
-bool wide_pieces(const SmallMlp& p) { return wgrad_items(p, 32).first[p.L] >= sm_count() / 2; }
-
 }  // namespace
 
 size_t small_pack_elems(mpode_dtype dt, int n, int k) {      // columns, reduction
@@ -1045,11 +906,8 @@ bool launch_small_forward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, lo
 }
 
 bool small_backward_ready(mpode_dtype dt, const SmallMlp& p) {
+    if (!small_wgrad_ready(dt, p)) return false;
     if (dt == MPODE_F32) return rows_tiles(dt, p.B) == 1 ? backward_t<float, 1>(p, nullptr, true) : backward_t<float, 2>(p, nullptr, true);
-    const bool wide = wide_pieces(p);
-    for (int check = 0; check < 2; ++check)
-        if (!(dt == MPODE_BF16 ? wgrad_t<__nv_bfloat16>(p, WgradItems{}, wide, check != 0, nullptr, true)
-                               : wgrad_t<__half>(p, WgradItems{}, wide, check != 0, nullptr, true))) return false;
     return dt == MPODE_BF16 ? backward_t<__nv_bfloat16, 1>(p, nullptr, true) : backward_t<__half, 1>(p, nullptr, true);
 }
 
@@ -1067,37 +925,6 @@ void launch_small_time(mpode_dtype dt, const SmallMlp& p, int blocks, cudaStream
     else if (dt == MPODE_F16) launch_chain(small_time_kernel<__half>, dim3(1), dim3(96), 0, st, p, blocks);
     else launch_chain(small_time_kernel<float>, dim3(1), dim3(96), 0, st, p, blocks);
     if (launches) ++*launches;
-}
-
-// float32: the CUDA-core contraction per layer and step (the rows of all stages are its reduction range; it takes the bias and the time
-// column along)
-static void small_wgrad_f32(const SmallMlp& p, cudaStream_t st, long long* launches) {
-    for (int s = 0; s < p.count; ++s)
-        for (int l = 0; l < p.L; ++l) {
-            const bool time = p.time && l == 0;
-            const size_t rows = (size_t)p.stages * p.B;
-            GemmArgs g{};
-            g.A = (const float*)p.zs[l + 1] + s * rows * p.wp[l + 1]; g.a_rs = 1; g.a_ks = p.wp[l + 1];
-            g.B = (const float*)p.xs[l] + s * rows * p.wp[l]; g.b_rs = 1; g.b_ks = p.wp[l];
-            g.M = p.wr[l + 1]; g.N = p.wr[l]; g.K = (int)rows;
-            g.epi = EPI_WGRAD; g.out = p.out + p.woff[l]; g.ldo = p.wr[l] + (time ? 1 : 0); g.beta = s == 0 ? p.beta : 1.f; g.alpha = p.coef[s];
-            g.split_k = 1; g.flag = p.flag;
-            g.row_sum = p.bias ? p.out + p.boff[l] : nullptr;
-            if (time) { g.row_sum_time = p.out + p.woff[l] + p.wr[l]; g.k_tau = p.scal[0].tau16 + (size_t)(p.step_hi - s) * (sizeof(RkStepScalars) / 4); g.k_per = p.B; }
-            // (the general kernel, which runs where this one cannot be launched, takes no sums along: the pass is not good)
-            if (!launch_gemm_simt(MPODE_F32, g, st, launches)) cudaMemsetAsync(p.err, 0xff, sizeof(unsigned), st);
-            if (tl_counters) ++tl_counters->simt;
-        }
-}
-
-void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
-    if (dt == MPODE_F32) { small_wgrad_f32(p, st, launches); return; }
-    const bool wide = wide_pieces(p);
-    const WgradItems items = wgrad_items(p, wide ? 32 : 16);
-    if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, items, wide, p.flag != nullptr, st);
-    else wgrad_t<__half>(p, items, wide, p.flag != nullptr, st);
-    if (launches) ++*launches;
-    if (tl_counters) ++tl_counters->fused;
 }
 
 }  // namespace mpode

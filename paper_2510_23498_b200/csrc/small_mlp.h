@@ -9,6 +9,7 @@ constexpr int SMALL_MAX_L = 4;
 
 struct SmallMlp {
     int B, L, stages, act, time, bias, round_increment;
+    int alone;                                         // every stage of the tableau depends on the one before it and no other
     int wr[SMALL_MAX_L + 1], wp[SMALL_MAX_L + 1];      // layer widths; rounded up to multiples of 8
     const float* theta; long long woff[SMALL_MAX_L], boff[SMALL_MAX_L];
     // weights in the order they are used (launch_small_pack): matrix instruction fragments, or rows in float32; forward: columns = outputs, reduction = inputs; backward: the other way round.  Biases and time column: low format, padded with zeros
@@ -50,6 +51,7 @@ bool small_backward_ready(mpode_dtype dt, const SmallMlp& p);
 void launch_small_backward(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 int small_blocks(mpode_dtype dt, int B);                               // blocks of the forward and backward kernels
 void launch_small_time(mpode_dtype dt, const SmallMlp& p, int blocks, cudaStream_t st, long long* launches);
+bool small_wgrad_ready(mpode_dtype dt, const SmallMlp& p);
 void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches);
 
 }  // namespace mpode

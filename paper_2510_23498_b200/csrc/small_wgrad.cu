@@ -1,0 +1,346 @@
+// Weight, bias and time-column gradients of the row-local paths: dW_l = sum over the rows of dZ_{l+1}^T X_l from the slabs of layer inputs and
+// cotangents, all layers and steps of a chunk in one launch.  The rows of all stages of a step are one matrix of stages * B rows, in pieces
+// of 64 (float32: 32) that the blocks of a cluster share out among themselves; a block keeps a 64 x 64 piece of a layer's gradient in
+// registers, its eight warps split over the piece and over the rows of a stage of the ring, and the cluster's sums meet in distributed shared
+// memory, added in a fixed order.  The bias gradient and the time column are two more columns (ones, stage times) of the pieces in the
+// first column of pieces.  CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of
+// the step's gradient that does not fit the format raises the flag.
+// What bounds it is the rows' way from the L2 (16 KB a stage at about 64 bytes a cycle and SM) and the fill of the ring.  16-bit formats multiply
+// with mma.sync.  float32 holds 8 x 8 sums a thread and reads four 16-byte words for 64 multiply-adds.
+#include "small_mlp.h"
+
+#include "profiler.h"
+#include "tc_ptx.cuh"
+#include "tensormap.h"
+
+namespace mpode {
+using namespace tc;
+namespace {
+
+constexpr int kThreads = 256, kTile = 64, kStages = 6, kMaxCluster = 8;
+constexpr int kRedRow = kTile + 3;                  // 64 columns, bias, time (odd stride)
+template <typename T> struct Geo {
+    static constexpr int E = 16 / sizeof(T), Pieces = kTile / E, Rows = 512 / Pieces;      // elements of 16 bytes; rows of a stage
+    static constexpr int LD = sizeof(T) == 4 ? kTile : kTile + 8;                          // (eight 16-bit rows hit eight 16-byte slots)
+    static constexpr int Groups = sizeof(T) == 4 ? 4 : 2;                                  // threads' groups that share out a stage's rows
+    static constexpr int StageBytes = 2 * Rows * LD * (int)sizeof(T);
+    static constexpr int Smem = kStages * StageBytes + Groups * kTile * kRedRow * 4;
+};
+
+struct Items { int first[SMALL_MAX_L + 1]; int S; };
+
+template <typename T> __device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
+template <> __device__ __forceinline__ void mma_k16<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+template <> __device__ __forceinline__ void mma_k16<__nv_bfloat16>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldm4_t(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, bool on) {      // off: 16 zero bytes
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float lds_of(uint32_t addr, int rank) {      // a word of another block's shared memory
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// A thread's share of the 64 x 64 piece and of the two columns of sums.
+// 16-bit: warp = 32 x 32 of the piece (two of two), half of the stage's rows.
+template <typename T> struct Sums {
+    float w[2][4][4], s[2][4];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[m][i] = 0.f;
+#pragma unroll
+                for (int n = 0; n < 4; ++n) w[m][n][i] = 0.f;
+            }
+    }
+    __device__ __forceinline__ void add(float c, const Sums& o) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[m][i] = fmaf(c, o.s[m][i], s[m][i]);
+#pragma unroll
+                for (int n = 0; n < 4; ++n) w[m][n][i] = fmaf(c, o.w[m][n][i], w[m][n][i]);
+            }
+    }
+    // rows 64 of a stage; tau: of each of this thread's rows; `sums`: whether the two columns are wanted
+    template <typename F>
+    __device__ __forceinline__ void stage(uint32_t A, uint32_t B, bool sums, F&& tau) {
+        constexpr int LD = Geo<T>::LD;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m0 = (warp & 1) * 32, n0 = ((warp >> 1) & 1) * 32;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k0 = ((warp >> 2) * 2 + q) * 16;
+            uint32_t a[2][4], b[2][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) ldm4_t(A + (uint32_t)(((k0 + (lane & 7) + (lane >> 4) * 8) * LD + m0 + m * 16 + ((lane >> 3) & 1) * 8) * 2), a[m]);
+#pragma unroll
+            for (int n = 0; n < 2; ++n) ldm4_t(B + (uint32_t)(((k0 + (lane & 7) + ((lane >> 3) & 1) * 8) * LD + n0 + n * 16 + (lane >> 4) * 8) * 2), b[n]);
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) mma_k16<T>(w[m][n], a[m], b[n >> 1][2 * (n & 1)], b[n >> 1][2 * (n & 1) + 1]);
+            if (sums && n0 == 0) {      // column 0: ones, column 1: the rounded stage time of the row
+                uint32_t o0 = 0u, o1 = 0u;
+                const int c = lane >> 2, k = k0 + 2 * (lane & 3);
+                if (c == 0) o0 = o1 = cvt_pack<T>(1.f, 1.f);
+                else if (c == 1) { o0 = cvt_pack<T>(tau(k), tau(k + 1)); o1 = cvt_pack<T>(tau(k + 8), tau(k + 9)); }
+#pragma unroll
+                for (int m = 0; m < 2; ++m) mma_k16<T>(s[m], a[m], o0, o1);
+            }
+        }
+    }
+    __device__ __forceinline__ void put(float* red) const {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m0 = (warp & 1) * 32, n0 = ((warp >> 1) & 1) * 32;
+        red += (warp >> 2) * kTile * kRedRow;
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float* row = red + (m0 + m * 16 + (lane >> 2) + (i >> 1) * 8) * kRedRow;
+                const int c = 2 * (lane & 3) + (i & 1);
+#pragma unroll
+                for (int n = 0; n < 4; ++n) row[n0 + n * 8 + c] = w[m][n][i];
+                if (n0 == 0 && c < 2) row[kTile + c] = s[m][i];
+            }
+    }
+};
+// float32: a group of 64 threads has the whole piece, 8 x 8 a thread (two by two squares of 4), and every fourth of the stage's rows
+template <> struct Sums<float> {
+    float w[8][8], b[8], t[8];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            b[i] = t[i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[i][j] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void add(float c, const Sums& o) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            b[i] = fmaf(c, o.b[i], b[i]);
+            t[i] = fmaf(c, o.t[i], t[i]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[i][j] = fmaf(c, o.w[i][j], w[i][j]);
+        }
+    }
+    template <typename F>
+    __device__ __forceinline__ void stage(uint32_t A, uint32_t B, bool sums, F&& tau) {
+        const int g = threadIdx.x >> 6, tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
+#pragma unroll 4
+        for (int q = 0; q < Geo<float>::Rows / 4; ++q) {
+            const int k = g * (Geo<float>::Rows / 4) + q;
+            const uint32_t ra = A + (uint32_t)((k * kTile + ty * 4) * 4), rb = B + (uint32_t)((k * kTile + tx * 4) * 4);
+            const uint4 a0 = lds128(ra), a1 = lds128(ra + 128), b0 = lds128(rb), b1 = lds128(rb + 128);
+            const float av[8] = {__uint_as_float(a0.x), __uint_as_float(a0.y), __uint_as_float(a0.z), __uint_as_float(a0.w),
+                                 __uint_as_float(a1.x), __uint_as_float(a1.y), __uint_as_float(a1.z), __uint_as_float(a1.w)};
+            const float bv[8] = {__uint_as_float(b0.x), __uint_as_float(b0.y), __uint_as_float(b0.z), __uint_as_float(b0.w),
+                                 __uint_as_float(b1.x), __uint_as_float(b1.y), __uint_as_float(b1.z), __uint_as_float(b1.w)};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) w[i][j] = fmaf(av[i], bv[j], w[i][j]);
+            if (sums && tx == 0) {
+                const float tk = tau(k);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { b[i] += av[i]; t[i] = fmaf(av[i], tk, t[i]); }
+            }
+        }
+    }
+    __device__ __forceinline__ void put(float* red) const {
+        const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
+        red += (threadIdx.x >> 6) * kTile * kRedRow;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float* row = red + (ty * 4 + (i & 3) + (i >> 2) * 32) * kRedRow;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) row[tx * 4 + (j & 3) + (j >> 2) * 32] = w[i][j];
+            if (tx == 0) { row[kTile] = b[i]; row[kTile + 1] = t[i]; }
+        }
+    }
+};
+
+template <typename T, bool CHECK>
+__global__ void __launch_bounds__(kThreads, 1) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ Items items) {
+    chain_begin();
+    using G = Geo<T>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ float taus[SMALL_MAX_CHUNK][RK_MAX_STAGES];
+    const int S = items.S, rank = (int)blockIdx.x % S, item = (int)blockIdx.x / S;
+    int l = 0;
+    while (item >= items.first[l + 1]) ++l;
+    const int M = p.wp[l + 1], N = p.wp[l], tn = (N + kTile - 1) / kTile;
+    const int m0 = (item - items.first[l]) / tn * kTile, n0 = (item - items.first[l]) % tn * kTile;
+    const bool time = p.time && l == 0, sums = n0 == 0 && (p.bias || time);
+    const int KR = p.stages * p.B, pieces = (KR + G::Rows - 1) / G::Rows;
+    const int mine = rank < pieces ? (pieces - rank + S - 1) / S : 0;      // pieces rank, rank + S, ... of every step
+    if ((int)threadIdx.x < p.count * RK_MAX_STAGES) taus[threadIdx.x >> 2][threadIdx.x & 3] = p.scal[p.step_hi - (int)(threadIdx.x >> 2)].tau16[threadIdx.x & 3];
+    const T* Z = (const T*)p.zs[l + 1];
+    const T* X = (const T*)p.xs[l];
+    const uint32_t ring = smem_u32(smem);
+    float* red = (float*)(smem + kStages * G::StageBytes);
+    // this thread's four pieces of 16 bytes of a stage: row, column, operand are the same for every stage
+    int fs = 0, fi = 0, fslot = 0;
+    auto fetch = [&]() {
+        if (fs < p.count && mine > 0) {
+            const int row0 = (rank + S * fi) * G::Rows;
+            const uint32_t dst = ring + (uint32_t)(fslot * G::StageBytes);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int id = (int)threadIdx.x + kThreads * (q & 1), r = id / G::Pieces, c = id % G::Pieces * G::E;
+                const bool isA = q < 2;
+                const int row = row0 + r, W = isA ? M : N, col = (isA ? m0 : n0) + c;
+                const bool on = row < KR && col < W;
+                const T* src = (isA ? Z : X) + ((long long)fs * KR + row) * W + col;
+                copy16(dst + (uint32_t)(((isA ? 0 : G::Rows) + r) * G::LD + c) * (uint32_t)sizeof(T), on ? src : Z, on);
+            }
+            if (++fi == mine) { fi = 0; ++fs; }
+            if (++fslot == kStages) fslot = 0;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    Sums<T> acc, tot;
+    acc.zero(); tot.zero();
+    const int in_full = p.wr[l] + (time ? 1 : 0);
+    auto param_of = [&](int r, int c) -> long long {
+        const int m = m0 + r, n = n0 + c;
+        if (m >= p.wr[l + 1]) return -1;
+        if (c < kTile) return n < p.wr[l] ? p.woff[l] + (long long)m * in_full + n : -1;
+        if (c == kTile) return sums && p.bias ? p.boff[l] + m : -1;
+        return sums && time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1;
+    };
+    const uint32_t red_u = smem_u32(red);
+    // the groups' sums meet in the block's own shared memory first: a word of another block's takes some 400 cycles
+    auto meet = [&](const Sums<T>& w) {
+        w.put(red);
+        __syncthreads();
+        for (int i = threadIdx.x; i < kTile * kRedRow; i += kThreads) {
+            float v = red[i];
+#pragma unroll
+            for (int g = 1; g < G::Groups; ++g) v += red[g * kTile * kRedRow + i];
+            red[i] = v;
+        }
+        cluster_sync();
+    };
+    auto cluster_sum = [&](int r, int c) {
+        float v[kMaxCluster], x = 0.f;
+#pragma unroll
+        for (int z = 0; z < kMaxCluster; ++z) v[z] = z < S ? lds_of(red_u + (uint32_t)(r * kRedRow + c) * 4u, z) : 0.f;
+#pragma unroll
+        for (int z = 0; z < kMaxCluster; ++z) x += v[z];
+        return x;
+    };
+    bool bad = false;
+    for (int k = 0; k < kStages - 1; ++k) fetch();
+    __syncthreads();
+    int slot = 0;
+    for (int s = 0; s < p.count; ++s) {
+        for (int i = 0; i < mine; ++i) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+            __syncthreads();
+            fetch();      // into the stage that every thread has left behind at this barrier
+            const int row0 = (rank + S * i) * G::Rows;
+            const uint32_t A = ring + (uint32_t)(slot * G::StageBytes);
+            acc.stage(A, A + (uint32_t)(G::Rows * G::LD * sizeof(T)), sums, [&](int k) {
+                const int row = row0 + k;
+                return taus[s][(row >= p.B) + (row >= 2 * p.B) + (row >= 3 * p.B)];      // (rows behind the last are zero)
+            });
+            if (++slot == kStages) slot = 0;
+        }
+        if (CHECK) {
+            meet(acc);
+            for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
+                const int r = i / (kTile + 2), c = i - r * (kTile + 2);
+                if (param_of(r, c) >= 0) bad |= Low<T>::nonfinite(Low<T>::from_f(cluster_sum(r, c)));
+            }
+            cluster_sync();
+        }
+        tot.add(p.coef[s], acc);
+        acc.zero();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    meet(tot);
+    for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
+        const int r = i / (kTile + 2), c = i - r * (kTile + 2);
+        const long long at = param_of(r, c);
+        if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + cluster_sum(r, c);
+    }
+    cluster_sync();      // (no block ends while another reads its sums)
+    if (CHECK) warp_flag_or(p.flag, bad);
+}
+
+template <typename T, bool CHECK>
+bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready) {
+    static bool done[kMaxDevices] = {false};
+    const int dev = current_device();
+    if (!done[dev]) {
+        if (cudaFuncSetAttribute(small_wgrad_kernel<T, CHECK>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<T>::Smem) != cudaSuccess) { cudaGetLastError(); return false; }
+        done[dev] = true;
+    }
+    if (ready) return true;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(items.first[p.L] * items.S));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Geo<T>::Smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)items.S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, small_wgrad_kernel<T, CHECK>, p, items) == cudaSuccess;
+}
+template <typename T>
+bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready, bool check) {
+    return check ? wgrad_t<T, true>(p, items, st, ready) : wgrad_t<T, false>(p, items, st, ready);
+}
+
+}  // namespace
+
+bool small_wgrad_ready(mpode_dtype dt, const SmallMlp& p) {
+    for (int check = 0; check < 2; ++check)
+        if (!(dt == MPODE_BF16  ? wgrad_t<__nv_bfloat16>(p, Items{}, nullptr, true, check != 0)
+              : dt == MPODE_F16 ? wgrad_t<__half>(p, Items{}, nullptr, true, check != 0)
+                                : wgrad_t<float>(p, Items{}, nullptr, true, check != 0))) return false;
+    return true;
+}
+
+// A cluster as large as it takes to give every SM a block, with two stages of rows for each of its blocks
+void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
+    Items it{};
+    for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + kTile - 1) / kTile) * ((p.wp[l] + kTile - 1) / kTile);
+    const int rows = dt == MPODE_F32 ? Geo<float>::Rows : Geo<__half>::Rows, pieces = (p.stages * p.B + rows - 1) / rows;
+    it.S = sm_count() / it.first[p.L];
+    if (it.S > kMaxCluster) it.S = kMaxCluster;
+    if (it.S > pieces / 2) it.S = pieces / 2;
+    if (it.S < 1) it.S = 1;
+    if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, it, st, false, p.flag != nullptr);
+    else if (dt == MPODE_F16) wgrad_t<__half>(p, it, st, false, p.flag != nullptr);
+    else wgrad_t<float>(p, it, st, false, p.flag != nullptr);
+    if (launches) ++*launches;
+    if (tl_counters) {
+        if (dt == MPODE_F32) tl_counters->simt += (long long)p.L * p.count;
+        else ++tl_counters->fused;
+    }
+}
+
+}  // namespace mpode

@@ -228,6 +228,10 @@ public:
         SmallMlp p = small_params(ws);
         p.stages = fs.stages; p.n_steps = fs.n_steps; p.round_increment = fs.round_increment; p.traj = const_cast<void*>(fs.traj);
         p.wait_ns = fs.wait_ns; p.starve = fs.starve;
+        p.alone = 1;
+        for (int j = 1; j < fs.stages; ++j)
+            for (int l = 0; l < j; ++l)
+                if ((fs.a[j * fs.stages + l] != 0.0) != (l == j - 1)) p.alone = 0;
         return p;
     }
     bool small_usable(const FusedSolve& fs) const {
