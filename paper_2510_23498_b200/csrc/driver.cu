@@ -26,6 +26,9 @@ const mpode_tableau kEuler = {1, kEulerA, kEulerB, kEulerC};
 const mpode_tableau kRk4 = {4, kRk4A, kRk4B, kRk4C};
 
 constexpr int kExpMin = -100, kExpMax = 100;
+// Page-locked block of a context with dynamic scaling: mirror of the scale state, then where the call's last copies land (scalar words, scale
+// log, t')
+constexpr size_t kMirrorBytes = 192;
 
 inline int precision_bits(mpode_dtype dt) { return dt == MPODE_F16 ? 11 : dt == MPODE_BF16 ? 8 : 24; }
 
@@ -511,7 +514,7 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
     const int* e_dev = dynamic ? sstate : nullptr;
     if (dynamic && c->mirror_host == nullptr && c->allow_side) {        // first dynamic pass through an entry point that may allocate
         void* mh = nullptr;
-        if (cudaHostAlloc(&mh, 64, cudaHostAllocMapped) == cudaSuccess) {
+        if (cudaHostAlloc(&mh, kMirrorBytes + (size_t)c->max_steps * 9 + ((size_t)c->max_steps + 1) * sizeof(float) + 16, cudaHostAllocMapped) == cudaSuccess) {
             void* md = nullptr;
             if (cudaHostGetDevicePointer(&md, mh, 0) == cudaSuccess &&
                 cudaEventCreateWithFlags(&c->ev_step[0], cudaEventDisableTiming) == cudaSuccess &&
@@ -573,6 +576,7 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
         v->fused_recompute(st, ws, fs, N - 1, L);
     }
 
+    bool seen = false;                          // the mapped words have told that the attempt of this round's last step failed
     int start = N - 1;                          // first step of this round of queueing (dynamic scaling: the step to repeat)
     int fail_step = -1, fail_count = 0;         // the step that failed last and how many of its attempts did
     int recomputed = -1;                        // the step whose stages the workspace holds
@@ -596,6 +600,7 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
         }
     };
     for (;;) {
+    seen = false;
     for (int i = start; i >= 0 && !all_done; --i) {
         if (recomputed != i) queue_recompute(i);     // a repeated attempt finds its step's stages still in place
         StepTimes tm = step_times(c, i);
@@ -693,6 +698,7 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
                     cudaEventSynchronize(c->ev_step[i & 1]);
                     ++c->stats.step_waits;
                     failed = mirror_h[1] >= 0 || mirror_h[2] != 0;
+                    seen = mirror_h[1] >= 0 && mirror_h[2] == 0;
                 } else {
                     cudaMemcpyAsync(hstate, sstate, sizeof hstate, cudaMemcpyDeviceToHost, st);
                     cudaStreamSynchronize(st);
@@ -710,22 +716,46 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
         }
     }
     if (!dynamic) break;
-    // one drain per round: the state and, should this have been the last round, everything else the host reads
-    cudaMemcpyAsync(hstate, sstate, sizeof hstate, cudaMemcpyDeviceToHost, st);
-    if (log) {
-        cudaMemcpyAsync(log->exp_used, slog_exp, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(log->attempts, slog_att, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(log->doubled, slog_dbl, (size_t)N, cudaMemcpyDeviceToHost, st);
-    }
-    if (tg) cudaMemcpyAsync(dt_host, tprime, ((size_t)N + 1) * sizeof(float), cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(&dev_err, flag + 2, 4, cudaMemcpyDeviceToHost, st);
-    if (c->ws_forward != nullptr && c->ws_forward != ws)     // the forward pass ran on another workspace: its error word lives there
-        cudaMemcpyAsync(&fwd_err, (unsigned*)at(c->ws_forward, c->lay.scal) + 2, 4, cudaMemcpyDeviceToHost, st);
-    cudaStreamSynchronize(st);
-    ++c->stats.host_syncs;
-    {
+    if (seen && (mirror_h[1] == fail_step ? fail_count : 0) + 1 < c->pol.k_max) {
+        // a repeat follows, and all that it needs is in the mapped words (five copies to pageable memory took 60 us for each overflow)
+        cudaStreamSynchronize(st);
+        ++c->stats.host_syncs;
+        hstate[0] = mirror_h[0]; hstate[1] = mirror_h[1]; hstate[2] = 0;
+    } else {
+        // one drain: the state and, should this have been the last round, everything else the host reads
+        unsigned char* pin = paced ? (unsigned char*)c->mirror_host : nullptr;
+        unsigned* words = paced ? (unsigned*)(pin + 64) : nullptr;               // the scalar slice: flag, norm, error word, ..., scale state
+        unsigned char* plog = paced ? pin + kMirrorBytes : nullptr;
+        float* pt = paced ? (float*)(pin + kMirrorBytes + ((size_t)c->max_steps * 9 + 15) / 16 * 16) : nullptr;
+        if (paced) {
+            cudaMemcpyAsync(words, flag, 64, cudaMemcpyDeviceToHost, st);
+            if (log) cudaMemcpyAsync(plog, slog_exp, (size_t)c->max_steps * 9, cudaMemcpyDeviceToHost, st);
+        } else {
+            cudaMemcpyAsync(hstate, sstate, sizeof hstate, cudaMemcpyDeviceToHost, st);
+            if (log) {
+                cudaMemcpyAsync(log->exp_used, slog_exp, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
+                cudaMemcpyAsync(log->attempts, slog_att, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
+                cudaMemcpyAsync(log->doubled, slog_dbl, (size_t)N, cudaMemcpyDeviceToHost, st);
+            }
+            cudaMemcpyAsync(&dev_err, flag + 2, 4, cudaMemcpyDeviceToHost, st);
+        }
+        if (tg) cudaMemcpyAsync(paced ? pt : dt_host, tprime, ((size_t)N + 1) * sizeof(float), cudaMemcpyDeviceToHost, st);
+        if (c->ws_forward != nullptr && c->ws_forward != ws)     // the forward pass ran on another workspace: its error word lives there
+            cudaMemcpyAsync(&fwd_err, (unsigned*)at(c->ws_forward, c->lay.scal) + 2, 4, cudaMemcpyDeviceToHost, st);
+        cudaStreamSynchronize(st);
+        ++c->stats.host_syncs;
         mpode_status cs = check_cuda(c, "mpode_backward");
         if (cs != MPODE_OK) return cs;
+        if (paced) {
+            for (int q = 0; q < 3; ++q) hstate[q] = (int)words[8 + q];
+            dev_err = words[2];
+            if (log) {
+                memcpy(log->exp_used, plog, (size_t)N * sizeof(int));
+                memcpy(log->attempts, plog + (size_t)c->max_steps * sizeof(int), (size_t)N * sizeof(int));
+                memcpy(log->doubled, plog + (size_t)c->max_steps * 2 * sizeof(int), (size_t)N);
+            }
+            if (tg) memcpy(dt_host, pt, ((size_t)N + 1) * sizeof(float));
+        }
     }
     dev_err |= fwd_err;
     if (dev_err != 0u) return fail(c, MPODE_ERR_CUDA, "a device-side wait timed out (code " + std::to_string(dev_err) + ")");

@@ -216,8 +216,11 @@ __global__ void __launch_bounds__(kThreads, 1) small_wgrad_kernel(const __grid_c
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    // A second set of sums holds what earlier steps gave.  float32 has no registers for it: its steps meet one by one, in memory.
+    constexpr bool kTotal = sizeof(T) == 2;
     Sums<T> acc, tot;
-    acc.zero(); tot.zero();
+    acc.zero();
+    if (kTotal) tot.zero();
     const int in_full = p.wr[l] + (time ? 1 : 0);
     auto param_of = [&](int r, int c) -> long long {
         const int m = m0 + r, n = n0 + c;
@@ -264,25 +267,32 @@ __global__ void __launch_bounds__(kThreads, 1) small_wgrad_kernel(const __grid_c
             });
             if (++slot == kStages) slot = 0;
         }
-        if (CHECK) {
+        if (CHECK || !kTotal) {
             meet(acc);
+            const float cf = p.coef[s], beta = s == 0 ? p.beta : 1.f;
             for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
                 const int r = i / (kTile + 2), c = i - r * (kTile + 2);
-                if (param_of(r, c) >= 0) bad |= Low<T>::nonfinite(Low<T>::from_f(cluster_sum(r, c)));
+                const long long at = param_of(r, c);
+                if (at < 0) continue;
+                const float v = cluster_sum(r, c);
+                if (CHECK) bad |= Low<T>::nonfinite(Low<T>::from_f(v));
+                if (!kTotal) p.out[at] = fmaf(cf, v, beta != 0.f ? beta * p.out[at] : 0.f);
             }
-            cluster_sync();
+            cluster_sync();      // (no block goes on, or ends, while another reads its sums)
         }
-        tot.add(p.coef[s], acc);
+        if (kTotal) tot.add(p.coef[s], acc);
         acc.zero();
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    meet(tot);
-    for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
-        const int r = i / (kTile + 2), c = i - r * (kTile + 2);
-        const long long at = param_of(r, c);
-        if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + cluster_sum(r, c);
+    if (kTotal) {
+        meet(tot);
+        for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
+            const int r = i / (kTile + 2), c = i - r * (kTile + 2);
+            const long long at = param_of(r, c);
+            if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + cluster_sum(r, c);
+        }
+        cluster_sync();
     }
-    cluster_sync();      // (no block ends while another reads its sums)
     if (CHECK) warp_flag_or(p.flag, bad);
 }
 
