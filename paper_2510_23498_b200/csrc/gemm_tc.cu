@@ -267,6 +267,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 // operands of the epilogue that live in global memory are requested before the accumulator is waited for
                 uint4 hv[4], uv[4];
                 float bl[32];
+                if (WG && p.direct && p.beta != 0.f && row_ok) {
+                    // what the sums are added to, eight requests at once (one after the other, each behind the store before it, they took half
+                    // of the kernel: 1024 x 1024 gradient of 1024 rows, 27 us)
+                    const float* orow32 = (const float*)p.out + (long long)m * p.ldo + n0 + c * 32;
+#pragma unroll
+                    for (int v = 0; v < 8; ++v)
+                        reinterpret_cast<float4*>(bl)[v] = n0 + c * 32 + v * 4 < p.N ? *reinterpret_cast<const float4*>(orow32 + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
                 if (!WG && row_ok && n0 + c * 32 < p.N) {
                     if (p.epi == EPI_DGRAD) load_h_chunk<T>(hrow, n0 + c * 32, p.N, hv);
                     if (PAIR == 2 && !tangent) load_h_chunk<T>(urow, n0 + c * 32, p.N, uv);
@@ -290,10 +298,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             if (nb + v * 4 < p.N) {
                                 float4 o = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
                                                        __uint_as_float(r[4 * v + 3]));
-                                if (p.beta != 0.f) {
-                                    const float4 old = *reinterpret_cast<const float4*>(orow32 + v * 4);
-                                    o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
-                                }
+                                if (p.beta != 0.f) { o.x += bl[4 * v]; o.y += bl[4 * v + 1]; o.z += bl[4 * v + 2]; o.w += bl[4 * v + 3]; }
                                 *reinterpret_cast<float4*>(orow32 + v * 4) = o;
                             }
                         }
@@ -536,26 +541,29 @@ bool launch_gemm_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lon
 }
 
 // ---------------------------------------------------------------- weight gradient
-// How the reduction range is sliced so that tiles x slices fills the SMs (few waves, little partial-sum traffic).
+// Tile width and slices of the reduction range, by estimated time in microseconds: waves of work items (two CTAs share an SM for widths of
+// at most 128), each its k-blocks and its epilogue (32 columns of a warp at a time, with or without the sums that it adds to), plus, with
+// more than one slice, the pass that reads the slices back and adds them.
 static void wgrad_plan(int M, int N, int K, int* bn_out, int* splits_out, int* kb_per_split_out) {
-    int bn = N >= 256 ? 256 : (N >= 128 ? 128 : 64);
-    int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
-    int kb_total = (K + BK - 1) / BK;
-    int sms = sm_count();
-    // estimated time in microseconds: waves of work items at ~0.5 us per k-block of a 128 x 256 tile, plus (with more
-    // than one slice) the pass that reads the slices back and adds them
-    int best = 1;
+    const int kb_total = (K + BK - 1) / BK, sms = sm_count();
+    int best = 1, best_bn = 64;
     double best_t = 1e30;
-    for (int s = 1; s <= 16 && s <= kb_total; ++s) {
-        int work = tiles * s;
-        int waves = (work + sms - 1) / sms;
-        int per_s = (kb_total + s - 1) / s;
-        double t = (double)waves * per_s * 0.5 * bn / 256.0;
-        if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
-        if (t < best_t) { best_t = t; best = s; }
+    for (int bn = 256; bn >= 64; bn /= 2) {
+        if (bn > 64 && N < bn) continue;
+        const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+        const double t_kb = bn == 256 ? 0.31 : bn == 128 ? 0.25 : 0.2, chunks = bn == 64 ? 2 : 4;
+        for (int s = 1; s <= 16 && s <= kb_total; ++s) {
+            const int work = tiles * s, per_s = (kb_total + s - 1) / s, slots = bn == 256 ? sms : 2 * sms;
+            const int waves = (work + slots - 1) / slots;
+            // (two CTAs of an SM share its tensor pipe and its way to the L2)
+            const double share = bn < 256 && work > sms ? (bn == 128 ? 1.7 : 1.4) : 1.0;
+            double t = waves * share * (per_s * t_kb + chunks * (s == 1 ? 0.5 : 0.25));
+            if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
+            if (t < best_t) { best_t = t; best = s; best_bn = bn; }
+        }
     }
-    int per = (kb_total + best - 1) / best;
-    *bn_out = bn;
+    const int per = (kb_total + best - 1) / best;
+    *bn_out = best_bn;
     *kb_per_split_out = per;
     *splits_out = (kb_total + per - 1) / per;
 }

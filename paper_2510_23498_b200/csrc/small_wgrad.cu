@@ -17,14 +17,15 @@ namespace mpode {
 using namespace tc;
 namespace {
 
-constexpr int kThreads = 256, kTile = 64, kStages = 6, kMaxCluster = 8;
+constexpr int kThreads = 256, kTile = 64, kMaxCluster = 8;
 constexpr int kRedRow = kTile + 3;                  // 64 columns, bias, time (odd stride)
 template <typename T> struct Geo {
     static constexpr int E = 16 / sizeof(T), Pieces = kTile / E, Rows = 512 / Pieces;      // elements of 16 bytes; rows of a stage
     static constexpr int LD = sizeof(T) == 4 ? kTile : kTile + 8;                          // (eight 16-bit rows hit eight 16-byte slots)
     static constexpr int Groups = sizeof(T) == 4 ? 4 : 2;                                  // threads' groups that share out a stage's rows
+    static constexpr int Stages = sizeof(T) == 4 ? 6 : 4, Blocks = sizeof(T) == 4 ? 1 : 2;  // of the ring; blocks that share an SM
     static constexpr int StageBytes = 2 * Rows * LD * (int)sizeof(T);
-    static constexpr int Smem = kStages * StageBytes + Groups * kTile * kRedRow * 4;
+    static constexpr int Smem = Stages * StageBytes + Groups * kTile * kRedRow * 4;
 };
 
 struct Items { int first[SMALL_MAX_L + 1]; int S; };
@@ -178,9 +179,10 @@ template <> struct Sums<float> {
 };
 
 template <typename T, bool CHECK>
-__global__ void __launch_bounds__(kThreads, 1) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ Items items) {
+__global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ Items items) {
     chain_begin();
     using G = Geo<T>;
+    constexpr int kStages = G::Stages;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float taus[SMALL_MAX_CHUNK][RK_MAX_STAGES];
     const int S = items.S, rank = (int)blockIdx.x % S, item = (int)blockIdx.x / S;
@@ -299,25 +301,39 @@ __global__ void __launch_bounds__(kThreads, 1) small_wgrad_kernel(const __grid_c
 template <typename T, bool CHECK>
 bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready) {
     static bool done[kMaxDevices] = {false};
+    static int at_once[kMaxDevices][kMaxCluster + 1] = {{0}};      // clusters of each size that the GPU holds at once
     const int dev = current_device();
-    if (!done[dev]) {
-        if (cudaFuncSetAttribute(small_wgrad_kernel<T, CHECK>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<T>::Smem) != cudaSuccess) { cudaGetLastError(); return false; }
-        done[dev] = true;
-    }
-    if (ready) return true;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(items.first[p.L] * items.S));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Geo<T>::Smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)items.S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
+    if (!done[dev]) {
+        if (cudaFuncSetAttribute(small_wgrad_kernel<T, CHECK>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<T>::Smem) != cudaSuccess) { cudaGetLastError(); return false; }
+        cfg.numAttrs = 1;
+        for (int S = 1; S <= kMaxCluster; ++S) {
+            at[0].val.clusterDim.x = (unsigned)S;
+            cfg.gridDim = dim3((unsigned)S);
+            if (cudaOccupancyMaxActiveClusters(&at_once[dev][S], small_wgrad_kernel<T, CHECK>, &cfg) != cudaSuccess) { cudaGetLastError(); at_once[dev][S] = 0; }
+        }
+        done[dev] = true;
+    }
+    if (ready) return true;
+    // the largest cluster of which all pieces' run at once, with two stages of rows for each of its blocks
+    const int n = items.first[p.L], stages = (p.stages * p.B + Geo<T>::Rows - 1) / Geo<T>::Rows;
+    Items it = items;
+    it.S = 1;
+    for (int S = 2; S <= kMaxCluster && 2 * S <= stages; ++S)
+        if (at_once[dev][S] >= n) it.S = S;
+    at[0].val.clusterDim.x = (unsigned)it.S;
+    cfg.gridDim = dim3((unsigned)(n * it.S));
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, small_wgrad_kernel<T, CHECK>, p, items) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, small_wgrad_kernel<T, CHECK>, p, it) == cudaSuccess;
 }
 template <typename T>
 bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready, bool check) {
@@ -334,15 +350,9 @@ bool small_wgrad_ready(mpode_dtype dt, const SmallMlp& p) {
     return true;
 }
 
-// A cluster as large as it takes to give every SM a block, with two stages of rows for each of its blocks
 void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
     Items it{};
     for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + kTile - 1) / kTile) * ((p.wp[l] + kTile - 1) / kTile);
-    const int rows = dt == MPODE_F32 ? Geo<float>::Rows : Geo<__half>::Rows, pieces = (p.stages * p.B + rows - 1) / rows;
-    it.S = sm_count() / it.first[p.L];
-    if (it.S > kMaxCluster) it.S = kMaxCluster;
-    if (it.S > pieces / 2) it.S = pieces / 2;
-    if (it.S < 1) it.S = 1;
     if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, it, st, false, p.flag != nullptr);
     else if (dt == MPODE_F16) wgrad_t<__half>(p, it, st, false, p.flag != nullptr);
     else wgrad_t<float>(p, it, st, false, p.flag != nullptr);
