@@ -31,6 +31,11 @@ __device__ __forceinline__ void st_v8(float* dst, const uint32_t* r) {
                  : "memory");
 }
 
+__device__ __forceinline__ void ld_v8(const float* src, float* r) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]) : "l"(src));
+}
+
 // Widest tiles (BN = 256): one CTA per SM, eight epilogue warps (two per TMEM lane quadrant, each half of the columns).
 // Narrower tiles (BN <= 128: the convolutions, thin layers): half the shared memory, four epilogue warps and a small register
 // footprint, so that two CTAs share an SM and one's loads and epilogue hide behind the other's MMAs.
@@ -58,7 +63,7 @@ struct TcParams {
     // at the tap's offset (out-of-image pixels read as zero)
     int conv, conv_h, conv_w, conv_c;   // conv_c: channels of the image (a multiple of 64; a k-block is 64 channels of one tap)
     const float* tbias;         // EPI_FWD with conv: [9][N] bias table per position class
-    int direct; float beta;     // weight gradient with one slice: write out = beta * out + acc directly
+    int direct; float beta;     // weight gradient with one slice: write out = beta * out + acc directly (2: rows on 32-byte boundaries)
     // flow with a trace estimate: a tile is 64 primal rows and the 64 tangent rows m_split further down (GemmArgs::cnf_pair)
     int pair; void* pair_out; const void* uprev;
 };
@@ -267,13 +272,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 // operands of the epilogue that live in global memory are requested before the accumulator is waited for
                 uint4 hv[4], uv[4];
                 float bl[32];
-                if (WG && p.direct && p.beta != 0.f && row_ok) {
-                    // what the sums are added to, eight requests at once (one after the other, each behind the store before it, they took half
-                    // of the kernel: 1024 x 1024 gradient of 1024 rows, 27 us)
+                if (WG && BN < 256 && p.direct && p.beta != 0.f && row_ok) {
+                    // What the sums are added to, requested at once and in whole sectors.  (The widest tiles, where eight warps share the work
+                    // and nothing else is waited for, are as fast with one 16-byte piece after the other: 2048 x 2048 gradient of 4096 rows 33 us
+                    // against 35.)
                     const float* orow32 = (const float*)p.out + (long long)m * p.ldo + n0 + c * 32;
+                    if (p.direct == 2) {      // rows on 32-byte boundaries: whole sectors
 #pragma unroll
-                    for (int v = 0; v < 8; ++v)
-                        reinterpret_cast<float4*>(bl)[v] = n0 + c * 32 + v * 4 < p.N ? *reinterpret_cast<const float4*>(orow32 + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int v = 0; v < 4; ++v)
+                            if (n0 + c * 32 + v * 8 < p.N) ld_v8(orow32 + v * 8, bl + 8 * v);
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < 8; ++v)
+                            if (n0 + c * 32 + v * 4 < p.N) reinterpret_cast<float4*>(bl)[v] = *reinterpret_cast<const float4*>(orow32 + v * 4);
+                    }
                 }
                 if (!WG && row_ok && n0 + c * 32 < p.N) {
                     if (p.epi == EPI_DGRAD) load_h_chunk<T>(hrow, n0 + c * 32, p.N, hv);
@@ -293,14 +305,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     // one reduction slice and an output whose rows are 16-byte aligned: out = beta * out + acc without scratch
                     if (row_ok && nb < p.N) {
                         float* orow32 = (float*)p.out + (long long)m * p.ldo + nb;
+                        if (BN < 256 && p.beta != 0.f) {
 #pragma unroll
-                        for (int v = 0; v < 8; ++v) {
-                            if (nb + v * 4 < p.N) {
-                                float4 o = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
-                                                       __uint_as_float(r[4 * v + 3]));
-                                if (p.beta != 0.f) { o.x += bl[4 * v]; o.y += bl[4 * v + 1]; o.z += bl[4 * v + 2]; o.w += bl[4 * v + 3]; }
-                                *reinterpret_cast<float4*>(orow32 + v * 4) = o;
+                            for (int v = 0; v < 32; ++v) r[v] = __float_as_uint(__uint_as_float(r[v]) + bl[v]);
+                        }
+                        if (BN == 256) {
+#pragma unroll
+                            for (int v = 0; v < 8; ++v) {
+                                if (nb + v * 4 < p.N) {
+                                    float4 o = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
+                                                           __uint_as_float(r[4 * v + 3]));
+                                    if (p.beta != 0.f) {
+                                        const float4 old = *reinterpret_cast<const float4*>(orow32 + v * 4);
+                                        o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
+                                    }
+                                    *reinterpret_cast<float4*>(orow32 + v * 4) = o;
+                                }
                             }
+                        } else if (p.direct == 2) {
+#pragma unroll
+                            for (int v = 0; v < 4; ++v)
+                                if (nb + v * 8 < p.N) st_v8(orow32 + v * 8, r + 8 * v);
+                        } else {
+#pragma unroll
+                            for (int v = 0; v < 8; ++v)
+                                if (nb + v * 4 < p.N) *reinterpret_cast<uint4*>(orow32 + v * 4) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
                         }
                     }
                 } else if (WG) {
@@ -541,29 +570,28 @@ bool launch_gemm_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lon
 }
 
 // ---------------------------------------------------------------- weight gradient
-// Tile width and slices of the reduction range, by estimated time in microseconds: waves of work items (two CTAs share an SM for widths of
-// at most 128), each its k-blocks and its epilogue (32 columns of a warp at a time, with or without the sums that it adds to), plus, with
-// more than one slice, the pass that reads the slices back and adds them.
+// How the reduction range is sliced so that tiles x slices fills the SMs (few waves, little partial-sum traffic).  Short reductions (up to 2048
+// rows) of which tiles of 256 columns are a quarter of the SMs at most get tiles of 64: four times the blocks, each with a quarter of the
+// epilogue, which is then most of the time (1024 x 1024 gradient of 1024 rows 27 -> 9.6 us; the flow 63-1024-1024-63 8.3 -> 7.2 ms a
+// pass).  Longer ones are cut into slices instead (784 x 2048 of 4096 rows: narrower tiles 31 us, two slices of 256 columns 26 and 5 for their sum).
 static void wgrad_plan(int M, int N, int K, int* bn_out, int* splits_out, int* kb_per_split_out) {
-    const int kb_total = (K + BK - 1) / BK, sms = sm_count();
-    int best = 1, best_bn = 64;
+    const int tiles256 = ((M + BM - 1) / BM) * ((N + 255) / 256), sms = sm_count(), kb_total = (K + BK - 1) / BK;
+    const int bn = kb_total <= 32 && 4 * tiles256 <= sms ? 64 : N >= 256 ? 256 : (N >= 128 ? 128 : 64);
+    const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+    // estimated time in microseconds: waves of work items at ~0.5 us per k-block of a 128 x 256 tile, plus (with more
+    // than one slice) the pass that reads the slices back and adds them
+    int best = 1;
     double best_t = 1e30;
-    for (int bn = 256; bn >= 64; bn /= 2) {
-        if (bn > 64 && N < bn) continue;
-        const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
-        const double t_kb = bn == 256 ? 0.31 : bn == 128 ? 0.25 : 0.2, chunks = bn == 64 ? 2 : 4;
-        for (int s = 1; s <= 16 && s <= kb_total; ++s) {
-            const int work = tiles * s, per_s = (kb_total + s - 1) / s, slots = bn == 256 ? sms : 2 * sms;
-            const int waves = (work + slots - 1) / slots;
-            // (two CTAs of an SM share its tensor pipe and its way to the L2)
-            const double share = bn < 256 && work > sms ? (bn == 128 ? 1.7 : 1.4) : 1.0;
-            double t = waves * share * (per_s * t_kb + chunks * (s == 1 ? 0.5 : 0.25));
-            if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
-            if (t < best_t) { best_t = t; best = s; best_bn = bn; }
-        }
+    for (int s = 1; s <= 16 && s <= kb_total; ++s) {
+        int work = tiles * s;
+        int waves = (work + sms - 1) / sms;
+        int per_s = (kb_total + s - 1) / s;
+        double t = (double)waves * per_s * 0.5 * bn / 256.0;
+        if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
+        if (t < best_t) { best_t = t; best = s; }
     }
-    const int per = (kb_total + best - 1) / best;
-    *bn_out = best_bn;
+    int per = (kb_total + best - 1) / best;
+    *bn_out = bn;
     *kb_per_split_out = per;
     *splits_out = (kb_total + per - 1) / per;
 }
@@ -596,6 +624,7 @@ bool launch_wgrad_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lo
     p.M = g.M; p.N = g.N; p.K = g.K; p.epi = EPI_WGRAD; p.err = g.err;
     p.splits = splits; p.kb_per_split = per; p.partial = g.partial;
     p.direct = splits == 1 && (g.crop_m == 0 || (g.crop_m == g.M && g.crop_n == g.N)) && g.ldo % 4 == 0 && (((uintptr_t)g.out) & 15) == 0;
+    if (p.direct && g.ldo % 8 == 0 && (((uintptr_t)g.out) & 31) == 0) p.direct = 2;
     p.out = g.out; p.ldo = g.ldo; p.beta = g.beta;
     bool ok;
     if (dt == MPODE_BF16) {
