@@ -146,11 +146,8 @@ struct GemmArgs {
     //     (both [m_split, N], leading dimension ldh): out = Q16(s hbar + s (1 - s) U gbar), out2 = Q16(s gbar), non-finite flagged.
     int cnf_pair; void* pair_out; const void* uprev;
     // EPI_WGRAD on the plain CUDA-core kernel: the row sums of A (bias gradient), row_sum[m] = beta row_sum[m] + sum; scaled by tau
-    // into row_sum_time[m * ldo] (the appended time column); and the bare sums into row_sum_raw[m].  Each may be null.  With `flag` a sum
-    // (before alpha) that does not fit the format raises it: for products over a whole step.
-    // `alpha` (0 = 1) scales what is added to the outputs; with k_tau the time column weighs the reduction index k by k_tau[k / k_per]
+    // into row_sum_time[m * ldo] (the appended time column); and the bare sums into row_sum_raw[m].  Each may be null.
     float *row_sum, *row_sum_time, *row_sum_raw;
-    float alpha; const float* k_tau; int k_per;
 };
 
 // returns whether the plain-operand kernel ran (the one that takes GemmArgs::row_sum)

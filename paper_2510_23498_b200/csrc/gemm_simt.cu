@@ -32,7 +32,7 @@ __device__ __forceinline__ float load_operand(const T* __restrict__ p, long long
     return Low<T>::to_f(p[((long long)pixel + (long long)dy * W + dx) * Cd + c]);
 }
 
-// The layer epilogue of one output element; returns whether the rounded value of an input gradient (with a flag: of a weight gradient)
+// The layer epilogue of one output element; returns whether the rounded value of an input gradient
 // is not finite.
 template <typename T>
 __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, float v) {
@@ -51,8 +51,7 @@ __device__ __forceinline__ bool finish_element(const GemmArgs& g, int m, int n, 
         return Low<T>::nonfinite(q);
     } else if (g.epi == EPI_WGRAD) {
         float* o = (float*)g.out + (long long)m * g.ldo + n;
-        *o = fmaf(g.alpha != 0.f ? g.alpha : 1.f, v, g.beta != 0.f ? *o : 0.f);
-        return g.flag != nullptr && Low<T>::nonfinite(Low<T>::from_f(v));
+        *o = v + (g.beta != 0.f ? *o : 0.f);
     } else {
         ((float*)g.out)[(long long)m * g.ldo + n] = v;
     }
@@ -169,7 +168,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     namespace cg = cooperative_groups;
     __shared__ __align__(16) float As[2][DK][kDenseLd];
     __shared__ __align__(16) float Bs[2][DK][kDenseLd];
-    __shared__ float rows[2][DM], tau_s[2][DK];
+    __shared__ float rows[DM];
     const T* A = (const T*)g.A;
     const T* B = (const T*)g.B;
     const int m0 = blockIdx.y * DM, n0 = blockIdx.x * DN, t = threadIdx.x;
@@ -177,7 +176,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     const int k_begin = blockIdx.z * per_slice, k_end = min(g.K, k_begin + per_slice);
     // the bias gradient is the row sum of A over the reduction range: taken along by the first column of tiles
     const bool sum_rows = !KFAST && (g.row_sum != nullptr || g.row_sum_time != nullptr) && blockIdx.x == 0;
-    float acc[4][4], rs[4] = {0.f, 0.f, 0.f, 0.f}, rt[4] = {0.f, 0.f, 0.f, 0.f};
+    float acc[4][4], rs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -198,8 +197,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             }
         }
     };
-    auto stash = [&](int buf, int k0) {
-        if (sum_rows && g.k_tau != nullptr && t < DK) tau_s[buf][t] = k0 + t < k_end ? g.k_tau[(k0 + t) / g.k_per] : 0.f;
+    auto stash = [&](int buf) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             if (KFAST) {
@@ -215,7 +213,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
     };
     if (k_begin < k_end) {
         fetch(k_begin);
-        stash(0, k_begin);
+        stash(0);
     }
     __syncthreads();
     int buf = 0;
@@ -234,29 +232,18 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             if (sum_rows) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) rs[i] += a[i];
-                if (g.k_tau != nullptr) {
-                    const float tk = tau_s[buf][kk];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) rt[i] = fmaf(tk, a[i], rt[i]);
-                }
             }
         }
-        if (more) stash(buf ^ 1, k0 + DK);
+        if (more) stash(buf ^ 1);
         __syncthreads();
     }
 
-    const float alpha = g.alpha != 0.f ? g.alpha : 1.f;
     bool bad = false;
-    auto put_row_sum = [&](int m, float s, float st) {
-        if (g.row_sum != nullptr) {
-            g.row_sum[m] = fmaf(alpha, s, g.beta != 0.f ? g.row_sum[m] : 0.f);
-            bad |= Low<T>::nonfinite(Low<T>::from_f(s));
-        }
+    auto put_row_sum = [&](int m, float s) {
+        if (g.row_sum != nullptr) g.row_sum[m] = s + (g.beta != 0.f ? g.row_sum[m] : 0.f);
         if (g.row_sum_time != nullptr) {
             float* o = g.row_sum_time + (long long)m * g.ldo;
-            const float v = g.k_tau != nullptr ? st : g.tau * s;
-            *o = fmaf(alpha, v, g.beta != 0.f ? *o : 0.f);
-            bad |= Low<T>::nonfinite(Low<T>::from_f(v));
+            *o = fmaf(g.tau, s, g.beta != 0.f ? *o : 0.f);
         }
         if (g.row_sum_raw != nullptr) g.row_sum_raw[m] = s;
     };
@@ -270,7 +257,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
                 const int n = n0 + tx * 4 + j;
                 if (m < g.M && n < g.N) bad |= finish_element<T>(g, m, n, acc[i][j]);
             }
-            if (sum_rows && tx == 0 && m < g.M) put_row_sum(m, rs[i], rt[i]);
+            if (sum_rows && tx == 0 && m < g.M) put_row_sum(m, rs[i]);
         }
     } else {      // the slices of one tile are one cluster: rank r adds up the tile's rows [r, r + 1) * DM / S
         cg::cluster_group cl = cg::this_cluster();
@@ -278,7 +265,7 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             *reinterpret_cast<float4*>(&tile[ty * 4 + i][tx * 4]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            if (sum_rows && tx == 0) { rows[0][ty * 4 + i] = rs[i]; rows[1][ty * 4 + i] = rt[i]; }
+            if (sum_rows && tx == 0) rows[ty * 4 + i] = rs[i];
         }
         cl.sync();
         const int rank = (int)blockIdx.z, per = DM / S;
@@ -290,16 +277,13 @@ __global__ void __launch_bounds__(kDenseThreads) gemm_dense_kernel(GemmArgs g, i
             bad |= finish_element<T>(g, m, n, v);
         }
         if (sum_rows && t < per && m0 + rank * per + t < g.M) {
-            float v = 0.f, vt = 0.f;
-            for (int z = 0; z < S; ++z) {
-                v += *cl.map_shared_rank(&rows[0][rank * per + t], z);
-                vt += *cl.map_shared_rank(&rows[1][rank * per + t], z);
-            }
-            put_row_sum(m0 + rank * per + t, v, vt);
+            float v = 0.f;
+            for (int z = 0; z < S; ++z) v += *cl.map_shared_rank(&rows[rank * per + t], z);
+            put_row_sum(m0 + rank * per + t, v);
         }
         cl.sync();      // no block leaves while another reads its shared memory
     }
-    if (g.epi == EPI_DGRAD || g.epi == EPI_WGRAD) warp_flag_or(g.flag, bad);
+    if (g.epi == EPI_DGRAD) warp_flag_or(g.flag, bad);
 }
 
 // Blocks of a cluster share a reduction of at least 64: as many (up to 8) as it takes to give every SM a block.
