@@ -716,46 +716,44 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
         }
     }
     if (!dynamic) break;
-    if (seen && (mirror_h[1] == fail_step ? fail_count : 0) + 1 < c->pol.k_max) {
-        // a repeat follows, and all that it needs is in the mapped words (five copies to pageable memory took 60 us for each overflow)
-        cudaStreamSynchronize(st);
-        ++c->stats.host_syncs;
-        hstate[0] = mirror_h[0]; hstate[1] = mirror_h[1]; hstate[2] = 0;
+    // One drain per round: the scalar words (error word, scale state) and, should this have been the last round, everything else the host reads.
+    // Into page-locked memory: to pageable memory every copy is a wait of its own, and five of them took 60 us for each overflow.
+    const bool again = seen && (mirror_h[1] == fail_step ? fail_count : 0) + 1 < c->pol.k_max;      // a repeat follows
+    unsigned char* pin = (unsigned char*)c->mirror_host;
+    unsigned* words = (unsigned*)(pin + 64);                                     // flag, norm, error word, ..., scale state
+    unsigned char* plog = pin + kMirrorBytes;
+    float* pt = (float*)(pin + kMirrorBytes + ((size_t)c->max_steps * 9 + 15) / 16 * 16);
+    const bool want_log = log != nullptr && !again, want_t = tg && !again;
+    if (paced) {
+        cudaMemcpyAsync(words, flag, 64, cudaMemcpyDeviceToHost, st);
+        if (want_log) cudaMemcpyAsync(plog, slog_exp, (size_t)c->max_steps * 9, cudaMemcpyDeviceToHost, st);
     } else {
-        // one drain: the state and, should this have been the last round, everything else the host reads
-        unsigned char* pin = paced ? (unsigned char*)c->mirror_host : nullptr;
-        unsigned* words = paced ? (unsigned*)(pin + 64) : nullptr;               // the scalar slice: flag, norm, error word, ..., scale state
-        unsigned char* plog = paced ? pin + kMirrorBytes : nullptr;
-        float* pt = paced ? (float*)(pin + kMirrorBytes + ((size_t)c->max_steps * 9 + 15) / 16 * 16) : nullptr;
-        if (paced) {
-            cudaMemcpyAsync(words, flag, 64, cudaMemcpyDeviceToHost, st);
-            if (log) cudaMemcpyAsync(plog, slog_exp, (size_t)c->max_steps * 9, cudaMemcpyDeviceToHost, st);
-        } else {
-            cudaMemcpyAsync(hstate, sstate, sizeof hstate, cudaMemcpyDeviceToHost, st);
-            if (log) {
-                cudaMemcpyAsync(log->exp_used, slog_exp, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
-                cudaMemcpyAsync(log->attempts, slog_att, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
-                cudaMemcpyAsync(log->doubled, slog_dbl, (size_t)N, cudaMemcpyDeviceToHost, st);
-            }
-            cudaMemcpyAsync(&dev_err, flag + 2, 4, cudaMemcpyDeviceToHost, st);
+        cudaMemcpyAsync(hstate, sstate, sizeof hstate, cudaMemcpyDeviceToHost, st);
+        if (want_log) {
+            cudaMemcpyAsync(log->exp_used, slog_exp, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
+            cudaMemcpyAsync(log->attempts, slog_att, (size_t)N * sizeof(int), cudaMemcpyDeviceToHost, st);
+            cudaMemcpyAsync(log->doubled, slog_dbl, (size_t)N, cudaMemcpyDeviceToHost, st);
         }
-        if (tg) cudaMemcpyAsync(paced ? pt : dt_host, tprime, ((size_t)N + 1) * sizeof(float), cudaMemcpyDeviceToHost, st);
-        if (c->ws_forward != nullptr && c->ws_forward != ws)     // the forward pass ran on another workspace: its error word lives there
-            cudaMemcpyAsync(&fwd_err, (unsigned*)at(c->ws_forward, c->lay.scal) + 2, 4, cudaMemcpyDeviceToHost, st);
-        cudaStreamSynchronize(st);
-        ++c->stats.host_syncs;
+        cudaMemcpyAsync(&dev_err, flag + 2, 4, cudaMemcpyDeviceToHost, st);
+    }
+    if (want_t) cudaMemcpyAsync(paced ? pt : dt_host, tprime, ((size_t)N + 1) * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (c->ws_forward != nullptr && c->ws_forward != ws)     // the forward pass ran on another workspace: its error word lives there
+        cudaMemcpyAsync(&fwd_err, (unsigned*)at(c->ws_forward, c->lay.scal) + 2, 4, cudaMemcpyDeviceToHost, st);
+    cudaStreamSynchronize(st);
+    ++c->stats.host_syncs;
+    {
         mpode_status cs = check_cuda(c, "mpode_backward");
         if (cs != MPODE_OK) return cs;
-        if (paced) {
-            for (int q = 0; q < 3; ++q) hstate[q] = (int)words[8 + q];
-            dev_err = words[2];
-            if (log) {
-                memcpy(log->exp_used, plog, (size_t)N * sizeof(int));
-                memcpy(log->attempts, plog + (size_t)c->max_steps * sizeof(int), (size_t)N * sizeof(int));
-                memcpy(log->doubled, plog + (size_t)c->max_steps * 2 * sizeof(int), (size_t)N);
-            }
-            if (tg) memcpy(dt_host, pt, ((size_t)N + 1) * sizeof(float));
+    }
+    if (paced) {
+        for (int q = 0; q < 3; ++q) hstate[q] = (int)words[8 + q];
+        dev_err = words[2];
+        if (want_log) {
+            memcpy(log->exp_used, plog, (size_t)N * sizeof(int));
+            memcpy(log->attempts, plog + (size_t)c->max_steps * sizeof(int), (size_t)N * sizeof(int));
+            memcpy(log->doubled, plog + (size_t)c->max_steps * 2 * sizeof(int), (size_t)N);
         }
+        if (want_t) memcpy(dt_host, pt, ((size_t)N + 1) * sizeof(float));
     }
     dev_err |= fwd_err;
     if (dev_err != 0u) return fail(c, MPODE_ERR_CUDA, "a device-side wait timed out (code " + std::to_string(dev_err) + ")");
