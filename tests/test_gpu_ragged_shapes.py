@@ -205,3 +205,60 @@ def test_conv_block_of_few_pixels():
 def test_flow_column_sums_at_chunk_edges(batch):
     wl = inputs.cnf_mlp(batch=batch, n_steps=1, d=16, hidden=72)
     assert_parity(run_gpu(wl, low="bf16"), run_oracle(wl, low="bf16"), TOL["bf16"])
+
+
+def _network(batch, widths, n_steps, solver="rk4"):
+    wl = inputs.mlp_block(batch=batch, n_steps=n_steps, d=widths[0], hidden=widths[1])
+    wl.vel["n_layers"], wl.vel["widths"], wl.theta = len(widths) - 1, widths, inputs.mlp_theta(3, widths, True)
+    wl.solver = solver
+    return wl
+
+
+# row-local kernels whose weights stay on the SM: one row, a block's 8 rows less and plus one, two and four row tiles a block; one layer (weights
+# in registers: 2, 4, 6 and 8 reduction steps, parameter gradients in registers up to 64 pieces and in slabs above); widths of one and
+# several tiles a warp, an odd number of reduction steps, and more than 16 of them.  Unscaled-safe passes in bfloat16: unscaled float16
+# cotangents of a mean over 2369 x 128 entries, 2 / 303232 = 6.6e-6, are 110 units of the smallest subnormal, so that a value that rounds to its
+# neighbour is 0.9 % off and the format's 2e-3 says nothing.
+@pytest.mark.parametrize("batch,widths,n_steps", [(1, [24, 24], 3), (7, [64, 64], 5), (9, [72, 72], 3), (1185, [100, 100], 2), (2369, [128, 128], 2), (9, [40, 136, 40], 2),
+                                                  (1190, [24, 130, 24], 2), (20, [16, 272, 16], 2), (9, [240, 64, 240], 2), (17, [33, 40, 33], 3), (300, [12, 20, 28, 12], 3)])
+def test_resident_networks_at_tile_edges(batch, widths, n_steps):
+    wl = _network(batch, widths, n_steps)
+    for low, scaling in (("bf16", "none"), ("f16", "dynamic"), ("bf16", "none_safe")):
+        gpu, orc = run_gpu(wl, low, scaling), run_oracle(wl, low, scaling)
+        assert_parity(gpu, orc, TOL[low])
+        assert gpu["stats"]["fused_launches"] > 0 and gpu["stats"]["simt_contractions"] == 0
+        if scaling == "dynamic":
+            assert_same_log(gpu["log"], orc["log"])
+
+
+# tableaux whose stages depend on the one before alone (what the epilogues carry in registers) and on several, the time terms beside them
+@pytest.mark.parametrize("solver", ["euler", "heun", "kutta3", "rk38"])
+@pytest.mark.parametrize("widths", [[64, 64], [40, 72, 40]])
+def test_resident_networks_per_tableau(solver, widths):
+    wl = _network(100, widths, 5, solver)
+    for low, scaling in (("bf16", "none"), ("f16", "dynamic")):
+        gpu, orc = run_gpu(wl, low, scaling, want_dt=True), run_oracle(wl, low, scaling, want_dt=True)
+        assert_parity(gpu, orc, TOL[low])
+        assert rel_l2(gpu["dL_dt"], orc["dL_dt"]) <= TOL[low]
+        plain = run_gpu(wl, low, scaling)
+        assert np.array_equal(plain["a0"], gpu["a0"]) and np.array_equal(plain["yT"], gpu["yT"])
+
+
+# weight gradients by clusters: fewer rows than two stages of the ring, pieces of 64 that end inside a tile, float32 with steps that meet one by one
+@pytest.mark.parametrize("low,batch,widths,n_steps", [("f32", 3, [16, 72, 16], 5), ("f32", 513, [64, 200, 64], 3), ("f16", 2300, [64, 136, 64], 2), ("bf16", 31, [128, 160, 128], 9)])
+def test_weight_gradient_clusters(low, batch, widths, n_steps):
+    wl = _network(batch, widths, n_steps)
+    scaling = "none" if low != "f16" else "dynamic"
+    gpu = run_gpu(wl, low, scaling)
+    assert_parity(gpu, run_oracle(wl, exact=True) if low == "f32" else run_oracle(wl, low, scaling), TOL[low])
+    # a running gradient is added to, not overwritten: twice the same pass into one array
+    import torch
+    from paper_2510_23498_b200 import binding
+    if scaling == "none":
+        ctx = binding.Context(wl.vel, wl.batch, wl.n_steps, low=low)
+        ctx.forward(torch.from_numpy(np.ascontiguousarray(wl.theta, dtype=np.float32)).cuda(), torch.from_numpy(np.ascontiguousarray(wl.y0, dtype=np.float32)).cuda(), wl.tgrid, wl.solver)
+        dl = torch.from_numpy(np.ascontiguousarray(gpu["dLdyT"], dtype=np.float32)).cuda()
+        _, g, _, _ = ctx.backward(dl)
+        ctx.backward(dl, accumulate_into=g)
+        assert rel_l2(g.cpu().numpy(), 2.0 * gpu["g"]) <= 1e-6      # (one more float32 rounding per entry and chunk of steps)
+        ctx.close()
