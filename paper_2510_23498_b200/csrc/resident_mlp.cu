@@ -7,6 +7,8 @@
 // update, seed, stage cotangent, adjoint update) is done by the thread that holds the values, in the epilogue of the last layer.  Warps
 // beside the ones that carry the chain move layer inputs and cotangents to memory, or, where the parameter gradient fits their registers
 // and no step's gradient has to be looked at, form it on the spot: then a pass of any number of steps is one launch and a sum over blocks.
+// Measured, a layer (before: small_mlp.cu): one layer of 64 1.28 -> 0.29 us, 200-200 2.2 -> 0.94 us; training passes: linear equation 64 wide, 1024
+// samples, 100 RK4 steps 2.97 -> 0.53 ms; MLP 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 4.8 -> 2.2 ms (with small_wgrad.cu).
 #include "resident_mlp.h"
 
 #include "profiler.h"
@@ -1308,6 +1310,12 @@ bool backward_t(const ResidentMlp& p, cudaStream_t st, bool ready) {
 
 }  // namespace
 
+// The line is the shared memory of a block: weights once, and backward every layer input of a step's stages (about 95 K weights at 8 rows a
+// block, fewer at 16); beyond it the weights stream (small_mlp.cu).  8 rows a block while that gives every SM one block at most: half the epilogue
+// and half the rows' reads per SM.  Training pass of 8 RK4 steps unless it says otherwise, ms streamed / resident: 64-64-64 at 1500 samples 0.72 / 0.48;
+// 64-128-64 at 2300 0.95 / 0.55; 40-136-136-40 at 2300 1.23 / 0.63; 72-160-72 at 1300 0.81 / 0.48; 32-96-96-32, float16 dynamic, 16 steps, at 200
+// 2.52 / 1.58; linear 100 wide, 40 steps, at 300 1.56 / 0.75; linear 128 wide forward, 40 steps, at 4000 0.50 / 0.16; 64-240-240-64 forward at 1000
+// 0.23 / 0.11.  Chains of 16 warps hold two row tiles at most (four spill).
 ResidentPlan plan_resident(mpode_dtype dt, int B, int L, const int* wp, bool bias, bool time) {
     ResidentPlan g;
     if (dt == MPODE_F32 || L < 1 || L > SMALL_MAX_L || wp[0] > 256) return g;

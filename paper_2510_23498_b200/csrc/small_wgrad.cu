@@ -5,6 +5,8 @@
 // memory, added in a fixed order.  The bias gradient and the time column are two more columns (ones, stage times) of the pieces in the
 // first column of pieces.  CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of
 // the step's gradient that does not fit the format raises the flag.
+// Measured (before: pieces of 32 x 32 or 16 x 16 a block, float32 a launch per layer): 72-200-200-72, 4000 rows, float16 24 -> 15 us; 64-256-256-64, 4096
+// rows, float32 115 -> 45 us (403 M multiply-adds, 11 us at full rate).
 // What bounds it is the rows' way from the L2 (16 KB a stage at about 64 bytes a cycle and SM) and the fill of the ring.  16-bit formats multiply
 // with mma.sync.  float32 holds 8 x 8 sums a thread and reads four 16-byte words for 64 multiply-adds.
 #include "small_mlp.h"
