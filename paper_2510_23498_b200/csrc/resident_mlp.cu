@@ -272,22 +272,23 @@ __device__ __forceinline__ void state_out(uint32_t buf, int sx, T* dst, int d, i
         if (r0 + r < B) reinterpret_cast<unsigned short*>(dst)[(long long)(r0 + r) * d + c] = v;
     }
 }
+// Rows behind the batch take the last row's values: they are integrated along with zero adjoint, and from a state of their own (y = 0) they
+// could overflow where no sample does, which zero cotangents turn into NaN (parameter gradients, time terms, overflow flag).
 template <typename T>
 __device__ __forceinline__ void state_in(uint32_t buf, int sx, const T* src, int d, int R, int r0, int B, int tid, int threads) {
+    auto row = [&](int r) { return (long long)(r0 + r < B ? r0 + r : B - 1); };
     if ((d & 7) == 0) {
         const int per = d / 8, n = R * per;
         for (int i = tid; i < n; i += threads) {
             const int r = i / per, c = (i - r * per) * 8;
-            if (r0 + r < B) copy16(buf + (uint32_t)((r * sx + c) * 2), src + (long long)(r0 + r) * d + c);
+            copy16(buf + (uint32_t)((r * sx + c) * 2), src + row(r) * d + c);
         }
         return;
     }
     for (int i = tid; i < R * d; i += threads) {
         const int r = i / d, c = i - r * d;
-        if (r0 + r < B) {
-            const unsigned short v = reinterpret_cast<const unsigned short*>(src)[(long long)(r0 + r) * d + c];
-            asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)((r * sx + c) * 2)), "h"(v) : "memory");
-        }
+        const unsigned short v = reinterpret_cast<const unsigned short*>(src)[row(r) * d + c];
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(buf + (uint32_t)((r * sx + c) * 2)), "h"(v) : "memory");
     }
 }
 

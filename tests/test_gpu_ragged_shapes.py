@@ -262,3 +262,40 @@ def test_weight_gradient_clusters(low, batch, widths, n_steps):
         ctx.backward(dl, accumulate_into=g)
         assert rel_l2(g.cpu().numpy(), 2.0 * gpu["g"]) <= 1e-6      # (one more float32 rounding per entry and chunk of steps)
         ctx.close()
+
+
+# Rows of a block that lie behind the batch must not reach a result: a velocity that leaves float16 along the trajectory from y = 0, but not
+# along the samples'.  Several layers: every fourth hidden unit is 60000 at y = 0 and off (-60000) at the samples' y = -16, its outgoing weights 4;
+# the other units see y + 16.  One layer: f = 0 at y = -15000 +- 8k, f(0) = 60000, slope 4.
+def _overflows_at_zero(batch, widths, n_steps=2):
+    wl = _network(batch, widths, n_steps)
+    d, h = widths[0], widths[1]
+    if len(widths) == 2:
+        wl.theta = np.concatenate([np.concatenate([np.full((d, d), 4.0 / d), np.zeros((d, 1))], axis=1).ravel(), np.full(d, 60000.0)]).astype(np.float32)
+        k = 8.0 * (np.arange(batch)[:, None] % 5 + np.arange(d // 2)[None, :] % 3)
+        wl.y0 = (-15000.0 + np.concatenate([k, -k], axis=1)).astype(np.float32)
+        return wl
+    wl.y0 = (-16.0 + 0.25 * wl.y0).astype(np.float32)
+    n0 = h * (d + 1)
+    W0, b0, W1 = wl.theta[:n0].reshape(h, d + 1), wl.theta[n0:n0 + h], wl.theta[n0 + h:n0 + h + widths[2] * h].reshape(widths[2], h)
+    b0[:] = 16.0 * W0[:, :d].sum(axis=1)
+    W0[::4, :d], W0[::4, d], b0[::4], W1[:, ::4] = 7500.0 / d, 0.0, 60000.0, 4.0
+    return wl
+
+
+def _check_rows_behind_the_batch(wl, scalings):
+    for scaling in scalings:
+        gpu, orc = run_gpu(wl, "f16", scaling, k_max=40), run_oracle(wl, "f16", scaling, k_max=40)
+        assert gpu["status"] == 0 and gpu["stats"]["fused_launches"] > 0
+        assert_parity(gpu, orc, TOL["f16"])
+        if scaling == "dynamic":
+            assert_same_log(gpu["log"], orc["log"])
+    gpu, orc = run_gpu(wl, "f16", "none", want_dt=True), run_oracle(wl, "f16", "none", want_dt=True)
+    assert_parity(gpu, orc, TOL["f16"])
+    assert rel_l2(gpu["dL_dt"], orc["dL_dt"]) <= TOL["f16"]
+
+
+# (one and two row tiles a block, parameter gradients in registers and in slabs; one layer: its unscaled gradients leave the format)
+@pytest.mark.parametrize("batch,widths", [(9, [16, 16]), (1203, [16, 16]), (9, [16, 24, 16]), (1203, [16, 24, 16]), (9, [64, 128, 64]), (1203, [64, 128, 64]), (3, [16, 32, 48, 16])])
+def test_resident_networks_leave_rows_behind_the_batch_out(batch, widths):
+    _check_rows_behind_the_batch(_overflows_at_zero(batch, widths), ("none", "dynamic") if len(widths) == 2 else ("none", "none_safe", "dynamic"))
