@@ -618,8 +618,9 @@ __global__ void __launch_bounds__(kThreads + 32, 1) small_backward_kernel(const 
         if (p.recompute) {
             const T* tn = traj + ((long long)n * p.B + r0) * d;
             for (int i = threadIdx.x; i < R * dp; i += kThreads) {
-                const int r = i / dp, c = i - r * dp;
-                sm.yb[i] = r0 + r < p.B && c < d ? tn[r * d + c] : Low<T>::from_f(0.f);
+                // (rows behind the batch follow the last one with zero adjoint: from y = 0 they could overflow where no sample does)
+                const int r = i / dp, c = i - r * dp, row = r0 + r < p.B ? r : p.B - 1 - r0;
+                sm.yb[i] = c < d ? tn[row * d + c] : Low<T>::from_f(0.f);
             }
             work_sync();
             small_stages<T, MT, true>(p, ring, sm, sc, r0, s, !want_t);

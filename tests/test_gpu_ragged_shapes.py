@@ -299,3 +299,8 @@ def _check_rows_behind_the_batch(wl, scalings):
 @pytest.mark.parametrize("batch,widths", [(9, [16, 16]), (1203, [16, 16]), (9, [16, 24, 16]), (1203, [16, 24, 16]), (9, [64, 128, 64]), (1203, [64, 128, 64]), (3, [16, 32, 48, 16])])
 def test_resident_networks_leave_rows_behind_the_batch_out(batch, widths):
     _check_rows_behind_the_batch(_overflows_at_zero(batch, widths), ("none", "dynamic") if len(widths) == 2 else ("none", "none_safe", "dynamic"))
+
+
+# (the streaming kernels, 128 K weights: the extra rows' stage derivatives meet zero adjoints in the time terms)
+def test_streaming_networks_leave_rows_behind_the_batch_out():
+    _check_rows_behind_the_batch(_overflows_at_zero(17, [128, 256, 256, 128]), ("none", "none_safe", "dynamic"))
