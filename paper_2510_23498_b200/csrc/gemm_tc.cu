@@ -570,25 +570,40 @@ bool launch_gemm_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lon
 }
 
 // ---------------------------------------------------------------- weight gradient
-// How the reduction range is sliced so that tiles x slices fills the SMs (few waves, little partial-sum traffic).  Short reductions (up to 2048
-// rows) of which tiles of 256 columns are a quarter of the SMs at most get tiles of 64: four times the blocks, each with a quarter of the
-// epilogue, which is then most of the time (1024 x 1024 gradient of 1024 rows 27 -> 9.6 us; the flow 63-1024-1024-63 8.3 -> 7.2 ms a
-// pass).  Longer ones are cut into slices instead (784 x 2048 of 4096 rows: narrower tiles 31 us, two slices of 256 columns 26 and 5 for their sum).
+// Tile width and slices of the reduction, so that tiles x slices fills the SMs (few waves, little partial-sum traffic).
+// Tiles are as wide as the output lets them be (256, 128, 64 columns), unless it has a quarter of the SMs' tiles of 128 x 256 at most and the
+// reduction either is short, up to 16 k-blocks (1024 rows), or up to 32 k-blocks and not sliced with wide tiles: then 64 columns, more blocks with
+// a shorter epilogue each.  Adding to an output of 1 MB or more in place is most of the time of wide tiles.  us a gradient, 64 columns / wide tiles (sliced: s):
+//   rows           1024           1536           2048
+//   128 x 128      7.4 / 10.2     8.8 / 7.4 s    10.3 / 8.0 s
+//   512 x 192      7.4 / 10.5     9.0 / 12.5     10.4 / 7.5 s
+//   128 x 1024     7.4 / 9.5 s    8.9 / 9.8 s    10.3 / 10.1 s
+//   64 x 1024      6.5 / 7.5 s    8.2 / 7.8 s    9.6 / 8.2 s
+//   512 x 1024     7.5 / 25.2     9.1 / 27.5     10.5 / 11.3 s
+// (sliced wide tiles and 64 columns cross between 16 and 32 k-blocks, for most shapes near 24; none of 400 shapes is slower than with wide tiles.)
+// The line at a quarter of the SMs is not where the two cross: 784 x 2048 of 1024 rows, 56 tiles, 11.5 / 25.6.
 static void wgrad_plan(int M, int N, int K, int* bn_out, int* splits_out, int* kb_per_split_out) {
     const int tiles256 = ((M + BM - 1) / BM) * ((N + 255) / 256), sms = sm_count(), kb_total = (K + BK - 1) / BK;
-    const int bn = kb_total <= 32 && 4 * tiles256 <= sms ? 64 : N >= 256 ? 256 : (N >= 128 ? 128 : 64);
-    const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
     // estimated time in microseconds: waves of work items at ~0.5 us per k-block of a 128 x 256 tile, plus (with more
     // than one slice) the pass that reads the slices back and adds them
-    int best = 1;
-    double best_t = 1e30;
-    for (int s = 1; s <= 16 && s <= kb_total; ++s) {
-        int work = tiles * s;
-        int waves = (work + sms - 1) / sms;
-        int per_s = (kb_total + s - 1) / s;
-        double t = (double)waves * per_s * 0.5 * bn / 256.0;
-        if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
-        if (t < best_t) { best_t = t; best = s; }
+    auto slices = [&](int bn) {
+        const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+        int best = 1;
+        double best_t = 1e30;
+        for (int s = 1; s <= 16 && s <= kb_total; ++s) {
+            int work = tiles * s;
+            int waves = (work + sms - 1) / sms;
+            int per_s = (kb_total + s - 1) / s;
+            double t = (double)waves * per_s * 0.5 * bn / 256.0;
+            if (s > 1) t += (double)(s + 2) * M * N * 4.0 / 3.0e6 + 5.0;
+            if (t < best_t) { best_t = t; best = s; }
+        }
+        return best;
+    };
+    int bn = N >= 256 ? 256 : (N >= 128 ? 128 : 64), best = slices(bn);
+    if (4 * tiles256 <= sms && (kb_total <= 16 || (kb_total <= 32 && best == 1))) {
+        bn = 64;
+        best = slices(bn);
     }
     int per = (kb_total + best - 1) / best;
     *bn_out = bn;

@@ -304,3 +304,11 @@ def test_resident_networks_leave_rows_behind_the_batch_out(batch, widths):
 # (the streaming kernels, 128 K weights: the extra rows' stage derivatives meet zero adjoints in the time terms)
 def test_streaming_networks_leave_rows_behind_the_batch_out():
     _check_rows_behind_the_batch(_overflows_at_zero(17, [128, 256, 256, 128]), ("none", "none_safe", "dynamic"))
+
+
+# weight gradients of the flow on both sides of the line between tiles of 64 columns and wider ones cut into slices: 16 and 17 k-blocks, outputs
+# 256 columns and more wide and between 128 and 255
+@pytest.mark.parametrize("batch,hidden", [(512, 264), (544, 264), (512, 136), (544, 136), (1024, 264)])
+def test_flow_weight_gradient_tile_widths(batch, hidden):
+    wl = inputs.cnf_mlp(batch=batch, n_steps=1, d=16, hidden=hidden)
+    assert_parity(run_gpu(wl, low="bf16"), run_oracle(wl, low="bf16"), TOL["bf16"])
