@@ -225,34 +225,52 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     Sums<T> acc, tot;
     acc.zero();
     if (kTotal) tot.zero();
-    const int in_full = p.wr[l] + (time ? 1 : 0);
-    auto param_of = [&](int r, int c) -> long long {
-        const int m = m0 + r, n = n0 + c;
-        if (m >= p.wr[l + 1]) return -1;
-        if (c < kTile) return n < p.wr[l] ? p.woff[l] + (long long)m * in_full + n : -1;
-        if (c == kTile) return sums && p.bias ? p.boff[l] + m : -1;
-        return sums && time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1;
-    };
+    // The entries of the piece that exist, mr rows of nc columns and the sums behind them: what of them this thread meets, adds and stores.  (All of the
+    // piece, 17 entries a thread one after the other, each with a read of the output of its own, was 8 us for a single block.)
+    const int in_full = p.wr[l] + (time ? 1 : 0), mr = min(kTile, p.wr[l + 1] - m0), nc = min(kTile, p.wr[l] - n0), cols = nc + (sums ? 2 : 0), entries = mr * cols;
     const uint32_t red_u = smem_u32(red);
+    auto all_sync = [&]() { if (S == 1) __syncthreads(); else cluster_sync(); };
     // the groups' sums meet in the block's own shared memory first: a word of another block's takes some 400 cycles
     auto meet = [&](const Sums<T>& w) {
         w.put(red);
         __syncthreads();
-        for (int i = threadIdx.x; i < kTile * kRedRow; i += kThreads) {
+        for (int i = threadIdx.x; i < mr * kRedRow; i += kThreads) {
             float v = red[i];
 #pragma unroll
             for (int g = 1; g < G::Groups; ++g) v += red[g * kTile * kRedRow + i];
             red[i] = v;
         }
-        cluster_sync();
+        all_sync();
     };
-    auto cluster_sum = [&](int r, int c) {
+    auto cluster_sum = [&](int at) {
+        if (S == 1) return red[at];
         float v[kMaxCluster], x = 0.f;
 #pragma unroll
-        for (int z = 0; z < kMaxCluster; ++z) v[z] = z < S ? lds_of(red_u + (uint32_t)(r * kRedRow + c) * 4u, z) : 0.f;
+        for (int z = 0; z < kMaxCluster; ++z) v[z] = z < S ? lds_of(red_u + (uint32_t)at * 4u, z) : 0.f;
 #pragma unroll
         for (int z = 0; z < kMaxCluster; ++z) x += v[z];
         return x;
+    };
+    // finish(parameter, beta times its gradient so far, the cluster's sum) for this thread's entries, four at a time
+    auto each_entry = [&](float beta, auto&& finish) {
+        const int step = kThreads * S;
+        for (int first = (int)threadIdx.x + kThreads * rank; first < entries; first += 4 * step) {
+            long long at[4];
+            int in_red[4];
+            float before[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = first + q * step, r = i / cols, c = i - r * cols, m = m0 + r;
+                in_red[q] = r * kRedRow + (c < nc ? c : kTile + c - nc);
+                at[q] = c < nc ? p.woff[l] + (long long)m * in_full + n0 + c
+                      : c == nc ? (p.bias ? p.boff[l] + m : -1) : (time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1);
+                if (i >= entries) at[q] = -1;
+                before[q] = at[q] >= 0 && beta != 0.f ? beta * p.out[at[q]] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (at[q] >= 0) finish(at[q], before[q], cluster_sum(in_red[q]));
+        }
     };
     bool bad = false;
     for (int k = 0; k < kStages - 1; ++k) fetch();
@@ -273,16 +291,12 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
         if (CHECK || !kTotal) {
             meet(acc);
-            const float cf = p.coef[s], beta = s == 0 ? p.beta : 1.f;
-            for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
-                const int r = i / (kTile + 2), c = i - r * (kTile + 2);
-                const long long at = param_of(r, c);
-                if (at < 0) continue;
-                const float v = cluster_sum(r, c);
+            const float cf = p.coef[s];
+            each_entry(kTotal ? 0.f : s == 0 ? p.beta : 1.f, [&](long long at, float before, float v) {
                 if (CHECK) bad |= Low<T>::nonfinite(Low<T>::from_f(v));
-                if (!kTotal) p.out[at] = fmaf(cf, v, beta != 0.f ? beta * p.out[at] : 0.f);
-            }
-            cluster_sync();      // (no block goes on, or ends, while another reads its sums)
+                if (!kTotal) p.out[at] = fmaf(cf, v, before);
+            });
+            all_sync();      // (no block goes on, or ends, while another reads its sums)
         }
         if (kTotal) tot.add(p.coef[s], acc);
         acc.zero();
@@ -290,12 +304,8 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     asm volatile("cp.async.wait_all;" ::: "memory");
     if (kTotal) {
         meet(tot);
-        for (int i = (int)threadIdx.x + kThreads * rank; i < kTile * (kTile + 2); i += kThreads * S) {
-            const int r = i / (kTile + 2), c = i - r * (kTile + 2);
-            const long long at = param_of(r, c);
-            if (at >= 0) p.out[at] = (p.beta != 0.f ? p.beta * p.out[at] : 0.f) + cluster_sum(r, c);
-        }
-        cluster_sync();
+        each_entry(p.beta, [&](long long at, float before, float v) { p.out[at] = before + v; });
+        all_sync();
     }
     if (CHECK) warp_flag_or(p.flag, bad);
 }
