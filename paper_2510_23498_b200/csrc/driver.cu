@@ -397,6 +397,7 @@ mpode_status mpode_forward(mpode_ctx* c, void* cuda_stream, const float* theta_d
         }
     }
     c->v->prepare(st, ws, theta_dev, probe_dev, L);                                         // Q16(theta)
+    c->v->pack_ahead(st, ws, false, L);
     launch_init_state(dt, y0_dev, yT_dev, traj_dev, c->B, c->d, c->D, st, L);                // y <- x, traj[0]
     // the whole loop in one persistent launch where the velocity has a fused kernel, else layer by layer
     FusedSolve fs = fused_solve(c, yT_dev);
@@ -547,6 +548,7 @@ static mpode_status run_backward(mpode_ctx* c, Velocity* v, const Layout& lay, v
                           sstate, mirror, st, L);
     }
     v->prepare(st, ws, c->theta, c->probe, L);                                            // weights in low precision
+    v->pack_ahead(st, ws, true, L);
     // fused kernels (one recompute launch per step, one VJP launch per attempt) where the velocity has them
     FusedSolve fs = fused_solve(c, nullptr);
     const bool fused = v->fused_backward_begin(st, ws, fs, L);

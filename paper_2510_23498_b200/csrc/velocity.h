@@ -77,6 +77,8 @@ public:
     virtual void plan(Layout& lay) = 0;
     // Q16(theta) into the workspace (and any per-pass constants such as the probe in low format)
     virtual void prepare(cudaStream_t st, void* ws, const float* theta, const signed char* probe, long long* L) = 0;
+    // weights in a form that only one direction's kernels read (right behind prepare)
+    virtual void pack_ahead(cudaStream_t, void*, bool /*backward*/, long long*) {}
     // k_j = f(tau_j, Y_j): reads the stage input, writes kbuf[j] (and klbuf[j]); keeps the layer outputs of stage j
     virtual void forward(cudaStream_t st, void* ws, int j, const void* yin, float tau16, long long* L) = 0;
     // (psi_j, dtheta_j) = VJP of stage j with the cotangent in the kappa buffer; dg = beta * dg + dtheta_j
