@@ -40,10 +40,6 @@ template <typename T> __device__ __forceinline__ T high_of(typename Pair<T>::W w
 }
 template <typename T> __device__ __forceinline__ float lo_w(typename Pair<T>::W w) { return lowf(low_of<T>(w)); }
 template <typename T> __device__ __forceinline__ float hi_w(typename Pair<T>::W w) { return lowf(high_of<T>(w)); }
-// |v| at or above this is not finite in the format
-template <typename T> __device__ __forceinline__ float low_limit() {
-    if constexpr (sizeof(T) == 4) return INFINITY; else return OverflowLimit<T>::value();
-}
 // rows of a block: 16 per row tile of the matrix instructions; float32 runs on the CUDA cores with 8
 template <typename T, int MT> constexpr int kRows = (sizeof(T) == 4 ? 8 : 16) * MT;
 

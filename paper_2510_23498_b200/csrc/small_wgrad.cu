@@ -5,29 +5,34 @@
 // memory, added in a fixed order.  The bias gradient and the time column are two more columns (ones, stage times) of the pieces in the
 // first column of pieces.  CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of
 // the step's gradient that does not fit the format raises the flag.
-// Measured (before: pieces of 32 x 32 or 16 x 16 a block, float32 a launch per layer): 72-200-200-72, 4000 rows, float16 24 -> 15 us; 64-256-256-64, 4096
-// rows, float32 115 -> 45 us (403 M multiply-adds, 11 us at full rate).
-// What bounds it is the rows' way from the L2 (16 KB a stage at about 64 bytes a cycle and SM) and the fill of the ring.  16-bit formats multiply
-// with mma.sync.  float32 holds 8 x 8 sums a thread and reads four 16-byte words for 64 multiply-adds.
+// Measured, us a launch (pieces of 32 x 32 or 16 x 16 a block, float32 a launch per layer and step): 72-200-200-72, 4000 rows 14.4 (35), four such steps
+// checked 55 (142); 64-64, two steps of 4096 rows 18.9 (57); 64-256-256-64, 4096 rows, float32 45 (111; 403 M multiply-adds, 11 us at full rate).  Few
+// rows: 200-200-200, 64 rows 6.5 (5.7); 120-392-120, 360 rows 6.9 (7.7); 128-256-128, 16 steps of 64 rows, checked 33 (31); 32-40-32, 5 steps of
+// 180 rows, checked 19.9 (15.6); 152-312-64-200-152, 2 steps of 237 rows, checked 13.4 (12.9).
+// What bounds it is the rows' way from the L2 (16 KB a stage at about 64 bytes a cycle and SM), the fill of the ring, and with few rows the
+// meeting of the sums.  16-bit formats multiply with mma.sync.  float32 holds 8 x 8 sums a thread and reads four 16-byte words for 64
+// multiply-adds.
 #include "small_mlp.h"
 
 #include "profiler.h"
 #include "tc_ptx.cuh"
 #include "tensormap.h"
 
+#include <type_traits>
+
 namespace mpode {
 using namespace tc;
 namespace {
 
 constexpr int kThreads = 256, kTile = 64, kMaxCluster = 8;
-constexpr int kRedRow = kTile + 3;                  // 64 columns, bias, time (odd stride)
 template <typename T> struct Geo {
     static constexpr int E = 16 / sizeof(T), Pieces = kTile / E, Rows = 512 / Pieces;      // elements of 16 bytes; rows of a stage
     static constexpr int LD = sizeof(T) == 4 ? kTile : kTile + 8;                          // (eight 16-bit rows hit eight 16-byte slots)
     static constexpr int Groups = sizeof(T) == 4 ? 4 : 2;                                  // threads' groups that share out a stage's rows
     static constexpr int Stages = sizeof(T) == 4 ? 6 : 4, Blocks = sizeof(T) == 4 ? 1 : 2;  // of the ring; blocks that share an SM
     static constexpr int StageBytes = 2 * Rows * LD * (int)sizeof(T);
-    static constexpr int Smem = Stages * StageBytes + Groups * kTile * kRedRow * 4;
+    static constexpr int GroupThreads = kThreads / Groups, Quads = sizeof(T) == 4 ? 20 : 10;      // of a group; sums of a thread, in fours
+    static constexpr int Smem = Stages * StageBytes + Groups * Quads * GroupThreads * 16;
 };
 
 struct Items { int first[SMALL_MAX_L + 1]; int S; };
@@ -50,11 +55,11 @@ __device__ __forceinline__ void copy16(uint32_t dst, const void* src, bool on) {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
-__device__ __forceinline__ float lds_of(uint32_t addr, int rank) {      // a word of another block's shared memory
+__device__ __forceinline__ float4 lds_of(uint32_t addr, int rank) {      // 16 bytes of another block's shared memory
     uint32_t a;
-    float v;
+    float4 v;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
     return v;
 }
 
@@ -109,20 +114,27 @@ template <typename T> struct Sums {
             }
         }
     }
-    __device__ __forceinline__ void put(float* red) const {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m0 = (warp & 1) * 32, n0 = ((warp >> 1) & 1) * 32;
-        red += (warp >> 2) * kTile * kRedRow;
+    // The sums in fours, as they lie in the registers: four f of thread t of a group at [f][t].  (Rows of the piece instead took three times as
+    // long to meet: scattered words, and an index worked out for each.)
+    __device__ __forceinline__ void put(float4* red) const {
+        red += (threadIdx.x >> 7) * 10 * 128 + (threadIdx.x & 127);
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < 2; ++m) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float* row = red + (m0 + m * 16 + (lane >> 2) + (i >> 1) * 8) * kRedRow;
-                const int c = 2 * (lane & 3) + (i & 1);
-#pragma unroll
-                for (int n = 0; n < 4; ++n) row[n0 + n * 8 + c] = w[m][n][i];
-                if (n0 == 0 && c < 2) row[kTile + c] = s[m][i];
-            }
+            for (int n = 0; n < 4; ++n) red[(m * 4 + n) * 128] = make_float4(w[m][n][0], w[m][n][1], w[m][n][2], w[m][n][3]);
+            red[(8 + m) * 128] = make_float4(s[m][0], s[m][1], s[m][2], s[m][3]);
+        }
     }
+    // where word i of four f of thread t goes: row r + 8 (i / 2), column c + i % 2; or, f >= 8, the bias (i even) and time column of that row
+    static __device__ __forceinline__ bool place(int f, int t, int& r, int& c) {      // whether it is one of the sums
+        const int warp = t >> 5, lane = t & 31, n0 = (warp >> 1) * 32;
+        r = (warp & 1) * 32 + (lane >> 2) + (f < 8 ? f >> 2 : f - 8) * 16;
+        c = f < 8 ? n0 + (f & 3) * 8 + 2 * (lane & 3) : n0 + (lane & 3);      // (of the sums: those of column 0)
+        return f >= 8;
+    }
+    static constexpr __device__ int row(int i, bool) { return 8 * (i >> 1); }
+    static constexpr __device__ int col(int i) { return i & 1; }
+    static constexpr __device__ bool time(int, int i) { return i & 1; }
 };
 // float32: a group of 64 threads has the whole piece, 8 x 8 a thread (two by two squares of 4), and every fourth of the stage's rows
 template <> struct Sums<float> {
@@ -167,17 +179,25 @@ template <> struct Sums<float> {
             }
         }
     }
-    __device__ __forceinline__ void put(float* red) const {
-        const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
-        red += (threadIdx.x >> 6) * kTile * kRedRow;
+    __device__ __forceinline__ void put(float4* red) const {
+        red += (threadIdx.x >> 6) * 20 * 64 + (threadIdx.x & 63);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float* row = red + (ty * 4 + (i & 3) + (i >> 2) * 32) * kRedRow;
+        for (int f = 0; f < 16; ++f) red[f * 64] = make_float4(w[f >> 1][4 * (f & 1)], w[f >> 1][4 * (f & 1) + 1], w[f >> 1][4 * (f & 1) + 2], w[f >> 1][4 * (f & 1) + 3]);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) row[tx * 4 + (j & 3) + (j >> 2) * 32] = w[i][j];
-            if (tx == 0) { row[kTile] = b[i]; row[kTile + 1] = t[i]; }
+        for (int h = 0; h < 2; ++h) {
+            red[(16 + h) * 64] = make_float4(b[4 * h], b[4 * h + 1], b[4 * h + 2], b[4 * h + 3]);
+            red[(18 + h) * 64] = make_float4(t[4 * h], t[4 * h + 1], t[4 * h + 2], t[4 * h + 3]);
         }
     }
+    static __device__ __forceinline__ bool place(int f, int t, int& r, int& c) {
+        const int tx = t & 7, ty = t >> 3;
+        r = ty * 4 + (f < 16 ? ((f >> 1) & 3) + (f >> 3) * 32 : (f & 1) * 32);
+        c = f < 16 ? tx * 4 + (f & 1) * 32 : tx;
+        return f >= 16;
+    }
+    static constexpr __device__ int row(int i, bool sum) { return sum ? i : 0; }
+    static constexpr __device__ int col(int i) { return i; }
+    static __device__ __forceinline__ bool time(int f, int) { return f >= 18; }
 };
 
 template <typename T, bool CHECK>
@@ -199,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     const T* Z = (const T*)p.zs[l + 1];
     const T* X = (const T*)p.xs[l];
     const uint32_t ring = smem_u32(smem);
-    float* red = (float*)(smem + kStages * G::StageBytes);
+    float4* red = (float4*)(smem + kStages * G::StageBytes);
     // this thread's four pieces of 16 bytes of a stage: row, column, operand are the same for every stage
     int fs = 0, fi = 0, fslot = 0;
     auto fetch = [&]() {
@@ -225,54 +245,122 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     Sums<T> acc, tot;
     acc.zero();
     if (kTotal) tot.zero();
-    // The entries of the piece that exist, mr rows of nc columns and the sums behind them: what of them this thread meets, adds and stores.  (All of the
-    // piece, 17 entries a thread one after the other, each with a read of the output of its own, was 8 us for a single block.)
-    const int in_full = p.wr[l] + (time ? 1 : 0), mr = min(kTile, p.wr[l + 1] - m0), nc = min(kTile, p.wr[l] - n0), cols = nc + (sums ? 2 : 0), entries = mr * cols;
+    const int in_full = p.wr[l] + (time ? 1 : 0), mr = min(kTile, p.wr[l + 1] - m0), nc = min(kTile, p.wr[l] - n0);
+    const int w_at = (int)p.woff[l] + m0 * in_full + n0, b_at = p.bias && sums ? (int)p.boff[l] + m0 : -1, t_at = time && sums ? (int)p.woff[l] + m0 * in_full + p.wr[l] : -1;
     const uint32_t red_u = smem_u32(red);
+    const int t = (int)threadIdx.x % G::GroupThreads;
     auto all_sync = [&]() { if (S == 1) __syncthreads(); else cluster_sync(); };
-    // the groups' sums meet in the block's own shared memory first: a word of another block's takes some 400 cycles
-    auto meet = [&](const Sums<T>& w) {
-        w.put(red);
-        __syncthreads();
-        for (int i = threadIdx.x; i < mr * kRedRow; i += kThreads) {
-            float v = red[i];
+    // The groups' and the blocks' sums meet in fours; each thread of the cluster takes up to kMine.  What a thread does here is a chain of single
+    // instructions, some five cycles each with two warps a scheduler: the parameters' places are worked out once a launch.
+    constexpr int kMine = G::Quads / G::Groups;
+    const int f0 = (int)threadIdx.x / G::GroupThreads + G::Groups * rank, step = G::Groups * S;
+    auto places = [&](int f, int (&at)[4]) {      // the parameters of four f, or -1
+        int r, c;
+        const bool sum = Sums<T>::place(f, t, r, c), on = f < G::Quads;
 #pragma unroll
-            for (int g = 1; g < G::Groups; ++g) v += red[g * kTile * kRedRow + i];
-            red[i] = v;
+        for (int i = 0; i < 4; ++i) {
+            const int ri = r + Sums<T>::row(i, sum);
+            const bool tm = Sums<T>::time(f, i);
+            at[i] = !on || ri >= mr ? -1
+                  : !sum ? (c + Sums<T>::col(i) < nc ? w_at + ri * in_full + c + Sums<T>::col(i) : -1)
+                  : c != 0 ? -1 : tm ? (t_at >= 0 ? t_at + ri * in_full : -1) : (b_at >= 0 ? b_at + ri : -1);
+        }
+    };
+    uint32_t mine_on = 0u;      // bit 4 u + i: word i of this thread's u-th four is a parameter's
+    if (CHECK) {
+#pragma unroll 1
+        for (int u = 0; u < kMine; ++u) {
+            int at[4];
+            places(f0 + u * step, at);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mine_on |= (at[i] >= 0 ? 1u : 0u) << (4 * u + i);
+        }
+    }
+    // before the blocks': the groups' sums, so that a four is one read of each block
+    auto own_sums = [&]() {
+        if (S == 1) return;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kMine; ++u) {
+            float4* q = red + u * kThreads + threadIdx.x;
+            float4 v = *q;
+#pragma unroll
+            for (int g = 1; g < G::Groups; ++g) { const float4 o = q[g * G::Quads * G::GroupThreads]; v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
+            *q = v;
+        }
+    };
+    auto sum_of = [&](int f, float (&v)[4], auto at_once) {      // groups first, then blocks, in ascending order; words of how many blocks in flight
+        v[0] = v[1] = v[2] = v[3] = 0.f;
+        auto take = [&](auto sets, auto&& word) {
+            float4 q[decltype(sets)::value];
+#pragma unroll
+            for (int g = 0; g < decltype(sets)::value; ++g) q[g] = word((g * G::Quads + f) * G::GroupThreads + t);
+#pragma unroll
+            for (int g = 1; g < decltype(sets)::value; ++g) { q[0].x += q[g].x; q[0].y += q[g].y; q[0].z += q[g].z; q[0].w += q[g].w; }
+            v[0] += q[0].x; v[1] += q[0].y; v[2] += q[0].z; v[3] += q[0].w;
+        };
+        if (S == 1) { take(std::integral_constant<int, G::Groups>(), [&](int w) { return red[w]; }); return; }
+#pragma unroll(decltype(at_once)::value)
+        for (int z = 0; z < S; ++z) take(std::integral_constant<int, 1>(), [&](int w) { return lds_of(red_u + (uint32_t)w * 16u, z); });
+    };
+    // whether this warp's part of the piece has any entry (float32: every thread's has)
+    const int part = (int)threadIdx.x >> 5;
+    const bool live = !kTotal || ((part & 1) * 32 < mr && (part >> 1 & 1) * 32 < nc);
+    bool bad = false;
+    auto check = [&](const Sums<T>& w) {      // a step's gradient, before the factor h / S
+        w.put(red);
+        own_sums();
+        all_sync();
+        auto look = [&](int u) {
+            const uint32_t on = mine_on >> (4 * u) & 15u;
+            if (on == 0u) return;
+            float v[4];
+            sum_of(f0 + u * step, v, std::integral_constant<int, 4>());
+#pragma unroll
+            for (int i = 0; i < 4; ++i) bad |= !(fabsf(v[i]) < low_limit<T>()) && (on >> i & 1u);
+        };
+        if (S == 1) {
+#pragma unroll
+            for (int u = 0; u < kMine; ++u) look(u);
+        } else {
+#pragma unroll 1
+            for (int u = 0; u * step < G::Quads; ++u) look(u);
+        }
+        all_sync();      // (no block goes on, or ends, while another reads its sums)
+    };
+    // out = beta out + cf sum; what is added to is requested before the barrier
+    auto add_to = [&](const Sums<T>& w, float beta, float cf) {
+        w.put(red);
+        int at[kMine][4];
+        float before[kMine][4];
+#pragma unroll
+        for (int u = 0; u < kMine; ++u) {
+            at[u][0] = at[u][1] = at[u][2] = at[u][3] = -1;
+            if (u * step >= G::Quads) continue;
+            places(f0 + u * step, at[u]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) before[u][i] = at[u][i] >= 0 && beta != 0.f ? beta * p.out[at[u][i]] : 0.f;
+        }
+        own_sums();
+        all_sync();
+#pragma unroll
+        for (int u = 0; u < kMine; ++u) {
+            if (u * step >= G::Quads) break;
+            bool any = false;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) any |= at[u][i] >= 0;
+            if (!any) continue;
+            float v[4];
+            sum_of(f0 + u * step, v, std::integral_constant<int, kMaxCluster>());
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (at[u][i] >= 0) {
+                    if (CHECK && !kTotal) bad |= !(fabsf(v[i]) < low_limit<T>());
+                    p.out[at[u][i]] = kTotal ? before[u][i] + v[i] : fmaf(cf, v[i], before[u][i]);
+                }
         }
         all_sync();
     };
-    auto cluster_sum = [&](int at) {
-        if (S == 1) return red[at];
-        float v[kMaxCluster], x = 0.f;
-#pragma unroll
-        for (int z = 0; z < kMaxCluster; ++z) v[z] = z < S ? lds_of(red_u + (uint32_t)at * 4u, z) : 0.f;
-#pragma unroll
-        for (int z = 0; z < kMaxCluster; ++z) x += v[z];
-        return x;
-    };
-    // finish(parameter, beta times its gradient so far, the cluster's sum) for this thread's entries, four at a time
-    auto each_entry = [&](float beta, auto&& finish) {
-        const int step = kThreads * S;
-        for (int first = (int)threadIdx.x + kThreads * rank; first < entries; first += 4 * step) {
-            long long at[4];
-            int in_red[4];
-            float before[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = first + q * step, r = i / cols, c = i - r * cols, m = m0 + r;
-                in_red[q] = r * kRedRow + (c < nc ? c : kTile + c - nc);
-                at[q] = c < nc ? p.woff[l] + (long long)m * in_full + n0 + c
-                      : c == nc ? (p.bias ? p.boff[l] + m : -1) : (time ? p.woff[l] + (long long)m * in_full + p.wr[l] : -1);
-                if (i >= entries) at[q] = -1;
-                before[q] = at[q] >= 0 && beta != 0.f ? beta * p.out[at[q]] : 0.f;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (at[q] >= 0) finish(at[q], before[q], cluster_sum(in_red[q]));
-        }
-    };
-    bool bad = false;
     for (int k = 0; k < kStages - 1; ++k) fetch();
     __syncthreads();
     int slot = 0;
@@ -283,30 +371,19 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
             fetch();      // into the stage that every thread has left behind at this barrier
             const int row0 = (rank + S * i) * G::Rows;
             const uint32_t A = ring + (uint32_t)(slot * G::StageBytes);
-            acc.stage(A, A + (uint32_t)(G::Rows * G::LD * sizeof(T)), sums, [&](int k) {
+            if (live) acc.stage(A, A + (uint32_t)(G::Rows * G::LD * sizeof(T)), sums, [&](int k) {
                 const int row = row0 + k;
                 return taus[s][(row >= p.B) + (row >= 2 * p.B) + (row >= 3 * p.B)];      // (rows behind the last are zero)
             });
             if (++slot == kStages) slot = 0;
         }
-        if (CHECK || !kTotal) {
-            meet(acc);
-            const float cf = p.coef[s];
-            each_entry(kTotal ? 0.f : s == 0 ? p.beta : 1.f, [&](long long at, float before, float v) {
-                if (CHECK) bad |= Low<T>::nonfinite(Low<T>::from_f(v));
-                if (!kTotal) p.out[at] = fmaf(cf, v, before);
-            });
-            all_sync();      // (no block goes on, or ends, while another reads its sums)
-        }
+        if (!kTotal) add_to(acc, s == 0 ? p.beta : 1.f, p.coef[s]);
+        else if (CHECK) check(acc);
         if (kTotal) tot.add(p.coef[s], acc);
         acc.zero();
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (kTotal) {
-        meet(tot);
-        each_entry(p.beta, [&](long long at, float before, float v) { p.out[at] = before + v; });
-        all_sync();
-    }
+    if (kTotal) add_to(tot, p.beta, 1.f);
     if (CHECK) warp_flag_or(p.flag, bad);
 }
 
@@ -336,11 +413,11 @@ bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready)
         done[dev] = true;
     }
     if (ready) return true;
-    // the largest cluster of which all pieces' run at once, with two stages of rows for each of its blocks
+    // the largest cluster of which all pieces' run at once, with a stage of rows for each of its blocks
     const int n = items.first[p.L], stages = (p.stages * p.B + Geo<T>::Rows - 1) / Geo<T>::Rows;
     Items it = items;
     it.S = 1;
-    for (int S = 2; S <= kMaxCluster && 2 * S <= stages; ++S)
+    for (int S = 2; S <= kMaxCluster && S <= stages; ++S)
         if (at_once[dev][S] >= n) it.S = S;
     at[0].val.clusterDim.x = (unsigned)it.S;
     cfg.gridDim = dim3((unsigned)(n * it.S));

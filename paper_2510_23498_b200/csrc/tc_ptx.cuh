@@ -237,6 +237,9 @@ template <> __device__ __forceinline__ uint32_t cvt_pack<__nv_bfloat16>(float a,
 template <typename T> struct OverflowLimit;
 template <> struct OverflowLimit<__half> { static __device__ __forceinline__ float value() { return 65520.f; } };
 template <> struct OverflowLimit<__nv_bfloat16> { static __device__ __forceinline__ float value() { return __uint_as_float(0x7F7F8000u); } };
+template <typename T> __device__ __forceinline__ float low_limit() {      // (float32: the limit itself is not finite)
+    if constexpr (sizeof(T) == 4) return INFINITY; else return OverflowLimit<T>::value();
+}
 
 // Whether a rounded value is not finite, noted for two values at once: 0 * Inf and 0 * NaN are NaN, which the sum keeps.  (Comparing
 // every value with the limit, a chain of predicates, was a third of the instructions of an input gradient's epilogue.)
