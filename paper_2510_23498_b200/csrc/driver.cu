@@ -150,6 +150,7 @@ FusedSolve fused_solve(const mpode_ctx* c, float* y) {
 void plan_workspace(const mpode_ctx* c, Velocity* v, Layout& lay) {
     lay.time_gradient = c->pol.time_gradient != 0;
     lay.stepwise = c->pol.scaling == MPODE_SCALE_DYNAMIC;
+    lay.checked = c->pol.scaling != MPODE_SCALE_NONE;
     v->plan(lay);
     if (c->pol.scaling == MPODE_SCALE_DYNAMIC)      // the device-side scale log: exponent, attempts (int each), doubled (byte) per step
         lay.slog = lay.take((size_t)c->max_steps * 9);

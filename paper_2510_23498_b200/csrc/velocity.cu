@@ -182,7 +182,7 @@ public:
         if (small_bwd_ok_) {
             if (lay.time_gradient) {
                 const int blocks = small_blocks(dt_, B_);
-                small_tpart_ = own.take((size_t)SMALL_MAX_CHUNK * (blocks > res_.blocks_b ? blocks : res_.blocks_b) * 3 * sizeof(float));
+                small_tpart_ = own.take((size_t)SMALL_MAX_CHUNK * (res_.backward && res_.blocks_b > blocks ? res_.blocks_b : blocks) * 3 * sizeof(float));
             }
             size_t per_step = 0;
             for (int l = 0; l < L_; ++l) per_step += (size_t)RK_MAX_STAGES * B_ * (small_w_[l] + small_w_[l + 1]) * es;
@@ -192,7 +192,8 @@ public:
             const size_t steps = lay.stepwise ? 1 : room / per_step;
             small_chunk_ = steps < 1 ? 1 : (steps > SMALL_MAX_CHUNK ? SMALL_MAX_CHUNK : (int)steps);
             if (small_chunk_ > max_steps_) small_chunk_ = max_steps_;
-            // (the blocks' parameter gradients, in passes that form them without the slabs)
+            // (the blocks' parameter gradients, in passes that form them without the slabs: those that look at no step's gradient)
+            if (lay.checked) res_.pieces = 0;
             const size_t partial = res_.backward && res_.pieces > 0 ? (size_t)res_.blocks_b * p_ * sizeof(float) : 0;
             Layout sums = own;
             small_partial_ = sums.take(partial);

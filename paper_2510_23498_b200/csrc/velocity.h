@@ -54,6 +54,7 @@ struct Layout {
     // <psi_j, k_l> terms [148], dtau_j [4], c_j [4], {Phi^T a, dt, dh} [4]
     bool time_gradient = false;
     bool stepwise = false;    // dynamic scaling: a pass goes step by step through psi and dg, whatever its path
+    bool checked = false;     // a policy that looks at each step's gradient (dynamic, unscaled-safe)
     size_t tprime = 0, tdots = 0;
     size_t take(size_t bytes) {
         size_t o = total;

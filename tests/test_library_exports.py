@@ -75,6 +75,21 @@ def test_convolutions_of_few_pixels_can_be_created():
         lib.mpode_destroy(h)
 
 
+def test_policies_that_look_at_every_step_plan_no_gradients_of_blocks():
+    # Small dense networks, MB: the buffers of a pass whose weight gradients come from slabs.  The parameter gradients of all blocks, which unscaled
+    # passes add up instead, are up to 0.9 MB more.
+    import ctypes as C
+    from paper_2510_23498_b200 import binding
+    lib = binding.load_library()
+    for scaling, low, batch, ws, steps, mb in (("dynamic", "bf16", 836, [80, 80], 5, 2.49), ("none_safe", "bf16", 602, [23, 88, 23], 30, 1.12), ("dynamic", "f16", 350, [80, 80], 5, 1.11)):
+        widths = (C.c_int * len(ws))(*ws)
+        desc = binding.VelocityDesc(binding.KINDS["mlp"], ws[0], len(ws) - 1, C.cast(widths, C.POINTER(C.c_int)), binding.ACTS["tanh"], 1, 1, 0, 0, 0, 0, 1)
+        h = C.c_void_p()
+        assert lib.mpode_create(C.byref(h), C.byref(desc), batch, steps, C.byref(binding.Policy(binding.DTYPES[low], binding.SCALINGS[scaling], 10, 0, 0, binding.NO_OVERRIDE, 0))) == 0
+        assert lib.mpode_workspace_bytes(h) <= mb * 1e6
+        lib.mpode_destroy(h)
+
+
 def test_a_refused_whole_solve_launch_fails_the_call_and_nothing_else_runs():
     # The hypernetwork flow plans its workspace for the whole-solve kernels alone: where the runtime refuses their launch (here every
     # launch, there is no device) the call fails with a status, and no kernel of another path is queued, for which no buffers exist.
