@@ -68,8 +68,8 @@ def test_tiny_network_variants(batch, d, hidden):
     assert_parity(run_gpu(wl, "f32", "none"), run_oracle(wl, exact=True), TOL["f32"])
 
 
-# row-local kernels of small dense networks: one row, a block's 16 rows less and plus one, two row tiles per block (more than 16 rows per
-# SM), 1 to 4 layers, state widths that are not multiples of 8 or 16, both sizes of gradient pieces, several chunks of steps
+# row-local kernels of small dense networks, weights resident: one row, an odd row, two row tiles of 8 per block (2500: forward, and the other path
+# backward), 1 to 4 layers, state widths that are not multiples of 8 or 16, several chunks of steps
 @pytest.mark.parametrize("batch,widths,n_steps", [(1, [16, 24, 16], 3), (15, [40, 72, 40], 3), (17, [9, 33, 65, 9], 3), (300, [64, 64], 20),
                                                   (200, [72, 200, 200, 72], 2), (2500, [24, 40, 24], 2), (130, [16, 32, 48, 32, 16], 3)])
 def test_small_networks_at_tile_edges(batch, widths, n_steps):
@@ -112,7 +112,7 @@ def test_small_float32_networks_at_tile_edges(batch, widths, n_steps):
 
 
 # unscaled-safe passes of small dense networks: the step's parameter gradient alone leaves the format (its sums run over the batch; the
-# cotangents and the adjoint stay finite), on both sizes of gradient pieces, in one chunk of steps and across chunks, in all formats
+# cotangents and the adjoint stay finite), in one and in several gradient pieces, in one chunk of steps and across chunks, in all formats
 @pytest.mark.parametrize("low,batch,widths,n_steps,size", [("f16", 1000, [64, 128, 64], 2, 100.0), ("f16", 1000, [64, 64], 20, 200.0), ("f16", 700, [72, 200, 200, 72], 2, 300.0),
                                                            ("bf16", 1000, [64, 128, 64], 2, 5e36), ("f32", 1000, [64, 128, 64], 2, 5e36)])
 def test_small_networks_report_a_parameter_gradient_that_overflows(low, batch, widths, n_steps, size):
@@ -312,3 +312,44 @@ def test_streaming_networks_leave_rows_behind_the_batch_out():
 def test_flow_weight_gradient_tile_widths(batch, hidden):
     wl = inputs.cnf_mlp(batch=batch, n_steps=1, d=16, hidden=hidden)
     assert_parity(run_gpu(wl, low="bf16"), run_oracle(wl, low="bf16"), TOL["bf16"])
+
+
+# The resident backward kernel with two row tiles of 8 a block (1185 to 2368 rows on 148 SMs): parameter gradients in registers (one layer and
+# two) and in slabs, with the time terms beside them
+@pytest.mark.parametrize("widths", [[64, 64], [40, 72, 40], [64, 128, 64]])
+@pytest.mark.parametrize("want_dt", [False, True])
+def test_resident_networks_with_two_row_tiles(widths, want_dt):
+    wl = _network(1503, widths, 3)
+    for low, scaling in (("bf16", "none"), ("f16", "dynamic")):
+        gpu, orc = run_gpu(wl, low, scaling, want_dt=want_dt), run_oracle(wl, low, scaling, want_dt=want_dt)
+        assert_parity(gpu, orc, TOL[low])
+        assert gpu["stats"]["fused_launches"] > 0 and gpu["stats"]["simt_contractions"] == 0
+        if want_dt:
+            assert rel_l2(gpu["dL_dt"], orc["dL_dt"]) <= TOL[low]
+
+
+# 16-bit networks whose weights stream (more than fit an SM, up to 160 K): one row, a block's 16 rows less and plus one, several blocks, two row
+# tiles a block (forward; the other path backward); and a network whose forward pass is resident and whose backward pass streams.  Unscaled passes
+# in bfloat16: unscaled float16 cotangents of a mean over 2401 x 128 entries, 2 / 307328 = 6.5e-6, are 109 units of the smallest subnormal, so
+# that their rounding alone, half a unit, is up to 0.5 % of them (measured 0.6 % in dL/dy0), above the format's 2e-3.
+@pytest.mark.parametrize("batch,widths,n_steps", [(1, [128, 256, 256, 128], 2), (15, [128, 256, 256, 128], 2), (17, [128, 256, 256, 128], 2), (200, [128, 256, 256, 128], 3), (2401, [128, 256, 256, 128], 1),
+                                                  (200, [64, 256, 256, 64], 3), (33, [129, 250, 260, 129], 2)])
+def test_streaming_networks_at_tile_edges(batch, widths, n_steps):
+    wl = _network(batch, widths, n_steps)
+    for low, scaling, want_dt in (("bf16", "none", False), ("f16", "dynamic", False), ("bf16", "none_safe", False), ("bf16", "none", True)):
+        gpu, orc = run_gpu(wl, low, scaling, want_dt=want_dt), run_oracle(wl, low, scaling, want_dt=want_dt)
+        assert_parity(gpu, orc, TOL[low])
+        assert gpu["stats"]["fused_launches"] > 0 and gpu["stats"]["simt_contractions"] == 0
+        if scaling == "dynamic":
+            assert_same_log(gpu["log"], orc["log"])
+        if want_dt:
+            assert rel_l2(gpu["dL_dt"], orc["dL_dt"]) <= TOL[low]
+
+
+# instance normalisation by the pixels of a plane: 4 and 16 of them a thread (up to 256 and 1024), read again and again above
+@pytest.mark.parametrize("H,W", [(16, 16), (17, 16), (32, 32), (33, 32)])
+@pytest.mark.parametrize("low", ["bf16", "f16"])
+def test_parabolic_planes_at_register_edges(H, W, low):
+    wl = inputs.parabolic_block(batch=2, n_steps=1, H=H, W=W, C=64, n_intervals=1, low=low, solver="euler")
+    scaling = "dynamic" if low == "f16" else "none"
+    assert_parity(run_gpu(wl, low, scaling), run_oracle(wl, low, scaling), TOL[low])
