@@ -28,6 +28,12 @@ inline bool aligned_to(const void* p, size_t a) { return ((uintptr_t)p % a) == 0
         else if ((dt) == MPODE_F16) { using T = __half; __VA_ARGS__; }       \
         else { using T = float; __VA_ARGS__; }                               \
     } while (0)
+// kernels that only the 16-bit formats have
+#define MPODE_DISPATCH_16(dt, T, ...)                                        \
+    do {                                                                     \
+        if ((dt) == MPODE_BF16) { using T = __nv_bfloat16; __VA_ARGS__; }    \
+        else { using T = __half; __VA_ARGS__; }                              \
+    } while (0)
 
 // ---------------------------------------------------------------- theta -> Q16(theta) (Alg. 1, Alg. 2: weights in low precision)
 // src: fp32 [rows, src_ld] (only the first `cols` columns are taken); dst: low [rp, cp]; dst_t: low [cp, rp], zero beyond [rows, cols].
@@ -1417,9 +1423,9 @@ void launch_instnorm_fwd(mpode_dtype dt, const void* S, void* Z, float* rstd, in
                          long long* launches) {
     if (dt != MPODE_F32 && C % 64 == 0 && aligned_to(S, 16) && aligned_to(Z, 16)) {
         dim3 grid8(C / 64, B);
-        if (HW <= 4 * kNorm8Lanes) MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_fwd8_kernel<T, 4>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
-        else if (HW <= 16 * kNorm8Lanes) MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_fwd8_kernel<T, 16>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
-        else MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_fwd8_long_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
+        if (HW <= 4 * kNorm8Lanes) MPODE_DISPATCH_16(dt, T, (launch_chain(instnorm_fwd8_kernel<T, 4>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
+        else if (HW <= 16 * kNorm8Lanes) MPODE_DISPATCH_16(dt, T, (launch_chain(instnorm_fwd8_kernel<T, 16>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
+        else MPODE_DISPATCH_16(dt, T, (launch_chain(instnorm_fwd8_long_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)S, (T*)Z, rstd, HW, C, eps)));
         COUNT(launches);
         return;
     }
@@ -1432,7 +1438,7 @@ void launch_instnorm_bwd(mpode_dtype dt, const void* dZ, const void* Z, const vo
                          int act, int norm, unsigned* flag, cudaStream_t st, long long* launches) {
     if (dt != MPODE_F32 && C % 64 == 0 && aligned_to(dZ, 16) && aligned_to(Z, 16) && aligned_to(S, 16) && aligned_to(dU, 16)) {
         dim3 grid8(C / 64, B);
-        MPODE_DISPATCH_T(dt, T, (launch_chain(instnorm_bwd8_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU,
+        MPODE_DISPATCH_16(dt, T, (launch_chain(instnorm_bwd8_kernel<T>, dim3(grid8), dim3(kNorm8Threads), 0, st, (const T*)dZ, (const T*)Z, (const T*)S, rstd, (T*)dU,
                                                                                             HW, C, act, norm, flag)));
         COUNT(launches);
         return;

@@ -63,7 +63,7 @@ struct TcParams {
     // at the tap's offset (out-of-image pixels read as zero)
     int conv, conv_h, conv_w, conv_c;   // conv_c: channels of the image (a multiple of 64; a k-block is 64 channels of one tap)
     const float* tbias;         // EPI_FWD with conv: [9][N] bias table per position class
-    int direct; float beta;     // weight gradient with one slice: write out = beta * out + acc directly (2: rows on 32-byte boundaries)
+    int direct; float beta;     // weight gradient with one slice and rows on 32-byte boundaries: write out = beta * out + acc directly
     // flow with a trace estimate: a tile is 64 primal rows and the 64 tangent rows m_split further down (GemmArgs::cnf_pair)
     int pair; void* pair_out; const void* uprev;
 };
@@ -277,15 +277,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     // and nothing else is waited for, are as fast with one 16-byte piece after the other: 2048 x 2048 gradient of 4096 rows 33 us
                     // against 35.)
                     const float* orow32 = (const float*)p.out + (long long)m * p.ldo + n0 + c * 32;
-                    if (p.direct == 2) {      // rows on 32-byte boundaries: whole sectors
 #pragma unroll
-                        for (int v = 0; v < 4; ++v)
-                            if (n0 + c * 32 + v * 8 < p.N) ld_v8(orow32 + v * 8, bl + 8 * v);
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < 8; ++v)
-                            if (n0 + c * 32 + v * 4 < p.N) reinterpret_cast<float4*>(bl)[v] = *reinterpret_cast<const float4*>(orow32 + v * 4);
-                    }
+                    for (int v = 0; v < 4; ++v)
+                        if (n0 + c * 32 + v * 8 < p.N) ld_v8(orow32 + v * 8, bl + 8 * v);
                 }
                 if (!WG && row_ok && n0 + c * 32 < p.N) {
                     if (p.epi == EPI_DGRAD) load_h_chunk<T>(hrow, n0 + c * 32, p.N, hv);
@@ -302,7 +296,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 tmem_ld_32x32(tcol + (uint32_t)(c * 32), r);
                 const int nb = n0 + c * 32;
                 if (WG && p.direct) {
-                    // one reduction slice and an output whose rows are 16-byte aligned: out = beta * out + acc without scratch
+                    // one reduction slice and an output whose rows are 32-byte aligned: out = beta * out + acc without scratch
                     if (row_ok && nb < p.N) {
                         float* orow32 = (float*)p.out + (long long)m * p.ldo + nb;
                         if (BN < 256 && p.beta != 0.f) {
@@ -322,14 +316,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                     *reinterpret_cast<float4*>(orow32 + v * 4) = o;
                                 }
                             }
-                        } else if (p.direct == 2) {
+                        } else {
 #pragma unroll
                             for (int v = 0; v < 4; ++v)
                                 if (nb + v * 8 < p.N) st_v8(orow32 + v * 8, r + 8 * v);
-                        } else {
-#pragma unroll
-                            for (int v = 0; v < 8; ++v)
-                                if (nb + v * 4 < p.N) *reinterpret_cast<uint4*>(orow32 + v * 4) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
                         }
                     }
                 } else if (WG) {
@@ -638,8 +628,9 @@ bool launch_wgrad_tc(mpode_dtype dt, const GemmArgs& g, cudaStream_t st, long lo
     TcParams p{};
     p.M = g.M; p.N = g.N; p.K = g.K; p.epi = EPI_WGRAD; p.err = g.err;
     p.splits = splits; p.kb_per_split = per; p.partial = g.partial;
-    p.direct = splits == 1 && (g.crop_m == 0 || (g.crop_m == g.M && g.crop_n == g.N)) && g.ldo % 4 == 0 && (((uintptr_t)g.out) & 15) == 0;
-    if (p.direct && g.ldo % 8 == 0 && (((uintptr_t)g.out) & 31) == 0) p.direct = 2;
+    // (the callers' outputs are parts of the step gradient in the workspace: where widths are multiples of 8 its rows are on 32-byte boundaries, but
+    // for a first layer with a time column)
+    p.direct = splits == 1 && (g.crop_m == 0 || (g.crop_m == g.M && g.crop_n == g.N)) && g.ldo % 8 == 0 && (((uintptr_t)g.out) & 31) == 0;
     p.out = g.out; p.ldo = g.ldo; p.beta = g.beta;
     bool ok;
     if (dt == MPODE_BF16) {

@@ -37,40 +37,6 @@ inline int chain_warps(int L, const int* wp) {
 template <typename T> __device__ __forceinline__ float lo_of(uint32_t w) { return Low<T>::to_f(from_bits<T>((unsigned short)(w & 0xFFFFu))); }
 template <typename T> __device__ __forceinline__ float hi_of(uint32_t w) { return Low<T>::to_f(from_bits<T>((unsigned short)(w >> 16))); }
 
-template <typename T> __device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
-template <> __device__ __forceinline__ void mma_k16<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-template <> __device__ __forceinline__ void mma_k16<__nv_bfloat16>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-template <typename T> __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0);
-template <> __device__ __forceinline__ void mma_k8<__half>(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
-}
-template <> __device__ __forceinline__ void mma_k8<__nv_bfloat16>(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
-}
-__device__ __forceinline__ void ldm4(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldm4_t(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldm2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void stm2_t(uint32_t addr, uint32_t r0, uint32_t r1) {
-    asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};" ::"r"(addr), "r"(r0), "r"(r1) : "memory");
-}
-__device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <typename T> __device__ __forceinline__ float act16(int act, float z) {
     switch (act) {
@@ -1293,9 +1259,12 @@ bool backward_t(const ResidentMlp& p, cudaStream_t st, bool ready) {
     if (p.s.L == 1 && p.s.wp[0] <= 128) {
         const int w = image_width(1, p.s.wp[0]);
         bool ok = true;
-        if (p.s.tpart == nullptr)
+        if (p.s.tpart == nullptr) {
             ok = w == 32 ? backward_t<T, MT, 8, REG, 2>(p, st, ready) : w == 64 ? backward_t<T, MT, 8, REG, 4>(p, st, ready)
-               : w == 96 ? backward_t<T, MT, 8, REG, 6>(p, st, ready) : backward_t<T, MT, 8, REG, 8>(p, st, ready);
+               : w == 96 ? backward_t<T, MT, 8, REG, 6>(p, st, ready) : false;
+            if constexpr (!REG)      // (97 wide and more have 91 pieces at least, and registers hold 64)
+                if (w == 128) ok = backward_t<T, MT, 8, REG, 8>(p, st, ready);
+        }
         if (p.s.tpart == nullptr && !ready) return ok;
         return ok && backward_t<T, MT, 8, REG, 0>(p, st, ready);      // the time terms are in the general code
     }
@@ -1348,7 +1317,7 @@ ResidentPlan plan_resident(mpode_dtype dt, int B, int L, const int* wp, bool bia
 
 void launch_resident_pack(mpode_dtype dt, const ResidentMlp& p, cudaStream_t st, long long* launches) {
     int blocks = (p.g.w_elems + 255) / 256;
-    if (blocks > 148 * 4) blocks = 148 * 4;
+    if (blocks > sm_count() * 4) blocks = sm_count() * 4;
     if (dt == MPODE_BF16) launch_chain(resident_pack_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, p);
     else launch_chain(resident_pack_kernel<__half>, dim3(blocks), dim3(256), 0, st, p);
     if (launches) ++*launches;

@@ -43,6 +43,8 @@ template <typename T> __device__ __forceinline__ float hi_w(typename Pair<T>::W 
 // rows of a block: 16 per row tile of the matrix instructions; float32 runs on the CUDA cores with 8
 template <typename T, int MT> constexpr int kRows = (sizeof(T) == 4 ? 8 : 16) * MT;
 
+
+// (mma_k16 kept where it is written, between the ring's waits: moved freely, passes were 1 to 2 % slower)
 template <typename T> __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
 template <> __device__ __forceinline__ void mma16816<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -52,10 +54,6 @@ template <> __device__ __forceinline__ void mma16816<__nv_bfloat16>(float (&d)[4
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-
 template <typename T> __device__ __forceinline__ float act_f(int act, float z) {
     if constexpr (sizeof(T) == 4) return act_fwd(act, z);
     switch (act) {
@@ -223,8 +221,8 @@ __device__ __forceinline__ void rows_gemm(Ring& ring, const T* A, int lda, int k
             uint32_t a[MT][2][4];
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
-                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32) * 2), a[m][0]);
-                ldmatrix4(a0 + (uint32_t)((m * 16 * lda + k * 32 + 16) * 2), a[m][1]);
+                ldm4(a0 + (uint32_t)((m * 16 * lda + k * 32) * 2), a[m][0]);
+                ldm4(a0 + (uint32_t)((m * 16 * lda + k * 32 + 16) * 2), a[m][1]);
             }
             ring_wait(ring);
             const uint4* W = (const uint4*)ring.stage() + warp * 32 + lane;
@@ -312,7 +310,7 @@ __device__ __forceinline__ void fetch_scalars(const SmallMlp& p, const SmallSmem
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(sm.scs + (n & 1) * kScalarWords + threadIdx.x)), "l"(src) : "memory");
     }
 }
-__device__ __forceinline__ void scalars_ready() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void scalars_ready() { copies_done(); }
 
 // float32 on the CUDA cores: a lane has four columns and all the block's rows, and a quarter of each unit's 16 reduction steps (8 lanes side
 // by side share a quarter): 12 shared-memory reads of 16 bytes for 128 multiply-adds (16 rows: 20 for 256).  (One column a thread was 12 reads,
