@@ -278,10 +278,11 @@ public:
         packed_ = 0;
         if (!small_ok_) quantize(st, ws, L);      // (the row-local kernels' form when they run, this one only if a pass turns out to need it)
     }
-    // Queued before anything else of the pass, in the form that its kernels are going to ask for: the GPU packs while the host queues what comes
-    // before them (packed when they ask, a pass took 4 to 12 us more).
+    // The streamed form (up to 640 KB) is queued before anything else of the pass: the GPU packs while the host queues what comes before its kernels
+    // (packed when they ask, a pass took 4 to 12 us more).  The resident form is packed when asked for, right in front of its kernel, which
+    // is launched meanwhile: ahead of the pass that took 1 us more.
     void pack_ahead(cudaStream_t st, void* ws, bool backward, long long* L) override {
-        if (small_ok_ && (small_bwd_ok_ || !backward)) pack((backward ? res_.backward : res_.forward) ? 2 : 1, small_params(ws), st, L);
+        if (small_ok_ && (backward ? small_bwd_ok_ && !res_.backward : !res_.forward)) pack(1, small_params(ws), st, L);
     }
     // the weights as the row-local kernels read them: 1 streamed, 2 resident
     void pack(int form, const SmallMlp& p, cudaStream_t st, long long* L) {
