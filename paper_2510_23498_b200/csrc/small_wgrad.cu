@@ -5,10 +5,10 @@
 // memory, added in a fixed order.  The bias gradient and the time column are two more columns (ones, stage times) of the pieces in the
 // first column of pieces.  CHECK (a policy that looks for overflow): the sums meet once per step, before the factor h / S, and an entry of
 // the step's gradient that does not fit the format raises the flag.
-// Measured, us a launch (pieces of 32 x 32 or 16 x 16 a block, float32 a launch per layer and step): 72-200-200-72, 4000 rows 14.4 (35), four such steps
-// checked 55 (142); 64-64, two steps of 4096 rows 18.9 (57); 64-256-256-64, 4096 rows, float32 45 (111; 403 M multiply-adds, 11 us at full rate).  Few
-// rows: 200-200-200, 64 rows 6.5 (5.7); 120-392-120, 360 rows 6.9 (7.7); 128-256-128, 16 steps of 64 rows, checked 33 (31); 32-40-32, 5 steps of
-// 180 rows, checked 19.9 (15.6); 152-312-64-200-152, 2 steps of 237 rows, checked 13.4 (12.9).
+// Measured, us a launch (pieces of 32 x 32 or 16 x 16 a block, float32 a launch per layer and step): 72-200-200-72, 4000 rows 13.9 (35), four such steps
+// checked 53 (142); 64-64, two steps of 4096 rows 18.0 (57); 64-256-256-64, 4096 rows, float32 43 (111; 403 M multiply-adds, 11 us at full rate);
+// 56-56, 11 steps of 46 rows, float32 30 (131).  Few rows: 120-392-120, 360 rows 6.9 (7.7); 128-256-128, 16 steps of 64 rows, checked 34 (31);
+// 32-40-32, 5 steps of 180 rows, checked 20 (15.6); 152-312-64-200-152, 2 steps of 237 rows, checked 14.3 (13.0).
 // What bounds it is the rows' way from the L2 (16 KB a stage at about 64 bytes a cycle and SM), the fill of the ring, and with few rows the
 // meeting of the sums.  16-bit formats multiply with mma.sync.  float32 holds 8 x 8 sums a thread and reads four 16-byte words for 64
 // multiply-adds.
@@ -101,7 +101,7 @@ template <typename T> struct Sums {
     }
     // The sums in fours, as they lie in the registers: four f of thread t of a group at [f][t].  (Rows of the piece instead took three times as
     // long to meet: scattered words, and an index worked out for each.)
-    __device__ __forceinline__ void put(float4* red) const {
+    __device__ __forceinline__ void put(float4* red, int, int, float = 1.f, bool = false) const {
         red += (threadIdx.x >> 7) * 10 * 128 + (threadIdx.x & 127);
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
@@ -164,15 +164,20 @@ template <> struct Sums<float> {
             }
         }
     }
-    __device__ __forceinline__ void put(float4* red) const {
+    // red = (or, with `add`, +=) k times the sums that lie in the piece; a thread's own words
+    __device__ __forceinline__ void put(float4* red, int rows, int cols, float k = 1.f, bool add = false) const {
+        const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
         red += (threadIdx.x >> 6) * 20 * 64 + (threadIdx.x & 63);
+        auto one = [&](int f, const float* v) {
+            const float4 o = add ? red[f * 64] : make_float4(0.f, 0.f, 0.f, 0.f);
+            red[f * 64] = make_float4(fmaf(k, v[0], o.x), fmaf(k, v[1], o.y), fmaf(k, v[2], o.z), fmaf(k, v[3], o.w));
+        };
 #pragma unroll
-        for (int f = 0; f < 16; ++f) red[f * 64] = make_float4(w[f >> 1][4 * (f & 1)], w[f >> 1][4 * (f & 1) + 1], w[f >> 1][4 * (f & 1) + 2], w[f >> 1][4 * (f & 1) + 3]);
+        for (int f = 0; f < 16; ++f)
+            if (ty * 4 + (f >> 3) * 32 < rows && tx * 4 + (f & 1) * 32 < cols) one(f, &w[f >> 1][4 * (f & 1)]);
+        if (tx != 0) return;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            red[(16 + h) * 64] = make_float4(b[4 * h], b[4 * h + 1], b[4 * h + 2], b[4 * h + 3]);
-            red[(18 + h) * 64] = make_float4(t[4 * h], t[4 * h + 1], t[4 * h + 2], t[4 * h + 3]);
-        }
+        for (int h = 0; h < 2; ++h) { one(16 + h, b + 4 * h); one(18 + h, t + 4 * h); }
     }
     static __device__ __forceinline__ bool place(int f, int t, int& r, int& c) {
         const int tx = t & 7, ty = t >> 3;
@@ -225,13 +230,15 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // A second set of sums holds what earlier steps gave.  float32 has no registers for it: its steps meet one by one, in memory.
-    constexpr bool kTotal = sizeof(T) == 2;
+    // What earlier steps gave: a second set of sums; in float32, which has no registers for it, the words that the sums meet in.  Checked float32
+    // passes need those for each step's sums: their steps meet one by one, in memory.
+    constexpr bool kTotal = sizeof(T) == 2, kBySteps = !kTotal && CHECK;
     Sums<T> acc, tot;
     acc.zero();
     if (kTotal) tot.zero();
-    const int in_full = p.wr[l] + (time ? 1 : 0), mr = min(kTile, p.wr[l + 1] - m0), nc = min(kTile, p.wr[l] - n0);
-    const int w_at = (int)p.woff[l] + m0 * in_full + n0, b_at = p.bias && sums ? (int)p.boff[l] + m0 : -1, t_at = time && sums ? (int)p.woff[l] + m0 * in_full + p.wr[l] : -1;
+    // the piece's rows and columns (worked out where they are used: no registers for them in the loop over the rows)
+    auto rows_in = [&]() { return min(kTile, p.wr[l + 1] - m0); };
+    auto cols_in = [&]() { return min(kTile, p.wr[l] - n0); };
     const uint32_t red_u = smem_u32(red);
     const int t = (int)threadIdx.x % G::GroupThreads;
     auto all_sync = [&]() { if (S == 1) __syncthreads(); else cluster_sync(); };
@@ -240,6 +247,8 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     constexpr int kMine = G::Quads / G::Groups;
     const int f0 = (int)threadIdx.x / G::GroupThreads + G::Groups * rank, step = G::Groups * S;
     auto places = [&](int f, int (&at)[4]) {      // the parameters of four f, or -1
+        const int in_full = p.wr[l] + (time ? 1 : 0), mr = rows_in(), nc = cols_in();
+        const int w_at = (int)p.woff[l] + m0 * in_full + n0, b_at = p.bias && sums ? (int)p.boff[l] + m0 : -1, t_at = time && sums ? (int)p.woff[l] + m0 * in_full + p.wr[l] : -1;
         int r, c;
         const bool sum = Sums<T>::place(f, t, r, c), on = f < G::Quads;
 #pragma unroll
@@ -265,14 +274,22 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     auto own_sums = [&]() {
         if (S == 1) return;
         __syncthreads();
+        const int mr = rows_in(), nc = cols_in();
+        float4 v[kMine];
 #pragma unroll
         for (int u = 0; u < kMine; ++u) {
-            float4* q = red + u * kThreads + threadIdx.x;
-            float4 v = *q;
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!kTotal) {
+                int r, c;
+                if (Sums<T>::place(u * G::Groups + (int)threadIdx.x / G::GroupThreads, t, r, c) ? c != 0 || !sums : r >= mr || c >= nc) continue;
+            }
+            const float4* q = red + u * kThreads + threadIdx.x;
+            v[u] = *q;
 #pragma unroll
-            for (int g = 1; g < G::Groups; ++g) { const float4 o = q[g * G::Quads * G::GroupThreads]; v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
-            *q = v;
+            for (int g = 1; g < G::Groups; ++g) { const float4 o = q[g * G::Quads * G::GroupThreads]; v[u].x += o.x; v[u].y += o.y; v[u].z += o.z; v[u].w += o.w; }
         }
+#pragma unroll
+        for (int u = 0; u < kMine; ++u) red[u * kThreads + threadIdx.x] = v[u];
     };
     auto sum_of = [&](int f, float (&v)[4], auto at_once) {      // groups first, then blocks, in ascending order; words of how many blocks in flight
         v[0] = v[1] = v[2] = v[3] = 0.f;
@@ -288,12 +305,9 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
 #pragma unroll(decltype(at_once)::value)
         for (int z = 0; z < S; ++z) take(std::integral_constant<int, 1>(), [&](int w) { return lds_of(red_u + (uint32_t)w * 16u, z); });
     };
-    // whether this warp's part of the piece has any entry (float32: every thread's has)
-    const int part = (int)threadIdx.x >> 5;
-    const bool live = !kTotal || ((part & 1) * 32 < mr && (part >> 1 & 1) * 32 < nc);
     bool bad = false;
     auto check = [&](const Sums<T>& w) {      // a step's gradient, before the factor h / S
-        w.put(red);
+        w.put(red, rows_in(), cols_in());
         own_sums();
         all_sync();
         auto look = [&](int u) {
@@ -313,9 +327,8 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
         all_sync();      // (no block goes on, or ends, while another reads its sums)
     };
-    // out = beta out + cf sum; what is added to is requested before the barrier
-    auto add_to = [&](const Sums<T>& w, float beta, float cf) {
-        w.put(red);
+    // out = beta out + cf times the sum of the words put; what is added to is requested before the barrier
+    auto add_to = [&](float beta, float cf) {
         int at[kMine][4];
         float before[kMine][4];
 #pragma unroll
@@ -340,8 +353,8 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (at[u][i] >= 0) {
-                    if (CHECK && !kTotal) bad |= !(fabsf(v[i]) < low_limit<T>());
-                    p.out[at[u][i]] = kTotal ? before[u][i] + v[i] : fmaf(cf, v[i], before[u][i]);
+                    if (kBySteps) bad |= !(fabsf(v[i]) < low_limit<T>());
+                    p.out[at[u][i]] = kBySteps ? fmaf(cf, v[i], before[u][i]) : before[u][i] + v[i];
                 }
         }
         all_sync();
@@ -356,19 +369,21 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
             fetch();      // into the stage that every thread has left behind at this barrier
             const int row0 = (rank + S * i) * G::Rows;
             const uint32_t A = ring + (uint32_t)(slot * G::StageBytes);
-            if (live) acc.stage(A, A + (uint32_t)(G::Rows * G::LD * sizeof(T)), sums, [&](int k) {
+            acc.stage(A, A + (uint32_t)(G::Rows * G::LD * sizeof(T)), sums, [&](int k) {
                 const int row = row0 + k;
                 return taus[s][(row >= p.B) + (row >= 2 * p.B) + (row >= 3 * p.B)];      // (rows behind the last are zero)
             });
             if (++slot == kStages) slot = 0;
         }
-        if (!kTotal) add_to(acc, s == 0 ? p.beta : 1.f, p.coef[s]);
-        else if (CHECK) check(acc);
+        if (CHECK && kTotal) check(acc);
         if (kTotal) tot.add(p.coef[s], acc);
+        else acc.put(red, rows_in(), cols_in(), kBySteps ? 1.f : p.coef[s], !kBySteps && s > 0);
+        if (kBySteps) add_to(s == 0 ? p.beta : 1.f, p.coef[s]);
         acc.zero();
     }
     copies_done();
-    if (kTotal) add_to(tot, p.beta, 1.f);
+    if (kTotal) tot.put(red, 0, 0);
+    if (!kBySteps) add_to(p.beta, 1.f);
     if (CHECK) warp_flag_or(p.flag, bad);
 }
 
