@@ -190,7 +190,9 @@ template <> struct Sums<float> {
     static __device__ __forceinline__ bool time(int f, int) { return f >= 18; }
 };
 
-template <typename T, bool CHECK>
+// look: 0 at no step's gradient, 1 at each of several, 2 at each as it is added (launches of one step; float32)
+enum { kNo, kEach, kAsAdded };
+template <typename T, int CHECK>
 __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(const __grid_constant__ SmallMlp p, const __grid_constant__ Items items) {
     chain_begin();
     using G = Geo<T>;
@@ -232,7 +234,9 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
     };
     // What earlier steps gave: a second set of sums; in float32, which has no registers for it, the words that the sums meet in.  Checked float32
     // passes need those for each step's sums: their steps meet one by one, in memory.
-    constexpr bool kTotal = sizeof(T) == 2, kBySteps = !kTotal && CHECK;
+    // (Checked 16-bit launches of one step too: the sums meet once instead of twice.)
+    constexpr bool kTotal = sizeof(T) == 2, kBySteps = CHECK == kAsAdded;
+    static_assert(kTotal || CHECK != kEach, "no second set of sums");
     Sums<T> acc, tot;
     acc.zero();
     if (kTotal) tot.zero();
@@ -261,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
     };
     uint32_t mine_on = 0u;      // bit 4 u + i: word i of this thread's u-th four is a parameter's
-    if (CHECK) {
+    if (CHECK == kEach) {
 #pragma unroll 1
         for (int u = 0; u < kMine; ++u) {
             int at[4];
@@ -327,15 +331,20 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
         all_sync();      // (no block goes on, or ends, while another reads its sums)
     };
-    // out = beta out + cf times the sum of the words put; what is added to is requested before the barrier
-    auto add_to = [&](float beta, float cf) {
-        int at[kMine][4];
-        float before[kMine][4];
+    int at[kMine][4];
+    auto find_places = [&]() {
 #pragma unroll
         for (int u = 0; u < kMine; ++u) {
             at[u][0] = at[u][1] = at[u][2] = at[u][3] = -1;
-            if (u * step >= G::Quads) continue;
-            places(f0 + u * step, at[u]);
+            if (u * step < G::Quads) places(f0 + u * step, at[u]);
+        }
+    };
+    // out = beta out + cf times the sum of the words put; what is added to is requested before the barrier
+    auto add_to = [&](float beta, float cf) {
+        float before[kMine][4];
+#pragma unroll
+        for (int u = 0; u < kMine; ++u) {
+            if (u * step >= G::Quads) break;
 #pragma unroll
             for (int i = 0; i < 4; ++i) before[u][i] = at[u][i] >= 0 && beta != 0.f ? beta * p.out[at[u][i]] : 0.f;
         }
@@ -359,6 +368,7 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
         }
         all_sync();
     };
+    if (kBySteps || !kTotal) find_places();      // (while the first rows are on their way; 16-bit loops have no registers for them)
     for (int k = 0; k < kStages - 1; ++k) fetch();
     __syncthreads();
     int slot = 0;
@@ -375,19 +385,25 @@ __global__ void __launch_bounds__(kThreads, Geo<T>::Blocks) small_wgrad_kernel(c
             });
             if (++slot == kStages) slot = 0;
         }
-        if (CHECK && kTotal) check(acc);
-        if (kTotal) tot.add(p.coef[s], acc);
-        else acc.put(red, rows_in(), cols_in(), kBySteps ? 1.f : p.coef[s], !kBySteps && s > 0);
-        if (kBySteps) add_to(s == 0 ? p.beta : 1.f, p.coef[s]);
+        if (kBySteps) {
+            acc.put(red, rows_in(), cols_in());
+            add_to(s == 0 ? p.beta : 1.f, p.coef[s]);
+        } else {
+            if (CHECK == kEach) check(acc);
+            if (kTotal) tot.add(p.coef[s], acc);
+            else acc.put(red, rows_in(), cols_in(), p.coef[s], s > 0);
+        }
         acc.zero();
     }
     copies_done();
-    if (kTotal) tot.put(red, 0, 0);
-    if (!kBySteps) add_to(p.beta, 1.f);
+    if (!kBySteps) {
+        if (kTotal) { tot.put(red, 0, 0); find_places(); }
+        add_to(p.beta, 1.f);
+    }
     if (CHECK) warp_flag_or(p.flag, bad);
 }
 
-template <typename T, bool CHECK>
+template <typename T, int CHECK>
 bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready) {
     static bool done[kMaxDevices] = {false};
     static int at_once[kMaxDevices][kMaxCluster + 1] = {{0}};      // clusters of each size that the GPU holds at once
@@ -425,26 +441,31 @@ bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready)
     return cudaLaunchKernelEx(&cfg, small_wgrad_kernel<T, CHECK>, p, it) == cudaSuccess;
 }
 template <typename T>
-bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st, bool ready, bool check) {
-    return check ? wgrad_t<T, true>(p, items, st, ready) : wgrad_t<T, false>(p, items, st, ready);
+bool wgrad_t(const SmallMlp& p, const Items& items, cudaStream_t st) {
+    if (p.flag == nullptr) return wgrad_t<T, kNo>(p, items, st, false);
+    if constexpr (sizeof(T) == 2)
+        if (p.count > 1) return wgrad_t<T, kEach>(p, items, st, false);
+    return wgrad_t<T, kAsAdded>(p, items, st, false);
+}
+template <typename T>
+bool wgrad_ready(const SmallMlp& p) {
+    if constexpr (sizeof(T) == 2)
+        if (!wgrad_t<T, kEach>(p, Items{}, nullptr, true)) return false;
+    return wgrad_t<T, kNo>(p, Items{}, nullptr, true) && wgrad_t<T, kAsAdded>(p, Items{}, nullptr, true);
 }
 
 }  // namespace
 
 bool small_wgrad_ready(mpode_dtype dt, const SmallMlp& p) {
-    for (int check = 0; check < 2; ++check)
-        if (!(dt == MPODE_BF16  ? wgrad_t<__nv_bfloat16>(p, Items{}, nullptr, true, check != 0)
-              : dt == MPODE_F16 ? wgrad_t<__half>(p, Items{}, nullptr, true, check != 0)
-                                : wgrad_t<float>(p, Items{}, nullptr, true, check != 0))) return false;
-    return true;
+    return dt == MPODE_BF16 ? wgrad_ready<__nv_bfloat16>(p) : dt == MPODE_F16 ? wgrad_ready<__half>(p) : wgrad_ready<float>(p);
 }
 
 void launch_small_wgrad(mpode_dtype dt, const SmallMlp& p, cudaStream_t st, long long* launches) {
     Items it{};
     for (int l = 0; l < p.L; ++l) it.first[l + 1] = it.first[l] + ((p.wp[l + 1] + kTile - 1) / kTile) * ((p.wp[l] + kTile - 1) / kTile);
-    if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, it, st, false, p.flag != nullptr);
-    else if (dt == MPODE_F16) wgrad_t<__half>(p, it, st, false, p.flag != nullptr);
-    else wgrad_t<float>(p, it, st, false, p.flag != nullptr);
+    if (dt == MPODE_BF16) wgrad_t<__nv_bfloat16>(p, it, st);
+    else if (dt == MPODE_F16) wgrad_t<__half>(p, it, st);
+    else wgrad_t<float>(p, it, st);
     if (launches) ++*launches;
     if (tl_counters) {
         if (dt == MPODE_F32) tl_counters->simt += (long long)p.L * p.count;
