@@ -315,7 +315,7 @@ __device__ __forceinline__ void scalars_ready() { copies_done(); }
 // float32 on the CUDA cores: a lane has four columns and all the block's rows, and a quarter of each unit's 16 reduction steps (8 lanes side
 // by side share a quarter): 12 shared-memory reads of 16 bytes for 128 multiply-adds (16 rows: 20 for 256).  (One column a thread was 12 reads,
 // 8 of 16 bytes, for 32, and bound by them.)  A warp covers 32 columns; where the pass has fewer than 256 the warps that are left
-// share out the units, as many of them as there are units (16-16 and narrower: no sums to meet).  The quarters meet by shuffles, each lane keeping a quarter of the rows, the warps' shares in shared memory; sums are
+// share out the units.  The quarters meet by shuffles, each lane keeping a quarter of the rows, the warps' shares in shared memory; sums are
 // added in a fixed order.
 template <int MT, typename P, typename F>
 __device__ __forceinline__ void rows_gemm_f32(Ring& ring, const SmallSmem<float>& sm, const float* A, int K, int N, P&& pre, F&& epi) {
@@ -325,8 +325,8 @@ __device__ __forceinline__ void rows_gemm_f32(Ring& ring, const SmallSmem<float>
         const int cols = min(kPassCols, N - c0);
         int cw = 1;                                               // warps side by side; the others of the 8 take other units
         while (cw * 32 < cols) cw *= 2;
-        const int kw = min(kWarps / cw, (K + 15) / 16), mine = warp / cw, col = (warp % cw) * 32 + (lane & 7) * 4;
-        const bool on = col < cols && mine < kw;                  // (widths are multiples of 8)
+        const int kw = kWarps / cw, mine = warp / cw, col = (warp % cw) * 32 + (lane & 7) * 4;
+        const bool on = col < cols;                               // (widths are multiples of 8)
         const int row0 = (kg >> 1) * (R / 2) + (kg & 1) * Q;      // the rows this lane keeps
         if (kw == 1 && on) {
 #pragma unroll
@@ -395,8 +395,7 @@ __device__ __forceinline__ void rows_gemm_f32(Ring& ring, const SmallSmem<float>
         const int ct = cw * 32;
         if (c0 > 0) work_sync();
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if (mine < kw) *reinterpret_cast<float4*>(sm.scratch + ((size_t)(mine * R + row0 + q) * ct + col)) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
+        for (int q = 0; q < Q; ++q) *reinterpret_cast<float4*>(sm.scratch + ((size_t)(mine * R + row0 + q) * ct + col)) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
         work_sync();
         const int hc = ct / 2;
         for (int i = threadIdx.x; i < R * hc; i += kThreads) {
