@@ -8,7 +8,7 @@
 // beside the ones that carry the chain move layer inputs and cotangents to memory, or, where the parameter gradient fits their registers
 // and no step's gradient has to be looked at, form it on the spot: then a pass of any number of steps is one launch and a sum over blocks.
 // Measured, a layer (before: small_mlp.cu): one layer of 64 1.28 -> 0.29 us, 200-200 2.2 -> 0.94 us; training passes: linear equation 64 wide, 1024
-// samples, 100 RK4 steps 2.97 -> 0.53 ms; MLP 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 4.8 -> 2.2 ms (with small_wgrad.cu).
+// samples, 100 RK4 steps 2.97 -> 0.53 ms; MLP 72-200-200-72, 1000 samples, 16 RK4 steps, float16 dynamic 4.8 -> 2.3 ms (with small_wgrad.cu).
 #include "resident_mlp.h"
 
 #include "profiler.h"
