@@ -44,16 +44,6 @@ template <typename T> __device__ __forceinline__ float hi_w(typename Pair<T>::W 
 template <typename T, int MT> constexpr int kRows = (sizeof(T) == 4 ? 8 : 16) * MT;
 
 
-// (mma_k16 kept where it is written, between the ring's waits: moved freely, passes were 1 to 2 % slower)
-template <typename T> __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1);
-template <> __device__ __forceinline__ void mma16816<__half>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-template <> __device__ __forceinline__ void mma16816<__nv_bfloat16>(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 template <typename T> __device__ __forceinline__ float act_f(int act, float z) {
     if constexpr (sizeof(T) == 4) return act_fwd(act, z);
     switch (act) {
@@ -237,13 +227,13 @@ __device__ __forceinline__ void rows_gemm(Ring& ring, const T* A, int lda, int k
             for (int g = 0; g < kNG; ++g)
                 if (warp + kWarps * g < in_pass) {
 #pragma unroll
-                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][0], b[g].x, b[g].y);
+                    for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m][g], a[m][0], b[g].x, b[g].y);
                 }
 #pragma unroll
             for (int g = 0; g < kNG; ++g)
                 if (warp + kWarps * g < in_pass) {
 #pragma unroll
-                    for (int m = 0; m < MT; ++m) mma16816<T>(acc[m][g], a[m][1], b[g].z, b[g].w);
+                    for (int m = 0; m < MT; ++m) mma_k16<T>(acc[m][g], a[m][1], b[g].z, b[g].w);
                 }
         }
 #pragma unroll
