@@ -353,3 +353,17 @@ def test_parabolic_planes_at_register_edges(H, W, low):
     wl = inputs.parabolic_block(batch=2, n_steps=1, H=H, W=W, C=64, n_intervals=1, low=low, solver="euler")
     scaling = "dynamic" if low == "f16" else "none"
     assert_parity(run_gpu(wl, low, scaling), run_oracle(wl, low, scaling), TOL[low])
+
+
+# weight gradients of unscaled-safe launches of one step, whose check goes with the addition to the output: clusters of one block and of several, and
+# a step's gradient that alone leaves the format (a constant cotangent, summed over the batch: 1000 rows of 100 or 5e36)
+@pytest.mark.parametrize("low,batch,widths,size", [("bf16", 9, [24, 40, 24], 5e36), ("bf16", 1000, [64, 128, 64], 5e36), ("f16", 1000, [72, 200, 200, 72], 300.0), ("f32", 1000, [16, 72, 16], 5e36)])
+def test_weight_gradients_of_one_checked_step(low, batch, widths, size):
+    wl = _network(batch, widths, 1)
+    gpu = run_gpu(wl, low, "none_safe")
+    if low != "f16":        # (unscaled float16 cotangents of a mean over 1000 x 72 entries are 466 units of the smallest subnormal: rounded to 0.1 % each)
+        assert_parity(gpu, run_oracle(wl, exact=True) if low == "f32" else run_oracle(wl, low, "none_safe"), TOL[low])
+    assert gpu["status"] == 0
+    if batch > 9:
+        gpu = run_gpu(wl, low, "none_safe", dLdyT=np.full((batch, widths[0]), size))
+        assert gpu["status"] == 8 and np.all(np.isposinf(gpu["g"])) and np.all(np.isposinf(gpu["a0"]))
